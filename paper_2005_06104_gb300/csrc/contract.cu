@@ -88,7 +88,7 @@ void env_right_fp64(cudaStream_t st, Scratch& s, const cplx* R, const WSparse& W
 
 void LanczosWork::init(DevicePool* pool) {
   c.reset(pool, 128);
-  y.reset(pool, 64);
+  y.reset(pool, 64 * 64);
   if (!real) TDVP_CUDA(cudaMalloc(&real, sizeof(double) * 384));
 }
 
@@ -107,51 +107,50 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
   nmax = std::min(std::max(1, nmax), 63);
   double* alpha = lw.real;
   double* beta = lw.real + 64;
-  double* nrm2 = lw.real + 130;
-  double* err = lw.real + 132;
-  double* errs = lw.real + 256;  // 2 per iteration of a speculative batch
+  double* nrm2 = lw.real + 130;  // |w|^2 and the factor 1 / |w|
+  double* start2 = lw.real + 255;  // |x|^2, read together with the first stopping test
+  double* errs = lw.real + 256;    // 2 per iteration of a batch
   lw.V.ensure(pool, (size_t)(nmax + 1) * n);
   lw.w.ensure(pool, (size_t)n);
   cplx* V = lw.V.data();
   cplx* wv = lw.w.data();
-  blas.norm2(st, x, n, nrm2);
-  double h_n2 = 0.0;
-  TDVP_CUDA(cudaMemcpyAsync(&h_n2, nrm2, sizeof(double), cudaMemcpyDeviceToHost, st));
-  TDVP_CUDA(cudaStreamSynchronize(st));
-  tdvp_require(std::isfinite(h_n2), TDVP_ERR_NONFINITE, "Lanczos: non-finite start vector");
-  const double beta0 = std::sqrt(h_n2);
-  if (beta0 == 0.0) {
-    TDVP_CUDA(cudaMemcpyAsync(out, x, n * sizeof(cplx), cudaMemcpyDeviceToDevice, st));
-    return 0;
-  }
-  scale_by_inv_sqrt(st, V, x, nrm2, n);
-  // A small local problem costs a host round trip per iteration more than its arithmetic.  With
-  // a hint, the first hint - 1 iterations go out in one batch (each next vector scaled with a
-  // guard, so an iteration after an invariant subspace only sees zeros) and their stopping
-  // tests are read together.  A run that stops inside the batch recomputes the small
-  // exponential at its stopping point (the same inputs and kernel, so the same result as
-  // stopping there) and ignores the iterations after it.
+  blas.norm2(st, x, n, start2);
+  scale_by_inv_sqrt(st, V, x, start2, n);
+  double beta0 = 0.0;
+  // A small local problem costs a host round trip per iteration more than its arithmetic: several
+  // iterations go out at once (each next vector scaled with a guard, so an iteration after an
+  // invariant subspace only sees zeros), their small exponentials run side by side in one launch
+  // and their stopping tests are read together.  A run that stops inside the batch takes the
+  // exponential of its stopping point and ignores the iterations after.  The first batch is the
+  // previous run's dimension (runs of one sweep rarely differ), or 4 without one (the time steps
+  // in use need 5 and more); each further batch is 2.
+  const bool small = n <= kSpeculateMaxN;
   int batch = 1;
-  if (hint && *hint > 2 && n <= kSpeculateMaxN)
-    batch = (int)std::min<long long>({(long long)*hint - 1, (long long)nmax, n});
-  int used = 0, last = -1;
+  if (small) batch = (int)std::min<long long>({(long long)(hint && *hint > 1 ? *hint : 4), (long long)nmax, n});
+  int used = 0;
+  const cplx* y = nullptr;  // exp(coef T) e_0 at the stopping point
   double last_err = 0.0;
   for (int j = 0; j < nmax;) {
     const int j0 = j;
     for (int b = 0; b < batch; ++b, ++j) {
-      if (b > 0) scale_by_inv_sqrt_guarded(st, V + (long long)j * n, wv, nrm2, n);
+      if (b > 0) scale_by(st, V + (long long)j * n, wv, nrm2 + 1, n);
       op(V + (long long)j * n, wv);
-      // alpha_j = Re <v_j, w>; w -= V (V^H w), twice (full re-orthogonalisation); beta = |w|
-      blas.lanczos_fused(st, 0, V, n, j + 1, wv, n, nullptr, lw.c.data(), alpha, j, nullptr, nullptr);
-      blas.lanczos_fused(st, 1, V, n, j + 1, wv, n, lw.c.data(), lw.c.data() + 64, nullptr, j, nullptr, nullptr);
-      blas.lanczos_fused(st, 2, V, n, j + 1, wv, n, lw.c.data() + 64, nullptr, nullptr, j, nrm2, beta + j + 1);
-      tridiag_expv(st, alpha, beta, j + 1, delta, kind, nrm2, lw.y.data(), batch > 1 ? errs + 2 * b : err);
+      // alpha_j = Re <v_j, w>, w made orthogonal to V[0..j], beta_{j+1} = |w|
+      blas.lanczos_step(st, V, n, j, wv, lw.c.data(), alpha, beta, nrm2);
     }
-    last = j - 1;
-    double h_err[2 * 64];
-    TDVP_CUDA(cudaMemcpyAsync(h_err, batch > 1 ? errs : err, sizeof(double) * 2 * batch, cudaMemcpyDeviceToHost,
-                              st));
+    tridiag_expv(st, alpha, beta, j0 + 1, batch, delta, kind, lw.y.data(), errs);
+    double h[1 + 2 * 64];
+    TDVP_CUDA(cudaMemcpyAsync(h, start2, sizeof(double) * (1 + 2 * batch), cudaMemcpyDeviceToHost, st));
     TDVP_CUDA(cudaStreamSynchronize(st));
+    const double* h_err = h + 1;
+    if (j0 == 0) {
+      tdvp_require(std::isfinite(h[0]), TDVP_ERR_NONFINITE, "Lanczos: non-finite start vector");
+      beta0 = std::sqrt(h[0]);
+      if (beta0 == 0.0) {
+        TDVP_CUDA(cudaMemcpyAsync(out, x, n * sizeof(cplx), cudaMemcpyDeviceToDevice, st));
+        return 0;
+      }
+    }
     for (int b = 0; b < batch; ++b) {
       const int jj = j0 + b;
       tdvp_require(std::isfinite(h_err[2 * b]) && std::isfinite(h_err[2 * b + 1]), TDVP_ERR_NONFINITE,
@@ -159,19 +158,19 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
       last_err = h_err[2 * b];
       if (h_err[2 * b] <= tol || h_err[2 * b + 1] <= kBreakdown || jj + 1 == n) {
         used = jj + 1;
+        y = lw.y.data() + 64 * b;
         break;
       }
     }
     if (used > 0 || j == nmax) break;
-    scale_by_inv_sqrt(st, V + (long long)j * n, wv, nrm2, n);
-    batch = 1;
+    scale_by(st, V + (long long)j * n, wv, nrm2 + 1, n);
+    if (small) batch = (int)std::min<long long>({2LL, (long long)(nmax - j), n - j});
   }
   if (used == 0)
     throw TdvpError(TDVP_ERR_LANCZOS_NOT_CONVERGED,
                     "Lanczos error estimate " + std::to_string(last_err) + " above tolerance after " +
                         std::to_string(nmax) + " steps");
-  if (used - 1 < last) tridiag_expv(st, alpha, beta, used, delta, kind, nrm2, lw.y.data(), err);
-  multi_combine(st, out, V, n, used, lw.y.data(), beta0, n);
+  multi_combine(st, out, V, n, used, y, beta0, n);
   if (hint) *hint = used;
   return used;
 }

@@ -440,46 +440,35 @@ __global__ void __launch_bounds__(RED_THREADS)
   }
 }
 
-__global__ void k_multi_axpy_sub(cplx* __restrict__ w, const cplx* __restrict__ V, long long ldv,
-                                 int nvec, const cplx* __restrict__ c, long long n) {
-  __shared__ cplx cs[64];
-  for (int k = threadIdx.x; k < nvec && k < 64; k += blockDim.x) cs[k] = c[k];
-  __syncthreads();
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  cplx acc = mkc(0.0, 0.0);
-  for (int k = 0; k < nvec; ++k) cfma(acc, V[(long long)k * ldv + i], cs[k]);
-  w[i] = csub(w[i], acc);
-}
-
 __global__ void k_multi_combine(cplx* __restrict__ y, const cplx* __restrict__ V, long long ldv,
                                 int nvec, const cplx* __restrict__ c, double scale, long long n) {
-  __shared__ cplx cs[64];
+  __shared__ cplx cs[64 + MD_CH];
   for (int k = threadIdx.x; k < nvec && k < 64; k += blockDim.x) cs[k] = c[k];
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   cplx acc = mkc(0.0, 0.0);
-  for (int k = 0; k < nvec; ++k) cfma(acc, V[(long long)k * ldv + i], cs[k]);
+  const unsigned active = __activemask();
+  for (int k0 = 0; k0 < nvec; k0 += MD_CH) {
+    cplx v[MD_CH];
+#pragma unroll
+    for (int q = 0; q < MD_CH; ++q) v[q] = k0 + q < nvec ? V[(long long)(k0 + q) * ldv + i] : mkc(0.0, 0.0);
+    // FP64 bound: entries that are zero in the whole warp (other charge sectors) cost no FMAs
+#pragma unroll
+    for (int q = 0; q < MD_CH; ++q)
+      if (__any_sync(active, v[q].x != 0.0 || v[q].y != 0.0)) cfma(acc, v[q], cs[k0 + q]);
+  }
   y[i] = cscale(acc, scale);
 }
 
+// FP64 division and square root cost tens of FP64 instructions: one thread per block forms the factor
 __global__ void k_scale_inv_sqrt(cplx* __restrict__ dst, const cplx* __restrict__ src,
                                  const double* __restrict__ nrm2, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double s = 1.0 / sqrt(*nrm2);
-  dst[i] = cscale(src[i], s);
-}
-
-// as k_scale_inv_sqrt, but a norm that is not a positive finite number above 1e-200 gives zeros
-__global__ void k_scale_inv_sqrt_guarded(cplx* __restrict__ dst, const cplx* __restrict__ src,
-                                         const double* __restrict__ nrm2, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double q = *nrm2;
-  const double s = (q > 1e-200 && q <= 1.7e308) ? 1.0 / sqrt(q) : 0.0;
-  dst[i] = cscale(src[i], s);
+  __shared__ double s;
+  if (threadIdx.x == 0) s = 1.0 / sqrt(*nrm2);
+  __syncthreads();
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    dst[i] = cscale(src[i], s);
 }
 
 __global__ void k_scale_host(cplx* __restrict__ dst, const cplx* __restrict__ src, cplx s, long long n) {
@@ -488,11 +477,11 @@ __global__ void k_scale_host(cplx* __restrict__ dst, const cplx* __restrict__ sr
   dst[i] = cmul(src[i], s);
 }
 
-__global__ void k_copy_real(const cplx* c, int j, double* alpha) { alpha[j] = c[j].x; }
-__global__ void k_store_beta(const double* nrm2, double* slot) { *slot = sqrt(*nrm2); }
 }  // namespace
 
-static int red_blocks(long long n, int max_blocks);
+static int red_blocks(long long n, int max_blocks) {
+  return std::max(1, std::min<int>(max_blocks, ceil_div(n, RED_THREADS * 4)));
+}
 
 void Blas1::init(DevicePool* p, int sm_count) {
   pool = p;
@@ -515,114 +504,257 @@ void Blas1::release() {
 // partial sums; the last block to finish (atomic ticket, no waiting) reduces
 // them in a fixed order, so results are deterministic and no block spins.
 namespace {
-__device__ __forceinline__ bool last_block(unsigned* counter) {
+__device__ __forceinline__ bool last_block(unsigned* counter, unsigned blocks) {
   __shared__ bool is_last;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
     const unsigned t = atomicAdd(counter, 1u);
-    is_last = (t == gridDim.x - 1);
+    is_last = (t == blocks - 1);
   }
   __syncthreads();
   return is_last;
 }
 
-// mode 0: c = V^H w                        (alpha[j] = Re c[j])
-// mode 1: w -= V cin;  c = V^H w
-// mode 2: w -= V cin;  nrm2 = |w|^2, beta_slot = sqrt(nrm2)
+// One warp sums NC complex accumulators over its 32 lanes.  Halving exchange: while more than one
+// value is left, a lane keeps one half of them and hands the other half to its partner, so 16
+// doubles take 16 FP64 adds per lane instead of 80 (a warp-wide FP64 instruction holds this part's
+// FP64 pipe for 16 cycles, which made the plain butterfly a large share of a short reduction).
+// Value v of the 2 NC doubles ends in the lanes whose top bits spell v; they store it to out[v].
+template <int NC>
+__device__ __forceinline__ void warp_sum_store(const cplx (&acc)[NC], double* out) {
+  constexpr int NV = 2 * NC;
+  double a[NV];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    a[2 * q] = acc[q].x;
+    a[2 * q + 1] = acc[q].y;
+  }
+  const int lane = threadIdx.x & 31;
+  int idx = 0, o = 16;
+#pragma unroll
+  for (int half = NV / 2; half >= 1; half >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int q = 0; q < half; ++q) {
+      const double send = up ? a[q] : a[q + half];
+      const double keep = up ? a[q + half] : a[q];
+      a[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    idx += up ? half : 0;
+  }
+  const int rest = 32 / NV - 1;  // the lane bits that no halving used
+#pragma unroll
+  for (; o >= 1; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+  if ((lane & rest) == 0) out[idx] = a[0];
+}
+
+__device__ __forceinline__ bool warp_nonzero(cplx v) {
+  return __any_sync(0xffffffffu, v.x != 0.0 || v.y != 0.0);
+}
+
+constexpr int TRI_MAX = 64;
+constexpr int CHEB_MAX = 1024;
+
+// The vector work of one Lanczos iteration (w = H v_j on entry): two full projections
+//   c = V^H w, w -= V c, twice (alpha_j = Re c_j of the first), then |w|.
+// Bound: GB300 runs 2 FP64 FMAs per cycle and SM, so a projection pair on j vectors (8 j FMAs per
+// entry) takes 26 ps per entry and vector on FP64 against 7 ps of HBM time: these kernels are FP64
+// bound at every size.  So
+//  - exact zeros cost no FMAs: a conserved charge leaves three quarters or more of a site vector
+//    zero, in runs longer than a warp, and a warp whose entries are all zero skips their
+//    multiply-adds (a skipped term is an exact zero unless v is not finite, which the norm of the
+//    iteration before has reported);
+//  - the reductions halve (warp_sum_store);
+//  - a short vector spreads its dot products over blocks by vector (grid.y) and its updates by
+//    entry, instead of sitting on the n / 1024 SMs that the partial sums need.
+// The sums keep one order whatever the spread: block g of G = n / 1024 (at most 2 per SM) adds the
+// entries g 256 + t, + 256 G, ... per thread t, then lanes, warps and blocks, and the fused
+// multiply-adds are written out, so every variant gives the same bits.  (A sweep of a split form
+// turns a last-bit change into 1e-7 of a site tensor: operand digits round at 2^-33, and a gauge
+// move divides by Schmidt values of 1e-6.)
+// Measured per iteration at n = 2.1e6, 7 vectors, charge-conserving: 0.61 ms -> 0.2 ms; at
+// n = 1.3e5: 60 us -> 25 us.
+
+// c[k] = <v_k, w>, k < nvec, KC vectors per block; alpha (when not null): alpha[j] = Re c[j]
+template <int KC>
 __global__ void __launch_bounds__(RED_THREADS)
-    k_lanczos_fused(int mode, const cplx* __restrict__ V, long long ldv, int nvec, cplx* __restrict__ w, long long n,
-                    const cplx* __restrict__ cin, cplx* __restrict__ cout, double* __restrict__ alpha, int j,
-                    double* __restrict__ nrm2, double* __restrict__ beta_slot, cplx* __restrict__ partial,
-                    unsigned* __restrict__ counter) {
-  __shared__ cplx cs[64];
-  __shared__ cplx red[MD_CH][RED_THREADS / 32];
-  __shared__ double dred[RED_THREADS / 32];
+    k_lanczos_dots(const cplx* __restrict__ V, long long ldv, int nvec, const cplx* __restrict__ w, long long n,
+                   cplx* __restrict__ cout, double* __restrict__ alpha, cplx* __restrict__ partial,
+                   unsigned* __restrict__ counter) {
+  constexpr int W = RED_THREADS / 32;
+  __shared__ double red[W][2 * KC];
   const int G = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (mode >= 1) {
-    for (int k = threadIdx.x; k < nvec; k += blockDim.x) cs[k] = cin[k];
-    __syncthreads();
-    for (long long i = (long long)blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += (long long)G * RED_THREADS) {
-      cplx acc = mkc(0.0, 0.0);
-      for (int k = 0; k < nvec; ++k) cfma(acc, V[(long long)k * ldv + i], cs[k]);
-      w[i] = csub(w[i], acc);
-    }
-    // each thread re-reads only the w[i] it wrote: no block-wide barrier needed
+  const int k0 = blockIdx.y * KC;
+  cplx acc[KC];
+#pragma unroll
+  for (int q = 0; q < KC; ++q) acc[q] = mkc(0.0, 0.0);
+  const long long step = (long long)G * RED_THREADS;
+  for (long long base = (long long)blockIdx.x * RED_THREADS + warp * 32; base < n; base += step) {
+    const long long i = base + lane;
+    const bool in = i < n;
+    const cplx wi = in ? w[i] : mkc(0.0, 0.0);
+    if (!warp_nonzero(wi)) continue;
+#pragma unroll
+    for (int q = 0; q < KC; ++q)
+      if (k0 + q < nvec && in) cfma_conj(acc[q], V[(long long)(k0 + q) * ldv + i], wi);
   }
-  if (mode <= 1) {
-    for (int k0 = 0; k0 < nvec; k0 += MD_CH) {
-      cplx acc[MD_CH];
+  warp_sum_store(acc, red[warp]);
+  __syncthreads();
+  if (threadIdx.x < 2 * KC && k0 + (int)(threadIdx.x >> 1) < nvec) {
+    double t = 0.0;
 #pragma unroll
-      for (int q = 0; q < MD_CH; ++q) acc[q] = mkc(0.0, 0.0);
-      for (long long i = (long long)blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += (long long)G * RED_THREADS) {
-        const cplx wi = w[i];
-#pragma unroll
-        for (int q = 0; q < MD_CH; ++q)
-          if (k0 + q < nvec) cfma_conj(acc[q], V[(long long)(k0 + q) * ldv + i], wi);
+    for (int u = 0; u < W; ++u) t += red[u][threadIdx.x];
+    reinterpret_cast<double*>(partial)[2 * ((long long)(k0 + (threadIdx.x >> 1)) * G + blockIdx.x) +
+                                       (threadIdx.x & 1)] = t;
+  }
+  if (last_block(counter, gridDim.x * gridDim.y)) {
+    for (int k = warp; k < nvec; k += W) {
+      cplx t = mkc(0.0, 0.0);
+      for (int g = lane; g < G; g += 32) t = cadd(t, __ldcg(&partial[(long long)k * G + g]));
+      t = warp_sum(t);
+      if (lane == 0) {
+        cout[k] = t;
+        if (alpha && k == nvec - 1) alpha[k] = t.x;
       }
-#pragma unroll
-      for (int q = 0; q < MD_CH; ++q) {
-        cplx t = warp_sum(acc[q]);
-        if (lane == 0) red[q][warp] = t;
-      }
-      __syncthreads();
-      if (threadIdx.x < MD_CH && k0 + (int)threadIdx.x < nvec) {
-        cplx t = mkc(0.0, 0.0);
-        for (int u = 0; u < RED_THREADS / 32; ++u) t = cadd(t, red[threadIdx.x][u]);
-        partial[(long long)(k0 + threadIdx.x) * G + blockIdx.x] = t;
-      }
-      __syncthreads();
     }
-    if (last_block(counter)) {
-      for (int k = warp; k < nvec; k += RED_THREADS / 32) {
-        cplx t = mkc(0.0, 0.0);
-        for (int g = lane; g < G; g += 32) t = cadd(t, partial[(long long)k * G + g]);
-        t = warp_sum(t);
-        if (lane == 0) {
-          cout[k] = t;
-          if (mode == 0 && k == j) alpha[j] = t.x;
-        }
-      }
-      if (threadIdx.x == 0) *counter = 0;
-    }
-  } else {
-    double a = 0.0;
-    for (long long i = (long long)blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += (long long)G * RED_THREADS)
-      a += cabs2(w[i]);
-    a = warp_sum(a);
-    if (lane == 0) dred[warp] = a;
+    if (threadIdx.x == 0) *counter = 0;
+  }
+}
+
+// w[i] - sum_k c[k] v_k[i] for the entry of each lane; loads of a group are in flight before its tests
+__device__ __forceinline__ cplx lanczos_subtract(const cplx* __restrict__ V, long long ldv, int nvec, const cplx* cs,
+                                                 const cplx* __restrict__ w, long long i, bool in) {
+  cplx sub = mkc(0.0, 0.0);
+  for (int k0 = 0; k0 < nvec; k0 += MD_CH) {
+    cplx v[MD_CH];
+#pragma unroll
+    for (int q = 0; q < MD_CH; ++q)
+      v[q] = in && k0 + q < nvec ? V[(long long)(k0 + q) * ldv + i] : mkc(0.0, 0.0);
+#pragma unroll
+    for (int q = 0; q < MD_CH; ++q)
+      if (k0 + q < nvec && warp_nonzero(v[q])) cfma(sub, v[q], cs[k0 + q]);
+  }
+  return in ? csub(w[i], sub) : mkc(0.0, 0.0);
+}
+
+__global__ void __launch_bounds__(RED_THREADS)
+    k_lanczos_axpy(const cplx* __restrict__ V, long long ldv, int nvec, cplx* __restrict__ w, long long n,
+                   const cplx* __restrict__ c) {
+  __shared__ cplx cs[TRI_MAX];
+  for (int k = threadIdx.x; k < nvec; k += blockDim.x) cs[k] = c[k];
+  __syncthreads();
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const cplx r = lanczos_subtract(V, ldv, nvec, cs, w, i, i < n);
+  if (i < n) w[i] = r;
+}
+
+// (UPDATE: w -= V c, then) nrm2[0] = |w|^2, nrm2[1] = 1 / |w|, *beta = |w|
+template <bool UPDATE>
+__global__ void __launch_bounds__(RED_THREADS)
+    k_lanczos_norm(const cplx* __restrict__ V, long long ldv, int nvec, cplx* __restrict__ w, long long n,
+                   const cplx* __restrict__ c, double* __restrict__ nrm2, double* __restrict__ beta,
+                   double* __restrict__ partial, unsigned* __restrict__ counter) {
+  __shared__ cplx cs[TRI_MAX];
+  __shared__ double dred[RED_THREADS / 32], part[RED_THREADS];
+  const int G = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (UPDATE) {
+    for (int k = threadIdx.x; k < nvec; k += RED_THREADS) cs[k] = c[k];
     __syncthreads();
-    double* dpart = reinterpret_cast<double*>(partial);
+  }
+  double a = 0.0;
+  const long long step = (long long)G * RED_THREADS;
+  for (long long base = (long long)blockIdx.x * RED_THREADS + warp * 32; base < n; base += step) {
+    const long long i = base + lane;
+    const bool in = i < n;
+    cplx wi;
+    if (UPDATE) {
+      wi = lanczos_subtract(V, ldv, nvec, cs, w, i, in);
+      if (in) w[i] = wi;
+    } else {
+      wi = in ? w[i] : mkc(0.0, 0.0);
+    }
+    if (warp_nonzero(wi)) a = __dadd_rn(a, fma(wi.x, wi.x, __dmul_rn(wi.y, wi.y)));
+  }
+  a = warp_sum(a);
+  if (lane == 0) dred[warp] = a;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int u = 0; u < RED_THREADS / 32; ++u) t += dred[u];
+    partial[blockIdx.x] = t;
+  }
+  if (last_block(counter, gridDim.x)) {
+    double t = 0.0;
+    for (int g0 = 0; g0 < G; g0 += RED_THREADS) {
+      __syncthreads();
+      if (g0 + (int)threadIdx.x < G) part[threadIdx.x] = __ldcg(&partial[g0 + threadIdx.x]);
+      __syncthreads();
+      if (threadIdx.x == 0)
+        for (int g = 0; g < min(RED_THREADS, G - g0); ++g) t += part[g];
+    }
     if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int u = 0; u < RED_THREADS / 32; ++u) t += dred[u];
-      dpart[blockIdx.x] = t;
-    }
-    if (last_block(counter)) {
-      if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int g = 0; g < G; ++g) t += dpart[g];
-        *nrm2 = t;
-        *beta_slot = sqrt(t);
-        *counter = 0;
-      }
+      nrm2[0] = t;
+      // the factor of the next basis vector; zero (not NaN) after an invariant subspace, so that
+      // the later iterations of a batch launched ahead see zeros
+      nrm2[1] = (t > 1e-200 && t <= 1.7e308) ? 1.0 / sqrt(t) : 0.0;
+      *beta = sqrt(t);
+      *counter = 0;
     }
   }
+}
+
+// dst = src * *factor
+__global__ void k_scale_by(cplx* __restrict__ dst, const cplx* __restrict__ src, const double* __restrict__ factor,
+                           long long n) {
+  const double s = *factor;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    dst[i] = cscale(src[i], s);
 }
 }  // namespace
 
-void Blas1::lanczos_fused(cudaStream_t st, int mode, const cplx* V, long long ldv, int nvec, cplx* w, long long n,
-                          const cplx* cin, cplx* cout, double* alpha, int j, double* nrm2, double* beta_slot) {
-  tdvp_require(nvec >= 1 && nvec <= 64, TDVP_ERR_INVALID_ARG, "lanczos_fused: nvec out of range");
+void Blas1::lanczos_step(cudaStream_t st, const cplx* V, long long n, int j, cplx* w, cplx* c, double* alpha,
+                         double* beta, double* nrm2) {
+  const int nvec = j + 1;
+  tdvp_require(j >= 0 && nvec < TRI_MAX, TDVP_ERR_INVALID_ARG, "lanczos_step: too many vectors");
   const int G = red_blocks(n, max_blocks);
-  k_lanczos_fused<<<G, RED_THREADS, 0, st>>>(mode, V, ldv, nvec, w, n, cin, cout, alpha, j, nrm2, beta_slot,
-                                             partial.data(), counter);
+  auto dots = [&](cplx* out, double* al) {
+    // vectors per block: 8 share one read of w once the blocks of the sums fill half the device
+    // (FP64 bound either way), fewer below, so that a short vector still reaches every SM
+    if (G * ceil_div(nvec, 8) >= max_blocks / 4)
+      k_lanczos_dots<8><<<dim3(G, ceil_div(nvec, 8)), RED_THREADS, 0, st>>>(V, n, nvec, w, n, out, al, partial.data(),
+                                                                            counter);
+    else if (G * ceil_div(nvec, 2) >= max_blocks / 4)
+      k_lanczos_dots<2><<<dim3(G, ceil_div(nvec, 2)), RED_THREADS, 0, st>>>(V, n, nvec, w, n, out, al, partial.data(),
+                                                                            counter);
+    else
+      k_lanczos_dots<1><<<dim3(G, nvec), RED_THREADS, 0, st>>>(V, n, nvec, w, n, out, al, partial.data(), counter);
+    TDVP_CHECK_LAUNCH();
+  };
+  const int ta = n <= 32LL * 1024 ? 64 : RED_THREADS;
+  dots(c, alpha);
+  k_lanczos_axpy<<<ceil_div(n, ta), ta, 0, st>>>(V, n, nvec, w, n, c);
+  TDVP_CHECK_LAUNCH();
+  dots(c + TRI_MAX, nullptr);
+  double* dpart = reinterpret_cast<double*>(partial.data());
+  // the norm's n / 1024 blocks also do the last update when they fill the device; below that a
+  // launch of its own spreads it (n = 2048, 8 vectors: 8 us on 2 SMs against 1 us and a launch)
+  if (2 * G >= max_blocks) {
+    k_lanczos_norm<true><<<G, RED_THREADS, 0, st>>>(V, n, nvec, w, n, c + TRI_MAX, nrm2, beta + j + 1, dpart, counter);
+  } else {
+    k_lanczos_axpy<<<ceil_div(n, ta), ta, 0, st>>>(V, n, nvec, w, n, c + TRI_MAX);
+    TDVP_CHECK_LAUNCH();
+    k_lanczos_norm<false><<<G, RED_THREADS, 0, st>>>(V, n, nvec, w, n, nullptr, nrm2, beta + j + 1, dpart, counter);
+  }
   TDVP_CHECK_LAUNCH();
 }
 
-static int red_blocks(long long n, int max_blocks) {
-  return std::max(1, std::min<int>(max_blocks, ceil_div(n, RED_THREADS * 4)));
+void scale_by(cudaStream_t st, cplx* dst, const cplx* src, const double* factor, long long n) {
+  if (n == 0) return;
+  k_scale_by<<<(int)std::min<long long>(ceil_div(n, 256), 152 * 8), 256, 0, st>>>(dst, src, factor, n);
+  TDVP_CHECK_LAUNCH();
 }
+
 
 void Blas1::multi_dot(cudaStream_t st, const cplx* V, long long ldv, int nvec, const cplx* w,
                       long long n, cplx* out) {
@@ -643,14 +775,6 @@ void Blas1::norm2(cudaStream_t st, const cplx* x, long long n, double* out) {
   TDVP_CHECK_LAUNCH();
 }
 
-void multi_axpy_sub(cudaStream_t st, cplx* w, const cplx* V, long long ldv, int nvec, const cplx* c,
-                    long long n) {
-  tdvp_require(nvec <= 64, TDVP_ERR_INVALID_ARG, "multi_axpy: nvec > 64");
-  if (n == 0 || nvec == 0) return;
-  k_multi_axpy_sub<<<ceil_div(n, 256), 256, 0, st>>>(w, V, ldv, nvec, c, n);
-  TDVP_CHECK_LAUNCH();
-}
-
 void multi_combine(cudaStream_t st, cplx* y, const cplx* V, long long ldv, int nvec, const cplx* c,
                    double scale, long long n) {
   tdvp_require(nvec <= 64, TDVP_ERR_INVALID_ARG, "multi_combine: nvec > 64");
@@ -661,13 +785,7 @@ void multi_combine(cudaStream_t st, cplx* y, const cplx* V, long long ldv, int n
 
 void scale_by_inv_sqrt(cudaStream_t st, cplx* dst, const cplx* src, const double* nrm2, long long n) {
   if (n == 0) return;
-  k_scale_inv_sqrt<<<ceil_div(n, 256), 256, 0, st>>>(dst, src, nrm2, n);
-  TDVP_CHECK_LAUNCH();
-}
-
-void scale_by_inv_sqrt_guarded(cudaStream_t st, cplx* dst, const cplx* src, const double* nrm2, long long n) {
-  if (n == 0) return;
-  k_scale_inv_sqrt_guarded<<<ceil_div(n, 256), 256, 0, st>>>(dst, src, nrm2, n);
+  k_scale_inv_sqrt<<<(int)std::min<long long>(ceil_div(n, 256), 152 * 8), 256, 0, st>>>(dst, src, nrm2, n);
   TDVP_CHECK_LAUNCH();
 }
 
@@ -681,16 +799,6 @@ void fill_zero(cudaStream_t st, cplx* p, long long n) {
   if (n) TDVP_CUDA(cudaMemsetAsync(p, 0, n * sizeof(cplx), st));
 }
 
-void copy_real_part(cudaStream_t st, const cplx* c, int j, double* alpha) {
-  k_copy_real<<<1, 1, 0, st>>>(c, j, alpha);
-  TDVP_CHECK_LAUNCH();
-}
-
-void store_beta(cudaStream_t st, const double* nrm2, double* slot) {
-  k_store_beta<<<1, 1, 0, st>>>(nrm2, slot);
-  TDVP_CHECK_LAUNCH();
-}
-
 // ============================================================================
 // exp(coef T) e_0 for a small symmetric tridiagonal T (Lanczos matrix).
 //
@@ -701,61 +809,65 @@ void store_beta(cudaStream_t st, const double* nrm2, double* slot) {
 //                              = e^{|delta| hi} sum_k eps_k e^{-x} I_k(x) T_k(X),        delta < 0
 // with x = |delta| h, eps_0 = 1, eps_k = 2.  J_k and e^{-x} I_k come from Miller's
 // backward recurrence normalised by J_0 + 2 sum J_2k = 1 and I_0 + 2 sum I_k = e^x.
-// One block; thread i owns component i (n <= 64).
+// One warp: lane l owns the components l and l + 32 (n <= 63), neighbours by shuffles.
+// Bound: a serial chain of FP64 operations (K + M of them, each waiting for the last).  So the
+// chain holds nothing but its recurrences: the quotients 2 k / x and the divisions by the norm are
+// formed by all lanes beside it, and a single warp needs no block barrier per term (80 us -> 25 us
+// per exponential at n = 10).  Block b takes the leading n0 + b rows: the stopping tests of the
+// iterations of one batch run side by side.
 // ============================================================================
 namespace {
-constexpr int TRI_MAX = 64;
-constexpr int CHEB_MAX = 1024;
-
-__global__ void __launch_bounds__(TRI_MAX)
-    k_tridiag_expv(const double* __restrict__ alpha, const double* __restrict__ beta, int n,
-                   double delta, int kind, const double* __restrict__ nrm2_next,
+__global__ void __launch_bounds__(32)
+    k_tridiag_expv(const double* __restrict__ alpha, const double* __restrict__ beta, int n0, double delta, int kind,
                    cplx* __restrict__ y, double* __restrict__ err) {
-  __shared__ double d[TRI_MAX], o[TRI_MAX + 1];
-  __shared__ double tk[TRI_MAX];
+  constexpr unsigned FULL = 0xffffffffu;
   __shared__ double coef[CHEB_MAX + 1];
-  __shared__ double sh_c, sh_h, sh_lo, sh_hi;
-  __shared__ int sh_K, sh_bad;
-  const int i = threadIdx.x;
-  if (i < n) d[i] = alpha[i];
-  if (i <= n) o[i] = (i >= 1 && i < n) ? beta[i] : 0.0;
-  __syncthreads();
-  if (i == 0) {
-    double lo = 1e300, hi = -1e300;
-    for (int r = 0; r < n; ++r) {
-      const double rad = fabs(o[r]) + fabs(o[r + 1]);
-      lo = fmin(lo, d[r] - rad);
-      hi = fmax(hi, d[r] + rad);
+  const int n = n0 + blockIdx.x;
+  y += (long long)blockIdx.x * TRI_MAX;
+  err += 2 * blockIdx.x;
+  const int lane = threadIdx.x;
+  const bool two = n > 32;  // warp-uniform: components 32.. exist
+  double d[2], ol[2], orr[2];
+  double lo = 1e300, hi = -1e300;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int i = lane + 32 * c;
+    d[c] = i < n ? alpha[i] : 0.0;
+    ol[c] = (i >= 1 && i < n) ? beta[i] : 0.0;
+    orr[c] = (i + 1 < n) ? beta[i + 1] : 0.0;
+    if (i < n) {
+      const double rad = fabs(ol[c]) + fabs(orr[c]);
+      lo = fmin(lo, d[c] - rad);
+      hi = fmax(hi, d[c] + rad);
     }
-    const double c = 0.5 * (hi + lo), h = 0.5 * (hi - lo);
-    sh_c = c;
-    sh_h = h;
-    sh_lo = lo;
-    sh_hi = hi;
-    const double x = fabs(delta) * h;
-    int K = (int)(x + 10.0 * cbrt(x + 1.0) + 40.0);
-    sh_bad = 0;
-    if (K > CHEB_MAX) {
-      K = CHEB_MAX;
-      sh_bad = 1;
-    }
-    sh_K = K;
-    // Miller backward recurrence, start well above K
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(FULL, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(FULL, hi, o));
+  }
+  const double c = 0.5 * (hi + lo), h = 0.5 * (hi - lo);
+  const double x = fabs(delta) * h;
+  int K = (int)(x + 10.0 * cbrt(x + 1.0) + 40.0);
+  const bool bad = K > CHEB_MAX;
+  if (bad) K = CHEB_MAX;
+  for (int k = lane; k <= K; k += 32) coef[k] = 0.0;
+  __syncwarp();
+  if (x < 1e-300) {
+    if (lane == 0) coef[0] = 1.0;
+  } else {
+    // Miller backward recurrence, start well above K; every lane runs it, lane 0 keeps the values
     const int M = 2 * ((K + 40 + (int)x) / 2 + 1);
-    for (int k = 0; k <= K; ++k) coef[k] = 0.0;
-    if (x < 1e-300) {
-      coef[0] = 1.0;
-    } else {
-      double jp1 = 0.0, jk = 1e-280, norm = 0.0;
-      for (int k = M; k >= 1; --k) {
+    double jp1 = 0.0, jk = 1e-280, norm = 0.0;
+    for (int kb = M; kb >= 1; kb -= 32) {
+      const double quot = 2.0 * (double)max(kb - lane, 0) / x;
+      for (int l = 0; l < min(32, kb); ++l) {
+        const int k = kb - l;
         // value at index k is jk, at k+1 is jp1; produce index k-1
-        const double jm1 = (kind == 0) ? (2.0 * k / x) * jk - jp1 : (2.0 * k / x) * jk + jp1;
-        if (k <= K) coef[k] = jk;
-        if (kind == 0) {
-          if ((k & 1) == 0) norm += 2.0 * jk;
-        } else {
-          norm += 2.0 * jk;
-        }
+        const double tk = __shfl_sync(FULL, quot, l);
+        const double jm1 = fma(tk, jk, kind == 0 ? -jp1 : jp1);
+        if (lane == 0 && k <= K) coef[k] = jk;
+        if (kind != 0 || (k & 1) == 0) norm += 2.0 * jk;
         jp1 = jk;
         jk = jm1;
         if (fabs(jk) > 1e250) {  // rescale
@@ -763,81 +875,94 @@ __global__ void __launch_bounds__(TRI_MAX)
           jk *= f;
           jp1 *= f;
           norm *= f;
-          for (int q = k; q <= K; ++q) coef[q] *= f;
+          __syncwarp();
+          for (int q = k + lane; q <= K; q += 32) coef[q] *= f;
+          __syncwarp();
         }
       }
-      coef[0] = jk;
-      norm += jk;
-      for (int k = 0; k <= K; ++k) coef[k] /= norm;
     }
+    if (lane == 0) coef[0] = jk;
+    norm += jk;
+    __syncwarp();
+    for (int k = lane; k <= K; k += 32) coef[k] /= norm;
   }
-  __syncthreads();
-  const int K = sh_K;
-  const double c = sh_c, h = sh_h;
+  __syncwarp();
   const double inv_h = h > 0.0 ? 1.0 / h : 0.0;
-  // scaled matrix X = (T - c) / h
-  const double xd = (i < n) ? (d[i] - c) * inv_h : 0.0;
-  const double xl = (i < n && i >= 1) ? o[i] * inv_h : 0.0;
-  const double xr = (i + 1 < n) ? o[i + 1] * inv_h : 0.0;
-  double acc_re = 0.0, acc_im = 0.0;
-  // T_0 e0 = e0
-  double cur = (i == 0) ? 1.0 : 0.0, prev = 0.0;
-  for (int k = 0; k <= K; ++k) {
-    // coefficient eps_k * phase_k * coef[k]
-    const double ck = (k == 0 ? 1.0 : 2.0) * coef[k];
-    double pre, pim;
-    if (kind == 0) {
-      // (-i sgn)^k
-      const int m = k & 3;
-      const double sgn = delta >= 0 ? 1.0 : -1.0;
-      pre = (m == 0) ? 1.0 : (m == 2 ? -1.0 : 0.0);
-      pim = (m == 1) ? -sgn : (m == 3 ? sgn : 0.0);
-    } else {
-      pre = (delta >= 0 && (k & 1)) ? -1.0 : 1.0;
-      pim = 0.0;
-    }
-    acc_re += ck * pre * cur;
-    acc_im += ck * pim * cur;
-    if (k == K) break;
-    if (i < n) tk[i] = cur;
-    __syncthreads();
-    double xv = 0.0;
-    if (i < n) {
-      xv = xd * cur;
-      if (i >= 1) xv += xl * tk[i - 1];
-      if (i + 1 < n) xv += xr * tk[i + 1];
-    }
-    const double nxt = (k == 0) ? xv : 2.0 * xv - prev;
-    __syncthreads();
-    prev = cur;
-    cur = nxt;
+  double xd[2], xl[2], xr[2], cur[2], prev[2] = {0.0, 0.0}, are[2] = {0.0, 0.0}, aim[2] = {0.0, 0.0};
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {  // X = (T - c) / h
+    xd[q] = lane + 32 * q < n ? (d[q] - c) * inv_h : 0.0;
+    xl[q] = ol[q] * inv_h;
+    xr[q] = orr[q] * inv_h;
   }
-  if (i < n) {
-    double fre, fim;
-    if (kind == 0) {
-      const double ph = -delta * c;
-      fre = cos(ph);
-      fim = sin(ph);
+  cur[0] = lane == 0 ? 1.0 : 0.0;  // T_0 e_0
+  cur[1] = 0.0;
+  for (int k = 0; k <= K; ++k) {
+    double ck = (k == 0 ? 1.0 : 2.0) * coef[k];
+    const int m = k & 3;
+    if (kind == 0) {  // (-i sgn delta)^k
+      if (k & 1) {
+        if ((m == 1) == (delta >= 0)) ck = -ck;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) aim[q] = fma(ck, cur[q], aim[q]);
+      } else {
+        if (m == 2) ck = -ck;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) are[q] = fma(ck, cur[q], are[q]);
+      }
     } else {
-      const double e = (delta >= 0) ? exp(-delta * sh_lo) : exp(-delta * sh_hi);
-      fre = e;
-      fim = 0.0;
+      if (delta >= 0 && (k & 1)) ck = -ck;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) are[q] = fma(ck, cur[q], are[q]);
     }
-    y[i] = mkc(fre * acc_re - fim * acc_im, fre * acc_im + fim * acc_re);
-    if (i == n - 1) {
-      const double b = sqrt(*nrm2_next);
-      const double ylast = sqrt(cabs2(y[i]));
-      err[0] = sh_bad ? 1e300 : b * ylast;
-      err[1] = b;
+    if (k == K) break;
+    double nx[2] = {0.0, 0.0};
+    const double up0 = __shfl_up_sync(FULL, cur[0], 1);  // lane 0: xl is 0
+    double dn0 = __shfl_down_sync(FULL, cur[0], 1);
+    if (two) {
+      const double first1 = __shfl_sync(FULL, cur[1], 0), last0 = __shfl_sync(FULL, cur[0], 31);
+      const double up1 = __shfl_up_sync(FULL, cur[1], 1), dn1 = __shfl_down_sync(FULL, cur[1], 1);
+      if (lane == 31) dn0 = first1;
+      nx[1] = fma(xr[1], dn1, fma(xl[1], lane == 0 ? last0 : up1, __dmul_rn(xd[1], cur[1])));
+    }
+    nx[0] = fma(xr[0], dn0, fma(xl[0], up0, __dmul_rn(xd[0], cur[0])));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const double nxt = k == 0 ? nx[q] : 2.0 * nx[q] - prev[q];
+      prev[q] = cur[q];
+      cur[q] = nxt;
+    }
+  }
+  double fre, fim = 0.0;
+  if (kind == 0) {
+    const double ph = -delta * c;
+    fre = cos(ph);
+    fim = sin(ph);
+  } else {
+    fre = (delta >= 0) ? exp(-delta * lo) : exp(-delta * hi);
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    if (i < n) {
+      const double acc_re = are[q], acc_im = aim[q];
+      const cplx v = mkc(fma(fre, acc_re, -__dmul_rn(fim, acc_im)), fma(fre, acc_im, __dmul_rn(fim, acc_re)));
+      y[i] = v;
+      if (i == n - 1) {
+        const double b = beta[n];
+        err[0] = bad ? 1e300 : b * sqrt(cabs2(v));
+        err[1] = b;
+      }
     }
   }
 }
 }  // namespace
 
-void tridiag_expv(cudaStream_t st, const double* alpha, const double* beta, int n, double delta,
-                  int kind, const double* nrm2_next, cplx* y, double* err) {
-  tdvp_require(n >= 1 && n < TRI_MAX, TDVP_ERR_INVALID_ARG, "tridiag_expv: n out of range");
-  k_tridiag_expv<<<1, TRI_MAX, 0, st>>>(alpha, beta, n, delta, kind, nrm2_next, y, err);
+void tridiag_expv(cudaStream_t st, const double* alpha, const double* beta, int n0, int count, double delta, int kind,
+                  cplx* y, double* err) {
+  tdvp_require(n0 >= 1 && count >= 1 && n0 + count - 1 < TRI_MAX, TDVP_ERR_INVALID_ARG,
+               "tridiag_expv: n out of range");
+  k_tridiag_expv<<<count, 32, 0, st>>>(alpha, beta, n0, delta, kind, y, err);
   TDVP_CHECK_LAUNCH();
 }
 

@@ -144,36 +144,30 @@ struct Blas1 {
                  long long n, cplx* out);
   // *out = sum_i |x_i|^2 (double in device memory)
   void norm2(cudaStream_t st, const cplx* x, long long n, double* out);
-  // One launch of a fused Lanczos step (partials reduced by the last block):
-  //   mode 0: cout = V^H w, alpha[j] = Re cout[j]
-  //   mode 1: w -= V cin, then cout = V^H w
-  //   mode 2: w -= V cin, then *nrm2 = |w|^2, *beta_slot = sqrt(*nrm2)
-  void lanczos_fused(cudaStream_t st, int mode, const cplx* V, long long ldv, int nvec, cplx* w, long long n,
-                     const cplx* cin, cplx* cout, double* alpha, int j, double* nrm2, double* beta_slot);
+  // The vector work of Lanczos iteration j: on entry w = H V[j]; on return alpha[j] and beta[j + 1]
+  // are set, w is orthogonal to V[0..j], nrm2[0] = |w|^2 and nrm2[1] = 1 / |w| (0 when |w|^2 <=
+  // 1e-200 or not finite).  c: 2 x 64 entries of scratch.  V's vectors are n entries apart.
+  void lanczos_step(cudaStream_t st, const cplx* V, long long n, int j, cplx* w, cplx* c, double* alpha, double* beta,
+                    double* nrm2);
   unsigned* counter = nullptr;  // ticket of the last-block reductions (reset by that block)
   void release();
 };
-// w[i] -= sum_k V[k*ldv+i] c[k]
-void multi_axpy_sub(cudaStream_t st, cplx* w, const cplx* V, long long ldv, int nvec,
-                    const cplx* c, long long n);
 // y[i] = scale * sum_k V[k*ldv+i] c[k]  (scale read from host value)
 void multi_combine(cudaStream_t st, cplx* y, const cplx* V, long long ldv, int nvec,
                    const cplx* c, double scale, long long n);
 // dst = src * (1 / sqrt(*nrm2))   (nrm2 in device memory)
 void scale_by_inv_sqrt(cudaStream_t st, cplx* dst, const cplx* src, const double* nrm2,
                        long long n);
-// the same with zeros when *nrm2 is not a positive finite number above 1e-200
-void scale_by_inv_sqrt_guarded(cudaStream_t st, cplx* dst, const cplx* src, const double* nrm2, long long n);
+// dst = src * *factor   (factor in device memory)
+void scale_by(cudaStream_t st, cplx* dst, const cplx* src, const double* factor, long long n);
 void scale_host(cudaStream_t st, cplx* dst, const cplx* src, cplx s, long long n);
 void fill_zero(cudaStream_t st, cplx* p, long long n);
-// Lanczos bookkeeping: alpha[j] = Re c[j]
-void copy_real_part(cudaStream_t st, const cplx* c, int j, double* alpha);
-// y[0..n) = exp(coef * T) e_0 for T tridiagonal (diag alpha, off beta[1..n-1]);
-// kind 0: coef = -i delta, kind 1: coef = -delta.  err[0] = sqrt(nrm2_next) |y[n-1]|,
-// err[1] = sqrt(nrm2_next) (beta_n), both written to device memory.
-void tridiag_expv(cudaStream_t st, const double* alpha, const double* beta, int n,
-                  double delta, int kind, const double* nrm2_next, cplx* y, double* err);
-void store_beta(cudaStream_t st, const double* nrm2, double* beta_slot);
+// For n = n0 .. n0 + count - 1 (b = n - n0): y[64 b + (0..n)) = exp(coef * T_n) e_0 for the
+// leading n x n part of the tridiagonal T (diagonal alpha, off-diagonals beta[1..n-1]);
+// kind 0: coef = -i delta, kind 1: coef = -delta.  err[2 b] = beta[n] |y[n-1]|, err[2 b + 1] =
+// beta[n], both written to device memory.
+void tridiag_expv(cudaStream_t st, const double* alpha, const double* beta, int n0, int count, double delta, int kind,
+                  cplx* y, double* err);
 
 // One-sided Jacobi SVD of a complex FP64 matrix (row-major rows x cols).
 struct SvdOut {
