@@ -11,8 +11,14 @@
 #include "linalg.cuh"
 
 // ============================================================================
-// ZGEMM (CUDA cores).  64x64 output tile, 8-deep K slices, 256 threads, each
-// thread accumulates a 4x4 block (rows ty+16i, cols tx+16j).
+// ZGEMM (CUDA cores).  T x T output tile, 16 x 16 (8 x 8 for T = 8) threads, each thread
+// accumulates T/16 x T/16 entries (rows ty + 16 i, cols tx + 16 j).
+// Bound: the FP64 pipe at every size (2 FMAs per cycle and SM: one complex multiply-add of a warp
+// takes 64 cycles, the two shared-memory reads feeding it 8), so the tile is not chosen for reuse
+// but so that the blocks cover the SMs and little of a tile is padding.  80 x 32 x 16 (a site of
+// bond dimension 16, w = 5): 47 us on 64 x 64 tiles (2 SMs, half of each tile padding), 4 us on
+// 8 x 8.  512-wide operands stay on 64 x 64 tiles (1.13 TFLOP/s, the pipe's rate).
+// Every entry sums its K range in order, so the tile does not change a bit of the result.
 // ============================================================================
 namespace {
 constexpr int GB_M = 64, GB_N = 64, GB_K = 8;
@@ -20,14 +26,17 @@ constexpr int GB_M = 64, GB_N = 64, GB_K = 8;
 // nsplit > 1: blockIdx.z = batch * nsplit + split; split s sums K range
 // [s*kchunk, min(K, (s+1)*kchunk)) into the partial buffer P[s][batch][M][N]
 // (alpha applied, beta left to the reduction).
-template <int OPA, int OPB>
-__global__ void __launch_bounds__(256)
+template <int OPA, int OPB, int T>
+__global__ void __launch_bounds__(T == 8 ? 64 : 256)
     k_zgemm(int M, int N, int K, cplx alpha, const cplx* __restrict__ A, long long lda,
             long long sA, const cplx* __restrict__ B, long long ldb, long long sB, cplx beta,
             cplx* __restrict__ C, long long ldc, long long sC, int nsplit, int kchunk, int nbatch,
             cplx* __restrict__ P) {
-  __shared__ cplx As[GB_K][GB_M + 1];
-  __shared__ cplx Bs[GB_K][GB_N + 1];
+  constexpr int TD = T == 8 ? 8 : 16;  // threads per side
+  constexpr int NT = TD * TD, R = T / TD;
+  constexpr int TK = T >= 64 ? GB_K : 16;
+  __shared__ cplx As[TK][T + 1];
+  __shared__ cplx Bs[TK][T + 1];
   const int split = blockIdx.z % nsplit;
   const long long bz = blockIdx.z / nsplit;
   A += bz * sA;
@@ -41,24 +50,24 @@ __global__ void __launch_bounds__(256)
   }
   const int kbeg = split * kchunk;
   const int kend = min(K, kbeg + kchunk);
-  const int m0 = blockIdx.y * GB_M, n0 = blockIdx.x * GB_N;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  cplx acc[4][4];
+  const int m0 = blockIdx.y * T, n0 = blockIdx.x * T;
+  const int tid = threadIdx.x, tx = tid % TD, ty = tid / TD;
+  cplx acc[R][R];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = mkc(0.0, 0.0);
+    for (int j = 0; j < R; ++j) acc[i][j] = mkc(0.0, 0.0);
 
-  for (int k0 = kbeg; k0 < kend; k0 += GB_K) {
+  for (int k0 = kbeg; k0 < kend; k0 += TK) {
 #pragma unroll
-    for (int e = tid; e < GB_M * GB_K; e += 256) {
+    for (int e = tid; e < T * TK; e += NT) {
       int m, k;
       if (OPA == OP_N || OPA == OP_R) {
-        m = e / GB_K;
-        k = e % GB_K;
+        m = e / TK;
+        k = e % TK;
       } else {
-        k = e / GB_M;
-        m = e % GB_M;
+        k = e / T;
+        m = e % T;
       }
       const int gm = m0 + m, gk = k0 + k;
       cplx v = mkc(0.0, 0.0);
@@ -69,14 +78,14 @@ __global__ void __launch_bounds__(256)
       As[k][m] = v;
     }
 #pragma unroll
-    for (int e = tid; e < GB_K * GB_N; e += 256) {
+    for (int e = tid; e < TK * T; e += NT) {
       int k, n;
       if (OPB == OP_N || OPB == OP_R) {
-        k = e / GB_N;
-        n = e % GB_N;
+        k = e / T;
+        n = e % T;
       } else {
-        n = e / GB_K;
-        k = e % GB_K;
+        n = e / TK;
+        k = e % TK;
       }
       const int gn = n0 + n, gk = k0 + k;
       cplx v = mkc(0.0, 0.0);
@@ -87,28 +96,30 @@ __global__ void __launch_bounds__(256)
       Bs[k][n] = v;
     }
     __syncthreads();
+    const int kn = T >= 64 ? TK : min(TK, kend - k0);  // the padding past K is zeros
 #pragma unroll
-    for (int kk = 0; kk < GB_K; ++kk) {
-      cplx a[4], b[4];
+    for (int kk = 0; kk < TK; ++kk) {
+      if (kk >= kn) break;
+      cplx a[R], b[R];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+      for (int i = 0; i < R; ++i) a[i] = As[kk][ty + TD * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+      for (int j = 0; j < R; ++j) b[j] = Bs[kk][tx + TD * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cfma(acc[i][j], a[i], b[j]);
+        for (int j = 0; j < R; ++j) cfma(acc[i][j], a[i], b[j]);
     }
     __syncthreads();
   }
   const bool use_beta = (beta.x != 0.0 || beta.y != 0.0);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty + 16 * i;
+  for (int i = 0; i < R; ++i) {
+    const int gm = m0 + ty + TD * i;
     if (gm >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx + 16 * j;
+    for (int j = 0; j < R; ++j) {
+      const int gn = n0 + tx + TD * j;
       if (gn >= N) continue;
       cplx r = cmul(alpha, acc[i][j]);
       cplx* c = C + (long long)gm * ldc + gn;
@@ -118,19 +129,29 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-#define ZG_ARGS M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, ns, kc, nb, P
-template <int OPA>
-void zgemm_b(int opB, dim3 g, cudaStream_t st, int M, int N, int K, cplx alpha, const cplx* A,
-             long long lda, long long sA, const cplx* B, long long ldb, long long sB, cplx beta,
-             cplx* C, long long ldc, long long sC, int ns, int kc, int nb, cplx* P) {
-  switch (opB) {
-    case OP_N: k_zgemm<OPA, OP_N><<<g, 256, 0, st>>>(ZG_ARGS); break;
-    case OP_T: k_zgemm<OPA, OP_T><<<g, 256, 0, st>>>(ZG_ARGS); break;
-    case OP_C: k_zgemm<OPA, OP_C><<<g, 256, 0, st>>>(ZG_ARGS); break;
-    default:   k_zgemm<OPA, OP_R><<<g, 256, 0, st>>>(ZG_ARGS); break;
+#define ZG_ARGS M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, ns, kc, batch, P
+template <int OPA, int OPB>
+void zgemm_t(int tile, dim3 g, cudaStream_t st, int M, int N, int K, cplx alpha, const cplx* A, long long lda,
+             long long sA, const cplx* B, long long ldb, long long sB, cplx beta, cplx* C, long long ldc, long long sC,
+             int ns, int kc, int batch, cplx* P) {
+  switch (tile) {
+    case 8: k_zgemm<OPA, OPB, 8><<<g, 64, 0, st>>>(ZG_ARGS); break;
+    case 16: k_zgemm<OPA, OPB, 16><<<g, 256, 0, st>>>(ZG_ARGS); break;
+    case 32: k_zgemm<OPA, OPB, 32><<<g, 256, 0, st>>>(ZG_ARGS); break;
+    default: k_zgemm<OPA, OPB, 64><<<g, 256, 0, st>>>(ZG_ARGS); break;
   }
 }
-#undef ZG_ARGS
+template <int OPA>
+void zgemm_b(int opB, int tile, dim3 g, cudaStream_t st, int M, int N, int K, cplx alpha, const cplx* A,
+             long long lda, long long sA, const cplx* B, long long ldb, long long sB, cplx beta,
+             cplx* C, long long ldc, long long sC, int ns, int kc, int batch, cplx* P) {
+  switch (opB) {
+    case OP_N: zgemm_t<OPA, OP_N>(tile, g, st, ZG_ARGS); break;
+    case OP_T: zgemm_t<OPA, OP_T>(tile, g, st, ZG_ARGS); break;
+    case OP_C: zgemm_t<OPA, OP_C>(tile, g, st, ZG_ARGS); break;
+    default:   zgemm_t<OPA, OP_R>(tile, g, st, ZG_ARGS); break;
+  }
+}
 
 // C[b][m][n] = sum_s P[s][b][m][n] + beta C[b][m][n]  (fixed summation order)
 __global__ void k_splitk_reduce(const cplx* __restrict__ P, int nsplit, int nbatch, int M, int N, cplx beta,
@@ -179,13 +200,18 @@ void zgemm(cudaStream_t st, int opA, int opB, int M, int N, int K, cplx alpha, c
   }
   DArr part;
   if (ns > 1) part.reset(ws, (size_t)ns * batch * M * N);
-  dim3 g(ceil_div(N, GB_N), ceil_div(M, GB_M), batch * ns);
+  // the largest tile whose blocks still give every SM two (the work of a tile is FP64 time, so
+  // smaller ones only cost when the blocks cover the device anyway)
+  int tile = 64;
+  while (tile > 8 && (long long)ceil_div(N, tile) * ceil_div(M, tile) * batch * ns < 2LL * sms) tile /= 2;
+  while (tile < 64 && ceil_div(M, tile) > 65535) tile *= 2;
+  dim3 g(ceil_div(N, tile), ceil_div(M, tile), batch * ns);
   cplx* P = part.data();
   switch (opA) {
-    case OP_N: zgemm_b<OP_N>(opB, g, st, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, ns, kc, batch, P); break;
-    case OP_T: zgemm_b<OP_T>(opB, g, st, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, ns, kc, batch, P); break;
-    case OP_C: zgemm_b<OP_C>(opB, g, st, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, ns, kc, batch, P); break;
-    default:   zgemm_b<OP_R>(opB, g, st, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, ns, kc, batch, P); break;
+    case OP_N: zgemm_b<OP_N>(opB, tile, g, st, ZG_ARGS); break;
+    case OP_T: zgemm_b<OP_T>(opB, tile, g, st, ZG_ARGS); break;
+    case OP_C: zgemm_b<OP_C>(opB, tile, g, st, ZG_ARGS); break;
+    default:   zgemm_b<OP_R>(opB, tile, g, st, ZG_ARGS); break;
   }
   TDVP_CHECK_LAUNCH();
   if (ns > 1) {
@@ -194,6 +220,7 @@ void zgemm(cudaStream_t st, int opA, int opB, int M, int N, int K, cplx alpha, c
     TDVP_CHECK_LAUNCH();
   }
 }
+#undef ZG_ARGS
 
 // ============================================================================
 // MPO-tensor stages
@@ -360,6 +387,11 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
+// Whether v is not +-0, from its bits: an FP64 compare would run on the FP64 pipe the test spares
+__device__ __forceinline__ bool nonzero_bits(cplx v) {
+  return ((__double2hiint(v.x) | __double2hiint(v.y)) << 1 | __double2loint(v.x) | __double2loint(v.y)) != 0;
+}
+__device__ __forceinline__ bool warp_nonzero(cplx v) { return __any_sync(0xffffffffu, nonzero_bits(v)); }
 
 __global__ void __launch_bounds__(RED_THREADS)
     k_multidot_partial(const cplx* __restrict__ V, long long ldv, int nvec, const cplx* __restrict__ w,
@@ -456,9 +488,9 @@ __global__ void k_multi_combine(cplx* __restrict__ y, const cplx* __restrict__ V
     // FP64 bound: entries that are zero in the whole warp (other charge sectors) cost no FMAs
 #pragma unroll
     for (int q = 0; q < MD_CH; ++q)
-      if (__any_sync(active, v[q].x != 0.0 || v[q].y != 0.0)) cfma(acc, v[q], cs[k0 + q]);
+      if (__any_sync(active, nonzero_bits(v[q]))) cfma(acc, v[q], cs[k0 + q]);
   }
-  y[i] = cscale(acc, scale);
+  y[i] = __any_sync(active, nonzero_bits(acc)) ? cscale(acc, scale) : acc;
 }
 
 // FP64 division and square root cost tens of FP64 instructions: one thread per block forms the factor
@@ -549,9 +581,6 @@ __device__ __forceinline__ void warp_sum_store(const cplx (&acc)[NC], double* ou
   if ((lane & rest) == 0) out[idx] = a[0];
 }
 
-__device__ __forceinline__ bool warp_nonzero(cplx v) {
-  return __any_sync(0xffffffffu, v.x != 0.0 || v.y != 0.0);
-}
 
 constexpr int TRI_MAX = 64;
 constexpr int CHEB_MAX = 1024;
@@ -635,7 +664,8 @@ __device__ __forceinline__ cplx lanczos_subtract(const cplx* __restrict__ V, lon
     for (int q = 0; q < MD_CH; ++q)
       if (k0 + q < nvec && warp_nonzero(v[q])) cfma(sub, v[q], cs[k0 + q]);
   }
-  return in ? csub(w[i], sub) : mkc(0.0, 0.0);
+  const cplx wi = in ? w[i] : mkc(0.0, 0.0);
+  return warp_nonzero(sub) ? csub(wi, sub) : wi;
 }
 
 __global__ void __launch_bounds__(RED_THREADS)

@@ -256,3 +256,15 @@ def test_keff_apply_precision_forms_through_a_handle(g, prec):
     h.keff_apply(bond, xd, yd, code)
     assert _rel(yd.cpu().numpy(), O.keff_apply(Ls[bond], R_incl, x)) < tol
     h.close()
+
+
+@pytest.mark.parametrize("ml,mr,w", [(1, 7, 3), (8, 8, 1), (9, 17, 5), (16, 16, 5), (33, 31, 8), (63, 65, 14),
+                                     (150, 70, 14)])
+def test_fp64_tiles_match_oracle(g, ml, mr, w):
+    """The FP64 GEMM at the edges of its 8, 16, 32 and 64-wide tiles, with and without a split K."""
+    rng = np.random.default_rng(ml)
+    L, R, x = _rand(rng, ml, w, ml), _rand(rng, mr, w, mr), _rand(rng, ml, mr)
+    Ld, Rd, xd = _dev(L, R, x)
+    yd = torch.empty_like(xd)
+    g.keff_contract(Ld, Rd, xd, yd)
+    assert _rel(yd.cpu().numpy(), O.keff_apply(L, R, x)) < TOL64
