@@ -485,7 +485,7 @@ tdvp_status tdvp_heff_contract_cached(const tdvp_site_dims* dims, const void* L,
     op.d = dims->d;
     // a tag names the (L, R) content for the operand caches of the tensor-core paths;
     // tags are kept apart from nothing else (this context serves only these calls)
-    op.env_key = env_tag;
+    op.env_key = precision == TDVP_PREC_FP64 ? -1 : env_tag;  // FP64 ignores the tag
     heff_apply_prec(st, c.scr, op, static_cast<const cplx*>(x), static_cast<cplx*>(y), precision);
     TDVP_CUDA(cudaStreamSynchronize(st));
     w.free_device();
@@ -502,6 +502,7 @@ tdvp_status tdvp_keff_contract(int ml, int mr, int wb, const void* L, const void
     keff_fp64(st, c.scr, static_cast<const cplx*>(L), ml, static_cast<const cplx*>(R), mr, wb,
               static_cast<const cplx*>(x), static_cast<cplx*>(y));
     TDVP_CUDA(cudaStreamSynchronize(st));
+    tc_check(st, c.scr);
   });
 }
 
@@ -521,6 +522,7 @@ tdvp_status tdvp_env_contract(const tdvp_site_dims* dims, int side, const void* 
                      dims->d, static_cast<cplx*>(out));
     TDVP_CUDA(cudaStreamSynchronize(st));
     w.free_device();
+    tc_check(st, c.scr);
   });
 }
 

@@ -16,8 +16,21 @@ double heff_flops(const SiteOp& op) {
   return 8.0 * (ml * d * mr * (ml * op.wl + mr * op.wr) + ml * mr * (double)op.W->nnz);
 }
 
+void zgemm_fp64(cudaStream_t st, Scratch& s, int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A,
+                long long lda, const cplx* B, long long ldb, cplx beta, cplx* C, long long ldc) {
+  if (f64_on_tensor_cores(M, N, K))
+    zgemm_f64s(st, s, opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+  else
+    zgemm(st, opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 1, 0, 0, 0, s.pool);
+}
+
 void heff_fp64(cudaStream_t st, Scratch& s, const SiteOp& op, const cplx* x, cplx* y) {
   const int ml = op.ml, mr = op.mr, wl = op.wl, wr = op.wr, d = op.d;
+  if (f64_on_tensor_cores((long long)ml * wl, (long long)d * mr, ml) &&
+      f64_on_tensor_cores((long long)ml * d, mr, (long long)wr * mr)) {
+    heff_f64s(st, s, op, x, y);
+    return;
+  }
   s.t1.ensure(s.pool, (size_t)ml * wl * d * mr);
   s.t2.ensure(s.pool, (size_t)ml * d * wr * mr);
   // T1[(a,w),(s',b')] = L[(a,w),a'] x[a',(s',b')]
@@ -48,7 +61,7 @@ void zgemm_prec(cudaStream_t st, Scratch& s, int precision, int opA, int opB, in
   else if (big && precision != TDVP_PREC_FP64)
     zgemm_tc(st, s, opA, opB, M, N, K, A, lda, B, ldb, C, ldc);
   else
-    zgemm(st, opA, opB, M, N, K, kOne, A, lda, B, ldb, kZero, C, ldc, 1, 0, 0, 0, s.pool);
+    zgemm_fp64(st, s, opA, opB, M, N, K, kOne, A, lda, B, ldb, kZero, C, ldc);
 }
 
 void keff_fp64(cudaStream_t st, Scratch& s, const cplx* L, int ml, const cplx* R, int mr, int w, const cplx* x,

@@ -17,6 +17,7 @@ struct SiteOp {
   long long env_key = -1;      // identifies the (L, R) content for operand caching; -1 = never cache
 };
 
+struct F64EnvDigits;  // digits of the environments of the FP64 tensor-core path (tc_f64.cu)
 struct TcSliceCache;  // sliced operands of the BF16 tensor-core path (tc_bf16.cu)
 
 // Work buffers reused across calls (drawn from a pool).
@@ -25,6 +26,7 @@ struct Scratch {
   DArr t1, t2, t3;
   TcEnvCache tc;
   std::shared_ptr<TcSliceCache> tcs;
+  std::shared_ptr<F64EnvDigits> f64;
 };
 
 // Algorithmic flop count of one H_eff apply (8 real flops per complex multiply-add):
@@ -51,6 +53,17 @@ void zgemm_tc(cudaStream_t st, Scratch& s, int opA, int opB, int M, int N, int K
 // C = opA(A) opB(B) on the BF16 exact-slice tensor-core GEMM (S slices, FP64 output).
 void zgemm_bf16s(cudaStream_t st, Scratch& s, int S, int opA, int opB, int M, int N, int K, const cplx* A,
                  long long lda, const cplx* B, long long ldb, cplx* C, long long ldc);
+// FP64 on the tensor cores by exact 8-bit digits (tc_f64.cu): whether a complex product of this
+// size belongs there, C = alpha opA(A) opB(B) + beta C, and H_eff.
+bool f64_on_tensor_cores(long long M, long long N, long long K);
+void zgemm_f64s(cudaStream_t st, Scratch& s, int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A,
+                long long lda, const cplx* B, long long ldb, cplx beta, cplx* C, long long ldc);
+void heff_f64s(cudaStream_t st, Scratch& s, const SiteOp& op, const cplx* x, cplx* y);
+// The FP64 product by size: exact digits on the tensor cores, or the CUDA-core GEMM.
+void zgemm_fp64(cudaStream_t st, Scratch& s, int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A,
+                long long lda, const cplx* B, long long ldb, cplx beta, cplx* C, long long ldc);
+// The error word of the tensor-core kernels' bounded waits (read by tc_check); marks it pending.
+int* tc_error_word(cudaStream_t st, Scratch& s);
 // The tensor-core GEMM of `precision` (zgemm_tc for the TF32 modes, zgemm_bf16s for
 // the BF16 modes) when the product is large enough to fill its tiles, the FP64
 // GEMM otherwise (alpha = 1, beta = 0).

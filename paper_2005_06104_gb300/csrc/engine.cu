@@ -362,6 +362,20 @@ void Engine::apply_op(const SiteOp& op, const cplx* x, cplx* y, int precision) {
 // gauge moves: a block QR / LQ when nothing is cut (R1), else a truncated SVD
 // (numerical rank 1e-10 s_max, cutoff eps, cap)
 // ============================================================================
+// The products of the gauge moves and the sweeps.  A handle in FP64 takes them by size (exact
+// digits on the tensor cores from 4 M multiply-adds on); one in a split form keeps the CUDA-core
+// order, so that its trajectories stay those of earlier releases bit by bit: its sweeps turn a
+// last-bit change into 1e-7 of a site tensor (operand digits round at 2^-33, and the next gauge
+// move divides by Schmidt values of 1e-6; measured at chi 256), far above what the product itself
+// could change.
+void Engine::gauge_gemm(int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A, long long lda, const cplx* B,
+                        long long ldb, cplx beta, cplx* C, long long ldc) {
+  if (opt.precision == TDVP_PREC_FP64)
+    zgemm_fp64(st, scr, opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+  else
+    zgemm(st, opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 1, 0, 0, 0, &pool);
+}
+
 void Engine::move_right(int i, double eps, int cap, bool trunc) {
   const int ml = psi.m[i], mr = psi.m[i + 1], mr2 = psi.m[i + 2];
   QrOut qo;
@@ -369,8 +383,8 @@ void Engine::move_right(int i, double eps, int cap, bool trunc) {
   if (!trunc && qo.full_rank(kRankRtol)) {  // R1: the QR keeps the numerical rank
     const int r = qo.k;
     DArr nxt(&pool, (size_t)r * d * mr2);
-    zgemm(st, OP_N, OP_N, r, d * mr2, mr, kOne, qo.C.data(), mr, psi.A[i + 1].data(), d * mr2, kZero, nxt.data(),
-          d * mr2, 1, 0, 0, 0, &pool);
+    gauge_gemm(OP_N, OP_N, r, d * mr2, mr, kOne, qo.C.data(), mr, psi.A[i + 1].data(), d * mr2, kZero, nxt.data(),
+          d * mr2);
     psi.A[i] = std::move(qo.Q);
     psi.A[i + 1] = std::move(nxt);
     psi.m[i + 1] = r;
@@ -391,11 +405,10 @@ void Engine::move_right(int i, double eps, int cap, bool trunc) {
   // C = U^+ A = S Vh (r x mr), one FP64 GEMM instead of rotating V in every Jacobi round;
   // A[i+1] <- C A[i+1]
   DArr C(&pool, (size_t)r * mr);
-  zgemm(st, OP_C, OP_N, r, mr, ml * d, kOne, sv.U.data(), r, psi.A[i].data(), mr, kZero, C.data(), mr, 1, 0, 0, 0,
-        &pool);
+  gauge_gemm(OP_C, OP_N, r, mr, ml * d, kOne, sv.U.data(), r, psi.A[i].data(), mr, kZero, C.data(), mr);
   DArr nxt(&pool, (size_t)r * d * mr2);
-  zgemm(st, OP_N, OP_N, r, d * mr2, mr, kOne, C.data(), mr, psi.A[i + 1].data(), d * mr2, kZero, nxt.data(),
-        d * mr2, 1, 0, 0, 0, &pool);
+  gauge_gemm(OP_N, OP_N, r, d * mr2, mr, kOne, C.data(), mr, psi.A[i + 1].data(), d * mr2, kZero, nxt.data(),
+        d * mr2);
   psi.A[i] = std::move(sv.U);
   psi.A[i + 1] = std::move(nxt);
   psi.m[i + 1] = r;
@@ -410,8 +423,7 @@ void Engine::move_left(int i, double eps, int cap, bool trunc) {
   if (!trunc && qo.full_rank(kRankRtol)) {  // R1: the LQ keeps the numerical rank
     const int r = qo.k;
     DArr prv(&pool, (size_t)ml0 * d * r);
-    zgemm(st, OP_N, OP_N, ml0 * d, r, ml, kOne, psi.A[i - 1].data(), ml, qo.C.data(), r, kZero, prv.data(), r, 1, 0,
-          0, 0, &pool);
+    gauge_gemm(OP_N, OP_N, ml0 * d, r, ml, kOne, psi.A[i - 1].data(), ml, qo.C.data(), r, kZero, prv.data(), r);
     psi.A[i] = std::move(qo.Q);
     psi.A[i - 1] = std::move(prv);
     psi.m[i] = r;
@@ -431,10 +443,9 @@ void Engine::move_left(int i, double eps, int cap, bool trunc) {
   tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "move_left: zero tensor");
   // C = A Vh^+ = U S (ml x r), one FP64 GEMM instead of rotating U in every Jacobi round
   DArr C(&pool, (size_t)ml * r);
-  zgemm(st, OP_N, OP_C, ml, r, d * mr, kOne, psi.A[i].data(), d * mr, sv.Vh.data(), d * mr, kZero, C.data(), r, 1, 0,
-        0, 0, &pool);
+  gauge_gemm(OP_N, OP_C, ml, r, d * mr, kOne, psi.A[i].data(), d * mr, sv.Vh.data(), d * mr, kZero, C.data(), r);
   DArr prv(&pool, (size_t)ml0 * d * r);
-  zgemm(st, OP_N, OP_N, ml0 * d, r, ml, kOne, psi.A[i - 1].data(), ml, C.data(), r, kZero, prv.data(), r, 1, 0, 0, 0, &pool);
+  gauge_gemm(OP_N, OP_N, ml0 * d, r, ml, kOne, psi.A[i - 1].data(), ml, C.data(), r, kZero, prv.data(), r);
   psi.A[i] = std::move(sv.Vh);
   psi.A[i - 1] = std::move(prv);
   psi.m[i] = r;
@@ -543,8 +554,7 @@ void Engine::sweep(double dt, int kind) {
         r = sv.rank;
         tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "sweep: zero site tensor");
         C.reset(&pool, (size_t)r * mold);
-        zgemm(st, OP_C, OP_N, r, mold, ml * d, kOne, sv.U.data(), r, psi.A[i].data(), mold, kZero, C.data(), mold,
-              1, 0, 0, 0, &pool);
+        gauge_gemm(OP_C, OP_N, r, mold, ml * d, kOne, sv.U.data(), r, psi.A[i].data(), mold, kZero, C.data(), mold);
         psi.A[i] = std::move(sv.U);
       } else {  // real time cuts nothing: block QR of full numerical rank (R1)
         r = qo.k;
@@ -565,8 +575,8 @@ void Engine::sweep(double dt, int kind) {
     }
     if (imag) normalize(C2.data(), (long long)r * mold);
     DArr nxt(&pool, (size_t)r * d * mr2);
-    zgemm(st, OP_N, OP_N, r, d * mr2, mold, kOne, C2.data(), mold, psi.A[i + 1].data(), d * mr2, kZero,
-          nxt.data(), d * mr2, 1, 0, 0, 0, &pool);
+    gauge_gemm(OP_N, OP_N, r, d * mr2, mold, kOne, C2.data(), mold, psi.A[i + 1].data(), d * mr2, kZero,
+          nxt.data(), d * mr2);
     psi.A[i + 1] = std::move(nxt);
     center = i + 1;
     for (int j = i + 2; j < N; ++j) Lok[j] = 0;
@@ -593,8 +603,8 @@ void Engine::sweep(double dt, int kind) {
         r = sv.rank;
         tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "sweep: zero site tensor");
         C.reset(&pool, (size_t)mold * r);
-        zgemm(st, OP_N, OP_C, mold, r, d * mr, kOne, psi.A[i].data(), d * mr, sv.Vh.data(), d * mr, kZero, C.data(),
-              r, 1, 0, 0, 0, &pool);
+        gauge_gemm(OP_N, OP_C, mold, r, d * mr, kOne, psi.A[i].data(), d * mr, sv.Vh.data(), d * mr, kZero, C.data(),
+              r);
         psi.A[i] = std::move(sv.Vh);
       } else {  // real time cuts nothing: block LQ of full numerical rank (R1)
         r = qo.k;
@@ -615,8 +625,8 @@ void Engine::sweep(double dt, int kind) {
     }
     if (imag) normalize(C2.data(), (long long)mold * r);
     DArr prv(&pool, (size_t)ml0 * d * r);
-    zgemm(st, OP_N, OP_N, ml0 * d, r, mold, kOne, psi.A[i - 1].data(), mold, C2.data(), r, kZero, prv.data(),
-          r, 1, 0, 0, 0, &pool);
+    gauge_gemm(OP_N, OP_N, ml0 * d, r, mold, kOne, psi.A[i - 1].data(), mold, C2.data(), r, kZero, prv.data(),
+          r);
     psi.A[i - 1] = std::move(prv);
     center = i - 1;
     for (int j = 0; j < i - 1; ++j) Rok[j] = 0;
@@ -669,8 +679,8 @@ void Engine::sweep2(double dt, int kind) {
     const long long n = (long long)ml * d * d * mr;
     theta.ensure(&pool, n);
     y.ensure(&pool, n);
-    zgemm(st, OP_N, OP_N, ml * d, d * mr, m, kOne, psi.A[i].data(), m, psi.A[i + 1].data(), d * mr, kZero,
-          theta.data(), d * mr, 1, 0, 0, 0, &pool);
+    gauge_gemm(OP_N, OP_N, ml * d, d * mr, m, kOne, psi.A[i].data(), m, psi.A[i + 1].data(), d * mr, kZero,
+          theta.data(), d * mr);
     const SiteOp op = pair_op(i);
     {
       PhaseScope ps(tracer, PH_LANCZOS_SITE);
@@ -700,8 +710,7 @@ void Engine::sweep2(double dt, int kind) {
     const int r = sv.rank;
     const int ml = psi.m[i];
     DArr C(&pool, (size_t)r * d * mr);  // U^+ Theta = S Vh: the centre on site i+1
-    zgemm(st, OP_C, OP_N, r, d * mr, ml * d, kOne, sv.U.data(), r, y.data(), d * mr, kZero, C.data(), d * mr, 1, 0,
-          0, 0, &pool);
+    gauge_gemm(OP_C, OP_N, r, d * mr, ml * d, kOne, sv.U.data(), r, y.data(), d * mr, kZero, C.data(), d * mr);
     psi.A[i] = std::move(sv.U);
     psi.m[i + 1] = r;
     env_left(i);  // L[i+1]
@@ -718,8 +727,7 @@ void Engine::sweep2(double dt, int kind) {
     const int r = sv.rank;
     const int mr = psi.m[i + 2];
     DArr C(&pool, (size_t)ml * d * r);  // Theta Vh^+ = U S: the centre on site i
-    zgemm(st, OP_N, OP_C, ml * d, r, d * mr, kOne, y.data(), d * mr, sv.Vh.data(), d * mr, kZero, C.data(), r, 1, 0,
-          0, 0, &pool);
+    gauge_gemm(OP_N, OP_C, ml * d, r, d * mr, kOne, y.data(), d * mr, sv.Vh.data(), d * mr, kZero, C.data(), r);
     psi.A[i + 1] = std::move(sv.Vh);
     psi.m[i + 1] = r;
     env_right(i + 1);  // R[i]
@@ -1061,11 +1069,10 @@ void Engine::krylov_zipup(const KrylovOp& kop, const MpsDev& src, MpsDev& out) {
     const int r = sv.rank;
     tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "zip-up: zero tensor in the compression");
     DArr C(&pool, (size_t)r * mr);
-    zgemm(st, OP_C, OP_N, r, mr, ml * d, kOne, sv.U.data(), r, t.A[i].data(), mr, kZero, C.data(), mr, 1, 0, 0, 0,
-          &pool);
+    gauge_gemm(OP_C, OP_N, r, mr, ml * d, kOne, sv.U.data(), r, t.A[i].data(), mr, kZero, C.data(), mr);
     DArr nxt(&pool, (size_t)r * d * mr2);
-    zgemm(st, OP_N, OP_N, r, d * mr2, mr, kOne, C.data(), mr, t.A[i + 1].data(), d * mr2, kZero, nxt.data(),
-          d * mr2, 1, 0, 0, 0, &pool);
+    gauge_gemm(OP_N, OP_N, r, d * mr2, mr, kOne, C.data(), mr, t.A[i + 1].data(), d * mr2, kZero, nxt.data(),
+          d * mr2);
     t.A[i] = std::move(sv.U);
     t.A[i + 1] = std::move(nxt);
     t.m[i + 1] = r;
@@ -1148,8 +1155,8 @@ void Engine::expand_basis(int k, const double* weights) {
       // Y P = Y - (Y B^H) B : rho_bar = (Y P)^H (Y P) = P rho~ P  (Eq. 6)
       DArr G(&pool, (size_t)rows * r);
       for (int pass = 0; pass < 2; ++pass) {
-        zgemm(st, OP_N, OP_C, rows, r, cols, kOne, Y.data(), cols, Bm.data(), cols, kZero, G.data(), r, 1, 0, 0, 0, &pool);
-        zgemm(st, OP_N, OP_N, rows, cols, r, kMinusOne, G.data(), r, Bm.data(), cols, kOne, Y.data(), cols, 1, 0, 0, 0, &pool);
+        zgemm_fp64(st, scr, OP_N, OP_C, rows, r, cols, kOne, Y.data(), cols, Bm.data(), cols, kZero, G.data(), r);
+        zgemm_fp64(st, scr, OP_N, OP_N, rows, cols, r, kMinusOne, G.data(), r, Bm.data(), cols, kOne, Y.data(), cols);
       }
       if (tr > 0.0) {
         const double eps_m = opt.eps_m;
@@ -1173,9 +1180,9 @@ void Engine::expand_basis(int k, const double* weights) {
           // enforce B_bar B^H = 0 to rounding: project off range(B) twice, re-orthonormalise
           DArr Gb(&pool, (size_t)nb * r);
           for (int pass = 0; pass < 2; ++pass) {
-            zgemm(st, OP_N, OP_C, nb, r, cols, kOne, sy.Vh.data(), cols, Bm.data(), cols, kZero, Gb.data(), r, 1, 0, 0, 0, &pool);
-            zgemm(st, OP_N, OP_N, nb, cols, r, kMinusOne, Gb.data(), r, Bm.data(), cols, kOne, sy.Vh.data(),
-                  cols, 1, 0, 0, 0, &pool);
+            zgemm_fp64(st, scr, OP_N, OP_C, nb, r, cols, kOne, sy.Vh.data(), cols, Bm.data(), cols, kZero, Gb.data(), r);
+            zgemm_fp64(st, scr, OP_N, OP_N, nb, cols, r, kMinusOne, Gb.data(), r, Bm.data(), cols, kOne, sy.Vh.data(),
+                  cols);
           }
           SvdOut so;
           struct KeepAll {
@@ -1206,10 +1213,10 @@ void Engine::expand_basis(int k, const double* weights) {
     }
     // centres move by Eq. 3: C_{i-1} = A_{i-1} (C_i B'^H), likewise for every psi~_l
     DArr G(&pool, (size_t)ml * mnew);
-    zgemm(st, OP_N, OP_C, ml, mnew, cols, kOne, X, cols, Bp.data(), cols, kZero, G.data(), mnew, 1, 0, 0, 0, &pool);
+    zgemm_fp64(st, scr, OP_N, OP_C, ml, mnew, cols, kOne, X, cols, Bp.data(), cols, kZero, G.data(), mnew);
     DArr prv(&pool, (size_t)ml0 * d * mnew);
-    zgemm(st, OP_N, OP_N, ml0 * d, mnew, ml, kOne, psi.A[i - 1].data(), ml, G.data(), mnew, kZero, prv.data(),
-          mnew, 1, 0, 0, 0, &pool);
+    zgemm_fp64(st, scr, OP_N, OP_N, ml0 * d, mnew, ml, kOne, psi.A[i - 1].data(), ml, G.data(), mnew, kZero, prv.data(),
+          mnew);
     for (int l = 0; l < nk; ++l) {
       MpsDev& ph = phis[l];
       const int mlp = ph.m[i], mlp0 = ph.m[i - 1];
@@ -1233,6 +1240,7 @@ void Engine::expand_basis(int k, const double* weights) {
   center = 0;
   for (int j = 0; j < N; ++j) Lok[j] = Rok[j] = 0;
   sync();
+  tc_check(st, scr);
 }
 
 void Engine::apply_krylov() {
@@ -1267,6 +1275,7 @@ double Engine::energy() {
   TDVP_CUDA(cudaMemcpyAsync(&e, lw.c.data(), sizeof(cplx), cudaMemcpyDeviceToHost, st));
   TDVP_CUDA(cudaMemcpyAsync(&nn, lw.real + 152, sizeof(double), cudaMemcpyDeviceToHost, st));
   sync();
+  tc_check(st, scr);
   return e.x / nn;
 }
 
@@ -1295,6 +1304,7 @@ cplx Engine::expect_local(const double* op, int site) {
   TDVP_CUDA(cudaMemcpyAsync(&e, lw.c.data(), sizeof(cplx), cudaMemcpyDeviceToHost, st));
   TDVP_CUDA(cudaMemcpyAsync(&nn, lw.real + 154, sizeof(double), cudaMemcpyDeviceToHost, st));
   sync();
+  tc_check(st, scr);
   return mkc(e.x / nn, e.y / nn);
 }
 
@@ -1326,5 +1336,6 @@ cplx Engine::expect_mpo(const tdvp_mpo_desc* op) {
   cplx v;
   TDVP_CUDA(cudaMemcpyAsync(&v, E.data(), sizeof(cplx), cudaMemcpyDeviceToHost, st));
   const double n = norm();
+  tc_check(st, scr);
   return mkc(v.x / (n * n), v.y / (n * n));
 }

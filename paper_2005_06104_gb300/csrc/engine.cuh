@@ -83,6 +83,8 @@ struct Engine {
   void env_left(int i);   // L[i+1] from L[i], A[i]
   void env_right(int i);  // R[i-1] from R[i], A[i]
   // gauge moves
+  void gauge_gemm(int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A, long long lda, const cplx* B,
+                  long long ldb, cplx beta, cplx* C, long long ldc);
   void move_right(int i, double eps, int cap, bool imag_trunc);
   void move_left(int i, double eps, int cap, bool imag_trunc);
   void canonicalize(int c);

@@ -304,7 +304,7 @@ void WSparse::free_device() {
 namespace {
 __global__ void k_wstage_left(const cplx* __restrict__ in, cplx* __restrict__ out, int WL, int WR,
                               int D, int C, const int* __restrict__ off, const int* __restrict__ idx,
-                              const cplx* __restrict__ val) {
+                              const cplx* __restrict__ val, long long sa, long long sw) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   const int sv = blockIdx.y;
   const long long a = blockIdx.z;
@@ -313,7 +313,7 @@ __global__ void k_wstage_left(const cplx* __restrict__ in, cplx* __restrict__ ou
   cplx acc = mkc(0.0, 0.0);
   for (int e = off[sv]; e < off[sv + 1]; ++e) {
     const int w = idx[2 * e], t = idx[2 * e + 1];
-    cfma(acc, val[e], in[((a * WL + w) * D + t) * C + c]);
+    cfma(acc, val[e], in[((a * sa + w * sw) * D + t) * C + c]);
   }
   out[((a * D + s) * WR + v) * C + c] = acc;
 }
@@ -346,10 +346,11 @@ __global__ void k_permute_asb(const cplx* __restrict__ in, cplx* __restrict__ ou
 }
 }  // namespace
 
-void wstage_left(cudaStream_t st, const WSparse& w, const cplx* in, cplx* out, int A, int C) {
+void wstage_left(cudaStream_t st, const WSparse& w, const cplx* in, cplx* out, int A, int C, bool wa) {
   tdvp_require(A <= 65535, TDVP_ERR_INVALID_ARG, "wstage_left: too many rows");
   dim3 g(ceil_div(C, 128), w.d * w.wr, A);
-  k_wstage_left<<<g, 128, 0, st>>>(in, out, w.wl, w.wr, w.d, C, w.d_l_off, w.d_l_idx, w.d_l_val);
+  k_wstage_left<<<g, 128, 0, st>>>(in, out, w.wl, w.wr, w.d, C, w.d_l_off, w.d_l_idx, w.d_l_val, wa ? 1 : w.wl,
+                                   wa ? A : 1);
   TDVP_CHECK_LAUNCH();
 }
 

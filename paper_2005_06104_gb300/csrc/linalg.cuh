@@ -41,8 +41,9 @@ struct WSparse {
   void free_device();
 };
 
-// out[a][s][v][c] = sum_{(w,t)} W[w,s,t,v] in[a][w][t][c]      (A = rows a, C = cols c)
-void wstage_left(cudaStream_t st, const WSparse& w, const cplx* in, cplx* out, int A, int C);
+// out[a][s][v][c] = sum_{(w,t)} W[w,s,t,v] in[a][w][t][c]      (A = rows a, C = cols c); with wa the
+// rows of `in` are in (w, a) order
+void wstage_left(cudaStream_t st, const WSparse& w, const cplx* in, cplx* out, int A, int C, bool wa = false);
 // out[s][b][w][c] = sum_{(v,t)} W[w,s,t,v] in[b][v][t][c]
 void wstage_right(cudaStream_t st, const WSparse& w, const cplx* in, cplx* out, int B, int C);
 

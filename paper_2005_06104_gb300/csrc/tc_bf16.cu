@@ -899,7 +899,9 @@ TcSliceCache& slice_cache(Scratch& s) {
   if (!s.tcs) s.tcs = std::make_shared<TcSliceCache>();
   return *s.tcs;
 }
-int* tc_err(cudaStream_t st, Scratch& s) {
+}  // namespace
+
+int* tc_error_word(cudaStream_t st, Scratch& s) {
   TcEnvCache& c = s.tc;
   if (c.err.bytes() == 0) {
     c.err.ensure(s.pool, sizeof(int));
@@ -908,7 +910,6 @@ int* tc_err(cudaStream_t st, Scratch& s) {
   c.pending = true;
   return c.err.as<int>();
 }
-}  // namespace
 
 int bf16_slices(int precision) { return precision == TDVP_PREC_BF16X6 ? 3 : 4; }
 
@@ -923,7 +924,7 @@ void heff_bf16s(cudaStream_t st, Scratch& s, const SiteOp& op, const cplx* x, cp
   const int ml = op.ml, mr = op.mr, wl = op.wl, wr = op.wr, d = op.d;
   TcSliceCache& c = slice_cache(s);
   DevicePool* pool = s.pool;
-  int* err = tc_err(st, s);
+  int* err = tc_error_word(st, s);
   if (op.env_key < 0 || c.key != op.env_key || c.S != S) {
     // L as the A operand: rows (w, a), K = (a', re/im)
     c.L.shape(pool, S, ml * wl, 2 * ml, false);
@@ -953,7 +954,7 @@ void zgemm_bf16s(cudaStream_t st, Scratch& s, int S, int opA, int opB, int M, in
                  long long lda, const cplx* B, long long ldb, cplx* C, long long ldc) {
   if (M <= 0 || N <= 0) return;
   DevicePool* pool = s.pool;
-  int* err = tc_err(st, s);
+  int* err = tc_error_word(st, s);
   Sliced a, b;
   a.shape(pool, S, M, 2 * std::max(K, 1), false);
   slice(st, SrcA{A, lda, M, K, opA}, a);

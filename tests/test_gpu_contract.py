@@ -268,3 +268,63 @@ def test_fp64_tiles_match_oracle(g, ml, mr, w):
     yd = torch.empty_like(xd)
     g.keff_contract(Ld, Rd, xd, yd)
     assert _rel(yd.cpu().numpy(), O.keff_apply(L, R, x)) < TOL64
+
+
+# FP64 products on the tensor cores (exact 8-bit digits): each result is held to 5e-15 of the
+# reference's norm.  The digits keep 56 bits below each row's largest entry and products to 2^-56
+# of the row maxima, 2.4e-16 norm-wise per product for Gaussian rows; two products are chained,
+# and the reference (numpy, FP64 sums of up to 14 * 400 terms) carries up to 2e-15 of its own.
+TOL_DIGITS = 5e-15
+DIGIT_SHAPES = [(64, 64, 14), (127, 129, 14), (128, 128, 8), (255, 130, 14), (70, 400, 5), (300, 96, 8)]
+
+
+@pytest.mark.parametrize("ml,mr,w", DIGIT_SHAPES)
+def test_fp64_digits_keff(g, ml, mr, w):
+    rng = np.random.default_rng(ml + mr)
+    L, R, x = _rand(rng, ml, w, ml), _rand(rng, mr, w, mr), _rand(rng, ml, mr)
+    Ld, Rd, xd = _dev(L, R, x)
+    yd = torch.empty_like(xd)
+    g.keff_contract(Ld, Rd, xd, yd)
+    assert _rel(yd.cpu().numpy(), O.keff_apply(L, R, x)) < TOL_DIGITS
+
+
+@pytest.mark.parametrize("ml,mr", [(96, 130), (129, 127), (64, 257)])
+def test_fp64_digits_site(g, ml, mr):
+    """H_eff and both environment updates (plain, transposed and conjugated operands)."""
+    rng = np.random.default_rng(ml)
+    W = W_CYL[10]
+    L, R, A = _rand(rng, ml, W.shape[0], ml), _rand(rng, mr, W.shape[3], mr), _rand(rng, ml, 2, mr)
+    Ld, Rd, Ad = _dev(L, R, A)
+    y, Lo, Ro = torch.empty_like(Ad), torch.empty(mr, W.shape[3], mr, dtype=Ad.dtype, device="cuda"), torch.empty_like(Ld)
+    g.heff_contract(Ld, W, Rd, Ad, y)
+    g.env_contract(0, Ld, W, Ad, Lo)
+    g.env_contract(1, Rd, W, Ad, Ro)
+    assert _rel(y.cpu().numpy(), O.heff_apply(L, W, R, A)) < TOL_DIGITS
+    assert _rel(Lo.cpu().numpy(), O.env_left_step(L, A, W)) < TOL_DIGITS
+    assert _rel(Ro.cpu().numpy(), O.env_right_step(R, A, W)) < TOL_DIGITS
+
+
+def test_fp64_digits_ranges_zeros_and_non_finite(g):
+    """Rows over hundreds of orders of magnitude keep their relative accuracy, zero rows and
+    columns stay exact zeros, a NaN or infinity reaches the outputs it reaches in FP64."""
+    rng = np.random.default_rng(3)
+    m, w = 160, 5
+    L, R, x = _rand(rng, m, w, m), _rand(rng, m, w, m), _rand(rng, m, m)
+    scale = 10.0 ** rng.integers(-140, 140, size=m)
+    L *= scale[:, None, None]
+    L[7], R[9] = 0.0, 0.0
+    Ld, Rd, xd = _dev(L, R, x)
+    yd = torch.empty_like(xd)
+    g.keff_contract(Ld, Rd, xd, yd)
+    got, ref = yd.cpu().numpy(), O.keff_apply(L / scale[:, None, None], R, x)
+    live = np.arange(m) != 7
+    assert np.all(got[7] == 0.0) and np.all(got[:, 9] == 0.0)
+    assert _rel((got / scale[:, None])[live], ref[live]) < TOL_DIGITS
+    Ld[5, 2, 3] = float("nan")
+    Rd[11, 1, 4] = float("inf")
+    g.keff_contract(Ld, Rd, xd, yd)
+    bad = ~np.isfinite(yd.cpu().numpy())
+    expect = np.zeros((m, m), dtype=bool)
+    expect[5], expect[:, 11] = True, True
+    expect[7, 11] = bad[7, 11]      # 0 * inf
+    assert np.array_equal(bad, expect)
