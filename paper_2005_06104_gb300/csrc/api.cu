@@ -448,11 +448,11 @@ void check_dims(const tdvp_site_dims* d) {
                "dims must be >= 1");
 }
 
-WSparse make_w(const tdvp_site_dims* d, const double* W_host) {
+WSparse make_w(cudaStream_t st, DevicePool* pool, const tdvp_site_dims* d, const double* W_host) {
   tdvp_require(W_host != nullptr, TDVP_ERR_INVALID_ARG, "null W");
   WSparse w;
   w.build(reinterpret_cast<const cplx*>(W_host), d->wl, d->wr, d->d);
-  w.upload();
+  w.upload(st, pool);
   return w;
 }
 }  // namespace
@@ -473,7 +473,7 @@ tdvp_status tdvp_heff_contract_cached(const tdvp_site_dims* dims, const void* L,
     tdvp_require(precision >= TDVP_PREC_FP64 && precision <= TDVP_PREC_BF16X6, TDVP_ERR_INVALID_ARG,
                  "unknown precision");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    WSparse w = make_w(dims, W);
+    WSparse w = make_w(st, &c.pool, dims, W);
     SiteOp op;
     op.L = static_cast<const cplx*>(L);
     op.R = static_cast<const cplx*>(R);
@@ -488,7 +488,6 @@ tdvp_status tdvp_heff_contract_cached(const tdvp_site_dims* dims, const void* L,
     op.env_key = precision == TDVP_PREC_FP64 ? -1 : env_tag;  // FP64 ignores the tag
     heff_apply_prec(st, c.scr, op, static_cast<const cplx*>(x), static_cast<cplx*>(y), precision);
     TDVP_CUDA(cudaStreamSynchronize(st));
-    w.free_device();
     tc_check(st, c.scr);
   });
 }
@@ -513,7 +512,7 @@ tdvp_status tdvp_env_contract(const tdvp_site_dims* dims, int side, const void* 
     tdvp_require(E && A && out && E != out, TDVP_ERR_INVALID_ARG, "null or aliased buffers");
     tdvp_require(side == 0 || side == 1, TDVP_ERR_INVALID_ARG, "side must be 0 or 1");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    WSparse w = make_w(dims, W);
+    WSparse w = make_w(st, &c.pool, dims, W);
     if (side == 0)
       env_left_fp64(st, c.scr, static_cast<const cplx*>(E), w, static_cast<const cplx*>(A), dims->ml, dims->mr,
                     dims->d, static_cast<cplx*>(out));
@@ -521,7 +520,6 @@ tdvp_status tdvp_env_contract(const tdvp_site_dims* dims, int side, const void* 
       env_right_fp64(st, c.scr, static_cast<const cplx*>(E), w, static_cast<const cplx*>(A), dims->ml, dims->mr,
                      dims->d, static_cast<cplx*>(out));
     TDVP_CUDA(cudaStreamSynchronize(st));
-    w.free_device();
     tc_check(st, c.scr);
   });
 }
@@ -538,7 +536,7 @@ tdvp_status tdvp_expm_contract(const tdvp_site_dims* dims, const void* L, const 
     tdvp_require(tol > 0 && nmax >= 1 && nmax <= 63 && std::isfinite(delta), TDVP_ERR_INVALID_ARG,
                  "bad Lanczos parameters");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    WSparse w = make_w(dims, W);
+    WSparse w = make_w(st, &c.pool, dims, W);
     SiteOp op;
     op.L = static_cast<const cplx*>(L);
     op.R = static_cast<const cplx*>(R);
@@ -556,12 +554,10 @@ tdvp_status tdvp_expm_contract(const tdvp_site_dims* dims, const void* L, const 
           st, &c.pool, c.blas, c.lw, [&](const cplx* a, cplx* b) { heff_apply_prec(st, c.scr, op, a, b, precision); },
           static_cast<const cplx*>(x), static_cast<cplx*>(y), n, delta, kind, tol, nmax);
     } catch (...) {
-      w.free_device();
       tc_check(st, c.scr);
       throw;
     }
     TDVP_CUDA(cudaStreamSynchronize(st));
-    w.free_device();
     tc_check(st, c.scr);
     if (iters) *iters = it;
   });

@@ -4,7 +4,9 @@
 #include <atomic>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <cstdint>
 #include <cstdio>
 #include <map>
@@ -69,8 +71,12 @@ inline void tdvp_require(bool ok, tdvp_status s, const std::string& msg) {
 // ---------------------------------------------------------------------------
 // Caching device allocator: blocks are rounded up to a power of two (>= 4 KiB)
 // and recycled per size class, so steady-state sweeps never call cudaMalloc.
+// Blocks up to 256 KiB are cut from 4 MiB slabs: a new handle needs some hundred of them, and
+// a cudaMalloc is 2 us alone but over 100 us while other threads launch (four chains created,
+// stepped and destroyed: 170 ms of cudaMalloc in a pass).  Slabs go back with the pool.
 class DevicePool {
  public:
+  static constexpr size_t kSlab = size_t(4) << 20, kSlabBlock = size_t(256) << 10;
   void* get(size_t bytes) {
     size_t cls = size_class(bytes);
     auto& fl = free_[cls];
@@ -79,29 +85,44 @@ class DevicePool {
       fl.pop_back();
       return p;
     }
-    void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, cls);
-    if (e != cudaSuccess) {
-      (void)cudaGetLastError();
-      trim();
-      TDVP_CUDA(cudaMalloc(&p, cls));
+    if (cls <= kSlabBlock) {
+      if (slab_left_ < cls) {
+        // the rest of the old slab (multiples of 4 KiB) stays in use as smaller blocks
+        for (size_t c = kSlabBlock; c >= 4096; c >>= 1)
+          while (slab_left_ >= c) {
+            free_[c].push_back(slab_);
+            slab_ += c;
+            slab_left_ -= c;
+          }
+        slab_ = static_cast<char*>(from_device(kSlab));
+        slabs_.push_back(slab_);
+        slab_left_ = kSlab;
+      }
+      void* p = slab_;
+      slab_ += cls;
+      slab_left_ -= cls;
+      return p;
     }
-    live_bytes_ += cls;
-    return p;
+    return from_device(cls);
   }
   void put(void* p, size_t bytes) {
     if (p) free_[size_class(bytes)].push_back(p);
   }
+  // returns the cached blocks that are allocations of their own to the device
   void trim() {
-    for (auto& kv : free_)
-      for (void* p : kv.second) {
-        cudaFree(p);
-        live_bytes_ -= kv.first;
-      }
-    free_.clear();
+    for (auto& kv : free_) {
+      if (kv.first <= kSlabBlock) continue;
+      for (void* p : kv.second) cudaFree(p);
+      kv.second.clear();
+    }
   }
-  ~DevicePool() { trim(); }
-  size_t live_bytes() const { return live_bytes_; }
+  DevicePool() = default;
+  DevicePool(const DevicePool&) = delete;
+  DevicePool& operator=(const DevicePool&) = delete;
+  ~DevicePool() {
+    trim();
+    for (void* p : slabs_) cudaFree(p);
+  }
   // bytes held in the free lists (allocated from the device, not in use)
   size_t cached_bytes() const {
     size_t b = 0;
@@ -122,8 +143,19 @@ class DevicePool {
   }
 
  private:
+  void* from_device(size_t bytes) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      (void)cudaGetLastError();
+      trim();
+      TDVP_CUDA(cudaMalloc(&p, bytes));
+    }
+    return p;
+  }
   std::map<size_t, std::vector<void*>> free_;
-  size_t live_bytes_ = 0;
+  std::vector<void*> slabs_;
+  char* slab_ = nullptr;
+  size_t slab_left_ = 0;
 };
 
 // A device array of complex numbers drawn from a pool (RAII).
@@ -182,7 +214,20 @@ class RawBuf {
   RawBuf() = default;
   RawBuf(const RawBuf&) = delete;
   RawBuf& operator=(const RawBuf&) = delete;
+  RawBuf(RawBuf&& o) noexcept { swap(o); }
+  RawBuf& operator=(RawBuf&& o) noexcept {
+    if (this != &o) {
+      release();
+      swap(o);
+    }
+    return *this;
+  }
   ~RawBuf() { release(); }
+  void swap(RawBuf& o) {
+    std::swap(p_, o.p_);
+    std::swap(bytes_, o.bytes_);
+    std::swap(pool_, o.pool_);
+  }
   void ensure(DevicePool* pool, size_t bytes) {
     if (p_ && DevicePool::size_class(bytes) == DevicePool::size_class(bytes_)) {
       bytes_ = bytes;
@@ -206,6 +251,38 @@ class RawBuf {
   void* p_ = nullptr;
   size_t bytes_ = 0;
   DevicePool* pool_ = nullptr;
+};
+
+// Host data of several arrays for one device buffer: parts at 256-byte offsets, one copy.  The
+// copy is from pageable memory, so the host data may go once upload() has returned.
+class Packed {
+ public:
+  template <class T>
+  size_t add(const T* p, size_t n) {
+    const size_t at = bytes_.size();
+    bytes_.resize(at + ((n * sizeof(T) + 255) & ~size_t(255)));
+    if (n) std::memcpy(bytes_.data() + at, p, n * sizeof(T));
+    return at;
+  }
+  template <class T>
+  size_t add(const std::vector<T>& v) {
+    return add(v.data(), v.size());
+  }
+  size_t zeros(size_t n) {  // n zero bytes
+    const size_t at = bytes_.size();
+    bytes_.resize(at + ((n + 255) & ~size_t(255)));
+    return at;
+  }
+  size_t size() const { return bytes_.size(); }
+  char* upload(cudaStream_t st, DevicePool* pool, RawBuf& buf) const {
+    buf.ensure(pool, std::max<size_t>(bytes_.size(), 256));
+    if (!bytes_.empty())
+      TDVP_CUDA(cudaMemcpyAsync(buf.as<char>(), bytes_.data(), bytes_.size(), cudaMemcpyHostToDevice, st));
+    return buf.as<char>();
+  }
+
+ private:
+  std::vector<char> bytes_;
 };
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }

@@ -191,7 +191,7 @@ void Engine::init(const tdvp_mps_desc* mps, const tdvp_mpo_desc* mpo, const tdvp
     for (const cplx& x : W_host[i])
       tdvp_require(std::isfinite(x.x) && std::isfinite(x.y), TDVP_ERR_NONFINITE, "non-finite MPO entry");
     Wsp[i].build(W_host[i].data(), w[i], w[i + 1], d);
-    Wsp[i].upload();
+    Wsp[i].upload(st, &pool);
   }
   L.resize(N);
   R.resize(N);
@@ -207,8 +207,6 @@ void Engine::init(const tdvp_mps_desc* mps, const tdvp_mpo_desc* mpo, const tdvp
 }
 
 void Engine::release() {
-  for (auto& ws : Wsp) ws.free_device();
-  for (auto& ws : Wsp2) ws.free_device();
   lw.release();
   blas.release();
   for (auto& p : ev_pairs) {
@@ -329,7 +327,7 @@ void Engine::build_pair_mpo() {
                 }
           }
     Wsp2[i].build(W2.data(), wl, wr, D);
-    Wsp2[i].upload();
+    Wsp2[i].upload(st, &pool);
   }
 }
 
@@ -778,11 +776,12 @@ void Engine::build_krylov_op(KrylovOp& kop) {
   kop.om_off.resize(N);
   kop.om_idx.resize(N);
   kop.om_val.resize(N);
+  kop.om.resize(N);
   for (int i = 0; i < N; ++i) {
     const int wl = w[i], wr = w[i + 1];
     auto h = one_minus_itau_h_site(W_host[i], i, N, wl, wr, d, opt.tau_re, opt.tau_im);
     kop.Wsp[i].build(h.data(), wl, wr, d);
-    kop.Wsp[i].upload();
+    kop.Wsp[i].upload(st, &pool);
     // Om[(w,wb),(t,v,tb,vb)] = sum_s W[w,s,t,v] conj(W[wb,s,tb,vb]), kept where nonzero
     std::vector<int> off(wl * wl + 1, 0), idx;
     std::vector<cplx> val;
@@ -802,27 +801,13 @@ void Engine::build_krylov_op(KrylovOp& kop) {
               }
         off[ww * wl + wb + 1] = (int)val.size();
       }
-    auto up = [&](auto& vec, auto** dst) {
-      using T = typename std::remove_reference<decltype(vec)>::type::value_type;
-      TDVP_CUDA(cudaMalloc((void**)dst, std::max<size_t>(1, vec.size()) * sizeof(T)));
-      if (!vec.empty())
-        TDVP_CUDA(cudaMemcpy(*dst, vec.data(), vec.size() * sizeof(T), cudaMemcpyHostToDevice));
-    };
-    up(off, &kop.om_off[i]);
-    up(idx, &kop.om_idx[i]);
-    up(val, &kop.om_val[i]);
+    Packed pk;
+    const size_t o_off = pk.add(off), o_idx = pk.add(idx), o_val = pk.add(val);
+    char* base = pk.upload(st, &pool, kop.om[i]);
+    kop.om_off[i] = reinterpret_cast<int*>(base + o_off);
+    kop.om_idx[i] = reinterpret_cast<int*>(base + o_idx);
+    kop.om_val[i] = reinterpret_cast<cplx*>(base + o_val);
   }
-}
-
-void KrylovOp::release() {
-  for (auto& ws : Wsp) ws.free_device();
-  for (auto* p : om_off) cudaFree(p);
-  for (auto* p : om_idx) cudaFree(p);
-  for (auto* p : om_val) cudaFree(p);
-  om_off.clear();
-  om_idx.clear();
-  om_val.clear();
-  Wsp.clear();
 }
 
 // One Krylov vector by the density-matrix approach (Sec. I.B): out = (1 - i tau H) src
@@ -1207,7 +1192,7 @@ void Engine::expand_basis(int k, const double* weights) {
       const std::vector<int> perm = sector_row_order(st, &pool, Bp.data(), mnew, cols);
       if (!perm.empty()) {
         DArr B2(&pool, (size_t)mnew * cols);
-        gather_rows(st, Bp.data(), mnew, cols, perm, B2.data());
+        gather_rows(st, &pool, Bp.data(), mnew, cols, perm, B2.data());
         Bp = std::move(B2);
       }
     }
@@ -1236,7 +1221,6 @@ void Engine::expand_basis(int k, const double* weights) {
     psi.A[i - 1] = std::move(prv);
     psi.m[i] = mnew;
   }
-  kop.release();
   center = 0;
   for (int j = 0; j < N; ++j) Lok[j] = Rok[j] = 0;
   sync();
@@ -1250,7 +1234,6 @@ void Engine::apply_krylov() {
   MpsDev out;
   disc_k = 0.0;
   krylov_apply(kop, psi, out);
-  kop.release();
   psi.m = out.m;
   for (int i = 0; i < N; ++i) psi.A[i] = std::move(out.A[i]);
   center = N - 1;
@@ -1325,12 +1308,10 @@ cplx Engine::expect_mpo(const tdvp_mpo_desc* op) {
       tdvp_require(std::isfinite(Wi[e].x) && std::isfinite(Wi[e].y), TDVP_ERR_NONFINITE, "non-finite MPO entry");
     WSparse ws;
     ws.build(Wi, wo[i], wo[i + 1], d);
-    ws.upload();
+    ws.upload(st, &pool);
     const int ml = psi.m[i], mr = psi.m[i + 1];
     En.reset(&pool, (size_t)mr * wo[i + 1] * mr);
     env_left_fp64(st, scr, E.data(), ws, psi.A[i].data(), ml, mr, d, En.data(), TDVP_PREC_FP64);
-    sync();
-    ws.free_device();
     E = std::move(En);
   }
   cplx v;

@@ -23,7 +23,7 @@ struct KrylovOp {
   std::vector<WSparse> Wsp;
   std::vector<int*> om_off, om_idx;
   std::vector<cplx*> om_val;
-  void release();
+  std::vector<RawBuf> om;  // the three arrays above, one buffer per site
 };
 
 struct Engine {

@@ -96,7 +96,7 @@ extern "C" tdvp_status tdvp_heff_contract_noalloc(const tdvp_site_dims* dims, co
       TDVP_CUDA(cudaMemcpyAsync(d_idx, h_idx, sizeof(int) * 2 * nnz, cudaMemcpyHostToDevice, st));
       TDVP_CUDA(cudaMemcpyAsync(d_val, h_val, sizeof(cplx) * nnz, cudaMemcpyHostToDevice, st));
     }
-    WSparse ws;  // views into the fixed array; never uploaded or freed (free_device is never called)
+    WSparse ws;  // views into the fixed array; never uploaded
     ws.wl = wl;
     ws.wr = wr;
     ws.d = d;

@@ -266,39 +266,23 @@ void WSparse::build(const cplx* W, int wl_, int wr_, int d_) {
   nnz = (int)l_val.size();
 }
 
-void WSparse::upload() {
-  free_device();
-  auto up = [](auto& vec, auto** dst) {
-    using T = typename std::remove_reference<decltype(vec)>::type::value_type;
-    size_t bytes = std::max<size_t>(1, vec.size()) * sizeof(T);
-    TDVP_CUDA(cudaMalloc((void**)dst, bytes));
-    if (!vec.empty()) TDVP_CUDA(cudaMemcpy(*dst, vec.data(), vec.size() * sizeof(T), cudaMemcpyHostToDevice));
-  };
-  up(l_off, &d_l_off);
-  up(l_idx, &d_l_idx);
-  up(l_val, &d_l_val);
+void WSparse::upload(cudaStream_t st, DevicePool* pool) {
   l_val_df.resize(l_val.size());
   for (size_t e = 0; e < l_val.size(); ++e) {
     const float rh = (float)l_val[e].x, ih = (float)l_val[e].y;
     l_val_df[e] = make_float4(rh, (float)(l_val[e].x - (double)rh), ih, (float)(l_val[e].y - (double)ih));
   }
-  up(l_val_df, &d_l_val_df);
-  up(r_off, &d_r_off);
-  up(r_idx, &d_r_idx);
-  up(r_val, &d_r_val);
-}
-
-void WSparse::free_device() {
-  cudaFree(d_l_off);
-  cudaFree(d_l_idx);
-  cudaFree(d_l_val);
-  cudaFree(d_l_val_df);
-  d_l_val_df = nullptr;
-  cudaFree(d_r_off);
-  cudaFree(d_r_idx);
-  cudaFree(d_r_val);
-  d_l_off = d_l_idx = d_r_off = d_r_idx = nullptr;
-  d_l_val = d_r_val = nullptr;
+  Packed pk;
+  const size_t o[7] = {pk.add(l_off), pk.add(l_idx), pk.add(l_val), pk.add(l_val_df),
+                       pk.add(r_off), pk.add(r_idx), pk.add(r_val)};
+  char* base = pk.upload(st, pool, dev);
+  d_l_off = reinterpret_cast<int*>(base + o[0]);
+  d_l_idx = reinterpret_cast<int*>(base + o[1]);
+  d_l_val = reinterpret_cast<cplx*>(base + o[2]);
+  d_l_val_df = reinterpret_cast<float4*>(base + o[3]);
+  d_r_off = reinterpret_cast<int*>(base + o[4]);
+  d_r_idx = reinterpret_cast<int*>(base + o[5]);
+  d_r_val = reinterpret_cast<cplx*>(base + o[6]);
 }
 
 namespace {
@@ -1422,8 +1406,9 @@ void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows,
   const double tol = std::max(1e-15, std::sqrt((double)p) * 2.2e-16);
   const int max_sweeps = 60;
   const size_t small_bytes = ((size_t)p * q + (need_acc ? (size_t)q * q : 0)) * sizeof(cplx);
-  int* d_flag = nullptr;
-  TDVP_CUDA(cudaMallocAsync(&d_flag, sizeof(int) + sizeof(double) * 2, st));
+  RawBuf flag_buf, bar_buf, s_buf, perm_buf, ss_buf;
+  flag_buf.ensure(pool, 256);
+  int* d_flag = flag_buf.as<int>();
   double* d_fro2 = reinterpret_cast<double*>(d_flag + 2);
   k_fro2<<<1, 256, 0, st>>>(X.data(), (long long)p * q, d_fro2);
   TDVP_CHECK_LAUNCH();
@@ -1442,7 +1427,6 @@ void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows,
       TDVP_CUDA(cudaMemcpyAsync(&sweeps, d_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
       TDVP_CUDA(cudaStreamSynchronize(st));
       if (sweeps > max_sweeps) {
-        cudaFreeAsync(d_flag, st);
         throw TdvpError(TDVP_ERR_SVD_NOT_CONVERGED, "Jacobi SVD did not converge");
       }
     } else {
@@ -1454,8 +1438,8 @@ void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows,
         return std::max(1, sms * std::max(1, per_sm));
       }();
       const int nblk = std::max(1, std::min(qpad / 2, coop_blocks));
-      GridBar* bar = nullptr;
-      TDVP_CUDA(cudaMallocAsync(&bar, sizeof(GridBar), st));
+      bar_buf.ensure(pool, sizeof(GridBar));
+      GridBar* bar = bar_buf.as<GridBar>();
       TDVP_CUDA(cudaMemsetAsync(bar, 0, sizeof(GridBar), st));
       cplx* xp = X.data();
       cplx* vp = Vx.data();
@@ -1469,24 +1453,20 @@ void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows,
       TDVP_CUDA(cudaMemcpyAsync(&sweeps, d_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
       TDVP_CUDA(cudaMemcpyAsync(&hb, bar, sizeof(GridBar), cudaMemcpyDeviceToHost, st));
       TDVP_CUDA(cudaStreamSynchronize(st));
-      TDVP_CUDA(cudaFreeAsync(bar, st));
       if (hb.err) {
-        cudaFreeAsync(d_flag, st);
         throw TdvpError(TDVP_ERR_TIMEOUT, "Jacobi SVD: a grid barrier wait ran out");
       }
       if (sweeps > max_sweeps) {
-        cudaFreeAsync(d_flag, st);
         throw TdvpError(TDVP_ERR_SVD_NOT_CONVERGED, "Jacobi SVD did not converge");
       }
     }
   }
-  TDVP_CUDA(cudaFreeAsync(d_flag, st));
   out.sweeps = sweeps;
   g_svd_counters.sweeps += sweeps;
   atomic_max(g_svd_counters.max_sweeps, sweeps);
   // singular values = column norms
-  double* d_s = nullptr;
-  TDVP_CUDA(cudaMallocAsync(&d_s, sizeof(double) * q, st));
+  s_buf.ensure(pool, sizeof(double) * q);
+  double* d_s = s_buf.as<double>();
   k_colnorms<<<q, 256, 0, st>>>(X.data(), p, q, d_s);
   TDVP_CHECK_LAUNCH();
   std::vector<double> s(q);
@@ -1501,14 +1481,11 @@ void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows,
   for (int r = 0; r < q; ++r) out.s[r] = s[perm[r]];
   const int keep = std::max(0, std::min(q, select(out.s, ctx)));
   out.rank = keep;
-  if (keep == 0) {
-    cudaFreeAsync(d_s, st);
-    return;
-  }
-  int* d_perm = nullptr;
-  double* d_ss = nullptr;
-  TDVP_CUDA(cudaMallocAsync(&d_perm, sizeof(int) * keep, st));
-  TDVP_CUDA(cudaMallocAsync(&d_ss, sizeof(double) * keep, st));
+  if (keep == 0) return;
+  perm_buf.ensure(pool, sizeof(int) * keep);
+  ss_buf.ensure(pool, sizeof(double) * keep);
+  int* d_perm = perm_buf.as<int>();
+  double* d_ss = ss_buf.as<double>();
   TDVP_CUDA(cudaMemcpyAsync(d_perm, perm.data(), sizeof(int) * keep, cudaMemcpyHostToDevice, st));
   TDVP_CUDA(cudaMemcpyAsync(d_ss, out.s.data(), sizeof(double) * keep, cudaMemcpyHostToDevice, st));
   if (want_u) {
@@ -1533,9 +1510,6 @@ void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows,
                                                       out.Vh.data());
     TDVP_CHECK_LAUNCH();
   }
-  TDVP_CUDA(cudaFreeAsync(d_perm, st));
-  TDVP_CUDA(cudaFreeAsync(d_ss, st));
-  TDVP_CUDA(cudaFreeAsync(d_s, st));
 }
 
 // ============================================================================
@@ -2191,7 +2165,7 @@ __global__ void k_to_c128(const float2* __restrict__ in, cplx* __restrict__ out,
   if (e < n) out[e] = mkc((double)in[e].x, (double)in[e].y);
 }
 
-void run_pchol_groups(cudaStream_t st, cplx* Xs, BlkDesc* d_desc, int* d_piv, std::vector<int> gsz) {
+void run_pchol_groups(cudaStream_t st, DevicePool* pool, cplx* Xs, BlkDesc* d_desc, int* d_piv, std::vector<int> gsz) {
   const int nblk = (int)gsz.size();
   static const int max_ctas = [] {
     int dev = 0, sms = 0, per_sm = 0;
@@ -2209,18 +2183,16 @@ void run_pchol_groups(cudaStream_t st, cplx* Xs, BlkDesc* d_desc, int* d_piv, st
   for (int b = 0; b < nblk; ++b) cta_off[b + 1] = cta_off[b] + gsz[b];
   const int nctas = cta_off[nblk];
   tdvp_require(nctas <= budget, TDVP_ERR_INVALID_ARG, "Cholesky groups exceed the co-resident CTAs");
-  int* d_off = nullptr;
-  int* d_idx = nullptr;
-  double* d_val = nullptr;
-  GridBar* bars = nullptr;
-  TDVP_CUDA(cudaMallocAsync(&d_off, sizeof(int) * (nblk + 1), st));
-  TDVP_CUDA(cudaMallocAsync(&d_idx, sizeof(int) * (nctas + 1), st));  // + the error word
-  TDVP_CUDA(cudaMallocAsync(&d_val, sizeof(double) * nctas, st));
-  TDVP_CUDA(cudaMallocAsync(&bars, sizeof(GridBar) * nblk, st));
-  int* d_gerr = d_idx + nctas;
-  TDVP_CUDA(cudaMemsetAsync(bars, 0, sizeof(GridBar) * nblk, st));
-  TDVP_CUDA(cudaMemsetAsync(d_gerr, 0, sizeof(int), st));
-  TDVP_CUDA(cudaMemcpyAsync(d_off, cta_off.data(), sizeof(int) * (nblk + 1), cudaMemcpyHostToDevice, st));
+  Packed pk;
+  const size_t o_off = pk.add(cta_off), o_bar = pk.zeros(sizeof(GridBar) * nblk), o_err = pk.zeros(sizeof(int)),
+               o_idx = pk.zeros(sizeof(int) * nctas), o_val = pk.zeros(sizeof(double) * nctas);
+  RawBuf meta;
+  char* base = pk.upload(st, pool, meta);
+  int* d_off = reinterpret_cast<int*>(base + o_off);
+  int* d_idx = reinterpret_cast<int*>(base + o_idx);
+  double* d_val = reinterpret_cast<double*>(base + o_val);
+  GridBar* bars = reinterpret_cast<GridBar*>(base + o_bar);
+  int* d_gerr = reinterpret_cast<int*>(base + o_err);
   int nb = nblk;
   double rel = 1e-15;
   const int* po = d_off;
@@ -2230,15 +2202,11 @@ void run_pchol_groups(cudaStream_t st, cplx* Xs, BlkDesc* d_desc, int* d_piv, st
   int herr = 0;
   TDVP_CUDA(cudaMemcpyAsync(&herr, d_gerr, sizeof(int), cudaMemcpyDeviceToHost, st));
   TDVP_CUDA(cudaStreamSynchronize(st));
-  TDVP_CUDA(cudaFreeAsync(d_off, st));
-  TDVP_CUDA(cudaFreeAsync(d_idx, st));
-  TDVP_CUDA(cudaFreeAsync(d_val, st));
-  TDVP_CUDA(cudaFreeAsync(bars, st));
   if (herr) throw TdvpError(TDVP_ERR_TIMEOUT, "pivoted Cholesky: a group barrier wait ran out");
 }
 
 template <class T>
-void run_jacobi_multi(cudaStream_t st, typename Jac<T>::C* Xs, typename Jac<T>::C* Vs,
+void run_jacobi_multi(cudaStream_t st, DevicePool* pool, typename Jac<T>::C* Xs, typename Jac<T>::C* Vs,
                       const std::vector<BlkDesc>& desc, const BlkDesc* d_desc, double* d_s, int* d_stat) {
   const int nblk = (int)desc.size();
   static const int max_ctas = [] {
@@ -2264,20 +2232,17 @@ void run_jacobi_multi(cudaStream_t st, typename Jac<T>::C* Xs, typename Jac<T>::
   }
   tdvp_require(cta_off[nblk] <= budget, TDVP_ERR_INVALID_ARG, "Jacobi groups exceed the co-resident CTAs");
   const int nctas = cta_off[nblk];
-  int* d_off = nullptr;
-  int* d_flags = nullptr;
-  int* d_gerr = nullptr;
-  double* d_fro2 = nullptr;
-  GridBar* bars = nullptr;
-  TDVP_CUDA(cudaMallocAsync(&d_off, sizeof(int) * (nblk + 1), st));
-  TDVP_CUDA(cudaMallocAsync(&d_flags, sizeof(int) * 4 * nblk + sizeof(int), st));
-  TDVP_CUDA(cudaMallocAsync(&d_fro2, sizeof(double) * nblk, st));
-  TDVP_CUDA(cudaMallocAsync(&bars, sizeof(GridBar) * nblk, st));
-  d_gerr = d_flags + 4 * nblk;
-  TDVP_CUDA(cudaMemsetAsync(bars, 0, sizeof(GridBar) * nblk, st));
-  TDVP_CUDA(cudaMemsetAsync(d_flags, 0, sizeof(int) * 4 * nblk + sizeof(int), st));
+  Packed pk;
+  const size_t o_off = pk.add(cta_off), o_flags = pk.zeros(sizeof(int) * (4 * nblk + 1)),
+               o_bar = pk.zeros(sizeof(GridBar) * nblk), o_fro = pk.zeros(sizeof(double) * nblk);
+  RawBuf meta;
+  char* base = pk.upload(st, pool, meta);
+  int* d_off = reinterpret_cast<int*>(base + o_off);
+  int* d_flags = reinterpret_cast<int*>(base + o_flags);
+  int* d_gerr = d_flags + 4 * nblk;
+  double* d_fro2 = reinterpret_cast<double*>(base + o_fro);
+  GridBar* bars = reinterpret_cast<GridBar*>(base + o_bar);
   TDVP_CUDA(cudaMemsetAsync(d_stat, 0, 3 * sizeof(int), st));
-  TDVP_CUDA(cudaMemcpyAsync(d_off, cta_off.data(), sizeof(int) * (nblk + 1), cudaMemcpyHostToDevice, st));
   int nb = nblk, ms = 60;
   const BlkDesc* dd = d_desc;
   const int* po = d_off;
@@ -2287,10 +2252,6 @@ void run_jacobi_multi(cudaStream_t st, typename Jac<T>::C* Xs, typename Jac<T>::
   int herr = 0;
   TDVP_CUDA(cudaMemcpyAsync(&herr, d_gerr, sizeof(int), cudaMemcpyDeviceToHost, st));
   TDVP_CUDA(cudaStreamSynchronize(st));
-  TDVP_CUDA(cudaFreeAsync(d_off, st));
-  TDVP_CUDA(cudaFreeAsync(d_flags, st));
-  TDVP_CUDA(cudaFreeAsync(d_fro2, st));
-  TDVP_CUDA(cudaFreeAsync(bars, st));
   if (herr) throw TdvpError(TDVP_ERR_TIMEOUT, "Jacobi SVD: a group barrier wait ran out");
 }
 }  // namespace
@@ -2389,15 +2350,15 @@ std::vector<int> sector_row_order(cudaStream_t st, DevicePool* pool, const cplx*
   return perm;
 }
 
-void gather_rows(cudaStream_t st, const cplx* M, int rows, int cols, const std::vector<int>& perm, cplx* out) {
+void gather_rows(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols, const std::vector<int>& perm, cplx* out) {
   tdvp_require((int)perm.size() == rows, TDVP_ERR_INVALID_ARG, "gather_rows: permutation length");
-  int* d_perm = nullptr;
-  TDVP_CUDA(cudaMallocAsync(&d_perm, sizeof(int) * rows, st));
+  RawBuf buf;
+  buf.ensure(pool, sizeof(int) * rows);
+  int* d_perm = buf.as<int>();
   TDVP_CUDA(cudaMemcpyAsync(d_perm, perm.data(), sizeof(int) * rows, cudaMemcpyHostToDevice, st));
   const long long n = (long long)rows * cols;
   k_gather_rows<<<(int)std::min<long long>(ceil_div(n, 256), 152 * 16), 256, 0, st>>>(M, cols, d_perm, rows, out);
   TDVP_CHECK_LAUNCH();
-  TDVP_CUDA(cudaFreeAsync(d_perm, st));
 }
 
 void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols,
@@ -2474,6 +2435,7 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
   BlkDesc* d_desc = nullptr;
   int *d_ridx = nullptr, *d_cidx = nullptr, *d_bad = nullptr, *d_piv = nullptr;
   double* d_s = nullptr;
+  RawBuf meta, sel_buf;
   psd = psd && rows == cols && !want_v;
   // the factorisation reads each block as a square n x n matrix: a Hermitian pattern
   // gives square blocks; anything else takes the plain SVD (same eigen data for PSD)
@@ -2481,15 +2443,17 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
   if (nsmall) {
     Xs.reset(pool, (size_t)std::max<long long>(1, xo));
     Vs.reset(pool, (size_t)std::max<long long>(1, vo));
-    TDVP_CUDA(cudaMallocAsync(&d_desc, sizeof(BlkDesc) * nsmall, st));
-    TDVP_CUDA(cudaMallocAsync(&d_ridx, sizeof(int) * std::max<size_t>(1, ridx.size()), st));
-    TDVP_CUDA(cudaMallocAsync(&d_cidx, sizeof(int) * std::max<size_t>(1, cidx.size()), st));
-    TDVP_CUDA(cudaMallocAsync(&d_s, sizeof(double) * std::max(1, so) + 3 * sizeof(int), st));
+    Packed pk;
+    const size_t o_desc = pk.add(desc), o_r = pk.add(ridx), o_c = pk.add(cidx),
+                 o_s = pk.zeros(sizeof(double) * std::max(1, so) + 3 * sizeof(int)),
+                 o_piv = pk.zeros(psd ? sizeof(int) * std::max<size_t>(1, ridx.size()) : 0);
+    char* base = pk.upload(st, pool, meta);
+    d_desc = reinterpret_cast<BlkDesc*>(base + o_desc);
+    d_ridx = reinterpret_cast<int*>(base + o_r);
+    d_cidx = reinterpret_cast<int*>(base + o_c);
+    d_s = reinterpret_cast<double*>(base + o_s);
     d_bad = reinterpret_cast<int*>(d_s + std::max(1, so));
-    TDVP_CUDA(cudaMemcpyAsync(d_desc, desc.data(), sizeof(BlkDesc) * nsmall, cudaMemcpyHostToDevice, st));
-    TDVP_CUDA(cudaMemcpyAsync(d_ridx, ridx.data(), sizeof(int) * ridx.size(), cudaMemcpyHostToDevice, st));
-    TDVP_CUDA(cudaMemcpyAsync(d_cidx, cidx.data(), sizeof(int) * cidx.size(), cudaMemcpyHostToDevice, st));
-    TDVP_CUDA(cudaMemsetAsync(d_bad, 0, 3 * sizeof(int), st));
+    if (psd) d_piv = reinterpret_cast<int*>(base + o_piv);
     k_gather_batched<<<nsmall, 256, 0, st>>>(M, cols, d_desc, d_ridx, d_cidx, Xs.data(), Vs.data());
     TDVP_CHECK_LAUNCH();
     prep.reset();
@@ -2498,8 +2462,6 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
       // eigendecomposition of a Hermitian PSD matrix: Jacobi SVD of its pivoted Cholesky
       // factor per block; eigenvalues below 1e-15 of the block's largest diagonal entry
       // (under every keep floor of the method) end the factorisation
-      TDVP_CUDA(cudaMallocAsync(&d_piv, sizeof(int) * std::max<size_t>(1, ridx.size()), st));
-      TDVP_CUDA(cudaMemsetAsync(d_s, 0, sizeof(double) * std::max(1, so), st));
       // blocks wider than one SM's FP64 pipe handles quickly get a group of CTAs each
       std::vector<int> gsz(nsmall);
       bool grouped = false;
@@ -2508,7 +2470,7 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
         grouped = grouped || gsz[b] > 1;
       }
       if (grouped) {
-        run_pchol_groups(st, Xs.data(), d_desc, d_piv, gsz);
+        run_pchol_groups(st, pool, Xs.data(), d_desc, d_piv, gsz);
       } else {
         k_pchol_batched<<<nsmall, 256, 0, st>>>(Xs.data(), d_desc, d_piv, 1e-15);
         TDVP_CHECK_LAUNCH();
@@ -2538,7 +2500,7 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
                                                                    d_s, d_bad);
         TDVP_CHECK_LAUNCH();
       } else {
-        run_jacobi_multi<float>(st, x32.as<float2>(), v32.as<float2>(), desc, d_desc, d_s, d_bad);
+        run_jacobi_multi<float>(st, pool, x32.as<float2>(), v32.as<float2>(), desc, d_desc, d_s, d_bad);
       }
       k_to_c128<<<ceil_div(std::max<long long>(1, xo), 256), 256, 0, st>>>(x32.as<float2>(), Xs.data(), xo);
       TDVP_CHECK_LAUNCH();
@@ -2546,7 +2508,7 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
       k_jacobi_batched<double><<<nsmall, 256, smem_need, st>>>(Xs.data(), Vs.data(), d_desc, 60, d_s, d_bad);
       TDVP_CHECK_LAUNCH();
     } else {
-      run_jacobi_multi<double>(st, Xs.data(), Vs.data(), desc, d_desc, d_s, d_bad);
+      run_jacobi_multi<double>(st, pool, Xs.data(), Vs.data(), desc, d_desc, d_s, d_bad);
     }
     jac.reset();
     std::vector<double> hs(so);
@@ -2601,23 +2563,15 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
       sel.push_back({c.blk, c.j, k, psd ? std::sqrt(c.s) : c.s});
     }
     if (!sel.empty()) {
-      SelEntry* d_sel = nullptr;
-      TDVP_CUDA(cudaMallocAsync(&d_sel, sizeof(SelEntry) * sel.size(), st));
+      sel_buf.ensure(pool, sizeof(SelEntry) * sel.size());
+      SelEntry* d_sel = sel_buf.as<SelEntry>();
       TDVP_CUDA(cudaMemcpyAsync(d_sel, sel.data(), sizeof(SelEntry) * sel.size(), cudaMemcpyHostToDevice, st));
       k_scatter_batched<<<(int)sel.size(), 128, 0, st>>>(Xs.data(), Vs.data(), d_desc, d_sel, d_ridx, d_cidx,
                                                           want_u ? out.U.data() : nullptr, keep,
                                                           want_v ? out.Vh.data() : nullptr, cols, want_u ? 1 : 0,
                                                           want_v ? 1 : 0, psd ? d_piv : nullptr);
       TDVP_CHECK_LAUNCH();
-      TDVP_CUDA(cudaFreeAsync(d_sel, st));
     }
-  }
-  if (nsmall) {
-    TDVP_CUDA(cudaFreeAsync(d_desc, st));
-    TDVP_CUDA(cudaFreeAsync(d_ridx, st));
-    TDVP_CUDA(cudaFreeAsync(d_cidx, st));
-    TDVP_CUDA(cudaFreeAsync(d_s, st));
-    if (d_piv) TDVP_CUDA(cudaFreeAsync(d_piv, st));
   }
 }
 
@@ -2890,19 +2844,15 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
   const int nctas = cta_off[nblk];
   tdvp_require(nctas <= budget, TDVP_ERR_INVALID_ARG, "QR groups exceed the co-resident CTAs");
   DArr X(pool, (size_t)xo), Qb(pool, (size_t)std::max<long long>(1, qo));
-  RawBuf meta;
-  const size_t b_desc = sizeof(QrDesc) * nblk, b_r = sizeof(int) * ridx.size(), b_c = sizeof(int) * cidx.size();
-  const size_t b_off = sizeof(int) * (nblk + 1), b_tau = sizeof(double) * to, b_bar = sizeof(GridBar) * nblk;
   std::vector<int2> ent;
   for (int b = 0; b < nblk; ++b)
     for (int j = 0; j < desc[b].kq; ++j) ent.push_back(make_int2(b, j));
-  const size_t b_ent = sizeof(int2) * ent.size();
-  auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-  const size_t o_desc = 0, o_r = al(b_desc), o_c = o_r + al(b_r), o_off = o_c + al(b_c), o_tau = o_off + al(b_off),
-               o_bar = o_tau + al(b_tau), o_ent = o_bar + al(b_bar), o_diag = o_ent + al(b_ent),
-               o_err = o_diag + al(sizeof(double) * K);
-  meta.ensure(pool, o_err + 256);
-  char* base = meta.as<char>();
+  Packed pk;
+  const size_t o_desc = pk.add(desc), o_r = pk.add(ridx), o_c = pk.add(cidx), o_off = pk.add(cta_off),
+               o_ent = pk.add(ent), o_bar = pk.zeros(sizeof(GridBar) * nblk), o_tau = pk.zeros(sizeof(double) * to),
+               o_diag = pk.zeros(sizeof(double) * (K + 1));  // |R_jj| and the error word
+  RawBuf meta;
+  char* base = pk.upload(st, pool, meta);
   auto* d_desc = reinterpret_cast<QrDesc*>(base + o_desc);
   auto* d_r = reinterpret_cast<int*>(base + o_r);
   auto* d_c = reinterpret_cast<int*>(base + o_c);
@@ -2910,15 +2860,8 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
   auto* d_tau = reinterpret_cast<double*>(base + o_tau);
   auto* d_bar = reinterpret_cast<GridBar*>(base + o_bar);
   auto* d_ent = reinterpret_cast<int2*>(base + o_ent);
-  auto* d_err = reinterpret_cast<int*>(base + o_err);
   auto* d_diag = reinterpret_cast<double*>(base + o_diag);
-  TDVP_CUDA(cudaMemcpyAsync(d_desc, desc.data(), b_desc, cudaMemcpyHostToDevice, st));
-  TDVP_CUDA(cudaMemcpyAsync(d_r, ridx.data(), b_r, cudaMemcpyHostToDevice, st));
-  TDVP_CUDA(cudaMemcpyAsync(d_c, cidx.data(), b_c, cudaMemcpyHostToDevice, st));
-  TDVP_CUDA(cudaMemcpyAsync(d_off, cta_off.data(), b_off, cudaMemcpyHostToDevice, st));
-  TDVP_CUDA(cudaMemcpyAsync(d_ent, ent.data(), b_ent, cudaMemcpyHostToDevice, st));
-  TDVP_CUDA(cudaMemsetAsync(d_bar, 0, b_bar, st));
-  TDVP_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int), st));
+  auto* d_err = reinterpret_cast<int*>(d_diag + K);
   k_qr_gather<<<nblk, 256, 0, st>>>(M, cols, d_desc, d_r, d_c, X.data());
   TDVP_CHECK_LAUNCH();
   {
@@ -2940,11 +2883,12 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
   k_qr_scatter<<<(int)ent.size(), 128, 0, st>>>(X.data(), Qb.data(), d_desc, d_ent, d_r, d_c, out.Q.data(),
                                                   out.C.data(), cols, K, d_diag);
   TDVP_CHECK_LAUNCH();
-  int herr = 0;
-  std::vector<double> diag(K);
-  TDVP_CUDA(cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  TDVP_CUDA(cudaMemcpyAsync(diag.data(), d_diag, sizeof(double) * K, cudaMemcpyDeviceToHost, st));
+  std::vector<double> diag(K + 1);
+  TDVP_CUDA(cudaMemcpyAsync(diag.data(), d_diag, sizeof(double) * (K + 1), cudaMemcpyDeviceToHost, st));
   TDVP_CUDA(cudaStreamSynchronize(st));
+  int herr = 0;
+  std::memcpy(&herr, &diag[K], sizeof(int));
+  diag.pop_back();
   if (herr) throw TdvpError(TDVP_ERR_TIMEOUT, "QR: a group barrier wait ran out");
   out.k = K;
   out.diag_min = *std::min_element(diag.begin(), diag.end());

@@ -28,7 +28,8 @@ struct WSparse {
   std::vector<int> r_off;           // d*wl + 1
   std::vector<int> r_idx;
   std::vector<cplx> r_val;
-  // device copies
+  // device copies (one pool buffer)
+  RawBuf dev;
   int* d_l_off = nullptr;
   int* d_l_idx = nullptr;
   cplx* d_l_val = nullptr;
@@ -37,8 +38,7 @@ struct WSparse {
   int* d_r_idx = nullptr;
   cplx* d_r_val = nullptr;
   void build(const cplx* W, int wl, int wr, int d);  // host W
-  void upload();
-  void free_device();
+  void upload(cudaStream_t st, DevicePool* pool);
 };
 
 // out[a][s][v][c] = sum_{(w,t)} W[w,s,t,v] in[a][w][t][c]      (A = rows a, C = cols c); with wa the
@@ -259,4 +259,4 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
 // rows last.  Empty when M is one block or already in that order.
 std::vector<int> sector_row_order(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols);
 // out[r, :] = M[perm[r], :]  (out and M must not overlap)
-void gather_rows(cudaStream_t st, const cplx* M, int rows, int cols, const std::vector<int>& perm, cplx* out);
+void gather_rows(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols, const std::vector<int>& perm, cplx* out);
