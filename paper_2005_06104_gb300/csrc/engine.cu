@@ -360,15 +360,16 @@ void Engine::apply_op(const SiteOp& op, const cplx* x, cplx* y, int precision) {
 // gauge moves: a block QR / LQ when nothing is cut (R1), else a truncated SVD
 // (numerical rank 1e-10 s_max, cutoff eps, cap)
 // ============================================================================
-// The products of the gauge moves and the sweeps.  A handle in FP64 takes them by size (exact
-// digits on the tensor cores from 4 M multiply-adds on); one in a split form keeps the CUDA-core
-// order, so that its trajectories stay those of earlier releases bit by bit: its sweeps turn a
-// last-bit change into 1e-7 of a site tensor (operand digits round at 2^-33, and the next gauge
-// move divides by Schmidt values of 1e-6; measured at chi 256), far above what the product itself
-// could change.
+// FP64 products of gauge moves, sweeps and the extension.  A handle in FP64 takes them by size
+// (exact digits on the tensor cores from 4 M multiply-adds on).  One in a split form stays on the
+// CUDA-core order up to 2^28 (bond dimension about 500; 2 ms on CUDA cores there, 16 ms and a third
+// of a sweep's moves at 1024, where the digits take 1 ms): its sweeps turn a last-bit change into
+// 1e-7 of a site tensor (operand digits round at 2^-33, and the next gauge move divides by Schmidt
+// values of 1e-6; measured at chi 256), so below that line its trajectories stay those of earlier
+// releases bit by bit.
 void Engine::gauge_gemm(int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A, long long lda, const cplx* B,
                         long long ldb, cplx beta, cplx* C, long long ldc) {
-  if (opt.precision == TDVP_PREC_FP64)
+  if (opt.precision == TDVP_PREC_FP64 || (long long)M * N * K >= (1LL << 28))
     zgemm_fp64(st, scr, opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
   else
     zgemm(st, opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 1, 0, 0, 0, &pool);
@@ -1140,8 +1141,8 @@ void Engine::expand_basis(int k, const double* weights) {
       // Y P = Y - (Y B^H) B : rho_bar = (Y P)^H (Y P) = P rho~ P  (Eq. 6)
       DArr G(&pool, (size_t)rows * r);
       for (int pass = 0; pass < 2; ++pass) {
-        zgemm_fp64(st, scr, OP_N, OP_C, rows, r, cols, kOne, Y.data(), cols, Bm.data(), cols, kZero, G.data(), r);
-        zgemm_fp64(st, scr, OP_N, OP_N, rows, cols, r, kMinusOne, G.data(), r, Bm.data(), cols, kOne, Y.data(), cols);
+        gauge_gemm(OP_N, OP_C, rows, r, cols, kOne, Y.data(), cols, Bm.data(), cols, kZero, G.data(), r);
+        gauge_gemm(OP_N, OP_N, rows, cols, r, kMinusOne, G.data(), r, Bm.data(), cols, kOne, Y.data(), cols);
       }
       if (tr > 0.0) {
         const double eps_m = opt.eps_m;
@@ -1165,8 +1166,8 @@ void Engine::expand_basis(int k, const double* weights) {
           // enforce B_bar B^H = 0 to rounding: project off range(B) twice, re-orthonormalise
           DArr Gb(&pool, (size_t)nb * r);
           for (int pass = 0; pass < 2; ++pass) {
-            zgemm_fp64(st, scr, OP_N, OP_C, nb, r, cols, kOne, sy.Vh.data(), cols, Bm.data(), cols, kZero, Gb.data(), r);
-            zgemm_fp64(st, scr, OP_N, OP_N, nb, cols, r, kMinusOne, Gb.data(), r, Bm.data(), cols, kOne, sy.Vh.data(),
+            gauge_gemm(OP_N, OP_C, nb, r, cols, kOne, sy.Vh.data(), cols, Bm.data(), cols, kZero, Gb.data(), r);
+            gauge_gemm(OP_N, OP_N, nb, cols, r, kMinusOne, Gb.data(), r, Bm.data(), cols, kOne, sy.Vh.data(),
                   cols);
           }
           SvdOut so;
@@ -1198,9 +1199,9 @@ void Engine::expand_basis(int k, const double* weights) {
     }
     // centres move by Eq. 3: C_{i-1} = A_{i-1} (C_i B'^H), likewise for every psi~_l
     DArr G(&pool, (size_t)ml * mnew);
-    zgemm_fp64(st, scr, OP_N, OP_C, ml, mnew, cols, kOne, X, cols, Bp.data(), cols, kZero, G.data(), mnew);
+    gauge_gemm(OP_N, OP_C, ml, mnew, cols, kOne, X, cols, Bp.data(), cols, kZero, G.data(), mnew);
     DArr prv(&pool, (size_t)ml0 * d * mnew);
-    zgemm_fp64(st, scr, OP_N, OP_N, ml0 * d, mnew, ml, kOne, psi.A[i - 1].data(), ml, G.data(), mnew, kZero, prv.data(),
+    gauge_gemm(OP_N, OP_N, ml0 * d, mnew, ml, kOne, psi.A[i - 1].data(), ml, G.data(), mnew, kZero, prv.data(),
           mnew);
     for (int l = 0; l < nk; ++l) {
       MpsDev& ph = phis[l];

@@ -113,26 +113,22 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int nchunks = (nkb + KC_KB - 1) / KC_KB;
   // Chunks whose A tile (these BM rows) or B tile (these BN rows) holds only zeros add exact
   // zeros to this output tile: the list of the others, built once (the slicing kernels set a
-  // bit per 128-row tile and chunk that holds a nonzero entry).  All three roles walk it.
+  // bit per 128-row tile and chunk that holds a nonzero entry) by one warp.  All three roles walk it.
   __shared__ int act[kMaxChunks];
   __shared__ int n_act;
-  if (threadIdx.x == 0) {
-    int n = 0;
-    for (int c = 0; c < nchunks; ++c) {
-      const int g = c0 + c;
-      bool on = true;
-      if (maskA) {
-        on = (maskA[(long long)blockIdx.y * mwords + (g >> 5)] >> (g & 31)) & 1u;
-        on = on && ((maskB[(long long)blockIdx.x * mwords + (g >> 5)] >> (g & 31)) & 1u);
-      }
-      if (on && n < kMaxChunks) act[n++] = c;
+  if (warp == 0) {
+    const int n = active_chunks(maskA + (long long)blockIdx.y * mwords, maskB + (long long)blockIdx.x * mwords, c0,
+                                nchunks, kMaxChunks, act);
+    if (lane == 0) {
+      n_act = n;
+      atomicAdd(&g_chunk_pairs[0], (unsigned long long)nchunks);
+      atomicAdd(&g_chunk_pairs[1], (unsigned long long)n);
     }
-    n_act = n;
-    atomicAdd(&g_chunk_pairs[0], (unsigned long long)nchunks);
-    atomicAdd(&g_chunk_pairs[1], (unsigned long long)n);
   }
 
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 32) {
+    prefetch_map(&tmA);
+    prefetch_map(&tmB);
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(smem_u32(&full[s]), 1);
       mbar_init(smem_u32(&empty[s]), 1);
@@ -798,18 +794,39 @@ void launch_bf16s(cudaStream_t st, const CUtensorMap& ma, const CUtensorMap& mb,
   TDVP_CHECK_LAUNCH();
 }
 
+// a float as a double by its bits (exact; an FP64 conversion would run on the FP64 pipe)
+__device__ __forceinline__ double float_bits_to_double(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+  if (e == 0 || e == 255) return (double)x;  // zero, subnormal, not finite
+  return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
+}
+
 // Sum of the split-K partials (double-float pairs, one [M][N] slab per split) into
 // the output: FP64, or double-float pairs when out_df.
-__global__ void k_splitk_df(const float2* __restrict__ ws, int splits, int M, int N, void* __restrict__ out,
-                            long long ldo, int out_df) {
+// Bound: FP64 (2 operations per cycle and SM against 8 bytes per partial).  So partials that are
+// zero in the whole warp (tiles of other charge sectors: most splits of most entries) cost
+// nothing, and the floats widen by integer operations: 2 FP64 additions per nonzero partial
+// where there were 4 operations for every one.
+// Average over a sweep at bond dimension 256: 37 -> 14 us.
+__global__ void __launch_bounds__(256) k_splitk_df(const float2* __restrict__ ws, int splits, int M, int N,
+                                                   void* __restrict__ out, long long ldo, int out_df) {
+  constexpr int U = 8;  // loads in flight per thread
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)M * N) return;
-  const long long m = e / N, n = e % N;
+  const long long per = (long long)M * N;
+  const bool in = e < per;
   double sum = 0.0;
-  for (int z = 0; z < splits; ++z) {
-    const float2 v = ws[(long long)z * M * N + e];
-    sum += (double)v.x + (double)v.y;
+  for (int z0 = 0; z0 < splits; z0 += U) {
+    float2 v[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      v[q] = in && z0 + q < splits ? __ldcs(&ws[(z0 + q) * per + e]) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (__any_sync(0xffffffffu, ((__float_as_uint(v[q].x) | __float_as_uint(v[q].y)) << 1) != 0u))
+        sum += float_bits_to_double(v[q].x) + float_bits_to_double(v[q].y);
   }
+  if (!in) return;
+  const long long m = e / N, n = e % N;
   if (out_df) {
     const float hi = (float)sum;
     static_cast<float2*>(out)[m * ldo + n] = make_float2(hi, (float)(sum - (double)hi));

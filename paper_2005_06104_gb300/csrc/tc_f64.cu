@@ -119,15 +119,14 @@ __global__ void __launch_bounds__(THREADS, 1)
   // chunks with a nonzero entry in both operand tiles (the others add exact zeros)
   __shared__ unsigned short act[kMaxChunks];
   __shared__ int n_act;
-  if (threadIdx.x == 0) {
-    int n = 0;
-    for (int c = 0; c < nchunks; ++c) {
-      const int g = c0 + c;
-      const bool on = (maskA[(long long)blockIdx.y * mwords + (g >> 5)] >> (g & 31)) &
-                      (maskB[(long long)blockIdx.x * mwords + (g >> 5)] >> (g & 31)) & 1u;
-      if (on && n < kMaxChunks) act[n++] = (unsigned short)c;
-    }
-    n_act = n;
+  if (warp == 0) {
+    const int n = active_chunks(maskA + (long long)blockIdx.y * mwords, maskB + (long long)blockIdx.x * mwords, c0,
+                                nchunks, kMaxChunks, act);
+    if (lane == 0) n_act = n;
+  }
+  if (threadIdx.x == 32) {
+    prefetch_map(hi ? &tmA4 : &tmA7);
+    prefetch_map(hi ? &tmB4 : &tmB7);
     for (int s = 0; s < MAX_STAGES; ++s) {
       mbar_init(smem_u32(&full[s]), 1);
       mbar_init(smem_u32(&empty[s]), 1);
@@ -564,7 +563,7 @@ struct F64EnvDigits {
 // plain FP64 GEMM (6.6 ns per 1000 complex multiply-adds on the whole device) is faster under
 // about 4 M of them, and thin operands fill too little of a 128-wide tile.
 bool f64_on_tensor_cores(long long M, long long N, long long K) {
-  return M >= 48 && N >= 24 && K >= 32 && M * N * K >= (1LL << 22) && M < (1LL << 30) && N < (1LL << 29) &&
+  return M >= 64 && N >= 32 && K >= 32 && M * N * K >= (1LL << 22) && M < (1LL << 30) && N < (1LL << 29) &&
          K < (1LL << 29);
 }
 

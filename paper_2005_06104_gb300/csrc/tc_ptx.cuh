@@ -98,6 +98,29 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
+// One warp lists the chunks c in [0, nchunks) whose bits c0 + c are set in both masks, in order,
+// at most `most` of them; returns their number.  32 chunks per step (one thread reading two mask
+// words per chunk took 2 us at 56 chunks, of the 5-10 us a sparse tile takes).
+template <class I>
+__device__ __forceinline__ int active_chunks(const unsigned* maskA, const unsigned* maskB, int c0, int nchunks, int most,
+                                             I* list) {
+  const int lane = threadIdx.x & 31;
+  int n = 0;
+  for (int b = 0; b < nchunks; b += 32) {
+    const int c = b + lane, g = c0 + c;
+    const bool on = c < nchunks && ((maskA[g >> 5] & maskB[g >> 5]) >> (g & 31)) & 1u;
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    const int at = n + __popc(m & ((1u << lane) - 1u));
+    if (on && at < most) list[at] = (I)c;
+    n += __popc(m);
+  }
+  return min(n, most);
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link).
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn();
 }  // namespace tc
