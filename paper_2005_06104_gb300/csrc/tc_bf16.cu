@@ -61,19 +61,6 @@ struct SCfg {
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
 };
 
-// Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major, M x N.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-      "l"(da), "l"(db), "r"(idesc), "r"(acc)
-      : "memory");
-}
-
 // hi + lo += v without loss (Knuth's two-sum into hi, its error into lo)
 __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float v) {
   const float s = __fadd_rn(hi, v);
@@ -181,6 +168,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer
     const uint32_t idesc = idesc_bf16(BM, BN);
+    const uint64_t desc = sdesc<64>(smem_u32(smem));
+    const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32);
     int used = 0;  // running count of k-blocks consumed, in the producer's order
     for (int ai = 0; ai < n_act && !*abort_flag; ++ai) {
       const int c = act[ai];
@@ -201,21 +190,26 @@ __global__ void __launch_bounds__(THREADS, 1)
           break;
         }
         fence_after();
-        const uint32_t a0 = smem_u32(smem + s * STAGE_BYTES);
-        const uint32_t b0 = a0 + S * TILE;
+        const uint32_t a0 = desc_lo + s * (STAGE_BYTES >> 4);
+        const uint32_t b0 = a0 + (S * TILE >> 4);
+        const uint32_t cont = kb == c * KC_KB ? 0u : 1u;
 #pragma unroll
         for (int k = 0; k < BK / 16; ++k) {
-          const uint32_t off = k * 32;  // 16 bf16 = 32 bytes along K inside the 64-byte swizzle atom
-          const uint32_t first = (kb == c * KC_KB && k == 0) ? 0u : 1u;
-          mma_bf16(accP, sdesc<64>(a0 + off), sdesc<64>(b0 + off), idesc, first);
-          uint32_t qacc = first;
+          constexpr int KS = 2;  // 16 bf16 = 32 bytes along K inside the 64-byte swizzle atom
+          if (k == 0)
+            mma_bf16_first(accP, a0, b0, desc_hi, idesc, cont);
+          else
+            mma_bf16_acc(accP, a0 + k * KS, b0 + k * KS, desc_hi, idesc);
 #pragma unroll
           for (int sa = 0; sa < S; ++sa)
 #pragma unroll
             for (int sb = 0; sb + sa < S; ++sb) {
               if (sa == 0 && sb == 0) continue;
-              mma_bf16(accQ, sdesc<64>(a0 + sa * TILE + off), sdesc<64>(b0 + sb * TILE + off), idesc, qacc);
-              qacc = 1u;
+              const uint32_t da = a0 + (sa * TILE >> 4) + k * KS, db = b0 + (sb * TILE >> 4) + k * KS;
+              if (k == 0 && sa == 0 && sb == 1)
+                mma_bf16_first(accQ, da, db, desc_hi, idesc, cont);
+              else
+                mma_bf16_acc(accQ, da, db, desc_hi, idesc);
             }
         }
         mma_commit(smem_u32(&empty[s]));

@@ -58,16 +58,28 @@ constexpr int SMEM_BYTES = STAGE_AREA + 1024 + 256;
 static_assert(SMEM_BYTES + 2 * kMaxChunks + 64 <= 227 * 1024, "shared memory");
 constexpr int kBadRow = 1 << 20;            // row exponent of a row with a non-finite entry
 
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-      "l"(da), "l"(db), "r"(idesc), "r"(acc)
-      : "memory");
+// The MMAs of one stage for group G0 + g of a pass (G0 = 0 or 4): all digit pairs with s + t = G0 + g
+template <int G0>
+__device__ __forceinline__ void mma_group(int g, uint32_t d, uint32_t a0, uint32_t b0, uint32_t hi, uint32_t idesc,
+                                          uint32_t cont) {
+#pragma unroll
+  for (int gg = 0; gg < 4; ++gg) {
+    if (gg != g) continue;
+    constexpr int KS = 2;  // 16 bf16 along K
+    const int sum = G0 + gg, lo = sum > NS - 1 ? sum - (NS - 1) : 0, up = sum < NS - 1 ? sum : NS - 1;
+#pragma unroll
+    for (int sa = 0; sa < NS; ++sa) {
+      if (sa < lo || sa > up) continue;
+#pragma unroll
+      for (int k = 0; k < BK / 16; ++k) {
+        const uint32_t da = a0 + (sa * TILE >> 4) + k * KS, db = b0 + ((sum - sa) * TILE >> 4) + k * KS;
+        if (sa == lo && k == 0)
+          mma_bf16_first(d, da, db, hi, idesc, cont);
+        else
+          mma_bf16_acc(d, da, db, hi, idesc);
+      }
+    }
+  }
 }
 
 // a 2^e as a double, rounded to nearest even; integer arithmetic (an FP64 conversion and a
@@ -175,6 +187,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     } else if (warp == 1 && lane == 0) {
       // ---------------- MMA issuer
       const uint32_t idesc = idesc_bf16(BM, BN);
+      const uint64_t desc = sdesc<64>(smem_u32(smem));
+      const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32);
       int used = 0;
       for (int dr = 0; dr < ndrains && !*abort_flag; ++dr) {
         const int a_end = min(n_act, (dr + 1) * per_drain);
@@ -190,8 +204,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             fence_after();
             const bool first = ai == dr * per_drain && kb == kb_beg;
             const bool last = ai == a_end - 1 && kb == kb_end - 1;
-            const uint32_t a0 = smem_u32(smem + s * stage_bytes);
-            const uint32_t b0 = a0 + nS * TILE;
+            const uint32_t a0 = desc_lo + s * (stage_bytes >> 4);
+            const uint32_t b0 = a0 + nS * (TILE >> 4);
+            const uint32_t cont = first ? 0u : 1u;
+#pragma unroll
             for (int g = ng - 1; g >= 0; --g) {
               if (first && dr > 0) {
                 if (!mbar_wait(smem_u32(&tempty[g]), (dr - 1) & 1)) {
@@ -200,15 +216,10 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
                 fence_after();
               }
-              uint32_t acc = first ? 0u : 1u;
-              for (int sa = max(0, g0 + g - (NS - 1)); sa <= min(NS - 1, g0 + g); ++sa) {
-                const uint32_t at = a0 + sa * TILE, bt = b0 + (g0 + g - sa) * TILE;
-#pragma unroll
-                for (int k = 0; k < BK / 16; ++k) {
-                  mma_bf16(tmem + g * BN, sdesc<64>(at + k * 32), sdesc<64>(bt + k * 32), idesc, acc);
-                  acc = 1u;
-                }
-              }
+              if (hi)
+                mma_group<0>(g, tmem + g * BN, a0, b0, desc_hi, idesc, cont);
+              else
+                mma_group<4>(g, tmem + g * BN, a0, b0, desc_hi, idesc, cont);
               if (last) mma_commit(smem_u32(&tfull[g]));
             }
             mma_commit(smem_u32(&empty[s]));

@@ -64,6 +64,36 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
   d |= (uint64_t)(SWZ == 128 ? 2 : 4) << 61;       // layout: 128B or 64B swizzle
   return d;
 }
+// Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major, M x N.
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+// One BF16 MMA on operands 16 * da and 16 * db bytes into shared memory (the low words of their
+// descriptors; `hi` is the word they share).  One thread issues every MMA of a CTA, and a
+// 128 x 128 x 16 one takes 64 cycles: with both 64-bit descriptors and the predicate rebuilt for
+// each, issue took 95-105 cycles and set the pace of the kernels.  So a descriptor is one 32-bit
+// addition of a constant, and only the first MMA of an accumulator carries a runtime predicate.
+__device__ __forceinline__ void mma_bf16_acc(uint32_t tmem_d, uint32_t da, uint32_t db, uint32_t hi, uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+      "setp.eq.u32 p, 0, 0;\n\t"
+      "mov.b64 a, {%1, %3};\n\t"
+      "mov.b64 b, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}\n" ::"r"(tmem_d),
+      "r"(da), "r"(db), "r"(hi), "r"(idesc)
+      : "memory");
+}
+__device__ __forceinline__ void mma_bf16_first(uint32_t tmem_d, uint32_t da, uint32_t db, uint32_t hi, uint32_t idesc,
+                                               uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "mov.b64 a, {%1, %3};\n\t"
+      "mov.b64 b, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}\n" ::"r"(tmem_d),
+      "r"(da), "r"(db), "r"(hi), "r"(idesc), "r"(acc)
+      : "memory");
+}
 // Instruction descriptor, kind::tf32: D = F32, A = B = TF32, both K-major, M x N.
 __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
   return (1u << 4)                       // D format F32
