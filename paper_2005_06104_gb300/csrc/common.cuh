@@ -26,6 +26,14 @@ __host__ __device__ __forceinline__ cplx cmul(cplx a, cplx b) {
 }
 __host__ __device__ __forceinline__ cplx cconj(cplx a) { return mkc(a.x, -a.y); }
 __host__ __device__ __forceinline__ cplx cscale(cplx a, double s) { return mkc(a.x * s, a.y * s); }
+#ifdef __CUDACC__
+// |a|^2 and a b with the fused operations written out, for kernels whose results have to keep their
+// bits whatever the compiler contracts around them
+__device__ __forceinline__ double cabs2_fma(cplx a) { return fma(a.x, a.x, __dmul_rn(a.y, a.y)); }
+__device__ __forceinline__ cplx cmul_fma(cplx a, cplx b) {
+  return mkc(fma(a.x, b.x, -__dmul_rn(a.y, b.y)), fma(a.x, b.y, __dmul_rn(a.y, b.x)));
+}
+#endif
 // a += b * c
 __host__ __device__ __forceinline__ void cfma(cplx& a, cplx b, cplx c) {
   a.x = fma(b.x, c.x, fma(-b.y, c.y, a.x));

@@ -538,15 +538,8 @@ __device__ __forceinline__ bool last_block(unsigned* counter, unsigned blocks) {
 // doubles take 16 FP64 adds per lane instead of 80 (a warp-wide FP64 instruction holds this part's
 // FP64 pipe for 16 cycles, which made the plain butterfly a large share of a short reduction).
 // Value v of the 2 NC doubles ends in the lanes whose top bits spell v; they store it to out[v].
-template <int NC>
-__device__ __forceinline__ void warp_sum_store(const cplx (&acc)[NC], double* out) {
-  constexpr int NV = 2 * NC;
-  double a[NV];
-#pragma unroll
-  for (int q = 0; q < NC; ++q) {
-    a[2 * q] = acc[q].x;
-    a[2 * q + 1] = acc[q].y;
-  }
+template <class T, int NV>
+__device__ __forceinline__ void warp_sum_values(T (&a)[NV], T* out) {
   const int lane = threadIdx.x & 31;
   int idx = 0, o = 16;
 #pragma unroll
@@ -554,18 +547,27 @@ __device__ __forceinline__ void warp_sum_store(const cplx (&acc)[NC], double* ou
     const bool up = lane & o;
 #pragma unroll
     for (int q = 0; q < half; ++q) {
-      const double send = up ? a[q] : a[q + half];
-      const double keep = up ? a[q + half] : a[q];
+      const T send = up ? a[q] : a[q + half];
+      const T keep = up ? a[q + half] : a[q];
       a[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
     }
     idx += up ? half : 0;
   }
-  const int rest = 32 / NV - 1;  // the lane bits that no halving used
+  constexpr int rest = 32 / NV - 1;  // the lane bits that no halving used
 #pragma unroll
   for (; o >= 1; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
   if ((lane & rest) == 0) out[idx] = a[0];
 }
-
+template <int NC>
+__device__ __forceinline__ void warp_sum_store(const cplx (&acc)[NC], double* out) {
+  double a[2 * NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    a[2 * q] = acc[q].x;
+    a[2 * q + 1] = acc[q].y;
+  }
+  warp_sum_values(a, out);
+}
 
 constexpr int TRI_MAX = 64;
 constexpr int CHEB_MAX = 1024;
@@ -689,7 +691,7 @@ __global__ void __launch_bounds__(RED_THREADS)
     } else {
       wi = in ? w[i] : mkc(0.0, 0.0);
     }
-    if (warp_nonzero(wi)) a = __dadd_rn(a, fma(wi.x, wi.x, __dmul_rn(wi.y, wi.y)));
+    if (warp_nonzero(wi)) a = __dadd_rn(a, cabs2_fma(wi));
   }
   a = warp_sum(a);
   if (lane == 0) dred[warp] = a;
@@ -1113,8 +1115,7 @@ template <class T>
 __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename Jac<T>::C* __restrict__ V, int p, int q,
                                   int P, int Q, T tol, T floor2, int want_v) {
   typedef typename Jac<T>::C C;
-  __shared__ T ra[8], rb[8];
-  __shared__ C rc[8];
+  __shared__ T rs[8][4];
   __shared__ T s_cs;
   __shared__ C s_sne;
   __shared__ int s_do;
@@ -1129,15 +1130,9 @@ __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename J
     cfma_conj(c, u, v);
   }
   const int warp = threadIdx.x >> 5;
-  if (warp * 32 < p) {  // warps past the last row hold zeros: no FP64 reduction for them
-    a = warp_sum(a);
-    b = warp_sum(b);
-    c = warp_sum(c);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    ra[warp] = a;
-    rb[warp] = b;
-    rc[warp] = c;
+  if (warp * 32 < p) {  // warps past the last row hold zeros and are not read
+    T h[4] = {a, b, c.x, c.y};
+    warp_sum_values(h, rs[warp]);  // halving: 6 additions per lane instead of 20
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1145,9 +1140,9 @@ __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename J
     C Cc = Jac<T>::make(0, 0);
     const int active = min((int)(blockDim.x >> 5), (p + 31) >> 5);  // the others hold exact zeros
     for (int u = 0; u < active; ++u) {
-      A += ra[u];
-      B += rb[u];
-      Cc = cadd(Cc, rc[u]);
+      A += rs[u][0];
+      B += rs[u][1];
+      Cc = cadd(Cc, Jac<T>::make(rs[u][2], rs[u][3]));
     }
     T cs;
     C sne;
@@ -2607,12 +2602,25 @@ __global__ void k_qr_gather(const cplx* __restrict__ M, int cols, const QrDesc* 
 
 constexpr int kQrChunk = 8;  // columns whose dot products one block reduction serves
 
-// Block-wide sums of n <= kQrChunk complex partials; the totals land in out[0..n).
+// Block-wide sums of n <= kQrChunk complex partials; the totals land in out[0..n).  The lane sums
+// halve (warp_sum_store): 6 FP64 additions for two columns instead of 20, which were the larger part
+// of a step's time on the FP64 pipe.
 __device__ __forceinline__ void qr_block_sums(cplx* acc, int n, cplx (*red)[kQrChunk], cplx* out) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int t = 0; t < n; ++t) {
-    const cplx v = warp_sum(acc[t]);
-    if (lane == 0) red[warp][t] = v;
+  const int warp = threadIdx.x >> 5;
+  double* r = reinterpret_cast<double*>(red[warp]);
+  if (n <= 2) {
+    cplx h[2] = {acc[0], n > 1 ? acc[1] : mkc(0.0, 0.0)};
+    warp_sum_store(h, r);
+  } else if (n <= 4) {
+    cplx h[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) h[t] = t < n ? acc[t] : mkc(0.0, 0.0);
+    warp_sum_store(h, r);
+  } else {
+    cplx h[kQrChunk];
+#pragma unroll
+    for (int t = 0; t < kQrChunk; ++t) h[t] = t < n ? acc[t] : mkc(0.0, 0.0);
+    warp_sum_store(h, r);
   }
   __syncthreads();
   if (threadIdx.x < n) {
@@ -2630,7 +2638,7 @@ __device__ void qr_make_reflector(cplx* __restrict__ Xb, int p, int j, double* _
   __shared__ int s_zero;
   cplx* x = Xb + (long long)j * p;
   cplx acc[1] = {mkc(0.0, 0.0)};
-  for (int r = j + threadIdx.x; r < p; r += blockDim.x) acc[0].x += cabs2(x[r]);
+  for (int r = j + threadIdx.x; r < p; r += blockDim.x) acc[0].x = __dadd_rn(acc[0].x, cabs2_fma(x[r]));
   qr_block_sums(acc, 1, red, tot);
   if (threadIdx.x == 0) {
     const double nrm = sqrt(tot[0].x);
@@ -2639,7 +2647,7 @@ __device__ void qr_make_reflector(cplx* __restrict__ Xb, int p, int j, double* _
     if (s_zero) {
       tau[j] = 0.0;
     } else {
-      const double aa = sqrt(cabs2(a));
+      const double aa = sqrt(cabs2_fma(a));
       const cplx ph = aa > 0.0 ? cscale(a, 1.0 / aa) : mkc(1.0, 0.0);
       const double den = aa + nrm;
       s_inv = cscale(cconj(ph), 1.0 / den);  // 1 / (x_j - beta) = e^{-i arg x_j} / (|x_j| + |x|)
@@ -2650,7 +2658,7 @@ __device__ void qr_make_reflector(cplx* __restrict__ Xb, int p, int j, double* _
   __syncthreads();
   if (!s_zero) {
     const cplx inv = s_inv;
-    for (int r = j + 1 + threadIdx.x; r < p; r += blockDim.x) x[r] = cmul(x[r], inv);
+    for (int r = j + 1 + threadIdx.x; r < p; r += blockDim.x) x[r] = cmul_fma(x[r], inv);
   }
   __syncthreads();
 }
@@ -2677,7 +2685,7 @@ __device__ __forceinline__ void qr_apply(cplx* __restrict__ Y, int p, int j, con
     for (int t = 0; t < kQrChunk; ++t)
       if (t < n) {
         cplx& y = Y[(long long)cols[t] * p + r];
-        y = csub(y, cmul(w[t], v));
+        y = csub(y, cmul_fma(w[t], v));
       }
   }
   __syncthreads();
@@ -2749,6 +2757,140 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+constexpr int kClQ = 96, kClP = 256, kClWarps = 8, kClU = kClP / 32;
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// Blocks of at most kClQ columns and kClP rows: one cluster per block, one warp per column, the
+// column in the warp's shared memory.  Bound: the chain of a reflector (its barrier, the reflector's
+// way through L2, one dot product, one norm, its square roots and divisions); a cluster barrier and
+// warp reductions take the place of the L2 barrier and of three block reductions.  Q is formed
+// without barriers.  Sums in the order of k_qr_groups: the same bits.
+// 80 x 40: 415 -> 295 us; the moves of a 24-site state at bond dimension 384 (blocks to 200 x 95):
+// 705 -> 530 us each.
+// tot = sum over virtual threads of part(u) with u < nu, in the block kernel's order
+__device__ __forceinline__ cplx qr_warp_total(const cplx (&acc)[kClU], int nu, double* sums) {
+  __syncwarp();
+  if (nu <= 2) {
+    cplx h[2] = {acc[0], acc[1]};
+    warp_sum_store(h, sums);
+  } else if (nu <= 4) {
+    cplx h[4] = {acc[0], acc[1], acc[2], acc[3]};
+    warp_sum_store(h, sums);
+  } else {
+    warp_sum_store(acc, sums);
+  }
+  __syncwarp();
+  cplx t = mkc(0.0, 0.0);
+  for (int u = 0; u < nu; ++u) t = cadd(t, mkc(sums[2 * u], sums[2 * u + 1]));
+  return t;
+}
+
+// y <- H_j y on a warp's column (shared memory); v: the reflector's rows j.. (row j reads as 1)
+__device__ __forceinline__ void qr_warp_apply(cplx* y, const cplx* __restrict__ vcol, int p, int j, double tj,
+                                              double* sums) {
+  const int lane = threadIdx.x & 31, nu = (p - j + 31) >> 5;
+  cplx v[kClU], acc[kClU];
+#pragma unroll
+  for (int u = 0; u < kClU; ++u) {
+    const int r = j + 32 * u + lane;
+    v[u] = r < p ? (r == j ? mkc(1.0, 0.0) : __ldcg(vcol + r)) : mkc(0.0, 0.0);
+  }
+#pragma unroll
+  for (int u = 0; u < kClU; ++u) {
+    const int r = j + 32 * u + lane;
+    acc[u] = mkc(0.0, 0.0);
+    if (u < nu && r < p) cfma_conj(acc[u], v[u], y[r]);
+  }
+  const cplx w = cscale(qr_warp_total(acc, nu, sums), tj);
+#pragma unroll
+  for (int u = 0; u < kClU; ++u) {
+    const int r = j + 32 * u + lane;
+    if (r < p) y[r] = csub(y[r], cmul_fma(w, v[u]));
+  }
+  __syncwarp();
+}
+
+__global__ void __launch_bounds__(32 * kClWarps)
+    k_qr_cluster(cplx* __restrict__ X, cplx* __restrict__ Qb, double* __restrict__ tau,
+                 const QrDesc* __restrict__ desc, int pmax) {
+  extern __shared__ cplx cols[];
+  __shared__ double sums_all[kClWarps][2 * kClU];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nc = (int)cluster_size(), rank = (int)cluster_rank();
+  const QrDesc d = desc[blockIdx.x / nc];
+  const int p = d.p, q = d.q, kq = d.kq;
+  cplx* Xb = X + d.x_off;
+  double* tb = tau + d.t_off;
+  double* sums = sums_all[warp];
+  const int c = rank + nc * warp;  // this warp's column: nc * kClWarps >= kClQ of them
+  cplx* y = cols + warp * pmax;
+  const bool own = c < q;
+  if (own)
+    for (int r = lane; r < p; r += 32) y[r] = Xb[(long long)c * p + r];
+  __syncwarp();
+  for (int j = 0; j < kq; ++j) {
+    if (own && c == j) {  // reflector j from this column
+      const int nu = (p - j + 31) >> 5;
+      cplx acc[kClU];
+#pragma unroll
+      for (int u = 0; u < kClU; ++u) {
+        const int r = j + 32 * u + lane;
+        acc[u] = mkc(0.0, 0.0);
+        if (r < p) acc[u].x = cabs2_fma(y[r]);
+      }
+      const double nrm = sqrt(qr_warp_total(acc, nu, sums).x);
+      const cplx a = y[j];
+      __syncwarp();
+      if (!(nrm > 0.0)) {
+        if (lane == 0) tb[j] = 0.0;
+      } else {
+        const double aa = sqrt(cabs2_fma(a));
+        const cplx ph = aa > 0.0 ? cscale(a, 1.0 / aa) : mkc(1.0, 0.0);
+        const double den = aa + nrm;
+        const cplx inv = cscale(cconj(ph), 1.0 / den);
+        if (lane == 0) {
+          tb[j] = den / nrm;
+          y[j] = cscale(ph, -nrm);
+        }
+        for (int r = j + 1 + lane; r < p; r += 32) y[r] = cmul_fma(y[r], inv);
+      }
+      __syncwarp();
+      for (int r = lane; r < p; r += 32) Xb[(long long)c * p + r] = y[r];
+    }
+    cluster_sync();
+    if (own && c > j) {
+      const double tj = __ldcg(tb + j);
+      if (tj != 0.0) qr_warp_apply(y, Xb + (long long)j * p, p, j, tj, sums);
+    }
+  }
+  if (own && c >= kq)  // columns right of the last reflector: rows of R only
+    for (int r = lane; r < p; r += 32) Xb[(long long)c * p + r] = y[r];
+  // Q_b: column c < kq starts as e_c; H_j applies to the columns c >= j
+  if (c < kq) {
+    for (int r = lane; r < p; r += 32) y[r] = mkc(r == c ? 1.0 : 0.0, 0.0);
+    __syncwarp();
+    for (int j = c; j >= 0; --j) {
+      const double tj = __ldcg(tb + j);
+      if (tj != 0.0) qr_warp_apply(y, Xb + (long long)j * p, p, j, tj, sums);
+    }
+    cplx* Qc = Qb + d.q_off + (long long)c * p;
+    for (int r = lane; r < p; r += 32) Qc[r] = y[r];
+  }
+}
+
 // Entry (blk, j): column j of Q_b and row j of R_b into the outputs.
 //   orient 0: Qout rows x K  (Qout[row, k_off + j] = Q_b[i, j]),
 //             Cout K x cols  (Cout[k_off + j, col] = R_b[j, c], c >= j)
@@ -2777,6 +2919,28 @@ __global__ void k_qr_scatter(const cplx* __restrict__ X, const cplx* __restrict_
 }
 }  // namespace
 
+namespace {
+// One launch of `kernel` with a cluster of nc CTAs per block.
+template <class F>
+void launch_clusters(cudaStream_t st, F* kernel, int nblk, int nc, size_t smem, void** args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nblk * nc);
+  cfg.blockDim = dim3(32 * kClWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nc;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  TDVP_CUDA(cudaLaunchKernelExC(&cfg, (const void*)kernel, args));
+  TDVP_CHECK_LAUNCH();
+}
+// CTAs per cluster: 16 (not portable, allowed by attribute) once 8 would hold more than four columns each
+inline int cluster_ctas(int qmax) { return qmax > 32 ? 16 : 8; }
+}  // namespace
+
 void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols, int orient, QrOut& out) {
   ActivePhase phase(PH_QR);
   out.k = 0;
@@ -2786,7 +2950,7 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
   std::vector<QrDesc> desc;
   std::vector<int> ridx, cidx;
   long long xo = 0, qo = 0;
-  int to = 0, K = 0, pmax = 1;
+  int to = 0, K = 0, pmax = 1, qmax = 1;
   for (auto& kv : comp) {
     auto& rr = kv.second.first;
     auto& cc = kv.second.second;
@@ -2809,10 +2973,13 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
     to += d.kq;
     K += d.kq;
     pmax = std::max(pmax, d.p);
+    qmax = std::max(qmax, d.q);
     desc.push_back(d);
   }
   if (K == 0) return;
   const int nblk = (int)desc.size();
+  const bool clusters = qmax <= kClQ && pmax <= kClP;
+  const int cl = cluster_ctas(qmax);
   const size_t smem = (size_t)pmax * sizeof(cplx);
   tdvp_require(smem <= 200 * 1024, TDVP_ERR_INVALID_ARG, "QR: block too tall for the staged reflector");
   static const bool attr = [] {
@@ -2864,7 +3031,20 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
   auto* d_err = reinterpret_cast<int*>(d_diag + K);
   k_qr_gather<<<nblk, 256, 0, st>>>(M, cols, d_desc, d_r, d_c, X.data());
   TDVP_CHECK_LAUNCH();
-  {
+  if (clusters) {
+    static const bool cattr = [] {
+      TDVP_CUDA(cudaFuncSetAttribute(k_qr_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      TDVP_CUDA(cudaFuncSetAttribute(k_qr_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(kClWarps * kClP * sizeof(cplx))));
+      return true;
+    }();
+    (void)cattr;
+    cplx* xp = X.data();
+    cplx* qp = Qb.data();
+    const QrDesc* dd = d_desc;
+    void* args[] = {&xp, &qp, &d_tau, &dd, &pmax};
+    launch_clusters(st, k_qr_cluster, nblk, cl, kClWarps * (size_t)pmax * sizeof(cplx), args);
+  } else {
     cplx* xp = X.data();
     cplx* qp = Qb.data();
     const QrDesc* dd = d_desc;
