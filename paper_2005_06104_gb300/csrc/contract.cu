@@ -112,6 +112,7 @@ void LanczosWork::release() {
   w.release();
   c.release();
   y.release();
+  live.release();
 }
 
 int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw,
@@ -127,8 +128,17 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
   lw.w.ensure(pool, (size_t)n);
   cplx* V = lw.V.data();
   cplx* wv = lw.w.data();
+  // long vectors keep a bitmap of the groups of 32 entries where the basis is nonzero (see
+  // Blas1::lanczos_step); short ones would pay its clearing for nothing
+  unsigned* live = nullptr;
+  if (n > kSpeculateMaxN) {
+    const size_t bytes = sizeof(unsigned) * (size_t)((n + 1023) / 1024);
+    lw.live.ensure(pool, bytes);
+    live = lw.live.as<unsigned>();
+    TDVP_CUDA(cudaMemsetAsync(live, 0, bytes, st));
+  }
   blas.norm2(st, x, n, start2);
-  scale_by_inv_sqrt(st, V, x, start2, n);
+  scale_by(st, V, x, start2, true, n, live);
   double beta0 = 0.0;
   // A small local problem costs a host round trip per iteration more than its arithmetic: several
   // iterations go out at once (each next vector scaled with a guard, so an iteration after an
@@ -146,10 +156,10 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
   for (int j = 0; j < nmax;) {
     const int j0 = j;
     for (int b = 0; b < batch; ++b, ++j) {
-      if (b > 0) scale_by(st, V + (long long)j * n, wv, nrm2 + 1, n);
+      if (b > 0) scale_by(st, V + (long long)j * n, wv, nrm2 + 1, false, n, live);
       op(V + (long long)j * n, wv);
       // alpha_j = Re <v_j, w>, w made orthogonal to V[0..j], beta_{j+1} = |w|
-      blas.lanczos_step(st, V, n, j, wv, lw.c.data(), alpha, beta, nrm2);
+      blas.lanczos_step(st, V, n, j, wv, live, lw.c.data(), alpha, beta, nrm2);
     }
     tridiag_expv(st, alpha, beta, j0 + 1, batch, delta, kind, lw.y.data(), errs);
     double h[1 + 2 * 64];
@@ -176,14 +186,14 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
       }
     }
     if (used > 0 || j == nmax) break;
-    scale_by(st, V + (long long)j * n, wv, nrm2 + 1, n);
+    scale_by(st, V + (long long)j * n, wv, nrm2 + 1, false, n, live);
     if (small) batch = (int)std::min<long long>({2LL, (long long)(nmax - j), n - j});
   }
   if (used == 0)
     throw TdvpError(TDVP_ERR_LANCZOS_NOT_CONVERGED,
                     "Lanczos error estimate " + std::to_string(last_err) + " above tolerance after " +
                         std::to_string(nmax) + " steps");
-  multi_combine(st, out, V, n, used, y, beta0, n);
+  multi_combine(st, out, V, n, used, y, beta0, n, live);
   if (hint) *hint = used;
   return used;
 }

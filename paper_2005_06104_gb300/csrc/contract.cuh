@@ -90,6 +90,7 @@ void env_right_fp64(cudaStream_t st, Scratch& s, const cplx* R, const WSparse& W
 // steps do not bring the error estimate below tol.
 struct LanczosWork {
   DArr V, w, c, y;
+  RawBuf live;             // bitmap of the nonzero 32-entry groups of the basis
   double* real = nullptr;  // device: alpha[64], beta[65], nrm2[2] at 130, scratch norms; |x|^2 at 255 and
                            // from 256 the error estimates of each iteration of a batch
   void init(DevicePool* pool);

@@ -458,13 +458,18 @@ __global__ void __launch_bounds__(RED_THREADS)
 }
 
 __global__ void k_multi_combine(cplx* __restrict__ y, const cplx* __restrict__ V, long long ldv,
-                                int nvec, const cplx* __restrict__ c, double scale, long long n) {
+                                int nvec, const cplx* __restrict__ c, double scale, long long n,
+                                const unsigned* __restrict__ live) {
   __shared__ cplx cs[64 + MD_CH];
   for (int k = threadIdx.x; k < nvec && k < 64; k += blockDim.x) cs[k] = c[k];
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   cplx acc = mkc(0.0, 0.0);
+  if (live && !((live[i >> 10] >> ((i >> 5) & 31)) & 1u)) {
+    y[i] = acc;
+    return;
+  }
   const unsigned active = __activemask();
   for (int k0 = 0; k0 < nvec; k0 += MD_CH) {
     cplx v[MD_CH];
@@ -476,16 +481,6 @@ __global__ void k_multi_combine(cplx* __restrict__ y, const cplx* __restrict__ V
       if (__any_sync(active, nonzero_bits(v[q]))) cfma(acc, v[q], cs[k0 + q]);
   }
   y[i] = __any_sync(active, nonzero_bits(acc)) ? cscale(acc, scale) : acc;
-}
-
-// FP64 division and square root cost tens of FP64 instructions: one thread per block forms the factor
-__global__ void k_scale_inv_sqrt(cplx* __restrict__ dst, const cplx* __restrict__ src,
-                                 const double* __restrict__ nrm2, long long n) {
-  __shared__ double s;
-  if (threadIdx.x == 0) s = 1.0 / sqrt(*nrm2);
-  __syncthreads();
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    dst[i] = cscale(src[i], s);
 }
 
 __global__ void k_scale_host(cplx* __restrict__ dst, const cplx* __restrict__ src, cplx s, long long n) {
@@ -584,6 +579,8 @@ constexpr int CHEB_MAX = 1024;
 //  - the reductions halve (warp_sum_store);
 //  - a short vector spreads its dot products over blocks by vector (grid.y) and its updates by
 //    entry, instead of sitting on the n / 1024 SMs that the partial sums need.
+//  - long vectors carry a bitmap of the groups of 32 entries in which some basis vector is nonzero
+//    (set when a vector is stored): groups outside it are not read at all.
 // The sums keep one order whatever the spread: block g of G = n / 1024 (at most 2 per SM) adds the
 // entries g 256 + t, + 256 G, ... per thread t, then lanes, warps and blocks, and the fused
 // multiply-adds are written out, so every variant gives the same bits.  (A sweep of a split form
@@ -592,12 +589,17 @@ constexpr int CHEB_MAX = 1024;
 // Measured per iteration at n = 2.1e6, 7 vectors, charge-conserving: 0.61 ms -> 0.2 ms; at
 // n = 1.3e5: 60 us -> 25 us.
 
+// whether some basis vector is nonzero in the 32 entries from `base` on (no bitmap: maybe)
+__device__ __forceinline__ bool group_live(const unsigned* live, long long base) {
+  return !live || ((live[base >> 10] >> ((base >> 5) & 31)) & 1u);
+}
+
 // c[k] = <v_k, w>, k < nvec, KC vectors per block; alpha (when not null): alpha[j] = Re c[j]
 template <int KC>
 __global__ void __launch_bounds__(RED_THREADS)
     k_lanczos_dots(const cplx* __restrict__ V, long long ldv, int nvec, const cplx* __restrict__ w, long long n,
-                   cplx* __restrict__ cout, double* __restrict__ alpha, cplx* __restrict__ partial,
-                   unsigned* __restrict__ counter) {
+                   const unsigned* __restrict__ live, cplx* __restrict__ cout, double* __restrict__ alpha,
+                   cplx* __restrict__ partial, unsigned* __restrict__ counter) {
   constexpr int W = RED_THREADS / 32;
   __shared__ double red[W][2 * KC];
   const int G = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -607,13 +609,17 @@ __global__ void __launch_bounds__(RED_THREADS)
   for (int q = 0; q < KC; ++q) acc[q] = mkc(0.0, 0.0);
   const long long step = (long long)G * RED_THREADS;
   for (long long base = (long long)blockIdx.x * RED_THREADS + warp * 32; base < n; base += step) {
+    if (!group_live(live, base)) continue;
     const long long i = base + lane;
     const bool in = i < n;
     const cplx wi = in ? w[i] : mkc(0.0, 0.0);
     if (!warp_nonzero(wi)) continue;
+    cplx v[KC];  // all loads in flight before the first multiply-add
+#pragma unroll
+    for (int q = 0; q < KC; ++q) v[q] = k0 + q < nvec && in ? V[(long long)(k0 + q) * ldv + i] : mkc(0.0, 0.0);
 #pragma unroll
     for (int q = 0; q < KC; ++q)
-      if (k0 + q < nvec && in) cfma_conj(acc[q], V[(long long)(k0 + q) * ldv + i], wi);
+      if (k0 + q < nvec) cfma_conj(acc[q], v[q], wi);
   }
   warp_sum_store(acc, red[warp]);
   __syncthreads();
@@ -657,41 +663,34 @@ __device__ __forceinline__ cplx lanczos_subtract(const cplx* __restrict__ V, lon
 
 __global__ void __launch_bounds__(RED_THREADS)
     k_lanczos_axpy(const cplx* __restrict__ V, long long ldv, int nvec, cplx* __restrict__ w, long long n,
-                   const cplx* __restrict__ c) {
+                   const unsigned* __restrict__ live, const cplx* __restrict__ c) {
   __shared__ cplx cs[TRI_MAX];
   for (int k = threadIdx.x; k < nvec; k += blockDim.x) cs[k] = c[k];
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i - (threadIdx.x & 31) >= n || !group_live(live, i & ~31LL)) return;
   const cplx r = lanczos_subtract(V, ldv, nvec, cs, w, i, i < n);
   if (i < n) w[i] = r;
 }
 
-// (UPDATE: w -= V c, then) nrm2[0] = |w|^2, nrm2[1] = 1 / |w|, *beta = |w|
-template <bool UPDATE>
+// nrm2[0] = |w|^2, nrm2[1] = 1 / |w|, *beta = |w|
 __global__ void __launch_bounds__(RED_THREADS)
-    k_lanczos_norm(const cplx* __restrict__ V, long long ldv, int nvec, cplx* __restrict__ w, long long n,
-                   const cplx* __restrict__ c, double* __restrict__ nrm2, double* __restrict__ beta,
+    k_lanczos_norm(const cplx* __restrict__ w, long long n, double* __restrict__ nrm2, double* __restrict__ beta,
                    double* __restrict__ partial, unsigned* __restrict__ counter) {
-  __shared__ cplx cs[TRI_MAX];
   __shared__ double dred[RED_THREADS / 32], part[RED_THREADS];
   const int G = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (UPDATE) {
-    for (int k = threadIdx.x; k < nvec; k += RED_THREADS) cs[k] = c[k];
-    __syncthreads();
-  }
   double a = 0.0;
   const long long step = (long long)G * RED_THREADS;
-  for (long long base = (long long)blockIdx.x * RED_THREADS + warp * 32; base < n; base += step) {
-    const long long i = base + lane;
-    const bool in = i < n;
-    cplx wi;
-    if (UPDATE) {
-      wi = lanczos_subtract(V, ldv, nvec, cs, w, i, in);
-      if (in) w[i] = wi;
-    } else {
-      wi = in ? w[i] : mkc(0.0, 0.0);
+  for (long long base = (long long)blockIdx.x * RED_THREADS + warp * 32; base < n; base += 4 * step) {
+    cplx wi[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const long long i = base + q * step + lane;
+      wi[q] = i < n ? w[i] : mkc(0.0, 0.0);
     }
-    if (warp_nonzero(wi)) a = __dadd_rn(a, cabs2_fma(wi));
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (warp_nonzero(wi[q])) a = __dadd_rn(a, cabs2_fma(wi[q]));
   }
   a = warp_sum(a);
   if (lane == 0) dred[warp] = a;
@@ -721,54 +720,69 @@ __global__ void __launch_bounds__(RED_THREADS)
   }
 }
 
-// dst = src * *factor
-__global__ void k_scale_by(cplx* __restrict__ dst, const cplx* __restrict__ src, const double* __restrict__ factor,
-                           long long n) {
-  const double s = *factor;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    dst[i] = cscale(src[i], s);
+// dst = src * *factor, or src / sqrt(*factor) when `root`; sets the bits of `live` (when not null) of
+// the 32-entry groups with a nonzero entry.  FP64 division and square root cost tens of FP64
+// instructions: one thread per block forms the factor.
+__global__ void __launch_bounds__(256)
+    k_scale_by(cplx* __restrict__ dst, const cplx* __restrict__ src, const double* __restrict__ factor, int root,
+               long long n, unsigned* __restrict__ live) {
+  __shared__ double sh;
+  if (threadIdx.x == 0) sh = root ? 1.0 / sqrt(*factor) : *factor;
+  __syncthreads();
+  const double s = sh;
+  const int lane = threadIdx.x & 31;
+  for (long long base = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; base < n;
+       base += (long long)gridDim.x * blockDim.x) {
+    const long long i = base + lane;
+    cplx v = i < n ? src[i] : mkc(0.0, 0.0);
+    const bool nz = warp_nonzero(v);
+    if (nz) v = cscale(v, s);
+    if (i < n) dst[i] = v;
+    if (live && nz && lane == 0) {
+      const unsigned bit = 1u << ((base >> 5) & 31);
+      if (!(__ldcg(&live[base >> 10]) & bit)) atomicOr(&live[base >> 10], bit);
+    }
+  }
 }
 }  // namespace
 
-void Blas1::lanczos_step(cudaStream_t st, const cplx* V, long long n, int j, cplx* w, cplx* c, double* alpha,
-                         double* beta, double* nrm2) {
+void Blas1::lanczos_step(cudaStream_t st, const cplx* V, long long n, int j, cplx* w, const unsigned* live, cplx* c,
+                         double* alpha, double* beta, double* nrm2) {
   const int nvec = j + 1;
   tdvp_require(j >= 0 && nvec < TRI_MAX, TDVP_ERR_INVALID_ARG, "lanczos_step: too many vectors");
   const int G = red_blocks(n, max_blocks);
   auto dots = [&](cplx* out, double* al) {
-    // vectors per block: 8 share one read of w once the blocks of the sums fill half the device
-    // (FP64 bound either way), fewer below, so that a short vector still reaches every SM
-    if (G * ceil_div(nvec, 8) >= max_blocks / 4)
-      k_lanczos_dots<8><<<dim3(G, ceil_div(nvec, 8)), RED_THREADS, 0, st>>>(V, n, nvec, w, n, out, al, partial.data(),
-                                                                            counter);
+    // vectors per block: 8 share one read of w when that still gives every SM four blocks; fewer
+    // below, so that the loads of a long vector overlap its FP64 work (2 blocks per SM: 37 % of
+    // the FP64 pipe) and a short one reaches every SM
+    if (G * ceil_div(nvec, 8) >= 2 * max_blocks)
+      k_lanczos_dots<8><<<dim3(G, ceil_div(nvec, 8)), RED_THREADS, 0, st>>>(V, n, nvec, w, n, live, out, al,
+                                                                            partial.data(), counter);
     else if (G * ceil_div(nvec, 2) >= max_blocks / 4)
-      k_lanczos_dots<2><<<dim3(G, ceil_div(nvec, 2)), RED_THREADS, 0, st>>>(V, n, nvec, w, n, out, al, partial.data(),
-                                                                            counter);
+      k_lanczos_dots<2><<<dim3(G, ceil_div(nvec, 2)), RED_THREADS, 0, st>>>(V, n, nvec, w, n, live, out, al,
+                                                                            partial.data(), counter);
     else
-      k_lanczos_dots<1><<<dim3(G, nvec), RED_THREADS, 0, st>>>(V, n, nvec, w, n, out, al, partial.data(), counter);
+      k_lanczos_dots<1><<<dim3(G, nvec), RED_THREADS, 0, st>>>(V, n, nvec, w, n, live, out, al, partial.data(), counter);
     TDVP_CHECK_LAUNCH();
   };
   const int ta = n <= 32LL * 1024 ? 64 : RED_THREADS;
   dots(c, alpha);
-  k_lanczos_axpy<<<ceil_div(n, ta), ta, 0, st>>>(V, n, nvec, w, n, c);
+  k_lanczos_axpy<<<ceil_div(n, ta), ta, 0, st>>>(V, n, nvec, w, n, live, c);
   TDVP_CHECK_LAUNCH();
   dots(c + TRI_MAX, nullptr);
   double* dpart = reinterpret_cast<double*>(partial.data());
-  // the norm's n / 1024 blocks also do the last update when they fill the device; below that a
-  // launch of its own spreads it (n = 2048, 8 vectors: 8 us on 2 SMs against 1 us and a launch)
-  if (2 * G >= max_blocks) {
-    k_lanczos_norm<true><<<G, RED_THREADS, 0, st>>>(V, n, nvec, w, n, c + TRI_MAX, nrm2, beta + j + 1, dpart, counter);
-  } else {
-    k_lanczos_axpy<<<ceil_div(n, ta), ta, 0, st>>>(V, n, nvec, w, n, c + TRI_MAX);
-    TDVP_CHECK_LAUNCH();
-    k_lanczos_norm<false><<<G, RED_THREADS, 0, st>>>(V, n, nvec, w, n, nullptr, nrm2, beta + j + 1, dpart, counter);
-  }
+  // (fused into the norm's n / 1024 blocks the second update took 84 us at n = 2.1e6, apart 39 + 14)
+  k_lanczos_axpy<<<ceil_div(n, ta), ta, 0, st>>>(V, n, nvec, w, n, live, c + TRI_MAX);
+  TDVP_CHECK_LAUNCH();
+  k_lanczos_norm<<<G, RED_THREADS, 0, st>>>(w, n, nrm2, beta + j + 1, dpart, counter);
   TDVP_CHECK_LAUNCH();
 }
 
-void scale_by(cudaStream_t st, cplx* dst, const cplx* src, const double* factor, long long n) {
+void scale_by(cudaStream_t st, cplx* dst, const cplx* src, const double* factor, bool root, long long n,
+              unsigned* live) {
   if (n == 0) return;
-  k_scale_by<<<(int)std::min<long long>(ceil_div(n, 256), 152 * 8), 256, 0, st>>>(dst, src, factor, n);
+  k_scale_by<<<(int)std::min<long long>(ceil_div(n, 256), 152 * 8), 256, 0, st>>>(dst, src, factor, root ? 1 : 0, n,
+                                                                                   live);
   TDVP_CHECK_LAUNCH();
 }
 
@@ -793,17 +807,15 @@ void Blas1::norm2(cudaStream_t st, const cplx* x, long long n, double* out) {
 }
 
 void multi_combine(cudaStream_t st, cplx* y, const cplx* V, long long ldv, int nvec, const cplx* c,
-                   double scale, long long n) {
+                   double scale, long long n, const unsigned* live) {
   tdvp_require(nvec <= 64, TDVP_ERR_INVALID_ARG, "multi_combine: nvec > 64");
   if (n == 0) return;
-  k_multi_combine<<<ceil_div(n, 256), 256, 0, st>>>(y, V, ldv, nvec, c, scale, n);
+  k_multi_combine<<<ceil_div(n, 256), 256, 0, st>>>(y, V, ldv, nvec, c, scale, n, live);
   TDVP_CHECK_LAUNCH();
 }
 
 void scale_by_inv_sqrt(cudaStream_t st, cplx* dst, const cplx* src, const double* nrm2, long long n) {
-  if (n == 0) return;
-  k_scale_inv_sqrt<<<(int)std::min<long long>(ceil_div(n, 256), 152 * 8), 256, 0, st>>>(dst, src, nrm2, n);
-  TDVP_CHECK_LAUNCH();
+  scale_by(st, dst, src, nrm2, true, n, nullptr);
 }
 
 void scale_host(cudaStream_t st, cplx* dst, const cplx* src, cplx s, long long n) {
@@ -870,12 +882,14 @@ __global__ void __launch_bounds__(32)
   if (bad) K = CHEB_MAX;
   for (int k = lane; k <= K; k += 32) coef[k] = 0.0;
   __syncwarp();
+  double norm = 1.0;
   if (x < 1e-300) {
     if (lane == 0) coef[0] = 1.0;
   } else {
     // Miller backward recurrence, start well above K; every lane runs it, lane 0 keeps the values
     const int M = 2 * ((K + 40 + (int)x) / 2 + 1);
-    double jp1 = 0.0, jk = 1e-280, norm = 0.0;
+    double jp1 = 0.0, jk = 1e-280;
+    norm = 0.0;
     for (int kb = M; kb >= 1; kb -= 32) {
       const double quot = 2.0 * (double)max(kb - lane, 0) / x;
       for (int l = 0; l < min(32, kb); ++l) {
@@ -884,24 +898,37 @@ __global__ void __launch_bounds__(32)
         const double tk = __shfl_sync(FULL, quot, l);
         const double jm1 = fma(tk, jk, kind == 0 ? -jp1 : jp1);
         if (lane == 0 && k <= K) coef[k] = jk;
-        if (kind != 0 || (k & 1) == 0) norm += 2.0 * jk;
+        if (kind != 0 || (k & 1) == 0) norm = fma(2.0, jk, norm);
         jp1 = jk;
         jk = jm1;
-        if (fabs(jk) > 1e250) {  // rescale
-          const double f = 1e-250;
-          jk *= f;
-          jp1 *= f;
-          norm *= f;
-          __syncwarp();
-          for (int q = k + lane; q <= K; q += 32) coef[q] *= f;
-          __syncwarp();
+        if ((__double2hiint(jk) & 0x7fffffff) >= 0x73e00000) {  // |jk| >= 2^831: look closer (integer test)
+          if (fabs(jk) > 1e250) {  // rescale
+            const double f = 1e-250;
+            jk *= f;
+            jp1 *= f;
+            norm *= f;
+            __syncwarp();
+            for (int q = k + lane; q <= K; q += 32) coef[q] *= f;
+            __syncwarp();
+          }
         }
       }
     }
     if (lane == 0) coef[0] = jk;
     norm += jk;
-    __syncwarp();
-    for (int k = lane; k <= K; k += 32) coef[k] /= norm;
+  }
+  __syncwarp();
+  // coefficient of T_k: eps_k (-i sgn delta)^k J_k or eps_k (-sgn)^k I_k, the factor i kept apart
+  for (int k = lane; k <= K; k += 32) {
+    double ck = coef[k];
+    if (x >= 1e-300) ck /= norm;
+    if (k > 0) ck *= 2.0;
+    bool neg;
+    if (kind == 0)
+      neg = (k & 1) ? (((k & 3) == 1) == (delta >= 0)) : (k & 3) == 2;
+    else
+      neg = delta >= 0 && (k & 1);
+    coef[k] = neg ? -ck : ck;
   }
   __syncwarp();
   const double inv_h = h > 0.0 ? 1.0 / h : 0.0;
@@ -915,40 +942,31 @@ __global__ void __launch_bounds__(32)
   cur[0] = lane == 0 ? 1.0 : 0.0;  // T_0 e_0
   cur[1] = 0.0;
   for (int k = 0; k <= K; ++k) {
-    double ck = (k == 0 ? 1.0 : 2.0) * coef[k];
-    const int m = k & 3;
-    if (kind == 0) {  // (-i sgn delta)^k
-      if (k & 1) {
-        if ((m == 1) == (delta >= 0)) ck = -ck;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) aim[q] = fma(ck, cur[q], aim[q]);
-      } else {
-        if (m == 2) ck = -ck;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) are[q] = fma(ck, cur[q], are[q]);
-      }
+    const double ck = coef[k];
+    const bool odd = kind == 0 && (k & 1);
+    if (odd) {
+      aim[0] = fma(ck, cur[0], aim[0]);
+      if (two) aim[1] = fma(ck, cur[1], aim[1]);
     } else {
-      if (delta >= 0 && (k & 1)) ck = -ck;
-#pragma unroll
-      for (int q = 0; q < 2; ++q) are[q] = fma(ck, cur[q], are[q]);
+      are[0] = fma(ck, cur[0], are[0]);
+      if (two) are[1] = fma(ck, cur[1], are[1]);
     }
     if (k == K) break;
-    double nx[2] = {0.0, 0.0};
     const double up0 = __shfl_up_sync(FULL, cur[0], 1);  // lane 0: xl is 0
     double dn0 = __shfl_down_sync(FULL, cur[0], 1);
     if (two) {
       const double first1 = __shfl_sync(FULL, cur[1], 0), last0 = __shfl_sync(FULL, cur[0], 31);
       const double up1 = __shfl_up_sync(FULL, cur[1], 1), dn1 = __shfl_down_sync(FULL, cur[1], 1);
       if (lane == 31) dn0 = first1;
-      nx[1] = fma(xr[1], dn1, fma(xl[1], lane == 0 ? last0 : up1, __dmul_rn(xd[1], cur[1])));
+      const double nx = fma(xr[1], dn1, fma(xl[1], lane == 0 ? last0 : up1, __dmul_rn(xd[1], cur[1])));
+      const double nxt = k == 0 ? nx : fma(2.0, nx, -prev[1]);
+      prev[1] = cur[1];
+      cur[1] = nxt;
     }
-    nx[0] = fma(xr[0], dn0, fma(xl[0], up0, __dmul_rn(xd[0], cur[0])));
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const double nxt = k == 0 ? nx[q] : 2.0 * nx[q] - prev[q];
-      prev[q] = cur[q];
-      cur[q] = nxt;
-    }
+    const double nx = fma(xr[0], dn0, fma(xl[0], up0, __dmul_rn(xd[0], cur[0])));
+    const double nxt = k == 0 ? nx : fma(2.0, nx, -prev[0]);
+    prev[0] = cur[0];
+    cur[0] = nxt;
   }
   double fre, fim = 0.0;
   if (kind == 0) {

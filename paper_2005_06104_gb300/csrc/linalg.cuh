@@ -147,20 +147,23 @@ struct Blas1 {
   void norm2(cudaStream_t st, const cplx* x, long long n, double* out);
   // The vector work of Lanczos iteration j: on entry w = H V[j]; on return alpha[j] and beta[j + 1]
   // are set, w is orthogonal to V[0..j], nrm2[0] = |w|^2 and nrm2[1] = 1 / |w| (0 when |w|^2 <=
-  // 1e-200 or not finite).  c: 2 x 64 entries of scratch.  V's vectors are n entries apart.
-  void lanczos_step(cudaStream_t st, const cplx* V, long long n, int j, cplx* w, cplx* c, double* alpha, double* beta,
-                    double* nrm2);
+  // 1e-200 or not finite).  c: 2 x 64 entries of scratch.  V's vectors are n entries apart.  live: null,
+  // or one bit per 32 entries, set where some V[0..j] is nonzero (scale_by sets them).
+  void lanczos_step(cudaStream_t st, const cplx* V, long long n, int j, cplx* w, const unsigned* live, cplx* c,
+                    double* alpha, double* beta, double* nrm2);
   unsigned* counter = nullptr;  // ticket of the last-block reductions (reset by that block)
   void release();
 };
-// y[i] = scale * sum_k V[k*ldv+i] c[k]  (scale read from host value)
+// y[i] = scale * sum_k V[k*ldv+i] c[k]  (scale read from host value; live as in lanczos_step)
 void multi_combine(cudaStream_t st, cplx* y, const cplx* V, long long ldv, int nvec,
-                   const cplx* c, double scale, long long n);
+                   const cplx* c, double scale, long long n, const unsigned* live = nullptr);
 // dst = src * (1 / sqrt(*nrm2))   (nrm2 in device memory)
 void scale_by_inv_sqrt(cudaStream_t st, cplx* dst, const cplx* src, const double* nrm2,
                        long long n);
-// dst = src * *factor   (factor in device memory)
-void scale_by(cudaStream_t st, cplx* dst, const cplx* src, const double* factor, long long n);
+// dst = src * *factor, or src / sqrt(*factor) with root   (factor in device memory); sets the bits of
+// live (when not null) of the 32-entry groups with a nonzero entry
+void scale_by(cudaStream_t st, cplx* dst, const cplx* src, const double* factor, bool root, long long n,
+              unsigned* live);
 void scale_host(cudaStream_t st, cplx* dst, const cplx* src, cplx s, long long n);
 void fill_zero(cudaStream_t st, cplx* p, long long n);
 // For n = n0 .. n0 + count - 1 (b = n - n0): y[64 b + (0..n)) = exp(coef * T_n) e_0 for the

@@ -371,31 +371,6 @@ struct SrcLwa {
     }
   }
 };
-// Rows (n, c') of the expanded real B operand built from opB(B)[k][n]:
-//   row (n, re): (Re, -Im) over K index (k, re/im); row (n, im): (Im, Re).
-struct SrcB {
-  static constexpr bool kDF = false;
-  const cplx* p;
-  long long ld;
-  int K, N, op;
-  __device__ void load4(long long n2, int k2, double v[4]) const {
-    const long long n = n2 >> 1;
-    const int cp = (int)(n2 & 1);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = (k2 >> 1) + h;
-      double re = 0.0, im = 0.0;
-      if (n < N && k < K) {
-        const cplx z = (op == OP_N || op == OP_R) ? p[(long long)k * ld + n] : p[n * ld + k];
-        re = z.x;
-        im = (op == OP_C || op == OP_R) ? -z.y : z.y;
-      }
-      v[2 * h] = cp == 0 ? re : im;
-      v[2 * h + 1] = cp == 0 ? -im : re;
-    }
-  }
-};
-
 // s_hi + s_lo += (a_hi + a_lo)(b_hi + b_lo) in double-float arithmetic (about 2^-48)
 __device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, float al, float bh, float bl) {
   const float p = __fmul_rn(ah, bh);
@@ -582,13 +557,6 @@ struct Seg {
       hi[i] = lo[i] = 0.f;
     }
   }
-  // any entry not exactly zero (a non-finite one counts)
-  __device__ bool nonzero() const {
-    bool nz = false;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) nz = nz || v[i] != 0.0 || !(v[i] == v[i]) || hi[i] != 0.f || lo[i] != 0.f;
-    return nz;
-  }
   // max key (FP64) or max |hi| (double-float); bad = non-finite seen
   __device__ unsigned long long key() const {
     unsigned long long k = 0;
@@ -638,9 +606,15 @@ __device__ __forceinline__ GroupScale warp_scale(const Seg<Src>& sg) {
   }
 }
 
+// Marks (row tile, chunk) as nonzero.  (Reading the word first to spare the atomic doubles the
+// slicing time: the atomic needs no answer, the read does.)
+__device__ __forceinline__ void mark_chunk(unsigned* mask, int mw, long long row, int ch) {
+  atomicOr(&mask[(row >> 7) * mw + (ch >> 5)], 1u << (ch & 31));
+}
+
 // A operands: one warp per (row, chunk of 128 K entries).
 // out: [S][rows_pad][ldk] bf16; scale: [nch][rows_pad] float.
-// mask (when non-null): bit ch of word (row / 128) * mw + ch / 32 is set when the group is not
+// mask: bit ch of word (row / 128) * mw + ch / 32 is set when the group is not
 // zero (its scale is nonzero or NaN), i.e. when the chunk holds a nonzero entry of the row tile.
 template <int S, class Src>
 __global__ void k_slice_chunks(Src src, int rows_pad, int ldk, int nch, __nv_bfloat16* __restrict__ out,
@@ -658,44 +632,122 @@ __global__ void k_slice_chunks(Src src, int rows_pad, int ldk, int nch, __nv_bfl
   if (k2 < ldk) sg.template write<S>(g, out + row * ldk + k2, (long long)rows_pad * ldk);
   if (lane == 0) {
     scale[(long long)ch * rows_pad + row] = g.sc;
-    if (mask && g.sc != 0.f) atomicOr(&mask[(row >> 7) * mw + (ch >> 5)], 1u << (ch & 31));
+    if (g.sc != 0.f) mark_chunk(mask, mw, row, ch);
   }
 }
 
-// B operands: one 128-thread block per row, one scale per row (two passes over
-// the source: the largest magnitude, then the slices).  scale: [rows_pad] float.
-template <int S, class Src>
-__global__ void __launch_bounds__(128) k_slice_rows(Src src, int rows_pad, int ldk, __nv_bfloat16* __restrict__ out,
-                                                    float* __restrict__ scale, unsigned* __restrict__ mask, int mw) {
-  static_assert(!Src::kDF, "row-scaled operands come from FP64 sources");
-  __shared__ unsigned long long red[4];
-  const long long row = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  unsigned long long k = 0;
-  Seg<Src> sg;
-  for (int k2 = 4 * tid; k2 < ldk; k2 += 512) {
-    sg.load(src, row, k2);
-    k = max(k, sg.key());
-  }
+__device__ __forceinline__ unsigned long long cplx_key(cplx z) { return max(abs_key(z.x), abs_key(z.y)); }
+__device__ __forceinline__ bool cplx_nonzero(cplx z) {
+  return z.x != 0.0 || z.y != 0.0 || !(z.x == z.x) || !(z.y == z.y);
+}
+
+// B operands, expanded to the real rows (n, re): (Re, -Im) and (n, im): (Im, Re) over the K index
+// (k, re/im), one scale for both rows of a complex row n < N of opB(B)[k][n] (two passes over the
+// source: the largest magnitude, then the slices).  Bound: HBM, 16 B read and 2 x 4 S B written per
+// entry (the first pass over a row leaves it in L1 or L2).
+// Two consecutive entries z of one complex row: 4 BF16 per slice and real row.
+template <int S>
+__device__ __forceinline__ void store_b(const cplx z[2], const GroupScale& g, __nv_bfloat16* out, long long n, int ldk,
+                                        int k2, long long slice) {
+  float re[2][S], im[2][S], ni[2][S];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) k = max(k, __shfl_xor_sync(0xffffffffu, k, o));
-  if (lane == 0) red[wid] = k;
-  __syncthreads();
-  k = max(max(red[0], red[1]), max(red[2], red[3]));
-  const GroupScale g = scale_from_key(k);
-  // warp wid covers the 128 entries [base, base + 128) of one chunk per pass (warp-uniform bound)
-  for (int base = 128 * wid; base < ldk; base += 512) {
-    const int k2 = base + 4 * lane;
-    const bool in = k2 < ldk;
-    if (in) sg.load(src, row, k2); else sg.zero();
-    if (in) sg.template write<S>(g, out + row * ldk + k2, (long long)rows_pad * ldk);
-    const bool nz = __any_sync(0xffffffffu, in && sg.nonzero());
-    if (mask && nz && lane == 0) {
-      const int ch = base >> 7;
-      atomicOr(&mask[(row >> 7) * mw + (ch >> 5)], 1u << (ch & 31));
-    }
+  for (int q = 0; q < 2; ++q) {
+    digits_fp64<S>(z[q].x, g, re[q]);
+    digits_fp64<S>(z[q].y, g, im[q]);
+    digits_fp64<S>(-z[q].y, g, ni[q]);
   }
-  if (tid == 0) scale[row] = g.sc;
+  float d[4][S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    d[0][s] = re[0][s];
+    d[1][s] = ni[0][s];
+    d[2][s] = re[1][s];
+    d[3][s] = ni[1][s];
+  }
+  store_slices<S>(d, out + 2 * n * ldk + k2, slice);
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    d[0][s] = im[0][s];
+    d[1][s] = re[0][s];
+    d[2][s] = im[1][s];
+    d[3][s] = re[1][s];
+  }
+  store_slices<S>(d, out + (2 * n + 1) * ldk + k2, slice);
+}
+
+// entry (n, k) at p[n * ld + k]: one block per complex row.  chi = 1024, w = 14 (235 MB): 436 -> 197 us
+// against one block per real row (each complex row read four times).
+template <int S>
+__global__ void __launch_bounds__(128)
+    k_slice_b_k(const cplx* __restrict__ p, long long ld, int N, int K, int conj, int rows_pad, int ldk,
+                __nv_bfloat16* __restrict__ out, float* __restrict__ scale, unsigned* __restrict__ mask, int mw) {
+  __shared__ unsigned long long red[4];
+  const long long n = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const bool live = n < N;
+  const cplx* x = p + (live ? n * ld : 0);
+  unsigned long long h = 0;
+  if (live)
+    for (int k = tid; k < K; k += 128) h = max(h, cplx_key(x[k]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
+  if (lane == 0) red[wid] = h;
+  __syncthreads();
+  const GroupScale g = scale_from_key(max(max(red[0], red[1]), max(red[2], red[3])));
+  const long long slice = (long long)rows_pad * ldk;
+  for (int base = 64 * wid; 2 * base < ldk; base += 256) {  // a warp covers one chunk: 64 complex entries
+    const int k = base + 2 * lane;
+    cplx z[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      z[q] = live && k + q < K ? x[k + q] : mkc(0.0, 0.0);
+      if (conj) z[q].y = -z[q].y;
+    }
+    if (2 * k < ldk) store_b<S>(z, g, out, n, ldk, 2 * k, slice);
+    if (__any_sync(0xffffffffu, cplx_nonzero(z[0]) || cplx_nonzero(z[1])) && lane == 0)
+      mark_chunk(mask, mw, 2 * n, base >> 6);
+  }
+  if (tid == 0) scale[2 * n] = scale[2 * n + 1] = g.sc;
+}
+
+// entry (n, k) at p[k * ld + n]: blocks of 8 complex rows (128-byte reads), turned in shared memory
+template <int S>
+__global__ void __launch_bounds__(256)
+    k_slice_b_r(const cplx* __restrict__ p, long long ld, int N, int K, int conj, int rows_pad, int ldk,
+                __nv_bfloat16* __restrict__ out, float* __restrict__ scale, unsigned* __restrict__ mask, int mw) {
+  constexpr int TR = 8;
+  __shared__ unsigned long long hmax[TR];
+  __shared__ cplx t[TR][65];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const long long n0 = (long long)blockIdx.x * TR;
+  const int rl = tid % TR, kk = tid / TR;  // 8 rows x 32 k
+  if (tid < TR) hmax[tid] = 0;
+  __syncthreads();
+  unsigned long long h = 0;
+  if (n0 + rl < N)
+    for (int k = kk; k < K; k += 32) h = max(h, cplx_key(p[(long long)k * ld + n0 + rl]));
+  atomicMax(&hmax[rl], h);
+  __syncthreads();
+  const long long n = n0 + wid;  // warp w turns row w
+  const GroupScale g = scale_from_key(hmax[wid]);
+  const long long slice = (long long)rows_pad * ldk;
+  for (int base = 0; 2 * base < ldk; base += 64) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int k = base + kk + 32 * q;
+      cplx z = n0 + rl < N && k < K ? p[(long long)k * ld + n0 + rl] : mkc(0.0, 0.0);
+      if (conj) z.y = -z.y;
+      t[rl][kk + 32 * q] = z;
+    }
+    __syncthreads();
+    const int k = base + 2 * lane;
+    const cplx z[2] = {t[wid][2 * lane], t[wid][2 * lane + 1]};
+    if (2 * k < ldk) store_b<S>(z, g, out, n, ldk, 2 * k, slice);
+    if (__any_sync(0xffffffffu, cplx_nonzero(z[0]) || cplx_nonzero(z[1])) && lane == 0)
+      mark_chunk(mask, mw, 2 * n, base >> 6);
+    __syncthreads();
+  }
+  if (lane == 0) scale[2 * n] = scale[2 * n + 1] = g.sc;
 }
 
 // ---------------------------------------------------------------- host side
@@ -722,27 +774,45 @@ struct Sliced {
   }
 };
 
+void clear_mask(cudaStream_t st, Sliced& o) {
+  TDVP_CUDA(cudaMemsetAsync(o.mask.as<void>(), 0, sizeof(unsigned) * (size_t)(o.rows_pad / 128) * o.mw, st));
+}
+
+// A operand
 template <class Src>
 void slice(cudaStream_t st, const Src& src, Sliced& o) {
-  __nv_bfloat16* d = o.data.as<__nv_bfloat16>();
+  tdvp_require(!o.row_scale, TDVP_ERR_INVALID_ARG, "slice: A operands carry chunk scales");
+  clear_mask(st, o);
+  auto* d = o.data.as<__nv_bfloat16>();
+  const int blocks = ceil_div((long long)o.rows_pad * o.nch * 32, 256);
+  if (o.S == 4)
+    k_slice_chunks<4, Src><<<blocks, 256, 0, st>>>(src, o.rows_pad, o.ldk, o.nch, d, o.scale.as<float>(),
+                                                   o.mask.as<unsigned>(), o.mw);
+  else
+    k_slice_chunks<3, Src><<<blocks, 256, 0, st>>>(src, o.rows_pad, o.ldk, o.nch, d, o.scale.as<float>(),
+                                                   o.mask.as<unsigned>(), o.mw);
+  TDVP_CHECK_LAUNCH();
+}
+
+// B operand from opB(B)[k][n] (B row-major with leading dimension ld)
+void slice_b(cudaStream_t st, const cplx* B, long long ld, int K, int N, int op, Sliced& o) {
+  tdvp_require(o.row_scale, TDVP_ERR_INVALID_ARG, "slice_b: B operands carry row scales");
+  clear_mask(st, o);
+  auto* d = o.data.as<__nv_bfloat16>();
   float* sc = o.scale.as<float>();
   unsigned* mk = o.mask.as<unsigned>();
-  TDVP_CUDA(cudaMemsetAsync(mk, 0, sizeof(unsigned) * (size_t)(o.rows_pad / 128) * o.mw, st));
-  if (o.row_scale) {
-    if constexpr (Src::kDF) {
-      throw TdvpError(TDVP_ERR_INVALID_ARG, "slice: row-scaled operands come from FP64 sources");
-    } else {
-      if (o.S == 4)
-        k_slice_rows<4, Src><<<o.rows_pad, 128, 0, st>>>(src, o.rows_pad, o.ldk, d, sc, mk, o.mw);
-      else
-        k_slice_rows<3, Src><<<o.rows_pad, 128, 0, st>>>(src, o.rows_pad, o.ldk, d, sc, mk, o.mw);
-    }
-  } else {
-    const int blocks = ceil_div((long long)o.rows_pad * o.nch * 32, 256);
+  const bool kcontig = op == OP_T || op == OP_C;
+  const int conj = op == OP_C || op == OP_R, rows = o.rows_pad / 2;
+  if (kcontig) {
     if (o.S == 4)
-      k_slice_chunks<4, Src><<<blocks, 256, 0, st>>>(src, o.rows_pad, o.ldk, o.nch, d, sc, mk, o.mw);
+      k_slice_b_k<4><<<rows, 128, 0, st>>>(B, ld, N, K, conj, o.rows_pad, o.ldk, d, sc, mk, o.mw);
     else
-      k_slice_chunks<3, Src><<<blocks, 256, 0, st>>>(src, o.rows_pad, o.ldk, o.nch, d, sc, mk, o.mw);
+      k_slice_b_k<3><<<rows, 128, 0, st>>>(B, ld, N, K, conj, o.rows_pad, o.ldk, d, sc, mk, o.mw);
+  } else {
+    if (o.S == 4)
+      k_slice_b_r<4><<<rows / 8, 256, 0, st>>>(B, ld, N, K, conj, o.rows_pad, o.ldk, d, sc, mk, o.mw);
+    else
+      k_slice_b_r<3><<<rows / 8, 256, 0, st>>>(B, ld, N, K, conj, o.rows_pad, o.ldk, d, sc, mk, o.mw);
   }
   TDVP_CHECK_LAUNCH();
 }
@@ -942,13 +1012,13 @@ void heff_bf16s(cudaStream_t st, Scratch& s, const SiteOp& op, const cplx* x, cp
     slice(st, SrcLwa{op.L, ml, wl}, c.L);
     // R[b][(v,b')] is B[k=(v,b')][n=b] stored n-major (op T)
     c.R.shape(pool, S, 2 * mr, 2 * wr * mr, true);
-    slice(st, SrcB{op.R, (long long)wr * mr, wr * mr, mr, OP_T}, c.R);
+    slice_b(st, op.R, (long long)wr * mr, wr * mr, mr, OP_T, c.R);
     c.key = op.env_key;
     c.S = S;
   }
   // stage 1: T1[(w,a)][(s',b',c)] = L x     (x[a'][(s',b')] is B[k=a'][n=(s',b')])
   c.X.shape(pool, S, 2 * d * mr, 2 * ml, true);
-  slice(st, SrcB{x, (long long)d * mr, ml, d * mr, OP_N}, c.X);
+  slice_b(st, x, (long long)d * mr, ml, d * mr, OP_N, c.X);
   const int M1 = ml * wl, N1 = 2 * d * mr;
   c.T1.ensure(pool, sizeof(float2) * (size_t)M1 * N1);  // double-float
   gemm_bf16s(st, pool, c.L, c.X, M1, N1, c.T1.as<void>(), N1, true, err);
@@ -970,6 +1040,6 @@ void zgemm_bf16s(cudaStream_t st, Scratch& s, int S, int opA, int opB, int M, in
   a.shape(pool, S, M, 2 * std::max(K, 1), false);
   slice(st, SrcA{A, lda, M, K, opA}, a);
   b.shape(pool, S, 2 * N, 2 * std::max(K, 1), true);
-  slice(st, SrcB{B, ldb, K, N, opB}, b);
+  slice_b(st, B, ldb, K, N, opB, b);
   gemm_bf16s(st, pool, a, b, M, 2 * N, C, 2 * ldc, false, err);
 }
