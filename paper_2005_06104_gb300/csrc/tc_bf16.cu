@@ -54,11 +54,13 @@ static_assert(128 * REGS_LOW + 32 * EPI_WARPS * REGS_HIGH <= THREADS * REGS_LAUN
 constexpr int TILE = BM * BK * 2;       // one slice of one operand tile (bytes); BM == BN
 constexpr int TMEM_COLS = 512;
 constexpr int EC = 64;                  // output columns per epilogue thread
+constexpr int EPI_ROW = EC * 8 + 16;    // bytes of a row of a warp's turned output (odd in 16-byte units)
 
 template <int S>
 struct SCfg {
   static constexpr int STAGE_BYTES = 2 * S * TILE;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+  static_assert(EPI_WARPS * 32 * EPI_ROW <= STAGES * STAGE_BYTES, "output tile in the stages");
 };
 
 // hi + lo += v without loss (Knuth's two-sum into hi, its error into lo)
@@ -68,6 +70,21 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float v) {
   const float e = __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -bb)), __fadd_rn(v, -bb));
   hi = s;
   lo = __fadd_rn(lo, e);
+}
+
+// a float as a double by its bits (exact; an FP64 conversion would run on the FP64 pipe)
+__device__ __forceinline__ double float_bits_to_double(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+  if (e == 0 || e == 255) return (double)x;  // zero, subnormal, not finite
+  return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
+}
+
+// x 2^e for a power of two s = 2^e given as a float, by the exponent bits when both sides are normal
+__device__ __forceinline__ double scale_pow2(double x, float s) {
+  const int e = (int)((__float_as_uint(s) >> 23) & 0xffu) - 127;
+  const int h = __double2hiint(x), ex = (h >> 20) & 0x7ff;
+  if (ex == 0 || ex == 0x7ff || ex + e <= 0 || ex + e >= 0x7ff || e == 128 || e == -127) return x * (double)s;
+  return __hiloint2double(h + (e << 20), __double2loint(x));
 }
 
 // (output tile, K chunk) pairs visited by k_gemm_bf16s since load: [0] all, [1] multiplied
@@ -225,7 +242,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int q = warp & 3;
     const int half = (warp - EPI_WARP0) >> 2;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const int gm = m0 + q * 32 + lane;
+    const int gm = m0 + q * 32 + lane;  // this thread's row in the accumulators
     const int nb = n0 + half * EC;
     float hi[EC], lo[EC];
 #pragma unroll
@@ -264,43 +281,42 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
     }
     if (ok) {  // warp-uniform
+      // A thread holds 64 columns of one row; written straight out, every store of a warp would touch
+      // 32 rows (8 us per tile).  The warp turns its 32 x 64 entries through its own part of the
+      // stages (all MMAs have read them) and stores whole 512-byte rows.
+      uint8_t* reg = smem + (warp - EPI_WARP0) * 32 * EPI_ROW;
+#pragma unroll
+      for (int j = 0; j < EC; j += 2)
+        *reinterpret_cast<float4*>(reg + lane * EPI_ROW + j * 8) = make_float4(hi[j], lo[j], hi[j + 1], lo[j + 1]);
+      __syncwarp();
       // column scales: lane i holds those of columns nb + 2i, nb + 2i + 1 (inside the padded rows)
       const float2 sbv = __ldg(reinterpret_cast<const float2*>(sB + nb) + lane);
-      const bool row_ok = gm < M;
-      const bool vec = nb + EC <= N && (ldo & 1) == 0;
-      if (out_df) {
-        // double-float output: (hi, lo) FP32 pairs, scaled exactly by the power-of-two column scale
-        float2* o = static_cast<float2*>(out) + blockIdx.z * split_stride + (long long)gm * ldo + nb;
-#pragma unroll
-        for (int j = 0; j < EC; j += 2) {
-          const float s0 = __shfl_sync(0xffffffffu, sbv.x, j >> 1);
-          const float s1 = __shfl_sync(0xffffffffu, sbv.y, j >> 1);
-          const float4 v = make_float4(__fmul_rn(hi[j], s0), __fmul_rn(lo[j], s0), __fmul_rn(hi[j + 1], s1),
-                                       __fmul_rn(lo[j + 1], s1));
-          if (row_ok) {
-            if (vec) {
-              *reinterpret_cast<float4*>(o + j) = v;
-            } else {
-              if (nb + j < N) o[j] = make_float2(v.x, v.y);
-              if (nb + j + 1 < N) o[j + 1] = make_float2(v.z, v.w);
-            }
+      const int col = nb + 2 * lane;
+      const bool vec = col + 1 < N && (ldo & 1) == 0;
+      const int rows = min(32, M - (m0 + q * 32));
+      for (int r = 0; r < rows; ++r) {
+        const float4 v = *reinterpret_cast<const float4*>(reg + r * EPI_ROW + lane * 16);
+        const long long at = (long long)(m0 + q * 32 + r) * ldo + col;
+        if (out_df) {
+          // double-float output: (hi, lo) FP32 pairs, scaled exactly by the power-of-two column scale
+          float2* o = static_cast<float2*>(out) + blockIdx.z * split_stride + at;
+          const float4 t = make_float4(__fmul_rn(v.x, sbv.x), __fmul_rn(v.y, sbv.x), __fmul_rn(v.z, sbv.y),
+                                       __fmul_rn(v.w, sbv.y));
+          if (vec) {
+            *reinterpret_cast<float4*>(o) = t;
+          } else {
+            if (col < N) o[0] = make_float2(t.x, t.y);
+            if (col + 1 < N) o[1] = make_float2(t.z, t.w);
           }
-        }
-      } else {
-        double* o = static_cast<double*>(out) + (long long)gm * ldo + nb;
-#pragma unroll
-        for (int j = 0; j < EC; j += 2) {
-          const float s0 = __shfl_sync(0xffffffffu, sbv.x, j >> 1);
-          const float s1 = __shfl_sync(0xffffffffu, sbv.y, j >> 1);
-          const double d0 = ((double)hi[j] + (double)lo[j]) * (double)s0;
-          const double d1 = ((double)hi[j + 1] + (double)lo[j + 1]) * (double)s1;
-          if (row_ok) {
-            if (vec) {
-              *reinterpret_cast<double2*>(o + j) = make_double2(d0, d1);
-            } else {
-              if (nb + j < N) o[j] = d0;
-              if (nb + j + 1 < N) o[j + 1] = d1;
-            }
+        } else {
+          double* o = static_cast<double*>(out) + at;
+          const double d0 = scale_pow2(float_bits_to_double(v.x) + float_bits_to_double(v.y), sbv.x);
+          const double d1 = scale_pow2(float_bits_to_double(v.z) + float_bits_to_double(v.w), sbv.y);
+          if (vec) {
+            *reinterpret_cast<double2*>(o) = make_double2(d0, d1);
+          } else {
+            if (col < N) o[0] = d0;
+            if (col + 1 < N) o[1] = d1;
           }
         }
       }
@@ -856,13 +872,6 @@ void launch_bf16s(cudaStream_t st, const CUtensorMap& ma, const CUtensorMap& mb,
   k_gemm_bf16s<S><<<grid, THREADS, SCfg<S>::SMEM_BYTES, st>>>(ma, mb, M, N, nkb, kb_split, sA, lsA, sB, out, ldo,
                                                               split_stride, out_df, d_err, maskA, maskB, mw);
   TDVP_CHECK_LAUNCH();
-}
-
-// a float as a double by its bits (exact; an FP64 conversion would run on the FP64 pipe)
-__device__ __forceinline__ double float_bits_to_double(float x) {
-  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
-  if (e == 0 || e == 255) return (double)x;  // zero, subnormal, not finite
-  return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
 }
 
 // Sum of the split-K partials (double-float pairs, one [M][N] slab per split) into

@@ -51,10 +51,12 @@ static_assert(128 * REGS_LOW + 32 * EPI_WARPS * REGS_HIGH <= THREADS * REGS_LAUN
 constexpr int TILE = BM * BK * 2;           // one slice of one operand tile (bytes)
 constexpr int TMEM_COLS = 512;
 constexpr int EC = 64;                      // output columns per epilogue thread
+constexpr int EPI_ROW = EC * 8 + 16;        // bytes of a row of a warp's turned output
 constexpr int MAX_STAGES = 3;
 constexpr int STAGE_AREA = 2 * 2 * NS * TILE;  // two stages of the 7-slice pass; three of the 4-slice one fit
 static_assert(3 * 2 * 4 * TILE <= STAGE_AREA, "stages of the first pass");
 constexpr int SMEM_BYTES = STAGE_AREA + 1024 + 256;
+static_assert(EPI_WARPS * 32 * EPI_ROW <= STAGE_AREA, "output tile in the stages");
 static_assert(SMEM_BYTES + 2 * kMaxChunks + 64 <= 227 * 1024, "shared memory");
 constexpr int kBadRow = 1 << 20;            // row exponent of a row with a non-finite entry
 
@@ -235,7 +237,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int q = warp & 3;
     const int half = (warp - EPI_WARP0) >> 2;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const int gm = m0 + q * 32 + lane;
     const int nb = n0 + half * EC;
     long long acc[EC];
 #pragma unroll
@@ -268,19 +269,24 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (lane == 0) mbar_arrive(smem_u32(&tempty[g]));
       }
     }
-    if (ok && gm < M) {
-      // d_s d_t weighs 2^(96 - 8 (s + t)) of 2^(EA + EB - 110); the unit of acc is the last group's
-      const int e0 = eA[gm] + (hi ? 72 - 110 : 40 - 110);
-      const bool bad = eA[gm] == kBadRow;
-      double* o = out + ((long long)blockIdx.z * M + gm) * N + nb;
+    if (ok) {
+      // the warp turns its 32 x 64 sums through the stages and stores whole rows (see tc_bf16.cu)
+      uint8_t* reg = smem + (warp - EPI_WARP0) * 32 * EPI_ROW;
 #pragma unroll
-      for (int j = 0; j < EC; j += 2) {
-        if (nb + j < N) {  // N is even
-          const int eb = eB[nb + j];  // the rows (n, re) and (n, im) of B share their exponent
-          double2 v = make_double2(scaled_int(acc[j], e0 + eb), scaled_int(acc[j + 1], e0 + eb));
-          if (bad || eb == kBadRow) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
-          *reinterpret_cast<double2*>(o + j) = v;
-        }
+      for (int j = 0; j < EC; j += 2)
+        *reinterpret_cast<longlong2*>(reg + lane * EPI_ROW + j * 8) = make_longlong2(acc[j], acc[j + 1]);
+      __syncwarp();
+      const int col = nb + 2 * lane;  // N is even
+      const int eb = col < N ? eB[col] : 0;  // the rows (n, re) and (n, im) of B share their exponent
+      const int rows = min(32, M - (m0 + q * 32));
+      for (int r = 0; r < rows; ++r) {
+        const longlong2 a = *reinterpret_cast<const longlong2*>(reg + r * EPI_ROW + lane * 16);
+        const int row = m0 + q * 32 + r, ea = eA[row];
+        // d_s d_t weighs 2^(96 - 8 (s + t)) of 2^(EA + EB - 110); the unit of acc is the last group's
+        const int e = ea + eb + (hi ? 72 - 110 : 40 - 110);
+        double2 v = make_double2(scaled_int(a.x, e), scaled_int(a.y, e));
+        if (ea == kBadRow || eb == kBadRow) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+        if (col < N) *reinterpret_cast<double2*>(out + ((long long)blockIdx.z * M + row) * N + col) = v;
       }
     }
   }
