@@ -63,13 +63,37 @@ struct SCfg {
   static_assert(EPI_WARPS * 32 * EPI_ROW <= STAGES * STAGE_BYTES, "output tile in the stages");
 };
 
-// hi + lo += v without loss (Knuth's two-sum into hi, its error into lo)
-__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float v) {
-  const float s = __fadd_rn(hi, v);
-  const float bb = __fadd_rn(s, -hi);
-  const float e = __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -bb)), __fadd_rn(v, -bb));
+// Two floats in one 64-bit register: sm_103a adds and multiplies both with one instruction (each
+// rounded to nearest as alone).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(uint32_t a, uint32_t b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// a - b (b times -1 plus a: one rounding)
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+  return r;
+}
+// hi + lo += v without loss (Knuth's two-sum into hi, its error into lo), two entries at once
+__device__ __forceinline__ void two_sum_acc(f32x2& hi, f32x2& lo, f32x2 v) {
+  const f32x2 s = add2(hi, v);
+  const f32x2 bb = sub2(s, hi);
+  const f32x2 e = add2(sub2(hi, sub2(s, bb)), sub2(v, bb));
   hi = s;
-  lo = __fadd_rn(lo, e);
+  lo = add2(lo, e);
 }
 
 // a float as a double by its bits (exact; an FP64 conversion would run on the FP64 pipe)
@@ -244,9 +268,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     const int gm = m0 + q * 32 + lane;  // this thread's row in the accumulators
     const int nb = n0 + half * EC;
-    float hi[EC], lo[EC];
+    f32x2 hi[EC / 2], lo[EC / 2];
 #pragma unroll
-    for (int j = 0; j < EC; ++j) hi[j] = lo[j] = 0.f;
+    for (int j = 0; j < EC / 2; ++j) hi[j] = lo[j] = 0ull;
     bool ok = true;
     for (int ai = 0; ai < n_act; ++ai) {
       const int c = act[ai];
@@ -256,24 +280,19 @@ __global__ void __launch_bounds__(THREADS, 1)
       ok = __all_sync(0xffffffffu, got && !*abort_flag);
       if (!ok) break;
       fence_after();
-      const float sa = sA[(long long)(c0 + c) * lsA + gm];
+      const uint32_t sab = __float_as_uint(sA[(long long)(c0 + c) * lsA + gm]);
+      const f32x2 sa = pack2(sab, sab);
 #pragma unroll
-      for (int c0 = 0; c0 < EC; c0 += 8) {
-        uint32_t vp[8], vq[8];
-        const uint32_t col = tmem + lane_base + (uint32_t)(b * 2 * BN + half * EC + c0);
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(vp[0]), "=r"(vp[1]), "=r"(vp[2]), "=r"(vp[3]), "=r"(vp[4]), "=r"(vp[5]), "=r"(vp[6]),
-                       "=r"(vp[7])
-                     : "r"(col));
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(vq[0]), "=r"(vq[1]), "=r"(vq[2]), "=r"(vq[3]), "=r"(vq[4]), "=r"(vq[5]), "=r"(vq[6]),
-                       "=r"(vq[7])
-                     : "r"(col + BN));
+      for (int e0 = 0; e0 < EC; e0 += 16) {
+        uint32_t vp[16], vq[16];
+        const uint32_t col = tmem + lane_base + (uint32_t)(b * 2 * BN + half * EC + e0);
+        tmem_ld16(vp, col);
+        tmem_ld16(vq, col + BN);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          two_sum_acc(hi[c0 + j], lo[c0 + j], __fmul_rn(__uint_as_float(vp[j]), sa));
-          two_sum_acc(hi[c0 + j], lo[c0 + j], __fmul_rn(__uint_as_float(vq[j]), sa));
+          two_sum_acc(hi[e0 / 2 + j], lo[e0 / 2 + j], mul2(pack2(vp[2 * j], vp[2 * j + 1]), sa));
+          two_sum_acc(hi[e0 / 2 + j], lo[e0 / 2 + j], mul2(pack2(vq[2 * j], vq[2 * j + 1]), sa));
         }
       }
       fence_before();
@@ -286,8 +305,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       // stages (all MMAs have read them) and stores whole 512-byte rows.
       uint8_t* reg = smem + (warp - EPI_WARP0) * 32 * EPI_ROW;
 #pragma unroll
-      for (int j = 0; j < EC; j += 2)
-        *reinterpret_cast<float4*>(reg + lane * EPI_ROW + j * 8) = make_float4(hi[j], lo[j], hi[j + 1], lo[j + 1]);
+      for (int j = 0; j < EC / 2; ++j)
+        *reinterpret_cast<uint4*>(reg + lane * EPI_ROW + j * 16) =
+            make_uint4((uint32_t)hi[j], (uint32_t)lo[j], (uint32_t)(hi[j] >> 32), (uint32_t)(lo[j] >> 32));
       __syncwarp();
       // column scales: lane i holds those of columns nb + 2i, nb + 2i + 1 (inside the padded rows)
       const float2 sbv = __ldg(reinterpret_cast<const float2*>(sB + nb) + lane);
