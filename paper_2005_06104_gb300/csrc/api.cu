@@ -218,6 +218,7 @@ tdvp_status tdvp_evolve_site(tdvp_handle* h, int site, const void* x, void* y, d
     const int it = e.lanczos([&](const cplx* a, cplx* b) { e.heff(site, a, b, precision); },
                              static_cast<const cplx*>(x), static_cast<cplx*>(y), n, delta, kind);
     e.sync();
+    tc_check(e.st, e.scr);
     if (iters) *iters = it;
   });
 }

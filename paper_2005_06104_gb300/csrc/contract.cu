@@ -9,6 +9,8 @@ const cplx kZero = {0.0, 0.0};
 constexpr double kBreakdown = 1e-13;  // Lanczos invariant-subspace threshold
 // local dimension up to which a Lanczos run may launch several iterations per host check
 constexpr long long kSpeculateMaxN = 1LL << 18;
+// local dimension from which a Lanczos run keeps a bitmap of the nonzero groups of its basis
+constexpr long long kBitmapMinN = 1LL << 14;
 }  // namespace
 
 double heff_flops(const SiteOp& op) {
@@ -131,7 +133,7 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
   // long vectors keep a bitmap of the groups of 32 entries where the basis is nonzero (see
   // Blas1::lanczos_step); short ones would pay its clearing for nothing
   unsigned* live = nullptr;
-  if (n > kSpeculateMaxN) {
+  if (n > kBitmapMinN) {
     const size_t bytes = sizeof(unsigned) * (size_t)((n + 1023) / 1024);
     lw.live.ensure(pool, bytes);
     live = lw.live.as<unsigned>();

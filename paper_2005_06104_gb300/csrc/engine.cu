@@ -494,7 +494,7 @@ int Engine::lanczos(const std::function<void(const cplx*, cplx*)>& op, const cpl
     tc_check(st, scr);  // a device timeout explains a failure better than what followed it
     throw;
   }
-  tc_check(st, scr);
+  // the error word of the bounded waits stays set until it is read: once per sweep, not per run
   lanczos_iters += used;
   lanczos_calls += 1;
   return used;
@@ -637,6 +637,7 @@ void Engine::sweep(double dt, int kind) {
     for (int j = 0; j < N; ++j) Lok[j] = Rok[j] = 0;
   env_prec = TDVP_PREC_FP64;
   sync();
+  tc_check(st, scr);
 }
 
 // ============================================================================
@@ -743,6 +744,7 @@ void Engine::sweep2(double dt, int kind) {
   env_prec = TDVP_PREC_FP64;
   ++env_epoch;
   sync();
+  tc_check(st, scr);
 }
 
 // ============================================================================

@@ -103,6 +103,53 @@ __device__ __forceinline__ double float_bits_to_double(float x) {
   return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
 }
 
+// (double)h + (double)l, the same bits, by integer operations on the sum's mantissa when l is the
+// smaller part: an FP64 addition holds the FP64 pipe for 16 cycles per warp, these 25 integer
+// operations for 7 issue slots of each scheduler.
+__device__ __forceinline__ double df_to_double(float h, float l) {
+  const unsigned hb = __float_as_uint(h), lb = __float_as_uint(l);
+  const int eh = (int)((hb >> 23) & 0xffu), el = (int)((lb >> 23) & 0xffu), sh = eh - el;
+  const double d = float_bits_to_double(h);
+  if (lb << 1 == 0u) return d;
+  if (eh == 0 || el == 0 || eh == 255 || sh < 1) return d + float_bits_to_double(l);
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+  const unsigned m = (lb & 0x7fffffu) | 0x800000u;  // l = m 2^(29 - sh) units in the last place of d
+  const bool minus = (hb ^ lb) >> 31;
+  unsigned long long t;
+  if (sh <= 29) {
+    t = (unsigned long long)m << (29 - sh);
+  } else {
+    const int k = min(sh - 29, 25);  // from 25 on l is below half a unit
+    const unsigned q = m >> k, rem = m & ((1u << k) - 1u), half = 1u << (k - 1);
+    const unsigned odd = (unsigned)(minus ? u - q : u + q) & 1u;
+    t = q + ((rem > half || (rem == half && odd)) ? 1u : 0u);  // to nearest even
+  }
+  const unsigned long long r = minus ? u - t : u + t;
+  // the exponent changes, or a power of two loses a part that only the finer half below it resolves
+  if ((r ^ u) >> 52 || (minus && !(u & 0xfffffffffffffull))) return d + float_bits_to_double(l);
+  return __longlong_as_double((long long)r);
+}
+
+// x as a float pair: hi = (float)x, lo = (float)(x - hi), the same bits by integer operations where
+// both parts are normal (four operations of the FP64 pipe otherwise)
+__device__ __forceinline__ float2 double_to_df(double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((u >> 52) & 0x7ff) - 1023;
+  if (e < -74 || e > 126) {
+    if (u << 1 == 0ull) return make_float2((float)x, 0.f);
+    const float hi = (float)x;
+    return make_float2(hi, (float)(x - (double)hi));
+  }
+  const unsigned sign = (unsigned)(u >> 63) << 31;
+  const unsigned top = (unsigned)((u & 0xfffffffffffffull) >> 29);  // 23 bits after the leading one
+  const unsigned rest = (unsigned)u & 0x1fffffffu;                  // 29 bits below
+  const unsigned up = rest > 0x10000000u || (rest == 0x10000000u && (top & 1u));  // to nearest even
+  const float hi = __uint_as_float((sign | ((unsigned)(e + 127) << 23) | top) + up);
+  const int rem = (int)rest - (up ? 0x20000000 : 0);  // x - hi in units 2^(e-52), of x's sign
+  const float lo = __int2float_rn(sign ? -rem : rem) * __uint_as_float((unsigned)(e - 52 + 127) << 23);
+  return make_float2(hi, rem == 0 ? 0.f : lo);
+}
+
 // x 2^e for a power of two s = 2^e given as a float, by the exponent bits when both sides are normal
 __device__ __forceinline__ double scale_pow2(double x, float s) {
   const int e = (int)((__float_as_uint(s) >> 23) & 0xffu) - 127;
@@ -119,7 +166,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     k_gemm_bf16s(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N,
                  int nkb_total, int kb_split, const float* __restrict__ sA, long long lsA,
                  const float* __restrict__ sB, void* __restrict__ out, long long ldo, long long split_stride,
-                 int out_df, int* __restrict__ err, const unsigned* __restrict__ maskA,
+                 int out_df, int skip_empty, int* __restrict__ err, const unsigned* __restrict__ maskA,
                  const unsigned* __restrict__ maskB, int mwords) {
   constexpr int STAGE_BYTES = SCfg<S>::STAGE_BYTES;
   extern __shared__ uint8_t smem_raw[];
@@ -313,7 +360,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       const float2 sbv = __ldg(reinterpret_cast<const float2*>(sB + nb) + lane);
       const int col = nb + 2 * lane;
       const bool vec = col + 1 < N && (ldo & 1) == 0;
-      const int rows = min(32, M - (m0 + q * 32));
+      // partials without a chunk are zeros that the reduction, which knows the masks, does not read
+      const int rows = skip_empty && n_act == 0 ? 0 : min(32, M - (m0 + q * 32));
       for (int r = 0; r < rows; ++r) {
         const float4 v = *reinterpret_cast<const float4*>(reg + r * EPI_ROW + lane * 16);
         const long long at = (long long)(m0 + q * 32 + r) * ldo + col;
@@ -330,8 +378,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
         } else {
           double* o = static_cast<double*>(out) + at;
-          const double d0 = scale_pow2(float_bits_to_double(v.x) + float_bits_to_double(v.y), sbv.x);
-          const double d1 = scale_pow2(float_bits_to_double(v.z) + float_bits_to_double(v.w), sbv.y);
+          const double d0 = scale_pow2(df_to_double(v.x, v.y), sbv.x);
+          const double d1 = scale_pow2(df_to_double(v.z, v.w), sbv.y);
           if (vec) {
             *reinterpret_cast<double2*>(o) = make_double2(d0, d1);
           } else {
@@ -432,34 +480,48 @@ struct SrcStage2 {
   __device__ void load4(long long row, int k2, float hi[4], float lo[4]) const {
     const long long a = row / D;
     const int s = (int)(row % D);
+    const int j = k2 >> 1;
+    const int vv = j / MR, b = j % MR;
+    float r[2][2], i[2][2];  // (hi, lo) of the real and imaginary parts of the entries j, j + 1
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int j = (k2 >> 1) + h;
-      const int vv = j / MR, b = j % MR;
-      float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-      if (a < ML && vv < WR) {
-        const int sv = s * WR + vv;
-        for (int e = off[sv]; e < off[sv + 1]; ++e) {
-          const int w = idx[2 * e], t = idx[2 * e + 1];
-          const float4 x = T1[((w * ML + a) * D + t) * (long long)MR + b];
-          const float4 c = val[e];
-          df_mac(rh, rl, c.x, c.y, x.x, x.y);     // + Re c Re x
-          df_mac(rh, rl, -c.z, -c.w, x.z, x.w);   // - Im c Im x
-          df_mac(ih, il, c.x, c.y, x.z, x.w);     // + Re c Im x
-          df_mac(ih, il, c.z, c.w, x.x, x.y);     // + Im c Re x
+    for (int h = 0; h < 2; ++h) r[h][0] = r[h][1] = i[h][0] = i[h][1] = 0.f;
+    auto add = [&](int h, const float4 c, const float4 x) {
+      df_mac(r[h][0], r[h][1], c.x, c.y, x.x, x.y);     // + Re c Re x
+      df_mac(r[h][0], r[h][1], -c.z, -c.w, x.z, x.w);   // - Im c Im x
+      df_mac(i[h][0], i[h][1], c.x, c.y, x.z, x.w);     // + Re c Im x
+      df_mac(i[h][0], i[h][1], c.z, c.w, x.x, x.y);     // + Im c Re x
+    };
+    if (a < ML && vv < WR && b + 1 < MR) {  // one MPO column: both loads of an entry in flight together
+      const int sv = s * WR + vv;
+      for (int e = off[sv]; e < off[sv + 1]; ++e) {
+        const float4* x = T1 + ((idx[2 * e] * ML + a) * D + idx[2 * e + 1]) * (long long)MR + b;
+        const float4 x0 = x[0], x1 = x[1], c = val[e];
+        add(0, c, x0);
+        add(1, c, x1);
+      }
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int v1 = (j + h) / MR, b1 = (j + h) % MR;
+        if (a < ML && v1 < WR) {
+          const int sv = s * WR + v1;
+          for (int e = off[sv]; e < off[sv + 1]; ++e)
+            add(h, val[e], T1[((idx[2 * e] * ML + a) * D + idx[2 * e + 1]) * (long long)MR + b1]);
         }
       }
-      // renormalise so that |lo| <= ulp(hi) / 2
-      float t = __fadd_rn(rh, rl);
-      rl = __fadd_rn(rl, -__fadd_rn(t, -rh));
-      rh = t;
-      t = __fadd_rn(ih, il);
-      il = __fadd_rn(il, -__fadd_rn(t, -ih));
-      ih = t;
-      hi[2 * h] = rh;
-      lo[2 * h] = rl;
-      hi[2 * h + 1] = ih;
-      lo[2 * h + 1] = il;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {  // renormalise so that |lo| <= ulp(hi) / 2
+      float t = __fadd_rn(r[h][0], r[h][1]);
+      r[h][1] = __fadd_rn(r[h][1], -__fadd_rn(t, -r[h][0]));
+      r[h][0] = t;
+      t = __fadd_rn(i[h][0], i[h][1]);
+      i[h][1] = __fadd_rn(i[h][1], -__fadd_rn(t, -i[h][0]));
+      i[h][0] = t;
+      hi[2 * h] = r[h][0];
+      lo[2 * h] = r[h][1];
+      hi[2 * h + 1] = i[h][0];
+      lo[2 * h + 1] = i[h][1];
     }
   }
 };
@@ -794,6 +856,7 @@ inline int pad128(int k) { return (k + 127) / 128 * 128; }
 // ([nch][rows_pad], A operands) or per row ([rows_pad], B operands).
 struct Sliced {
   RawBuf data, scale, mask;
+  unsigned* mk = nullptr;  // the mask in use: mask, or a part of a shared buffer
   int rows_pad = 0, ldk = 0, nch = 0, S = 0, mw = 0;
   bool row_scale = false;
   void shape(DevicePool* pool, int S_, int rows, int K2, bool per_row) {
@@ -806,37 +869,45 @@ struct Sliced {
     data.ensure(pool, sizeof(__nv_bfloat16) * (size_t)S * rows_pad * ldk);
     scale.ensure(pool, sizeof(float) * (size_t)(per_row ? 1 : nch) * rows_pad);
     // one bit per (128-row tile, chunk) holding a nonzero entry (exact zeros of conserved charges)
-    mask.ensure(pool, sizeof(unsigned) * (size_t)(rows_pad / 128) * mw);
+    mask.ensure(pool, mask_words() * sizeof(unsigned));
+    mk = mask.as<unsigned>();
   }
+  size_t mask_words() const { return (size_t)(rows_pad / 128) * mw; }
 };
 
 void clear_mask(cudaStream_t st, Sliced& o) {
-  TDVP_CUDA(cudaMemsetAsync(o.mask.as<void>(), 0, sizeof(unsigned) * (size_t)(o.rows_pad / 128) * o.mw, st));
+  TDVP_CUDA(cudaMemsetAsync(o.mk, 0, sizeof(unsigned) * o.mask_words(), st));
+}
+// gives two shaped operands masks side by side and clears both at once (a memset is a launch)
+void clear_masks(cudaStream_t st, DevicePool* pool, Sliced& a, Sliced& b) {
+  const size_t na = a.mask_words(), nb = b.mask_words();
+  a.mask.ensure(pool, (na + nb) * sizeof(unsigned));
+  a.mk = a.mask.as<unsigned>();
+  b.mk = a.mk + na;
+  TDVP_CUDA(cudaMemsetAsync(a.mk, 0, (na + nb) * sizeof(unsigned), st));
 }
 
-// A operand
+// A operand (its mask cleared before)
 template <class Src>
 void slice(cudaStream_t st, const Src& src, Sliced& o) {
   tdvp_require(!o.row_scale, TDVP_ERR_INVALID_ARG, "slice: A operands carry chunk scales");
-  clear_mask(st, o);
   auto* d = o.data.as<__nv_bfloat16>();
   const int blocks = ceil_div((long long)o.rows_pad * o.nch * 32, 256);
   if (o.S == 4)
     k_slice_chunks<4, Src><<<blocks, 256, 0, st>>>(src, o.rows_pad, o.ldk, o.nch, d, o.scale.as<float>(),
-                                                   o.mask.as<unsigned>(), o.mw);
+                                                   o.mk, o.mw);
   else
     k_slice_chunks<3, Src><<<blocks, 256, 0, st>>>(src, o.rows_pad, o.ldk, o.nch, d, o.scale.as<float>(),
-                                                   o.mask.as<unsigned>(), o.mw);
+                                                   o.mk, o.mw);
   TDVP_CHECK_LAUNCH();
 }
 
-// B operand from opB(B)[k][n] (B row-major with leading dimension ld)
+// B operand from opB(B)[k][n] (B row-major with leading dimension ld; its mask cleared before)
 void slice_b(cudaStream_t st, const cplx* B, long long ld, int K, int N, int op, Sliced& o) {
   tdvp_require(o.row_scale, TDVP_ERR_INVALID_ARG, "slice_b: B operands carry row scales");
-  clear_mask(st, o);
   auto* d = o.data.as<__nv_bfloat16>();
   float* sc = o.scale.as<float>();
-  unsigned* mk = o.mask.as<unsigned>();
+  unsigned* mk = o.mk;
   const bool kcontig = op == OP_T || op == OP_C;
   const int conj = op == OP_C || op == OP_R, rows = o.rows_pad / 2;
   if (kcontig) {
@@ -890,41 +961,76 @@ void launch_bf16s(cudaStream_t st, const CUtensorMap& ma, const CUtensorMap& mb,
   dim3 grid(ceil_div(N, BN), ceil_div(M, BM), splits);
   tdvp_require(grid.y <= 65535 && splits <= 65535, TDVP_ERR_INVALID_ARG, "gemm_bf16s: grid too large");
   k_gemm_bf16s<S><<<grid, THREADS, SCfg<S>::SMEM_BYTES, st>>>(ma, mb, M, N, nkb, kb_split, sA, lsA, sB, out, ldo,
-                                                              split_stride, out_df, d_err, maskA, maskB, mw);
+                                                              split_stride, out_df, splits > 1 ? 1 : 0, d_err, maskA, maskB,
+                                                              mw);
   TDVP_CHECK_LAUNCH();
 }
 
-// Sum of the split-K partials (double-float pairs, one [M][N] slab per split) into
-// the output: FP64, or double-float pairs when out_df.
-// Bound: FP64 (2 operations per cycle and SM against 8 bytes per partial).  So partials that are
-// zero in the whole warp (tiles of other charge sectors: most splits of most entries) cost
-// nothing, and the floats widen by integer operations: 2 FP64 additions per nonzero partial
-// where there were 4 operations for every one.
-// Average over a sweep at bond dimension 256: 37 -> 14 us.
-__global__ void __launch_bounds__(256) k_splitk_df(const float2* __restrict__ ws, int splits, int M, int N,
-                                                   void* __restrict__ out, long long ldo, int out_df) {
-  constexpr int U = 8;  // loads in flight per thread
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long per = (long long)M * N;
-  const bool in = e < per;
-  double sum = 0.0;
-  for (int z0 = 0; z0 < splits; z0 += U) {
-    float2 v[U];
+// Sum of the split-K partials (double-float pairs, one [M][N] slab per split of `cps` chunks) into
+// the output: FP64, or double-float pairs when out_df.  One block per row and 256 columns (N even).
+// Bound: FP64 (2 operations per cycle and SM against 8 bytes per partial) and, for the short sums,
+// latency.  So a warp first reads off the masks which splits of its tile hold a chunk (the GEMM has
+// not written the others: zeros of other charge sectors), loads those all at once, skips partials
+// that are zero in the whole warp, and joins hi and lo by integer operations: one FP64 addition per
+// nonzero partial after the first where there were 4 operations for every one.  The order of the
+// splits is kept.
+// Average over a sweep at bond dimension 256: 37 -> 13 us (the partials themselves are 58 MB there).
+__global__ void __launch_bounds__(128) k_splitk_df(const float2* __restrict__ ws, int splits, int cps, int nchunks,
+                                                   int M, int N, void* __restrict__ out, long long ldo, int out_df,
+                                                   const unsigned* __restrict__ maskA,
+                                                   const unsigned* __restrict__ maskB, int mwords) {
+  constexpr int U = 4;  // splits in flight per thread, two columns each
+  const int m = blockIdx.y, lane = threadIdx.x & 31;
+  const int n0 = blockIdx.x * 256 + 2 * (threadIdx.x & ~31), n = n0 + 2 * lane;
+  if (n0 >= N) return;  // warp-uniform; N is even
+  const long long per = (long long)M * N, e = (long long)m * N + n;
+  const bool in = n < N;
+  unsigned todo;  // splits with a chunk (at most 32); a warp's 64 columns lie in one 128-column tile
+  {
+    const unsigned* a = maskA + (long long)(m >> 7) * mwords;
+    const unsigned* b = maskB + (long long)(n0 >> 7) * mwords;
+    unsigned on = 0;
+    if (lane < splits) {
+      const int lo = lane * cps, hi = min(nchunks, lo + cps) - 1;  // first and last chunk
+      for (int w = lo >> 5; w <= hi >> 5; ++w) {
+        unsigned x = a[w] & b[w];
+        if (w == lo >> 5) x &= ~0u << (lo & 31);
+        if (w == hi >> 5) x &= ~0u >> (31 - (hi & 31));
+        on |= x;
+      }
+    }
+    todo = __ballot_sync(0xffffffffu, on != 0u);
+  }
+  double s0 = 0.0, s1 = 0.0;
+  bool first = true;  // no partial added yet (warp-uniform)
+  while (todo) {
+    float4 v[U];
 #pragma unroll
-    for (int q = 0; q < U; ++q)
-      v[q] = in && z0 + q < splits ? __ldcs(&ws[(z0 + q) * per + e]) : make_float2(0.f, 0.f);
+    for (int q = 0; q < U; ++q) {
+      const int z = __ffs(todo) - 1;  // -1: none left
+      todo &= todo - 1;
+      v[q] = in && z >= 0 ? *reinterpret_cast<const float4*>(ws + z * per + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 #pragma unroll
-    for (int q = 0; q < U; ++q)
-      if (__any_sync(0xffffffffu, ((__float_as_uint(v[q].x) | __float_as_uint(v[q].y)) << 1) != 0u))
-        sum += float_bits_to_double(v[q].x) + float_bits_to_double(v[q].y);
+    for (int q = 0; q < U; ++q) {
+      const unsigned bits = __float_as_uint(v[q].x) | __float_as_uint(v[q].y) | __float_as_uint(v[q].z) |
+                            __float_as_uint(v[q].w);
+      if (!__any_sync(0xffffffffu, (bits << 1) != 0u)) continue;
+      const double t0 = df_to_double(v[q].x, v[q].y), t1 = df_to_double(v[q].z, v[q].w);
+      s0 = first ? t0 : s0 + t0;
+      s1 = first ? t1 : s1 + t1;
+      first = false;
+    }
   }
   if (!in) return;
-  const long long m = e / N, n = e % N;
   if (out_df) {
-    const float hi = (float)sum;
-    static_cast<float2*>(out)[m * ldo + n] = make_float2(hi, (float)(sum - (double)hi));
+    float2* o = static_cast<float2*>(out) + m * ldo + n;
+    o[0] = double_to_df(s0);
+    o[1] = double_to_df(s1);
   } else {
-    static_cast<double*>(out)[m * ldo + n] = sum;
+    double* o = static_cast<double*>(out) + m * ldo + n;
+    o[0] = s0;
+    o[1] = s1;
   }
 }
 
@@ -964,7 +1070,7 @@ void gemm_bf16s(cudaStream_t st, DevicePool* pool, const Sliced& A, const Sliced
   const int nkb = A.ldk / BK;
   const int nchunks = (nkb + KC_KB - 1) / KC_KB;
   const long long tiles = (long long)ceil_div(N, BN) * ceil_div(M, BM);
-  const int splits = pool ? choose_splits(tiles, nchunks) : 1;
+  const int splits = pool && M <= 65535 ? choose_splits(tiles, nchunks) : 1;  // at most 32
   const int kb_split = splits > 1 ? ((nchunks + splits - 1) / splits) * KC_KB : nkb;
   RawBuf ws;
   void* dst = out;
@@ -979,8 +1085,8 @@ void gemm_bf16s(cudaStream_t st, DevicePool* pool, const Sliced& A, const Sliced
   }
   tdvp_require(A.mw == B.mw && (kb_split + KC_KB - 1) / KC_KB <= kMaxChunks, TDVP_ERR_INVALID_ARG,
                "gemm_bf16s: chunk masks or chunks per split out of range");
-  const unsigned* mA = A.mask.as<unsigned>();
-  const unsigned* mB = B.mask.as<unsigned>();
+  const unsigned* mA = A.mk;
+  const unsigned* mB = B.mk;
   if (A.S == 4)
     launch_bf16s<4>(st, ma, mb, M, N, nkb, kb_split, splits, A.scale.as<float>(), A.rows_pad, B.scale.as<float>(),
                     dst, ld, stride, df, d_err, mA, mB, A.mw);
@@ -988,8 +1094,8 @@ void gemm_bf16s(cudaStream_t st, DevicePool* pool, const Sliced& A, const Sliced
     launch_bf16s<3>(st, ma, mb, M, N, nkb, kb_split, splits, A.scale.as<float>(), A.rows_pad, B.scale.as<float>(),
                     dst, ld, stride, df, d_err, mA, mB, A.mw);
   if (splits > 1) {
-    const long long n = (long long)M * N;
-    k_splitk_df<<<ceil_div(n, 256), 256, 0, st>>>(ws.as<float2>(), splits, M, N, out, ldo, out_df ? 1 : 0);
+    k_splitk_df<<<dim3(ceil_div(N, 256), M), 128, 0, st>>>(ws.as<float2>(), splits, kb_split / KC_KB, nchunks, M, N, out,
+                                                          ldo, out_df ? 1 : 0, mA, mB, A.mw);
     TDVP_CHECK_LAUNCH();
   }
 }
@@ -1038,22 +1144,25 @@ void heff_bf16s(cudaStream_t st, Scratch& s, const SiteOp& op, const cplx* x, cp
   if (op.env_key < 0 || c.key != op.env_key || c.S != S) {
     // L as the A operand: rows (w, a), K = (a', re/im)
     c.L.shape(pool, S, ml * wl, 2 * ml, false);
+    c.R.shape(pool, S, 2 * mr, 2 * wr * mr, true);
+    clear_mask(st, c.L);
+    clear_mask(st, c.R);
     slice(st, SrcLwa{op.L, ml, wl}, c.L);
     // R[b][(v,b')] is B[k=(v,b')][n=b] stored n-major (op T)
-    c.R.shape(pool, S, 2 * mr, 2 * wr * mr, true);
     slice_b(st, op.R, (long long)wr * mr, wr * mr, mr, OP_T, c.R);
     c.key = op.env_key;
     c.S = S;
   }
   // stage 1: T1[(w,a)][(s',b',c)] = L x     (x[a'][(s',b')] is B[k=a'][n=(s',b')])
   c.X.shape(pool, S, 2 * d * mr, 2 * ml, true);
+  c.T2.shape(pool, S, ml * d, 2 * wr * mr, false);
+  clear_masks(st, pool, c.X, c.T2);
   slice_b(st, x, (long long)d * mr, ml, d * mr, OP_N, c.X);
   const int M1 = ml * wl, N1 = 2 * d * mr;
   c.T1.ensure(pool, sizeof(float2) * (size_t)M1 * N1);  // double-float
   gemm_bf16s(st, pool, c.L, c.X, M1, N1, c.T1.as<void>(), N1, true, err);
   // stage 2: MPO tensor, sliced straight into the stage-3 A operand
   const WSparse& ws = *op.W;
-  c.T2.shape(pool, S, ml * d, 2 * wr * mr, false);
   tdvp_require(ws.d_l_val_df != nullptr, TDVP_ERR_INVALID_ARG, "heff_bf16s: MPO site without double-float values");
   slice(st, SrcStage2{c.T1.as<float4>(), ws.d_l_off, ws.d_l_idx, ws.d_l_val_df, ml, wl, wr, d, mr}, c.T2);
   // stage 3: y[(a,s)][(b,c)] = T2 R^T
@@ -1067,8 +1176,9 @@ void zgemm_bf16s(cudaStream_t st, Scratch& s, int S, int opA, int opB, int M, in
   int* err = tc_error_word(st, s);
   Sliced a, b;
   a.shape(pool, S, M, 2 * std::max(K, 1), false);
-  slice(st, SrcA{A, lda, M, K, opA}, a);
   b.shape(pool, S, 2 * N, 2 * std::max(K, 1), true);
+  clear_masks(st, pool, a, b);
+  slice(st, SrcA{A, lda, M, K, opA}, a);
   slice_b(st, B, ldb, K, N, opB, b);
   gemm_bf16s(st, pool, a, b, M, 2 * N, C, 2 * ldc, false, err);
 }
