@@ -838,48 +838,23 @@ void fill_zero(cudaStream_t st, cplx* p, long long n) {
 //                              = e^{|delta| hi} sum_k eps_k e^{-x} I_k(x) T_k(X),        delta < 0
 // with x = |delta| h, eps_0 = 1, eps_k = 2.  J_k and e^{-x} I_k come from Miller's
 // backward recurrence normalised by J_0 + 2 sum J_2k = 1 and I_0 + 2 sum I_k = e^x.
-// One warp: lane l owns the components l and l + 32 (n <= 63), neighbours by shuffles.
-// Bound: a serial chain of FP64 operations (K + M of them, each waiting for the last).  So the
-// chain holds nothing but its recurrences: the quotients 2 k / x and the divisions by the norm are
-// formed by all lanes beside it, and a single warp needs no block barrier per term (80 us -> 25 us
-// per exponential at n = 10).  Block b takes the leading n0 + b rows: the stopping tests of the
-// iterations of one batch run side by side.
+// Lane l of a warp owns the components l and l + 32 (n <= 63), neighbours by shuffles.
+// Bound: serial chains of FP64 instructions, 65 cycles each on the FP64 unit of a warp's scheduler
+// (a division 1800, a cosine 1300).  So the chains run on different schedulers: Miller recurrence and
+// norm, Chebyshev vectors, phase; the quotients 2 k / x and the divisions by the norm are formed by
+// all lanes.  80 us -> 46 us by one warp -> 22 us at n = 10.  Block b takes the leading n0 + b rows:
+// the stopping tests of the iterations of one batch run side by side.
 // ============================================================================
 namespace {
-__global__ void __launch_bounds__(32)
-    k_tridiag_expv(const double* __restrict__ alpha, const double* __restrict__ beta, int n0, double delta, int kind,
-                   cplx* __restrict__ y, double* __restrict__ err) {
+constexpr int PAR_K = 95;  // orders the parallel path keeps vectors for (x up to about 15)
+
+// T_k(X) e_0 and the coefficients one after the other, by one warp: are, aim of its components
+__device__ __noinline__ void tridiag_serial(int n, int K, double x, double delta, int kind, double c, double h,
+                                            const double (&d)[2], const double (&ol)[2], const double (&orr)[2],
+                                            double* coef, double (&are)[2], double (&aim)[2]) {
   constexpr unsigned FULL = 0xffffffffu;
-  __shared__ double coef[CHEB_MAX + 1];
-  const int n = n0 + blockIdx.x;
-  y += (long long)blockIdx.x * TRI_MAX;
-  err += 2 * blockIdx.x;
-  const int lane = threadIdx.x;
-  const bool two = n > 32;  // warp-uniform: components 32.. exist
-  double d[2], ol[2], orr[2];
-  double lo = 1e300, hi = -1e300;
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    const int i = lane + 32 * c;
-    d[c] = i < n ? alpha[i] : 0.0;
-    ol[c] = (i >= 1 && i < n) ? beta[i] : 0.0;
-    orr[c] = (i + 1 < n) ? beta[i + 1] : 0.0;
-    if (i < n) {
-      const double rad = fabs(ol[c]) + fabs(orr[c]);
-      lo = fmin(lo, d[c] - rad);
-      hi = fmax(hi, d[c] + rad);
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fmin(lo, __shfl_xor_sync(FULL, lo, o));
-    hi = fmax(hi, __shfl_xor_sync(FULL, hi, o));
-  }
-  const double c = 0.5 * (hi + lo), h = 0.5 * (hi - lo);
-  const double x = fabs(delta) * h;
-  int K = (int)(x + 10.0 * cbrt(x + 1.0) + 40.0);
-  const bool bad = K > CHEB_MAX;
-  if (bad) K = CHEB_MAX;
+  const int lane = threadIdx.x & 31;
+  const bool two = n > 32;
   for (int k = lane; k <= K; k += 32) coef[k] = 0.0;
   __syncwarp();
   double norm = 1.0;
@@ -932,7 +907,8 @@ __global__ void __launch_bounds__(32)
   }
   __syncwarp();
   const double inv_h = h > 0.0 ? 1.0 / h : 0.0;
-  double xd[2], xl[2], xr[2], cur[2], prev[2] = {0.0, 0.0}, are[2] = {0.0, 0.0}, aim[2] = {0.0, 0.0};
+  double xd[2], xl[2], xr[2], cur[2], prev[2] = {0.0, 0.0};
+  are[0] = are[1] = aim[0] = aim[1] = 0.0;
 #pragma unroll
   for (int q = 0; q < 2; ++q) {  // X = (T - c) / h
     xd[q] = lane + 32 * q < n ? (d[q] - c) * inv_h : 0.0;
@@ -968,13 +944,131 @@ __global__ void __launch_bounds__(32)
     prev[0] = cur[0];
     cur[0] = nxt;
   }
+}
+
+__global__ void __launch_bounds__(128)
+    k_tridiag_expv(const double* __restrict__ alpha, const double* __restrict__ beta, int n0, double delta, int kind,
+                   cplx* __restrict__ y, double* __restrict__ err) {
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ double coef[CHEB_MAX + 1];
+  __shared__ double quot[128], jv[128], tk[PAR_K + 1][32], im_sum[32], phase[2];
+  __shared__ int rescaled;
+  const int n = n0 + blockIdx.x;
+  y += (long long)blockIdx.x * TRI_MAX;
+  err += 2 * blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool two = n > 32;  // warp-uniform: components 32.. exist
+  double d[2], ol[2], orr[2];
+  double lo = 1e300, hi = -1e300;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int i = lane + 32 * c;
+    d[c] = i < n ? alpha[i] : 0.0;
+    ol[c] = (i >= 1 && i < n) ? beta[i] : 0.0;
+    orr[c] = (i + 1 < n) ? beta[i + 1] : 0.0;
+    if (i < n) {
+      const double rad = fabs(ol[c]) + fabs(orr[c]);
+      lo = fmin(lo, d[c] - rad);
+      hi = fmax(hi, d[c] + rad);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(FULL, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(FULL, hi, o));
+  }
+  const double c = 0.5 * (hi + lo), h = 0.5 * (hi - lo);
+  const double x = fabs(delta) * h;
+  int K = (int)(x + 10.0 * cbrt(x + 1.0) + 40.0);
+  const bool bad = K > CHEB_MAX;
+  if (bad) K = CHEB_MAX;
+  const int M = 2 * ((K + 40 + (int)fmin(x, 4096.0)) / 2 + 1);
+  double are[2] = {0.0, 0.0}, aim[2] = {0.0, 0.0};
+  // The usual case: the Miller recurrence (warp 0), the Chebyshev vectors (warp 1) and the phase (warp 3)
+  // run side by side, each on its scheduler's FP64 unit; then the two sums.
+  bool par = n <= 32 && K <= PAR_K && M < 128 && x >= 1e-300;
+  if (par) {
+    if (threadIdx.x < M) quot[threadIdx.x + 1] = 2.0 * (double)(threadIdx.x + 1) / x;
+    if (threadIdx.x == 0) rescaled = 0;
+    __syncthreads();
+    if (warp == 0) {
+      double jp1 = 0.0, jk = 1e-280;
+      bool big = false;
+      for (int k = M; k >= 1; --k) {
+        if (lane == 0) jv[k] = jk;
+        const double jm1 = fma(quot[k], jk, kind == 0 ? -jp1 : jp1);
+        jp1 = jk;
+        jk = jm1;
+        big = big || (__double2hiint(jk) & 0x7fffffff) >= 0x73e00000;  // near 1e250: the serial path rescales
+      }
+      if (lane == 0) {
+        jv[0] = jk;
+        rescaled = big;
+      }
+      __syncwarp();
+      double norm = 0.0;
+      for (int k = M; k >= 1; --k)
+        if (kind != 0 || (k & 1) == 0) norm = fma(2.0, jv[k], norm);
+      norm += jk;
+      for (int k = lane; k <= K; k += 32) {
+        double ck = jv[k] / norm;
+        if (k > 0) ck *= 2.0;
+        const bool neg = kind == 0 ? ((k & 1) ? (((k & 3) == 1) == (delta >= 0)) : (k & 3) == 2) : delta >= 0 && (k & 1);
+        coef[k] = neg ? -ck : ck;
+      }
+    } else if (warp == 1) {
+      const double inv_h = h > 0.0 ? 1.0 / h : 0.0;
+      const double xd = lane < n ? (d[0] - c) * inv_h : 0.0, xl = ol[0] * inv_h, xr = orr[0] * inv_h;
+      double cur = lane == 0 ? 1.0 : 0.0, prev = 0.0;
+      for (int k = 0; k <= K; ++k) {
+        tk[k][lane] = cur;
+        const double up = __shfl_up_sync(FULL, cur, 1), dn = __shfl_down_sync(FULL, cur, 1);
+        const double nx = fma(xr, dn, fma(xl, up, __dmul_rn(xd, cur)));
+        const double nxt = k == 0 ? nx : fma(2.0, nx, -prev);
+        prev = cur;
+        cur = nxt;
+      }
+    } else if (warp == 3) {
+      double fre, fim = 0.0;
+      if (kind == 0) {
+        const double ph = -delta * c;
+        fre = cos(ph);
+        fim = sin(ph);
+      } else {
+        fre = (delta >= 0) ? exp(-delta * lo) : exp(-delta * hi);
+      }
+      if (lane == 0) {
+        phase[0] = fre;
+        phase[1] = fim;
+      }
+    }
+    __syncthreads();
+    par = !rescaled;
+  }
+  if (par) {
+    if (warp == 0)
+      for (int k = 0; k <= K; k += kind == 0 ? 2 : 1) are[0] = fma(coef[k], tk[k][lane], are[0]);
+    if (warp == 1 && kind == 0) {
+      for (int k = 1; k <= K; k += 2) aim[0] = fma(coef[k], tk[k][lane], aim[0]);
+      im_sum[lane] = aim[0];
+    }
+    __syncthreads();
+    if (warp == 0 && kind == 0) aim[0] = im_sum[lane];
+  }
+  if (warp != 0) return;
   double fre, fim = 0.0;
-  if (kind == 0) {
-    const double ph = -delta * c;
-    fre = cos(ph);
-    fim = sin(ph);
+  if (par) {
+    fre = phase[0];
+    fim = phase[1];
   } else {
-    fre = (delta >= 0) ? exp(-delta * lo) : exp(-delta * hi);
+    tridiag_serial(n, K, x, delta, kind, c, h, d, ol, orr, coef, are, aim);
+    if (kind == 0) {
+      const double ph = -delta * c;
+      fre = cos(ph);
+      fim = sin(ph);
+    } else {
+      fre = (delta >= 0) ? exp(-delta * lo) : exp(-delta * hi);
+    }
   }
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -997,7 +1091,7 @@ void tridiag_expv(cudaStream_t st, const double* alpha, const double* beta, int 
                   cplx* y, double* err) {
   tdvp_require(n0 >= 1 && count >= 1 && n0 + count - 1 < TRI_MAX, TDVP_ERR_INVALID_ARG,
                "tridiag_expv: n out of range");
-  k_tridiag_expv<<<count, 32, 0, st>>>(alpha, beta, n0, delta, kind, y, err);
+  k_tridiag_expv<<<count, 128, 0, st>>>(alpha, beta, n0, delta, kind, y, err);
   TDVP_CHECK_LAUNCH();
 }
 
@@ -1103,6 +1197,56 @@ __device__ __forceinline__ bool jacobi_params(T a, T b, C c, T tol, T floor2, T&
   return true;
 }
 
+// The same rotation from an angle good to FP32, for a = |x_p|^2, b = |x_q|^2 in FP64: any complex
+// tangent tau = t e^{i phi} gives a unitary rotation, cs = 1 / sqrt(1 + |tau|^2), sne = cs tau, so only
+// that normalisation has to be exact.  A coupling |c| is then left at 6e-8 |c| instead of at rounding,
+// which the sweep after it removes; the last sweep's angles are below 1e-8, so it leaves 6e-16 of
+// sqrt(a b), under the tolerance (sqrt(p) 2.2e-16 or more) below which pairs are not rotated at all.
+// 15 FP64 instructions of 65 cycles each, where the exact angle's two reciprocal roots, root and
+// division are about 70.
+__device__ __forceinline__ float high_float(double x, int add) {  // x 2^add towards zero; 0 below FP32's range
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ff) - 1023 + 127 + add;
+  if (e <= 0) return 0.f;
+  if (e >= 255) return __uint_as_float((h & 0x80000000u) | 0x7f7fffffu);
+  return __uint_as_float((h & 0x80000000u) | ((unsigned)e << 23) | ((h & 0xfffffu) << 3) | (l >> 29));
+}
+__device__ __forceinline__ double wide_double(float x) {  // (double)x by its bits; 0 for a subnormal
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+  if (e == 0) return 0.0;
+  return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
+}
+__device__ __forceinline__ bool jacobi_params_quick(double a, double b, double2 c, double tol2, double floor2,
+                                                    double& cs, double2& sne) {
+  // comparisons of non-negative doubles by their bits
+  const long long la = __double_as_longlong(a), lb = __double_as_longlong(b);
+  const double big = la > lb ? a : b, small = la > lb ? b : a;
+  if (__double_as_longlong(big) <= __double_as_longlong(floor2) ||
+      __double_as_longlong(small) <= __double_as_longlong(kJacobiFloor * big))
+    return false;
+  const double ac2 = cabs2_fma(c);
+  if (__double_as_longlong(ac2) <= __double_as_longlong(tol2 * a * b)) return false;
+  if ((__double2hiint(ac2) & 0x7ff00000) == 0x7ff00000) return false;  // not finite: the norms will say so
+  const int sh = -((((__double2hiint(ac2) >> 20) & 0x7ff) - 1023) >> 1);  // |c| 2^sh in [1, 2)
+  const float cx = high_float(c.x, sh), cy = high_float(c.y, sh);
+  const float inv = rsqrtf(cx * cx + cy * cy);
+  const float zeta = 0.5f * high_float(b - a, sh) * inv;
+  const float az = fabsf(zeta);
+  const float t = copysignf(az > 1e9f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az)), zeta) * inv;
+  const double tx = wide_double(t * cx), ty = wide_double(t * cy);
+  const double m = fma(tx, tx, fma(ty, ty, 1.0));  // [1, 2]
+  // 1 / sqrt(m): FP32 seed, one third-order step (error (5/16) (2^-22)^3)
+  const double r = wide_double(rsqrtf(high_float(m, 0)));
+  const double e = fma(-(m * r), r, 1.0);
+  cs = fma(r, e * fma(0.375, e, 0.5), r);
+  sne = make_double2(cs * tx, cs * ty);
+  return true;
+}
+__device__ __forceinline__ bool jacobi_params_quick(float a, float b, float2 c, float tol2, float floor2, float& cs,
+                                                    float2& sne) {
+  return jacobi_params(a, b, c, sqrtf(tol2), floor2, cs, sne);  // FP32 rotations have no shorter form
+}
+
 template <class T, class C>
 __device__ __forceinline__ void rotate_pair(C& xp, C& xq, T cs, C sne) {
   // xp' = cs xp - conj(sne) xq ; xq' = sne xp + cs xq
@@ -1131,7 +1275,7 @@ __global__ void k_svd_prepare(const cplx* __restrict__ M, int rows, int cols, in
 // |sin theta| above 1e-8 was applied (kJacobiSmallAngle2).
 template <class T>
 __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename Jac<T>::C* __restrict__ V, int p, int q,
-                                  int P, int Q, T tol, T floor2, int want_v) {
+                                  int P, int Q, T tol, T floor2, int want_v, int quick = 0) {
   typedef typename Jac<T>::C C;
   __shared__ T rs[8][4];
   __shared__ T s_cs;
@@ -1153,20 +1297,21 @@ __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename J
     warp_sum_values(h, rs[warp]);  // halving: 6 additions per lane instead of 20
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    T A = 0, B = 0;
-    C Cc = Jac<T>::make(0, 0);
+  if (threadIdx.x < 32) {
     const int active = min((int)(blockDim.x >> 5), (p + 31) >> 5);  // the others hold exact zeros
-    for (int u = 0; u < active; ++u) {
-      A += rs[u][0];
-      B += rs[u][1];
-      Cc = cadd(Cc, Jac<T>::make(rs[u][2], rs[u][3]));
-    }
+    T tot = 0;
+    for (int u = 0; u < active; ++u) tot += rs[u][threadIdx.x & 3];  // one of the four sums per lane
+    const T A = __shfl_sync(0xffffffffu, tot, 0), B = __shfl_sync(0xffffffffu, tot, 1);
+    const C Cc = Jac<T>::make(__shfl_sync(0xffffffffu, tot, 2), __shfl_sync(0xffffffffu, tot, 3));
     T cs;
     C sne;
-    s_do = jacobi_params(A, B, Cc, tol, floor2, cs, sne) ? 1 : 0;
-    s_cs = cs;
-    s_sne = sne;
+    const bool rot = quick ? jacobi_params_quick(A, B, Cc, tol * tol, floor2, cs, sne)
+                           : jacobi_params(A, B, Cc, tol, floor2, cs, sne);
+    if (threadIdx.x == 0) {
+      s_do = !rot ? 0 : cabs2(sne) > Jac<T>::small_angle2 ? 2 : 1;
+      s_cs = cs;
+      s_sne = sne;
+    }
   }
   __syncthreads();
   const int doit = s_do;
@@ -1180,7 +1325,6 @@ __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename J
     xp[r] = u;
     xq[r] = v;
   }
-  const bool significant = cabs2(sne) > Jac<T>::small_angle2;
   if (want_v) {
     C* vp = V + (long long)P * q;
     C* vq = V + (long long)Q * q;
@@ -1191,7 +1335,7 @@ __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename J
       vq[r] = v;
     }
   }
-  return significant;
+  return doit == 2;
 }
 
 // Grid-wide barrier for the cooperative path (all blocks co-resident by cooperative
@@ -1607,7 +1751,7 @@ __global__ void k_gather_batched(const cplx* __restrict__ M, int cols, const Blk
 template <class T>
 __global__ void __launch_bounds__(256)
     k_jacobi_batched(typename Jac<T>::C* __restrict__ X, typename Jac<T>::C* __restrict__ V,
-                     const BlkDesc* __restrict__ desc, int max_sweeps, double* __restrict__ s_out,
+                     const BlkDesc* __restrict__ desc, int max_sweeps, int quick, double* __restrict__ s_out,
                      int* __restrict__ bad) {
   typedef typename Jac<T>::C C;
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -1662,7 +1806,9 @@ __global__ void __launch_bounds__(256)
         }
         T cs;
         C sne;
-        if (!jacobi_params(a, b, c, tol, floor2, cs, sne)) continue;
+        if (!(quick ? jacobi_params_quick(a, b, c, tol * tol, floor2, cs, sne)
+                    : jacobi_params(a, b, c, tol, floor2, cs, sne)))
+          continue;
         if (lane == 0 && cabs2(sne) > Jac<T>::small_angle2) s_rot = 1;
         for (int r = lane; r < p; r += 32) {
           C u = xp[r], v = xq[r];
@@ -1715,7 +1861,7 @@ __global__ void __launch_bounds__(256)
     k_pchol_batched(cplx* __restrict__ X, BlkDesc* __restrict__ desc, int* __restrict__ piv, double rel_floor) {
   __shared__ double s_val[8];
   __shared__ int s_idx[8];
-  __shared__ double s_thr, s_piv;
+  __shared__ double s_thr, s_piv, s_ljj, s_inv;
   __shared__ int s_k;
   BlkDesc& dref = desc[blockIdx.x];
   const int n = dref.p;
@@ -1794,9 +1940,13 @@ __global__ void __launch_bounds__(256)
       }
       __syncthreads();
     }
-    const double ljj = sqrt(A[(long long)j * n + j].x);
-    const double inv = 1.0 / ljj;
+    // one warp's square root and division (2800 cycles of an FP64 unit), not eight
+    if (tid == 0) {
+      s_ljj = sqrt(A[(long long)j * n + j].x);
+      s_inv = 1.0 / s_ljj;
+    }
     __syncthreads();
+    const double ljj = s_ljj, inv = s_inv;
     for (int i = tid; i < n; i += blockDim.x) {
       cplx& a = A[(long long)j * n + i];
       if (i > j)
@@ -1930,7 +2080,7 @@ __device__ __forceinline__ bool group_sync(GridBar* b, unsigned n, int* gerr, un
 template <class T>
 __global__ void __launch_bounds__(256)
     k_jacobi_groups(typename Jac<T>::C* __restrict__ X, typename Jac<T>::C* __restrict__ V,
-                    const BlkDesc* __restrict__ desc, const int* __restrict__ cta_off, int nblk, int max_sweeps,
+                    const BlkDesc* __restrict__ desc, const int* __restrict__ cta_off, int nblk, int max_sweeps, int quick,
                     double* __restrict__ fro2, int* __restrict__ flags, GridBar* __restrict__ bars,
                     int* __restrict__ gerr, double* __restrict__ s_out, int* __restrict__ stat) {
   typedef typename Jac<T>::C C;
@@ -1976,7 +2126,7 @@ __global__ void __launch_bounds__(256)
         int P, Q;
         rr_pair(round, k, qpad, P, Q);
         if (Q >= d.q) continue;
-        if (jacobi_pair_block(X + d.x_off, V + d.v_off, d.p, d.q, P, Q, tol, floor2, d.need_v) && threadIdx.x == 0)
+        if (jacobi_pair_block(X + d.x_off, V + d.v_off, d.p, d.q, P, Q, tol, floor2, d.need_v, quick) && threadIdx.x == 0)
           rot[sweep % 3] = 1;
       }
       if (!group_sync(bar, n_b, gerr, epoch)) return;
@@ -2020,6 +2170,7 @@ __global__ void __launch_bounds__(256)
                    const int* __restrict__ cta_off, int nblk, double rel_floor, double* __restrict__ pval,
                    int* __restrict__ pidx, GridBar* __restrict__ bars, int* __restrict__ gerr) {
   __shared__ double s_val[8];
+  __shared__ double s_ljj, s_inv;
   __shared__ int s_idx[8];
   int lo = 0, hi = nblk - 1;
   while (lo < hi) {
@@ -2136,9 +2287,13 @@ __global__ void __launch_bounds__(256)
         }
         __syncthreads();
       }
-      const double ljj = sqrt(A[(long long)j * n + j].x);
-      const double inv = 1.0 / ljj;
+      // one warp's square root and division (2800 cycles of an FP64 unit), not eight
+      if (tid == 0) {
+        s_ljj = sqrt(A[(long long)j * n + j].x);
+        s_inv = 1.0 / s_ljj;
+      }
       __syncthreads();
+      const double ljj = s_ljj, inv = s_inv;
       for (int i = tid; i < n; i += blockDim.x) {
         cplx& a = A[(long long)j * n + i];
         if (i > j)
@@ -2220,7 +2375,7 @@ void run_pchol_groups(cudaStream_t st, DevicePool* pool, cplx* Xs, BlkDesc* d_de
 
 template <class T>
 void run_jacobi_multi(cudaStream_t st, DevicePool* pool, typename Jac<T>::C* Xs, typename Jac<T>::C* Vs,
-                      const std::vector<BlkDesc>& desc, const BlkDesc* d_desc, double* d_s, int* d_stat) {
+                      const std::vector<BlkDesc>& desc, const BlkDesc* d_desc, bool quick, double* d_s, int* d_stat) {
   const int nblk = (int)desc.size();
   static const int max_ctas = [] {
     int dev = 0, sms = 0, per_sm = 0;
@@ -2256,10 +2411,10 @@ void run_jacobi_multi(cudaStream_t st, DevicePool* pool, typename Jac<T>::C* Xs,
   double* d_fro2 = reinterpret_cast<double*>(base + o_fro);
   GridBar* bars = reinterpret_cast<GridBar*>(base + o_bar);
   TDVP_CUDA(cudaMemsetAsync(d_stat, 0, 3 * sizeof(int), st));
-  int nb = nblk, ms = 60;
+  int nb = nblk, ms = 60, qk = quick ? 1 : 0;
   const BlkDesc* dd = d_desc;
   const int* po = d_off;
-  void* args[] = {&Xs, &Vs, &dd, &po, &nb, &ms, &d_fro2, &d_flags, &bars, &d_gerr, &d_s, &d_stat};
+  void* args[] = {&Xs, &Vs, &dd, &po, &nb, &ms, &qk, &d_fro2, &d_flags, &bars, &d_gerr, &d_s, &d_stat};
   TDVP_CUDA(cudaLaunchCooperativeKernel((void*)k_jacobi_groups<T>, dim3(nctas), dim3(256), args, 0, st));
   g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
   int herr = 0;
@@ -2376,7 +2531,7 @@ void gather_rows(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int
 
 void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols,
                       int (*select)(const std::vector<double>& s, void* ctx), void* ctx, SvdOut& out, bool want_u,
-                      bool want_v, bool psd, bool jacobi_fp32) {
+                      bool want_v, bool psd, bool jacobi_fp32, bool quick) {
   g_svd_counters.calls++;
   const long long n = (long long)rows * cols;
   if (rows <= 1 || cols <= 1 || n > (1LL << 27)) {
@@ -2509,19 +2664,19 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
       k_to_c64<<<ceil_div(std::max<long long>(1, vo), 256), 256, 0, st>>>(Vs.data(), v32.as<float2>(), vo);
       TDVP_CHECK_LAUNCH();
       if (!multi) {
-        k_jacobi_batched<float><<<nsmall, 256, smem_need / 2, st>>>(x32.as<float2>(), v32.as<float2>(), d_desc, 60,
+        k_jacobi_batched<float><<<nsmall, 256, smem_need / 2, st>>>(x32.as<float2>(), v32.as<float2>(), d_desc, 60, 0,
                                                                    d_s, d_bad);
         TDVP_CHECK_LAUNCH();
       } else {
-        run_jacobi_multi<float>(st, pool, x32.as<float2>(), v32.as<float2>(), desc, d_desc, d_s, d_bad);
+        run_jacobi_multi<float>(st, pool, x32.as<float2>(), v32.as<float2>(), desc, d_desc, false, d_s, d_bad);
       }
       k_to_c128<<<ceil_div(std::max<long long>(1, xo), 256), 256, 0, st>>>(x32.as<float2>(), Xs.data(), xo);
       TDVP_CHECK_LAUNCH();
     } else if (!multi) {
-      k_jacobi_batched<double><<<nsmall, 256, smem_need, st>>>(Xs.data(), Vs.data(), d_desc, 60, d_s, d_bad);
+      k_jacobi_batched<double><<<nsmall, 256, smem_need, st>>>(Xs.data(), Vs.data(), d_desc, 60, quick ? 1 : 0, d_s, d_bad);
       TDVP_CHECK_LAUNCH();
     } else {
-      run_jacobi_multi<double>(st, pool, Xs.data(), Vs.data(), desc, d_desc, d_s, d_bad);
+      run_jacobi_multi<double>(st, pool, Xs.data(), Vs.data(), desc, d_desc, quick, d_s, d_bad);
     }
     jac.reset();
     std::vector<double> hs(so);
@@ -2649,6 +2804,23 @@ __device__ __forceinline__ void qr_block_sums(cplx* acc, int n, cplx (*red)[kQrC
   __syncthreads();
 }
 
+// The scalars of a reflector from |x|^2 and its leading entry a, by one whole warp: nrm = |x|, beta,
+// inv = 1 / (a - beta) = e^{-i arg a} / (|a| + |x|) and tau.  A warp's FP64 instruction takes 65 cycles
+// of its scheduler's unit whatever lanes are active, so a square root is 1000 and a division 1800: the
+// two roots run in two lanes of one sequence, the three divisions in three (7300 -> 2800 cycles).
+__device__ __forceinline__ void qr_scalars(double nrm2, cplx a, double& nrm, cplx& beta, cplx& inv, double& tau) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const double root = sqrt(lane == 1 ? cabs2_fma(a) : nrm2);
+  nrm = __shfl_sync(FULL, root, 0);
+  const double aa = __shfl_sync(FULL, root, 1), den = aa + nrm;
+  const double quot = (lane == 2 ? den : 1.0) / (lane == 0 ? (aa > 0.0 ? aa : 1.0) : lane == 1 ? den : nrm);
+  const cplx ph = aa > 0.0 ? cscale(a, __shfl_sync(FULL, quot, 0)) : mkc(1.0, 0.0);
+  inv = cscale(cconj(ph), __shfl_sync(FULL, quot, 1));
+  tau = __shfl_sync(FULL, quot, 2);
+  beta = cscale(ph, -nrm);
+}
+
 // Reflector j from column j of X_b (rows j..p-1), by the whole block.
 __device__ void qr_make_reflector(cplx* __restrict__ Xb, int p, int j, double* __restrict__ tau,
                                   cplx (*red)[kQrChunk], cplx* tot) {
@@ -2658,19 +2830,17 @@ __device__ void qr_make_reflector(cplx* __restrict__ Xb, int p, int j, double* _
   cplx acc[1] = {mkc(0.0, 0.0)};
   for (int r = j + threadIdx.x; r < p; r += blockDim.x) acc[0].x = __dadd_rn(acc[0].x, cabs2_fma(x[r]));
   qr_block_sums(acc, 1, red, tot);
-  if (threadIdx.x == 0) {
-    const double nrm = sqrt(tot[0].x);
+  if (threadIdx.x < 32) {
+    double nrm, t;
+    cplx beta, inv;
     const cplx a = x[j];
-    s_zero = !(nrm > 0.0);
-    if (s_zero) {
-      tau[j] = 0.0;
-    } else {
-      const double aa = sqrt(cabs2_fma(a));
-      const cplx ph = aa > 0.0 ? cscale(a, 1.0 / aa) : mkc(1.0, 0.0);
-      const double den = aa + nrm;
-      s_inv = cscale(cconj(ph), 1.0 / den);  // 1 / (x_j - beta) = e^{-i arg x_j} / (|x_j| + |x|)
-      tau[j] = den / nrm;
-      x[j] = cscale(ph, -nrm);  // beta
+    qr_scalars(tot[0].x, a, nrm, beta, inv, t);
+    __syncwarp();
+    if (threadIdx.x == 0) {
+      s_zero = !(nrm > 0.0);
+      tau[j] = s_zero ? 0.0 : t;
+      s_inv = inv;
+      if (!s_zero) x[j] = beta;
     }
   }
   __syncthreads();
@@ -2869,19 +3039,18 @@ __global__ void __launch_bounds__(32 * kClWarps)
         acc[u] = mkc(0.0, 0.0);
         if (r < p) acc[u].x = cabs2_fma(y[r]);
       }
-      const double nrm = sqrt(qr_warp_total(acc, nu, sums).x);
+      const double nrm2 = qr_warp_total(acc, nu, sums).x;
       const cplx a = y[j];
+      double nrm, t;
+      cplx beta, inv;
+      qr_scalars(nrm2, a, nrm, beta, inv, t);
       __syncwarp();
       if (!(nrm > 0.0)) {
         if (lane == 0) tb[j] = 0.0;
       } else {
-        const double aa = sqrt(cabs2_fma(a));
-        const cplx ph = aa > 0.0 ? cscale(a, 1.0 / aa) : mkc(1.0, 0.0);
-        const double den = aa + nrm;
-        const cplx inv = cscale(cconj(ph), 1.0 / den);
         if (lane == 0) {
-          tb[j] = den / nrm;
-          y[j] = cscale(ph, -nrm);
+          tb[j] = t;
+          y[j] = beta;
         }
         for (int r = j + 1 + lane; r < p; r += 32) y[r] = cmul_fma(y[r], inv);
       }

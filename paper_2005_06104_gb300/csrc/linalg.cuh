@@ -188,7 +188,7 @@ struct SvdOut {
 // want_u/want_v: which factors to materialise.
 template <class Select>
 void svd_jacobi(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols,
-                Select select, SvdOut& out, bool want_u = true, bool want_v = true);
+                Select select, SvdOut& out, bool want_u, bool want_v, bool quick);
 // implemented for this signature:
 void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols,
                      int (*select)(const std::vector<double>& s, void* ctx), void* ctx,
@@ -215,26 +215,28 @@ extern SvdCounters g_svd_counters;
 // (eigenvalues to about 1e-7 relative, eigenvectors to about 1e-7 / relative gap); for the
 // Krylov vectors of the precision forms, whose density matrices are formed to about that
 // accuracy by the tensor-core GEMMs.
+// quick: rotation angles of the FP64 sweeps by FP32 arithmetic (unitary to FP64; see
+// jacobi_params_quick); the factors agree with the exact angles' to rounding, not bit by bit.
 void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols,
                       int (*select)(const std::vector<double>& s, void* ctx), void* ctx,
-                      SvdOut& out, bool want_u, bool want_v, bool psd = false, bool jacobi_fp32 = false);
+                      SvdOut& out, bool want_u, bool want_v, bool psd, bool jacobi_fp32, bool quick);
 template <class Select>
 inline void svd_jacobi(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols,
-                       Select select, SvdOut& out, bool want_u, bool want_v) {
+                       Select select, SvdOut& out, bool want_u, bool want_v, bool quick) {
   auto thunk = [](const std::vector<double>& s, void* ctx) -> int {
     return (*static_cast<Select*>(ctx))(s);
   };
-  svd_blocked_keep(st, pool, M, rows, cols, thunk, &select, out, want_u, want_v);
+  svd_blocked_keep(st, pool, M, rows, cols, thunk, &select, out, want_u, want_v, false, false, quick);
 }
 // Eigendecomposition of a Hermitian positive semidefinite n x n matrix: out.s the
 // eigenvalues (descending), out.U the kept eigenvectors (n x keep).
 template <class Select>
 inline void eig_psd_jacobi(cudaStream_t st, DevicePool* pool, const cplx* M, int n, Select select, SvdOut& out,
-                           bool jacobi_fp32 = false) {
+                           bool jacobi_fp32, bool quick) {
   auto thunk = [](const std::vector<double>& s, void* ctx) -> int {
     return (*static_cast<Select*>(ctx))(s);
   };
-  svd_blocked_keep(st, pool, M, n, n, thunk, &select, out, true, false, true, jacobi_fp32);
+  svd_blocked_keep(st, pool, M, n, n, thunk, &select, out, true, false, true, jacobi_fp32, quick);
 }
 
 // copy a (rows x cols) block into a (rows x ldo) destination at column offset
