@@ -152,13 +152,14 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
   const bool small = n <= kSpeculateMaxN;
   int batch = 1;
   if (small) batch = (int)std::min<long long>({(long long)(hint && *hint > 1 ? *hint : 4), (long long)nmax, n});
+  const bool fused = Blas1::lanczos_step_fused(n);  // the step leaves the next basis vector scaled
   int used = 0;
   const cplx* y = nullptr;  // exp(coef T) e_0 at the stopping point
   double last_err = 0.0;
   for (int j = 0; j < nmax;) {
     const int j0 = j;
     for (int b = 0; b < batch; ++b, ++j) {
-      if (b > 0) scale_by(st, V + (long long)j * n, wv, nrm2 + 1, false, n, live);
+      if (b > 0 && !fused) scale_by(st, V + (long long)j * n, wv, nrm2 + 1, false, n, live);
       op(V + (long long)j * n, wv);
       // alpha_j = Re <v_j, w>, w made orthogonal to V[0..j], beta_{j+1} = |w|
       blas.lanczos_step(st, V, n, j, wv, live, lw.c.data(), alpha, beta, nrm2);
@@ -188,7 +189,7 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
       }
     }
     if (used > 0 || j == nmax) break;
-    scale_by(st, V + (long long)j * n, wv, nrm2 + 1, false, n, live);
+    if (!fused) scale_by(st, V + (long long)j * n, wv, nrm2 + 1, false, n, live);
     if (small) batch = (int)std::min<long long>({2LL, (long long)(nmax - j), n - j});
   }
   if (used == 0)

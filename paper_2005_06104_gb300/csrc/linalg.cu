@@ -720,6 +720,133 @@ __global__ void __launch_bounds__(RED_THREADS)
   }
 }
 
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// Blocks of at most kClQ columns and kClP rows: one cluster per block, one warp per column, the
+// column in the warp's shared memory.  Bound: the chain of a reflector (its barrier, the reflector's
+// way through L2, one dot product, one norm, its square roots and divisions); a cluster barrier and
+// warp reductions take the place of the L2 barrier and of three block reductions.  Q is formed
+// without barriers.  Sums in the order of k_qr_groups: the same bits.
+// 80 x 40: 415 -> 295 us; the moves of a 24-site state at bond dimension 384 (blocks to 200 x 95):
+// 705 -> 530 us each.
+
+// The whole vector work of a Lanczos iteration on a short vector in one launch, by one cluster: the
+// two projections, the norm and the next basis vector, with the partial sums and orders of the kernels
+// above (block g of G = n / 1024 there is task g of the dot products here), so the same bits.
+// Bound: latency.  As six launches the iteration took 24 us and 15 us of a host thread, and several
+// threads share one driver: four chains of bond dimension 16 issued 23 700 launches in 70 ms.  Cluster
+// barriers (0.3 us) take the launches' place; FP64 work goes to all four schedulers of 8 or 16 SMs,
+// which carries n = 4096.  n = 512, 8 vectors: 24 -> 16 us and five launches fewer.
+constexpr int kSmallN = 4096;
+__global__ void __launch_bounds__(RED_THREADS)
+    k_lanczos_small(cplx* __restrict__ V, int j, cplx* w, int n, double* __restrict__ alpha, double* __restrict__ beta,
+                    double* __restrict__ nrm2, cplx* partial) {
+  constexpr int W = RED_THREADS / 32;
+  __shared__ double red[W][2];
+  __shared__ cplx cs[TRI_MAX];
+  __shared__ double s_inv;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nc = (int)cluster_size(), rank = (int)cluster_rank();
+  const int nvec = j + 1, G = max(1, (n + 4 * RED_THREADS - 1) / (4 * RED_THREADS));
+  const int per = (n + nc - 1) / nc, e0 = rank * per, e1 = min(n, e0 + per);  // this CTA's entries
+  double* dpart = reinterpret_cast<double*>(partial);
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int task = rank; task < nvec * G; task += nc) {  // one vector, one block of the sums
+      const int k = task / G, g = task % G;
+      cplx acc[1] = {mkc(0.0, 0.0)};
+      for (int base = g * RED_THREADS + warp * 32; base < n; base += G * RED_THREADS) {
+        const int i = base + lane;
+        const cplx wi = i < n ? __ldcg(w + i) : mkc(0.0, 0.0);
+        if (!warp_nonzero(wi)) continue;
+        const cplx v = i < n ? V[(long long)k * n + i] : mkc(0.0, 0.0);
+        cfma_conj(acc[0], v, wi);
+      }
+      warp_sum_store(acc, red[warp]);
+      __syncthreads();
+      if (threadIdx.x < 2) {
+        double t = 0.0;
+#pragma unroll
+        for (int u = 0; u < W; ++u) t += red[u][threadIdx.x];
+        dpart[2 * (k * G + g) + threadIdx.x] = t;
+      }
+      __syncthreads();
+    }
+    cluster_sync();
+    for (int k = warp; k < nvec; k += W) {  // every CTA sums the partials it needs itself
+      cplx t = mkc(0.0, 0.0);
+      if (lane < G) t = cadd(t, __ldcg(&partial[k * G + lane]));  // G <= 4
+      t = warp_sum(t);
+      if (lane == 0) {
+        cs[k] = t;
+        if (pass == 0 && rank == 0 && k == j) alpha[j] = t.x;
+      }
+    }
+    __syncthreads();
+    for (int base = e0 + warp * 32; base < e1; base += RED_THREADS) {
+      const int i = base + lane;
+      const bool in = i < e1;
+      cplx sub = mkc(0.0, 0.0);
+      for (int k0 = 0; k0 < nvec; k0 += MD_CH) {
+        cplx v[MD_CH];
+#pragma unroll
+        for (int q = 0; q < MD_CH; ++q) v[q] = in && k0 + q < nvec ? V[(long long)(k0 + q) * n + i] : mkc(0.0, 0.0);
+#pragma unroll
+        for (int q = 0; q < MD_CH; ++q)
+          if (k0 + q < nvec && warp_nonzero(v[q])) cfma(sub, v[q], cs[k0 + q]);
+      }
+      if (in) {
+        const cplx wi = __ldcg(w + i);
+        w[i] = csub(wi, sub);
+      }
+    }
+    cluster_sync();
+  }
+  for (int g = rank; g < G; g += nc) {
+    double a = 0.0;
+    for (int base = g * RED_THREADS + warp * 32; base < n; base += G * RED_THREADS) {
+      const int i = base + lane;
+      const cplx wi = i < n ? __ldcg(w + i) : mkc(0.0, 0.0);
+      if (warp_nonzero(wi)) a = __dadd_rn(a, cabs2_fma(wi));
+    }
+    a = warp_sum(a);
+    if (lane == 0) red[warp][0] = a;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int u = 0; u < W; ++u) t += red[u][0];
+      dpart[2 * TRI_MAX * 4 + g] = t;  // past the partial sums of the dot products
+    }
+    __syncthreads();
+  }
+  cluster_sync();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int g = 0; g < G; ++g) t += __ldcg(&dpart[2 * TRI_MAX * 4 + g]);
+    const double root = sqrt(t), inv = (t > 1e-200 && t <= 1.7e308) ? 1.0 / root : 0.0;  // as k_lanczos_norm
+    s_inv = inv;
+    if (rank == 0) {
+      nrm2[0] = t;
+      nrm2[1] = inv;
+      beta[j + 1] = root;
+    }
+  }
+  __syncthreads();
+  const double inv = s_inv;
+  for (int i = e0 + threadIdx.x; i < e1; i += RED_THREADS) V[(long long)nvec * n + i] = cscale(__ldcg(w + i), inv);
+}
+
 // dst = src * *factor, or src / sqrt(*factor) when `root`; sets the bits of `live` (when not null) of
 // the 32-entry groups with a nonzero entry.  FP64 division and square root cost tens of FP64
 // instructions: one thread per block forms the factor.
@@ -746,10 +873,44 @@ __global__ void __launch_bounds__(256)
 }
 }  // namespace
 
-void Blas1::lanczos_step(cudaStream_t st, const cplx* V, long long n, int j, cplx* w, const unsigned* live, cplx* c,
+namespace {
+// One launch of `kernel` with a cluster of nc CTAs per block.
+template <class F>
+void launch_clusters(cudaStream_t st, F* kernel, int nblk, int nc, size_t smem, void** args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nblk * nc);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nc;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  TDVP_CUDA(cudaLaunchKernelExC(&cfg, (const void*)kernel, args));
+  TDVP_CHECK_LAUNCH();
+}
+}  // namespace
+
+bool Blas1::lanczos_step_fused(long long n) { return n <= kSmallN; }
+
+void Blas1::lanczos_step(cudaStream_t st, cplx* V, long long n, int j, cplx* w, const unsigned* live, cplx* c,
                          double* alpha, double* beta, double* nrm2) {
   const int nvec = j + 1;
   tdvp_require(j >= 0 && nvec < TRI_MAX, TDVP_ERR_INVALID_ARG, "lanczos_step: too many vectors");
+  if (lanczos_step_fused(n)) {
+    static const bool attr = [] {
+      TDVP_CUDA(cudaFuncSetAttribute(k_lanczos_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      return true;
+    }();
+    (void)attr;
+    int nn = (int)n;
+    cplx* pp = partial.data();
+    void* args[] = {&V, &j, &w, &nn, &alpha, &beta, &nrm2, &pp};
+    launch_clusters(st, k_lanczos_small, 1, n > 1024 ? 16 : 8, 0, args);
+    return;
+  }
   const int G = red_blocks(n, max_blocks);
   auto dots = [&](cplx* out, double* al) {
     // vectors per block: 8 share one read of w when that still gives every SM four blocks; fewer
@@ -2947,27 +3108,6 @@ __global__ void __launch_bounds__(256)
 
 constexpr int kClQ = 96, kClP = 256, kClWarps = 8, kClU = kClP / 32;
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ unsigned cluster_rank() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ unsigned cluster_size() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
-}
-// Blocks of at most kClQ columns and kClP rows: one cluster per block, one warp per column, the
-// column in the warp's shared memory.  Bound: the chain of a reflector (its barrier, the reflector's
-// way through L2, one dot product, one norm, its square roots and divisions); a cluster barrier and
-// warp reductions take the place of the L2 barrier and of three block reductions.  Q is formed
-// without barriers.  Sums in the order of k_qr_groups: the same bits.
-// 80 x 40: 415 -> 295 us; the moves of a 24-site state at bond dimension 384 (blocks to 200 x 95):
-// 705 -> 530 us each.
 // tot = sum over virtual threads of part(u) with u < nu, in the block kernel's order
 __device__ __forceinline__ cplx qr_warp_total(const cplx (&acc)[kClU], int nu, double* sums) {
   __syncwarp();
@@ -3107,23 +3247,6 @@ __global__ void k_qr_scatter(const cplx* __restrict__ X, const cplx* __restrict_
 }  // namespace
 
 namespace {
-// One launch of `kernel` with a cluster of nc CTAs per block.
-template <class F>
-void launch_clusters(cudaStream_t st, F* kernel, int nblk, int nc, size_t smem, void** args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nblk * nc);
-  cfg.blockDim = dim3(32 * kClWarps);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = nc;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  TDVP_CUDA(cudaLaunchKernelExC(&cfg, (const void*)kernel, args));
-  TDVP_CHECK_LAUNCH();
-}
 // CTAs per cluster: 16 (not portable, allowed by attribute) once 8 would hold more than four columns each
 inline int cluster_ctas(int qmax) { return qmax > 32 ? 16 : 8; }
 }  // namespace

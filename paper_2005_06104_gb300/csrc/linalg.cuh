@@ -149,8 +149,11 @@ struct Blas1 {
   // are set, w is orthogonal to V[0..j], nrm2[0] = |w|^2 and nrm2[1] = 1 / |w| (0 when |w|^2 <=
   // 1e-200 or not finite).  c: 2 x 64 entries of scratch.  V's vectors are n entries apart.  live: null,
   // or one bit per 32 entries, set where some V[0..j] is nonzero (scale_by sets them).
-  void lanczos_step(cudaStream_t st, const cplx* V, long long n, int j, cplx* w, const unsigned* live, cplx* c,
+  // When lanczos_step_fused(n), V[j + 1] = w / |w| is written too (zeros for nrm2[1] = 0); otherwise
+  // the caller scales.
+  void lanczos_step(cudaStream_t st, cplx* V, long long n, int j, cplx* w, const unsigned* live, cplx* c,
                     double* alpha, double* beta, double* nrm2);
+  static bool lanczos_step_fused(long long n);
   unsigned* counter = nullptr;  // ticket of the last-block reductions (reset by that block)
   void release();
 };
