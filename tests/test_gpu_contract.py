@@ -270,6 +270,17 @@ def test_fp64_tiles_match_oracle(g, ml, mr, w):
     assert _rel(yd.cpu().numpy(), O.keff_apply(L, R, x)) < TOL64
 
 
+@pytest.mark.parametrize("ml,mr,w", [(5, 32, 1), (1, 33, 1), (7, 32, 8), (7, 34, 8), (40, 128, 2), (17, 100, 14)])
+def test_fp64_split_sums(g, ml, mr, w):
+    """Sums of a split K at 2 splits, 16 (the most that one cluster adds up) and more."""
+    rng = np.random.default_rng(ml * mr)
+    L, R, x = _rand(rng, ml, w, ml), _rand(rng, mr, w, mr), _rand(rng, ml, mr)
+    Ld, Rd, xd = _dev(L, R, x)
+    yd = torch.empty_like(xd)
+    g.keff_contract(Ld, Rd, xd, yd)
+    assert _rel(yd.cpu().numpy(), O.keff_apply(L, R, x)) < TOL64
+
+
 # FP64 products on the tensor cores (exact 8-bit digits): each result is held to 5e-15 of the
 # reference's norm.  The digits keep 56 bits below each row's largest entry and products to 2^-56
 # of the row maxima, 2.4e-16 norm-wise per product for Gaussian rows; two products are chained,
