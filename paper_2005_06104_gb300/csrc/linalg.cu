@@ -1428,7 +1428,7 @@ __device__ __forceinline__ bool jacobi_params(T a, T b, C c, T tol, T floor2, T&
 // that normalisation has to be exact.  A coupling |c| is then left at 6e-8 |c| instead of at rounding,
 // which the sweep after it removes; the last sweep's angles are below 1e-8, so it leaves 6e-16 of
 // sqrt(a b), under the tolerance (sqrt(p) 2.2e-16 or more) below which pairs are not rotated at all.
-// 15 FP64 instructions of 65 cycles each, where the exact angle's two reciprocal roots, root and
+// 10 FP64 instructions of 65 cycles each, where the exact angle's two reciprocal roots, root and
 // division are about 70.
 __device__ __forceinline__ float high_float(double x, int add) {  // x 2^add towards zero; 0 below FP32's range
   const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
@@ -1437,6 +1437,7 @@ __device__ __forceinline__ float high_float(double x, int add) {  // x 2^add tow
   if (e >= 255) return __uint_as_float((h & 0x80000000u) | 0x7f7fffffu);
   return __uint_as_float((h & 0x80000000u) | ((unsigned)e << 23) | ((h & 0xfffffu) << 3) | (l >> 29));
 }
+__device__ __forceinline__ int biased_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 __device__ __forceinline__ double wide_double(float x) {  // (double)x by its bits; 0 for a subnormal
   const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
   if (e == 0) return 0.0;
@@ -1444,18 +1445,22 @@ __device__ __forceinline__ double wide_double(float x) {  // (double)x by its bi
 }
 __device__ __forceinline__ bool jacobi_params_quick(double a, double b, double2 c, double tol2, double floor2,
                                                     double& cs, double2& sne) {
-  // comparisons of non-negative doubles by their bits
+  // the tests on bits, exponents and FP32 mantissas (they decide to 1e-7 of their thresholds)
   const long long la = __double_as_longlong(a), lb = __double_as_longlong(b);
   const double big = la > lb ? a : b, small = la > lb ? b : a;
-  if (__double_as_longlong(big) <= __double_as_longlong(floor2) ||
-      __double_as_longlong(small) <= __double_as_longlong(kJacobiFloor * big))
-    return false;
-  const double ac2 = cabs2_fma(c);
-  if (__double_as_longlong(ac2) <= __double_as_longlong(tol2 * a * b)) return false;
-  if ((__double2hiint(ac2) & 0x7ff00000) == 0x7ff00000) return false;  // not finite: the norms will say so
-  const int sh = -((((__double2hiint(ac2) >> 20) & 0x7ff) - 1023) >> 1);  // |c| 2^sh in [1, 2)
+  if (__double_as_longlong(big) <= __double_as_longlong(floor2)) return false;
+  const int eb = biased_exponent(big), ec = max(biased_exponent(c.x), biased_exponent(c.y));
+  if (ec == 0 || ec == 0x7ff || eb == 0x7ff) return false;  // not finite: the norms will say so
+  if (high_float(small, 1023 - eb) <= (float)kJacobiFloor * high_float(big, 1023 - eb)) return false;
+  const int sh = 1023 - ec;  // |c| 2^sh in [1, 2.9)
   const float cx = high_float(c.x, sh), cy = high_float(c.y, sh);
-  const float inv = rsqrtf(cx * cx + cy * cy);
+  const float n2 = cx * cx + cy * cy;
+  // |c|^2 > tol2 a b
+  const int ea = biased_exponent(a), eq = biased_exponent(b), et = biased_exponent(tol2);
+  const int lead = ea + eq + et - 3 * 1023 + 2 * sh;
+  const float mant = high_float(a, 1023 - ea) * high_float(b, 1023 - eq) * high_float(tol2, 1023 - et);  // [1, 8)
+  if (lead >= 4 || (lead > -4 && n2 <= mant * __uint_as_float((unsigned)(lead + 127) << 23))) return false;
+  const float inv = rsqrtf(n2);
   const float zeta = 0.5f * high_float(b - a, sh) * inv;
   const float az = fabsf(zeta);
   const float t = copysignf(az > 1e9f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az)), zeta) * inv;
@@ -1472,6 +1477,16 @@ __device__ __forceinline__ bool jacobi_params_quick(float a, float b, float2 c, 
                                                     float2& sne) {
   return jacobi_params(a, b, c, sqrtf(tol2), floor2, cs, sne);  // FP32 rotations have no shorter form
 }
+
+// whether |sne|^2 is above the angle that asks for another sweep; FP64 only where FP32 cannot tell
+__device__ __forceinline__ bool large_angle(double2 sne) {
+  const float x = high_float(sne.x, 0), y = high_float(sne.y, 0), s = x * x + y * y;
+  constexpr float lim = (float)Jac<double>::small_angle2;
+  if (s > lim * 1.0001f) return true;
+  if (s < lim * 0.9999f) return false;
+  return cabs2(sne) > Jac<double>::small_angle2;
+}
+__device__ __forceinline__ bool large_angle(float2 sne) { return cabs2(sne) > Jac<float>::small_angle2; }
 
 template <class T, class C>
 __device__ __forceinline__ void rotate_pair(C& xp, C& xq, T cs, C sne) {
@@ -1534,7 +1549,7 @@ __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename J
     const bool rot = quick ? jacobi_params_quick(A, B, Cc, tol * tol, floor2, cs, sne)
                            : jacobi_params(A, B, Cc, tol, floor2, cs, sne);
     if (threadIdx.x == 0) {
-      s_do = !rot ? 0 : cabs2(sne) > Jac<T>::small_angle2 ? 2 : 1;
+      s_do = !rot ? 0 : large_angle(sne) ? 2 : 1;
       s_cs = cs;
       s_sne = sne;
     }
@@ -1983,7 +1998,7 @@ __global__ void __launch_bounds__(256)
   extern __shared__ __align__(16) unsigned char sm_raw[];
   C* sm = reinterpret_cast<C*>(sm_raw);
   __shared__ int s_rot;
-  __shared__ T s_fro[8];
+  __shared__ T s_fro[8], h4[8][4];
   const BlkDesc d = desc[blockIdx.x];
   const int p = d.p, q = d.q, qpad = q + (q & 1);
   C* Xs = sm;
@@ -2023,19 +2038,19 @@ __global__ void __launch_bounds__(256)
           b += cabs2(v);
           cfma_conj(c, u, v);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          a += __shfl_xor_sync(0xffffffffu, a, o);
-          b += __shfl_xor_sync(0xffffffffu, b, o);
-          c.x += __shfl_xor_sync(0xffffffffu, c.x, o);
-          c.y += __shfl_xor_sync(0xffffffffu, c.y, o);
-        }
+        T h[4] = {a, b, c.x, c.y};
+        warp_sum_values(h, h4[warp]);  // halving: 6 additions per lane instead of 20, in the same tree
+        __syncwarp();
+        a = h4[warp][0];
+        b = h4[warp][1];
+        c = Jac<T>::make(h4[warp][2], h4[warp][3]);
+        __syncwarp();  // read before the next pair's sums arrive
         T cs;
         C sne;
         if (!(quick ? jacobi_params_quick(a, b, c, tol * tol, floor2, cs, sne)
                     : jacobi_params(a, b, c, tol, floor2, cs, sne)))
           continue;
-        if (lane == 0 && cabs2(sne) > Jac<T>::small_angle2) s_rot = 1;
+        if (lane == 0 && large_angle(sne)) s_rot = 1;
         for (int r = lane; r < p; r += 32) {
           C u = xp[r], v = xq[r];
           rotate_pair(u, v, cs, sne);
