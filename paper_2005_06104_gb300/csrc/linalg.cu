@@ -52,10 +52,12 @@ __device__ __forceinline__ cplx ld_cluster(const cplx* p, unsigned rank) {
 
 // nsplit > 1: blockIdx.z = batch * nsplit + split; split s sums K range
 // [s*kchunk, min(K, (s+1)*kchunk)).  With a partial buffer it goes to P[s][batch][M][N]
-// (alpha applied, beta left to k_splitk_reduce).  Without one (P null, T < 64) the splits of
+// (alpha applied, beta left to k_splitk_reduce).  Without one (P null, T <= 16) the splits of
 // a tile are one cluster: each leaves its tile in shared memory and the CTAs add the tiles in
 // split order, entry by entry, as k_splitk_reduce does.  M = 16, N = 80, K = 160 in ten splits:
-// product 4.5 us, sum 2.8 us and the gap between them; in one cluster 5.6 us.
+// product 4.5 us, sum 2.8 us and the gap between them; in one cluster 5.6 us.  Wider tiles run for
+// 100 us and more, and there a cluster waits for its whole set of SMs: 210 us with the sum apart,
+// 243 us in clusters of 32-wide tiles (bond dimension 256).
 template <int OPA, int OPB, int T>
 __global__ void __launch_bounds__(T == 8 ? 64 : 256)
     k_zgemm(int M, int N, int K, cplx alpha, const cplx* __restrict__ A, long long lda,
@@ -72,7 +74,7 @@ __global__ void __launch_bounds__(T == 8 ? 64 : 256)
   const long long bz = blockIdx.z / nsplit;
   A += bz * sA;
   B += bz * sB;
-  const bool clustered = T < 64 && nsplit > 1 && P == nullptr;
+  const bool clustered = T <= 16 && nsplit > 1 && P == nullptr;
   if (nsplit > 1 && !clustered) {
     C = P + ((long long)split * nbatch + bz) * (long long)M * N;
     ldc = N;
@@ -146,7 +148,7 @@ __global__ void __launch_bounds__(T == 8 ? 64 : 256)
   }
   const bool use_beta = (beta.x != 0.0 || beta.y != 0.0);
   if (clustered) {
-    static_assert(T >= 64 || T * T <= 2 * TK * (T + 1), "a tile fits in the operands' shared memory");
+    static_assert(T > 16 || T * T <= 2 * TK * (T + 1), "a tile fits in the operands' shared memory");
 #pragma unroll
     for (int i = 0; i < R; ++i)
 #pragma unroll
@@ -207,7 +209,6 @@ void zgemm_t(int tile, dim3 g, cudaStream_t st, int M, int N, int K, cplx alpha,
   static const bool wide = [] {  // clusters of more than 8
     TDVP_CUDA(cudaFuncSetAttribute(k_zgemm<OPA, OPB, 8>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     TDVP_CUDA(cudaFuncSetAttribute(k_zgemm<OPA, OPB, 16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    TDVP_CUDA(cudaFuncSetAttribute(k_zgemm<OPA, OPB, 32>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return true;
   }();
   (void)wide;
@@ -281,8 +282,8 @@ void zgemm(cudaStream_t st, int opA, int opB, int M, int N, int K, cplx alpha, c
   while (tile > 8 && (long long)ceil_div(N, tile) * ceil_div(M, tile) * batch * ns < 2LL * sms) tile /= 2;
   while (tile < 64 && ceil_div(M, tile) > 65535) tile *= 2;
   dim3 g(ceil_div(N, tile), ceil_div(M, tile), batch * ns);
-  // up to 16 splits of a small tile add up inside a cluster, more go through a partial buffer
-  const bool partial = ns > 1 && (tile == 64 || ns > kMaxCluster);
+  // up to 16 splits of a small tile add up inside a cluster, others go through a partial buffer
+  const bool partial = ns > 1 && (tile > 16 || ns > kMaxCluster);
   DArr part;
   if (partial) part.reset(ws, (size_t)ns * batch * M * N);
   cplx* P = partial ? part.data() : nullptr;
