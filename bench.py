@@ -97,7 +97,7 @@ def parse():
 PRECISIONS = {"fp64": "PREC_FP64", "tf32x3": "PREC_TF32X3", "tf32x3_env": "PREC_TF32X3_ENV",
               "bf16x10": "PREC_BF16X10", "bf16x6": "PREC_BF16X6"}
 PRECISION_TEXT = {
-    "fp64": "FP64 on CUDA cores throughout",
+    "fp64": "FP64 throughout",
     "tf32x3": "tcgen05 split TF32 x3 (H_eff, K_eff, Krylov GEMMs); FP64 environments, Lanczos, SVD",
     "tf32x3_env": "tcgen05 split TF32 x3 (H_eff, K_eff, environments, Krylov GEMMs); FP64 Lanczos, SVD",
     "bf16x10": "tcgen05 BF16 exact slices x10 (H_eff, K_eff, environments, Krylov GEMMs); FP64 Lanczos, QR, SVD, "

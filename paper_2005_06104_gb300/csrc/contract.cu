@@ -1,4 +1,4 @@
-// One-site contractions (FP64 on CUDA cores) and the Lanczos exponential.
+// One-site contractions (FP64) and the Lanczos exponential.
 #include <algorithm>
 
 #include "contract.cuh"
