@@ -800,14 +800,6 @@ __global__ void __launch_bounds__(RED_THREADS)
   }
 }
 
-// Blocks of at most kClQ columns and kClP rows: one cluster per block, one warp per column, the
-// column in the warp's shared memory.  Bound: the chain of a reflector (its barrier, the reflector's
-// way through L2, one dot product, one norm, its square roots and divisions); a cluster barrier and
-// warp reductions take the place of the L2 barrier and of three block reductions.  Q is formed
-// without barriers.  Sums in the order of k_qr_groups: the same bits.
-// 80 x 40: 415 -> 295 us; the moves of a 24-site state at bond dimension 384 (blocks to 200 x 95):
-// 705 -> 530 us each.
-
 // The whole vector work of a Lanczos iteration on a short vector in one launch, by one cluster: the
 // two projections, the norm and the next basis vector, with the partial sums and orders of the kernels
 // above (block g of G = n / 1024 there is task g of the dot products here), so the same bits.
@@ -942,10 +934,10 @@ __global__ void __launch_bounds__(256)
 namespace {
 // One launch of `kernel` with a cluster of nc CTAs per block.
 template <class F>
-void launch_clusters(cudaStream_t st, F* kernel, int nblk, int nc, size_t smem, void** args) {
+void launch_clusters(cudaStream_t st, F* kernel, int nblk, int nc, int threads, size_t smem, void** args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nblk * nc);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -974,7 +966,7 @@ void Blas1::lanczos_step(cudaStream_t st, cplx* V, long long n, int j, cplx* w, 
     int nn = (int)n;
     cplx* pp = partial.data();
     void* args[] = {&V, &j, &w, &nn, &alpha, &beta, &nrm2, &pp};
-    launch_clusters(st, k_lanczos_small, 1, n > 1024 ? 16 : 8, 0, args);
+    launch_clusters(st, k_lanczos_small, 1, n > 1024 ? 16 : 8, 256, 0, args);
     return;
   }
   const int G = red_blocks(n, max_blocks);
@@ -3187,115 +3179,135 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-constexpr int kClQ = 96, kClP = 256, kClWarps = 8, kClU = kClP / 32;
+// Blocks of at most kClQ columns and kClP rows: one cluster per block, a team of two warps per
+// column, the column in the team's shared memory.  Bound: the chain of a reflector (its barrier,
+// the reflector's way through L2, one dot product, one norm, its square roots and divisions), every
+// FP64 instruction of a warp 65 cycles; a cluster barrier and warp reductions take the place of the
+// L2 barrier and of three block reductions, and the team halves the dot product, the update and the
+// sums.  Q is formed without barriers.  Sums in the order of k_qr_groups: the same bits.
+// The moves of a 24-site state at bond dimension 384 (blocks to 200 x 95): 705 us each by
+// k_qr_groups, 515 with one warp per column, 400 with two.
+// kClCols columns per CTA, kClTeam warps each; a column is kClU units of 32 rows from row j on,
+// unit u with warp u % kClTeam of its team
+constexpr int kClQ = 96, kClP = 256, kClCols = 8, kClTeam = 2, kClU = kClP / 32, kClUw = kClU / kClTeam;
 
-// tot = sum over virtual threads of part(u) with u < nu, in the block kernel's order
-__device__ __forceinline__ cplx qr_warp_total(const cplx (&acc)[kClU], int nu, double* sums) {
-  __syncwarp();
-  if (nu <= 2) {
+__device__ __forceinline__ void team_sync(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(32 * kClTeam) : "memory");
+}
+
+// sum over virtual threads of the units' parts, in the block kernel's order (lanes, then units);
+// acc[i]: unit kClTeam i + half.  Lane parity carries the real and the imaginary chain.
+__device__ __forceinline__ cplx qr_team_total(const cplx (&acc)[kClUw], int nu, int half, int team,
+                                              double (*sums)[2 * kClUw]) {
+  if (nu <= kClTeam) {
+    cplx h[1] = {acc[0]};
+    warp_sum_store(h, sums[half]);
+  } else if (nu <= 2 * kClTeam) {
     cplx h[2] = {acc[0], acc[1]};
-    warp_sum_store(h, sums);
-  } else if (nu <= 4) {
-    cplx h[4] = {acc[0], acc[1], acc[2], acc[3]};
-    warp_sum_store(h, sums);
+    warp_sum_store(h, sums[half]);
   } else {
-    warp_sum_store(acc, sums);
+    warp_sum_store(acc, sums[half]);
   }
-  __syncwarp();
-  cplx t = mkc(0.0, 0.0);
-  for (int u = 0; u < nu; ++u) t = cadd(t, mkc(sums[2 * u], sums[2 * u + 1]));
-  return t;
+  team_sync(team);
+  const int part = threadIdx.x & 1;
+  double t = 0.0;
+  for (int u = 0; u < nu; ++u) t += sums[u % kClTeam][2 * (u / kClTeam) + part];
+  return mkc(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 1));
 }
 
-// y <- H_j y on a warp's column (shared memory); v: the reflector's rows j.. (row j reads as 1)
-__device__ __forceinline__ void qr_warp_apply(cplx* y, const cplx* __restrict__ vcol, int p, int j, double tj,
-                                              double* sums) {
+// y <- H_j y on a team's column (shared memory); v: the reflector's rows j.. (row j reads as 1)
+__device__ __forceinline__ void qr_team_apply(cplx* y, const cplx* __restrict__ vcol, int p, int j, double tj, int half,
+                                              int team, double (*sums)[2 * kClUw]) {
   const int lane = threadIdx.x & 31, nu = (p - j + 31) >> 5;
-  cplx v[kClU], acc[kClU];
+  cplx v[kClUw], acc[kClUw];
 #pragma unroll
-  for (int u = 0; u < kClU; ++u) {
-    const int r = j + 32 * u + lane;
-    v[u] = r < p ? (r == j ? mkc(1.0, 0.0) : __ldcg(vcol + r)) : mkc(0.0, 0.0);
+  for (int i = 0; i < kClUw; ++i) {
+    const int r = j + 32 * (kClTeam * i + half) + lane;
+    v[i] = r < p ? (r == j ? mkc(1.0, 0.0) : __ldcg(vcol + r)) : mkc(0.0, 0.0);
   }
 #pragma unroll
-  for (int u = 0; u < kClU; ++u) {
-    const int r = j + 32 * u + lane;
-    acc[u] = mkc(0.0, 0.0);
-    if (u < nu && r < p) cfma_conj(acc[u], v[u], y[r]);
+  for (int i = 0; i < kClUw; ++i) {
+    const int u = kClTeam * i + half, r = j + 32 * u + lane;
+    acc[i] = mkc(0.0, 0.0);
+    if (u < nu && r < p) cfma_conj(acc[i], v[i], y[r]);
   }
-  const cplx w = cscale(qr_warp_total(acc, nu, sums), tj);
+  const cplx w = cscale(qr_team_total(acc, nu, half, team, sums), tj);
 #pragma unroll
-  for (int u = 0; u < kClU; ++u) {
-    const int r = j + 32 * u + lane;
-    if (r < p) y[r] = csub(y[r], cmul_fma(w, v[u]));
+  for (int i = 0; i < kClUw; ++i) {
+    const int r = j + 32 * (kClTeam * i + half) + lane;
+    if (r < p) y[r] = csub(y[r], cmul_fma(w, v[i]));
   }
-  __syncwarp();
+  team_sync(team);
 }
 
-__global__ void __launch_bounds__(32 * kClWarps)
+__global__ void __launch_bounds__(32 * kClTeam * kClCols)
     k_qr_cluster(cplx* __restrict__ X, cplx* __restrict__ Qb, double* __restrict__ tau,
                  const QrDesc* __restrict__ desc, int pmax) {
   extern __shared__ cplx cols[];
-  __shared__ double sums_all[kClWarps][2 * kClU];
+  __shared__ double sums_all[kClCols][kClTeam][2 * kClUw];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int team = warp / kClTeam, half = warp % kClTeam, tt = 32 * half + lane;
+  constexpr int TT = 32 * kClTeam;
   const int nc = (int)cluster_size(), rank = (int)cluster_rank();
   const QrDesc d = desc[blockIdx.x / nc];
   const int p = d.p, q = d.q, kq = d.kq;
   cplx* Xb = X + d.x_off;
   double* tb = tau + d.t_off;
-  double* sums = sums_all[warp];
-  const int c = rank + nc * warp;  // this warp's column: nc * kClWarps >= kClQ of them
-  cplx* y = cols + warp * pmax;
+  auto sums = sums_all[team];
+  const int c = rank + nc * team;  // this team's column: nc * kClCols >= kClQ of them
+  cplx* y = cols + team * pmax;
   const bool own = c < q;
   if (own)
-    for (int r = lane; r < p; r += 32) y[r] = Xb[(long long)c * p + r];
-  __syncwarp();
+    for (int r = tt; r < p; r += TT) y[r] = Xb[(long long)c * p + r];
+  team_sync(team);
   for (int j = 0; j < kq; ++j) {
     if (own && c == j) {  // reflector j from this column
       const int nu = (p - j + 31) >> 5;
-      cplx acc[kClU];
+      cplx acc[kClUw];
 #pragma unroll
-      for (int u = 0; u < kClU; ++u) {
-        const int r = j + 32 * u + lane;
-        acc[u] = mkc(0.0, 0.0);
-        if (r < p) acc[u].x = cabs2_fma(y[r]);
+      for (int i = 0; i < kClUw; ++i) {
+        const int r = j + 32 * (kClTeam * i + half) + lane;
+        acc[i] = mkc(0.0, 0.0);
+        if (r < p) acc[i].x = cabs2_fma(y[r]);
       }
-      const double nrm2 = qr_warp_total(acc, nu, sums).x;
+      const double nrm2 = qr_team_total(acc, nu, half, team, sums).x;
       const cplx a = y[j];
       double nrm, t;
       cplx beta, inv;
-      qr_scalars(nrm2, a, nrm, beta, inv, t);
-      __syncwarp();
+      qr_scalars(nrm2, a, nrm, beta, inv, t);  // in both warps: each has a scheduler of its own
+      team_sync(team);
       if (!(nrm > 0.0)) {
-        if (lane == 0) tb[j] = 0.0;
+        if (tt == 0) tb[j] = 0.0;
       } else {
-        if (lane == 0) {
+        if (tt == 0) {
           tb[j] = t;
           y[j] = beta;
         }
-        for (int r = j + 1 + lane; r < p; r += 32) y[r] = cmul_fma(y[r], inv);
+        for (int r = j + 1 + tt; r < p; r += TT) y[r] = cmul_fma(y[r], inv);
       }
-      __syncwarp();
-      for (int r = lane; r < p; r += 32) Xb[(long long)c * p + r] = y[r];
+      team_sync(team);
+      for (int r = tt; r < p; r += TT) Xb[(long long)c * p + r] = y[r];
     }
+    __syncwarp();
     cluster_sync();
     if (own && c > j) {
       const double tj = __ldcg(tb + j);
-      if (tj != 0.0) qr_warp_apply(y, Xb + (long long)j * p, p, j, tj, sums);
+      if (tj != 0.0) qr_team_apply(y, Xb + (long long)j * p, p, j, tj, half, team, sums);
     }
   }
   if (own && c >= kq)  // columns right of the last reflector: rows of R only
-    for (int r = lane; r < p; r += 32) Xb[(long long)c * p + r] = y[r];
+    for (int r = tt; r < p; r += TT) Xb[(long long)c * p + r] = y[r];
   // Q_b: column c < kq starts as e_c; H_j applies to the columns c >= j
   if (c < kq) {
-    for (int r = lane; r < p; r += 32) y[r] = mkc(r == c ? 1.0 : 0.0, 0.0);
-    __syncwarp();
+    team_sync(team);
+    for (int r = tt; r < p; r += TT) y[r] = mkc(r == c ? 1.0 : 0.0, 0.0);
+    team_sync(team);
     for (int j = c; j >= 0; --j) {
       const double tj = __ldcg(tb + j);
-      if (tj != 0.0) qr_warp_apply(y, Xb + (long long)j * p, p, j, tj, sums);
+      if (tj != 0.0) qr_team_apply(y, Xb + (long long)j * p, p, j, tj, half, team, sums);
     }
     cplx* Qc = Qb + d.q_off + (long long)c * p;
-    for (int r = lane; r < p; r += 32) Qc[r] = y[r];
+    for (int r = tt; r < p; r += TT) Qc[r] = y[r];
   }
 }
 
@@ -3426,7 +3438,7 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
     static const bool cattr = [] {
       TDVP_CUDA(cudaFuncSetAttribute(k_qr_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
       TDVP_CUDA(cudaFuncSetAttribute(k_qr_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(kClWarps * kClP * sizeof(cplx))));
+                                     (int)(kClCols * kClP * sizeof(cplx))));
       return true;
     }();
     (void)cattr;
@@ -3434,7 +3446,7 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
     cplx* qp = Qb.data();
     const QrDesc* dd = d_desc;
     void* args[] = {&xp, &qp, &d_tau, &dd, &pmax};
-    launch_clusters(st, k_qr_cluster, nblk, cl, kClWarps * (size_t)pmax * sizeof(cplx), args);
+    launch_clusters(st, k_qr_cluster, nblk, cl, 32 * kClTeam * kClCols, kClCols * (size_t)pmax * sizeof(cplx), args);
   } else {
     cplx* xp = X.data();
     cplx* qp = Qb.data();
