@@ -17,9 +17,9 @@
 // Measured against 113-bit sums, bond operator (two chained products), norm-wise: 1.15e-16 here
 // and 3.4e-16 on CUDA cores at 129 x 127, w = 14; 1.4e-16 and 5.2e-16 with rows falling over six
 // decades; 1.25e-16 and 2.3e-15 at 512.
-// Measured time, H_eff: 512 x 512, w = 14: 53.3 -> 3.0 ms (20 TFLOP/s of FP64, 24 % of the BF16
+// Measured time, H_eff: 512 x 512, w = 14: 53.4 -> 2.4 ms (25 TFLOP/s of FP64, 46 % of the BF16
 // peak per digit product); 129 x 127, w = 8: 630 -> 95 us; both environment updates and the bond
-// operator at 300 x 277, w = 14: 31.8 -> 2.4 ms.
+// operator at 300 x 277, w = 14: 31.8 -> 1.9 ms.
 //
 // The eight groups need 8 x 128 TMEM columns and the 64-bit sums two registers per entry and
 // set, so one CTA takes one of two passes over its K range: groups 0..3 (slices 0..3, 10
