@@ -82,8 +82,8 @@ struct Engine {
   void build_pair_mpo();
   void env_left(int i);   // L[i+1] from L[i], A[i]
   void env_right(int i);  // R[i-1] from R[i], A[i]
-  // FP32 rotation angles in FP64 Jacobi sweeps: not in a split form, whose trajectories keep their bits
-  // (see gauge_gemm)
+  // FP32 arithmetic for large rotation angles in FP64 Jacobi sweeps: not in a split form, whose
+  // trajectories keep their bits (see gauge_gemm)
   bool quick_jacobi() const { return opt.precision == TDVP_PREC_FP64; }
   // gauge moves
   void gauge_gemm(int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A, long long lda, const cplx* B,

@@ -1416,13 +1416,19 @@ __device__ __forceinline__ bool jacobi_params(T a, T b, C c, T tol, T floor2, T&
   return true;
 }
 
-// The same rotation from an angle good to FP32, for a = |x_p|^2, b = |x_q|^2 in FP64: any complex
-// tangent tau = t e^{i phi} gives a unitary rotation, cs = 1 / sqrt(1 + |tau|^2), sne = cs tau, so only
-// that normalisation has to be exact.  A coupling |c| is then left at 6e-8 |c| instead of at rounding,
-// which the sweep after it removes; the last sweep's angles are below 1e-8, so it leaves 6e-16 of
-// sqrt(a b), under the tolerance (sqrt(p) 2.2e-16 or more) below which pairs are not rotated at all.
-// 10 FP64 instructions of 65 cycles each, where the exact angle's two reciprocal roots, root and
-// division are about 70.
+// The same rotation with the angle's arithmetic in FP32 where that is enough.  GB300's FP64 unit takes 65
+// cycles per instruction of a warp: the exact angle's two reciprocal roots, root and division are about
+// 70 of them, these about 20 for a large angle and 10 for a small one.
+//  - |sin theta| > 1e-8: any complex tangent tau = t e^{i phi} gives a unitary rotation, cs = 1 / sqrt(1 +
+//    |tau|^2), sne = cs tau, so only that normalisation has to be exact.  With tau good to FP32 about
+//    3e-7 |c| of the coupling c stays, and the angle asks for another sweep, which removes it.
+//  - |sin theta| <= 1e-8, perhaps the pair's last rotation: tau = c / (b - a) with cs = 1 is the rotation
+//    to 1e-16 of itself (t = 1 / (2 zeta) (1 - 1 / (4 zeta^2) + ...)), with the quotient in FP64.  An FP32
+//    quotient would not do: a small angle does not mean a small coupling.  For |x_q| << |x_p| the angle
+//    is |cos(x_p, x_q)| |x_q| / |x_p|, and columns of norms 1 and 1e-8 kept a cosine of 2e-7.
+// The reciprocal of b - a is Newton's iteration from FP32's (1.8e-7, 3e-14, then rounding).
+// An imaginary-time step of 40 sites at bond dimension 40, two thirds of it Jacobi sweeps: 174 ms with the
+// exact angles, 154 ms with these.
 __device__ __forceinline__ float high_float(double x, int add) {  // x 2^add towards zero; 0 below FP32's range
   const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
   const int e = (int)((h >> 20) & 0x7ff) - 1023 + 127 + add;
@@ -1436,15 +1442,18 @@ __device__ __forceinline__ double wide_double(float x) {  // (double)x by its bi
   if (e == 0) return 0.0;
   return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
 }
-__device__ __forceinline__ bool jacobi_params_quick(double a, double b, double2 c, double tol2, double floor2,
-                                                    double& cs, double2& sne) {
+constexpr float kSmallZeta = 5e7f;  // |zeta| from which |sin theta| <= 1e-8
+// 0: the pair stays, 1: rotate, 2: rotate, and the sweep is not the last (Jac<double>::small_angle2), -1: out
+// of this function's range
+__device__ __forceinline__ int jacobi_params_quick(double a, double b, double2 c, double tol2, double floor2,
+                                                   double& cs, double2& sne) {
   // the tests on bits, exponents and FP32 mantissas (they decide to 1e-7 of their thresholds)
   const long long la = __double_as_longlong(a), lb = __double_as_longlong(b);
   const double big = la > lb ? a : b, small = la > lb ? b : a;
-  if (__double_as_longlong(big) <= __double_as_longlong(floor2)) return false;
+  if (__double_as_longlong(big) <= __double_as_longlong(floor2)) return 0;
   const int eb = biased_exponent(big), ec = max(biased_exponent(c.x), biased_exponent(c.y));
-  if (ec == 0 || ec == 0x7ff || eb == 0x7ff) return false;  // not finite: the norms will say so
-  if (high_float(small, 1023 - eb) <= (float)kJacobiFloor * high_float(big, 1023 - eb)) return false;
+  if (ec == 0 || ec == 0x7ff || eb == 0x7ff) return 0;  // not finite: the norms will say so
+  if (high_float(small, 1023 - eb) <= (float)kJacobiFloor * high_float(big, 1023 - eb)) return 0;
   const int sh = 1023 - ec;  // |c| 2^sh in [1, 2.9)
   const float cx = high_float(c.x, sh), cy = high_float(c.y, sh);
   const float n2 = cx * cx + cy * cy;
@@ -1452,34 +1461,41 @@ __device__ __forceinline__ bool jacobi_params_quick(double a, double b, double2 
   const int ea = biased_exponent(a), eq = biased_exponent(b), et = biased_exponent(tol2);
   const int lead = ea + eq + et - 3 * 1023 + 2 * sh;
   const float mant = high_float(a, 1023 - ea) * high_float(b, 1023 - eq) * high_float(tol2, 1023 - et);  // [1, 8)
-  if (lead >= 4 || (lead > -4 && n2 <= mant * __uint_as_float((unsigned)(lead + 127) << 23))) return false;
+  if (lead >= 4 || (lead > -4 && n2 <= mant * __uint_as_float((unsigned)(lead + 127) << 23))) return 0;
   const float inv = rsqrtf(n2);
-  const float zeta = 0.5f * high_float(b - a, sh) * inv;
+  const double diff = b - a;
+  const float zeta = 0.5f * high_float(diff, sh) * inv;
   const float az = fabsf(zeta);
-  const float t = copysignf(az > 1e9f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az)), zeta) * inv;
+  if (az >= kSmallZeta) {
+    const int ed = biased_exponent(diff);
+    if (ed < 50 || ed > 2000) return -1;  // 1 / (b - a) has to be a normal number
+    const double s = wide_double(1.0f / high_float(diff, 1023 - ed));  // 2^(ed - 1023) / (b - a)
+    double r = __hiloint2double(__double2hiint(s) + ((1023 - ed) << 20), __double2loint(s));
+    r = fma(r, fma(-diff, r, 1.0), r);
+    r = fma(r, fma(-diff, r, 1.0), r);
+    cs = 1.0;
+    sne = make_double2(c.x * r, c.y * r);
+    return 1;
+  }
+  const float t = copysignf(1.0f / (az + sqrtf(1.0f + az * az)), zeta) * inv;
   const double tx = wide_double(t * cx), ty = wide_double(t * cy);
-  const double m = fma(tx, tx, fma(ty, ty, 1.0));  // [1, 2]
-  // 1 / sqrt(m): FP32 seed, one third-order step (error (5/16) (2^-22)^3)
-  const double r = wide_double(rsqrtf(high_float(m, 0)));
-  const double e = fma(-(m * r), r, 1.0);
-  cs = fma(r, e * fma(0.375, e, 0.5), r);
+  cs = rsqrt(fma(tx, tx, fma(ty, ty, 1.0)));
   sne = make_double2(cs * tx, cs * ty);
-  return true;
-}
-__device__ __forceinline__ bool jacobi_params_quick(float a, float b, float2 c, float tol2, float floor2, float& cs,
-                                                    float2& sne) {
-  return jacobi_params(a, b, c, sqrtf(tol2), floor2, cs, sne);  // FP32 rotations have no shorter form
+  return 2;
 }
 
-// whether |sne|^2 is above the angle that asks for another sweep; FP64 only where FP32 cannot tell
-__device__ __forceinline__ bool large_angle(double2 sne) {
-  const float x = high_float(sne.x, 0), y = high_float(sne.y, 0), s = x * x + y * y;
-  constexpr float lim = (float)Jac<double>::small_angle2;
-  if (s > lim * 1.0001f) return true;
-  if (s < lim * 0.9999f) return false;
-  return cabs2(sne) > Jac<double>::small_angle2;
+// 0: the pair stays, 1: rotate, 2: rotate, and the sweep is not the last.
+template <class T, class C>
+__device__ __forceinline__ int jacobi_rotation(T a, T b, C c, T tol, T floor2, int quick, T& cs, C& sne) {
+  if constexpr (sizeof(T) == 8) {  // FP32 rotations have no shorter form
+    if (quick) {
+      const int r = jacobi_params_quick(a, b, c, tol * tol, floor2, cs, sne);
+      if (r >= 0) return r;
+    }
+  }
+  if (!jacobi_params(a, b, c, tol, floor2, cs, sne)) return 0;
+  return cabs2(sne) > Jac<T>::small_angle2 ? 2 : 1;
 }
-__device__ __forceinline__ bool large_angle(float2 sne) { return cabs2(sne) > Jac<float>::small_angle2; }
 
 template <class T, class C>
 __device__ __forceinline__ void rotate_pair(C& xp, C& xq, T cs, C sne) {
@@ -1539,10 +1555,9 @@ __device__ bool jacobi_pair_block(typename Jac<T>::C* __restrict__ X, typename J
     const C Cc = Jac<T>::make(__shfl_sync(0xffffffffu, tot, 2), __shfl_sync(0xffffffffu, tot, 3));
     T cs;
     C sne;
-    const bool rot = quick ? jacobi_params_quick(A, B, Cc, tol * tol, floor2, cs, sne)
-                           : jacobi_params(A, B, Cc, tol, floor2, cs, sne);
+    const int rot = jacobi_rotation(A, B, Cc, tol, floor2, quick, cs, sne);
     if (threadIdx.x == 0) {
-      s_do = !rot ? 0 : large_angle(sne) ? 2 : 1;
+      s_do = rot;
       s_cs = cs;
       s_sne = sne;
     }
@@ -2040,10 +2055,9 @@ __global__ void __launch_bounds__(256)
         __syncwarp();  // read before the next pair's sums arrive
         T cs;
         C sne;
-        if (!(quick ? jacobi_params_quick(a, b, c, tol * tol, floor2, cs, sne)
-                    : jacobi_params(a, b, c, tol, floor2, cs, sne)))
-          continue;
-        if (lane == 0 && large_angle(sne)) s_rot = 1;
+        const int rot = jacobi_rotation(a, b, c, tol, floor2, quick, cs, sne);
+        if (rot == 0) continue;
+        if (lane == 0 && rot == 2) s_rot = 1;
         for (int r = lane; r < p; r += 32) {
           C u = xp[r], v = xq[r];
           rotate_pair(u, v, cs, sne);

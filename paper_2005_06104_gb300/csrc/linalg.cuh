@@ -218,8 +218,9 @@ extern SvdCounters g_svd_counters;
 // (eigenvalues to about 1e-7 relative, eigenvectors to about 1e-7 / relative gap); for the
 // Krylov vectors of the precision forms, whose density matrices are formed to about that
 // accuracy by the tensor-core GEMMs.
-// quick: rotation angles of the FP64 sweeps by FP32 arithmetic (unitary to FP64; see
-// jacobi_params_quick); the factors agree with the exact angles' to rounding, not bit by bit.
+// quick: large rotation angles of the FP64 sweeps by FP32 arithmetic, small ones (the last sweep's) in
+// FP64 by a shorter formula (see jacobi_params_quick); the factors are as orthogonal as with the exact
+// angles, not the same bit by bit.
 void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int cols,
                       int (*select)(const std::vector<double>& s, void* ctx), void* ctx,
                       SvdOut& out, bool want_u, bool want_v, bool psd, bool jacobi_fp32, bool quick);
