@@ -1427,7 +1427,7 @@ __device__ __forceinline__ bool jacobi_params(T a, T b, C c, T tol, T floor2, T&
 //    quotient would not do: a small angle does not mean a small coupling.  For |x_q| << |x_p| the angle
 //    is |cos(x_p, x_q)| |x_q| / |x_p|, and columns of norms 1 and 1e-8 kept a cosine of 2e-7.
 // The reciprocal of b - a is Newton's iteration from FP32's (1.8e-7, 3e-14, then rounding).
-// An imaginary-time step of 40 sites at bond dimension 40, two thirds of it Jacobi sweeps: 174 ms with the
+// An imaginary-time step of 20 sites at bond dimension 40, two fifths of it Jacobi sweeps: 174 ms with the
 // exact angles, 154 ms with these.
 __device__ __forceinline__ float high_float(double x, int add) {  // x 2^add towards zero; 0 below FP32's range
   const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
