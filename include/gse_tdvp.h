@@ -418,6 +418,12 @@ TDVP_API tdvp_status tdvp_expm_contract(const tdvp_site_dims* dims, const void* 
  * a later call with another device current returns TDVP_ERR_INVALID_ARG. */
 TDVP_API const char* tdvp_contract_last_error(void);
 
+/* Failure injection for tests: marks the handle (h = NULL: the context of the handle-free calls, after
+ * its first call) as a tensor-core kernel does whose bounded wait ran out.  The next call on it
+ * returns TDVP_ERR_TIMEOUT, whatever else it met (a sweep stops at its next Lanczos run), and clears
+ * the mark.  The state is then what a time-out leaves: not usable without a checkpoint. */
+TDVP_API tdvp_status tdvp_inject_timeout(tdvp_handle* h);
+
 /* y = H_eff x by the same FP64 contraction as tdvp_heff_contract(...,
  * TDVP_PREC_FP64, ...) (the summation order may differ: the results agree to
  * about 1e-12 relative), but without allocating device memory.  The paper has no counterpart: this entry

@@ -9,6 +9,36 @@
 
 
 namespace {
+// f() as a status.  Every call reads the error word of the tensor-core kernels' bounded waits, if it
+// launched any, whether f returned or threw: a wait that ran out left wrong values, which explain
+// whatever followed, and the word must not wait for the next call.
+template <class F>
+tdvp_status checked(cudaStream_t st, Scratch& scr, std::string& err, F&& f) {
+  tdvp_status s = TDVP_OK;
+  try {
+    f();
+    err.clear();
+  } catch (const TdvpError& e) {
+    err = e.what();
+    s = e.status;
+  } catch (const std::bad_alloc&) {
+    err = "host allocation failed";
+    s = TDVP_ERR_OUT_OF_MEMORY;
+  } catch (const std::exception& e) {
+    err = e.what();
+    s = TDVP_ERR_CUDA;
+  }
+  try {
+    tc_check(st, scr);
+  } catch (const TdvpError& e) {
+    if (s == TDVP_OK || e.status == TDVP_ERR_TIMEOUT) {
+      err = e.what();
+      s = e.status;
+    }
+  }
+  return s;
+}
+
 template <class F>
 tdvp_status guarded(tdvp_handle* h, F&& f) {
   if (!h) return TDVP_ERR_INVALID_ARG;
@@ -18,20 +48,8 @@ tdvp_status guarded(tdvp_handle* h, F&& f) {
     explicit Bind(Tracer* t) : prev(t_tracer) { t_tracer = t; }
     ~Bind() { t_tracer = prev; }
   } bind(h->eng.tracer.on ? &h->eng.tracer : nullptr);
-  try {
-    f();
-    h->err.clear();
-    return TDVP_OK;
-  } catch (const TdvpError& e) {
-    h->err = e.what();
-    return e.status;
-  } catch (const std::bad_alloc&) {
-    h->err = "host allocation failed";
-    return TDVP_ERR_OUT_OF_MEMORY;
-  } catch (const std::exception& e) {
-    h->err = e.what();
-    return TDVP_ERR_CUDA;
-  }
+  Engine& e = h->eng;
+  return checked(e.st, e.scr, h->err, f);
 }
 
 void check_options(const tdvp_options& o) {
@@ -411,10 +429,10 @@ RawCtx& raw() {
 }
 
 template <class F>
-tdvp_status raw_guarded(F&& f) {
+tdvp_status raw_guarded(void* stream, F&& f) {
   RawCtx& c = raw();
   std::lock_guard<std::mutex> lk(c.mu);
-  try {
+  return checked(static_cast<cudaStream_t>(stream), c.scr, c.err, [&] {
     int dev = 0;
     TDVP_CUDA(cudaGetDevice(&dev));
     if (!c.ready) {
@@ -432,15 +450,7 @@ tdvp_status raw_guarded(F&& f) {
                  "handle-free contractions run on the device current at their first call (" +
                      std::to_string(c.device) + "), not on device " + std::to_string(dev));
     f(c);
-    c.err.clear();
-    return TDVP_OK;
-  } catch (const TdvpError& e) {
-    c.err = e.what();
-    return e.status;
-  } catch (const std::exception& e) {
-    c.err = e.what();
-    return TDVP_ERR_CUDA;
-  }
+  });
 }
 
 void check_dims(const tdvp_site_dims* d) {
@@ -467,7 +477,7 @@ tdvp_status tdvp_heff_contract(const tdvp_site_dims* dims, const void* L, const 
 
 tdvp_status tdvp_heff_contract_cached(const tdvp_site_dims* dims, const void* L, const double* W, const void* R,
                                       const void* x, void* y, int precision, long long env_tag, void* stream) {
-  return raw_guarded([&](RawCtx& c) {
+  return raw_guarded(stream, [&](RawCtx& c) {
     tdvp_require(env_tag >= -1, TDVP_ERR_INVALID_ARG, "env_tag must be >= -1");
     check_dims(dims);
     tdvp_require(L && R && x && y && x != y, TDVP_ERR_INVALID_ARG, "null or aliased buffers");
@@ -495,7 +505,7 @@ tdvp_status tdvp_heff_contract_cached(const tdvp_site_dims* dims, const void* L,
 
 tdvp_status tdvp_keff_contract(int ml, int mr, int wb, const void* L, const void* R, const void* x, void* y,
                                void* stream) {
-  return raw_guarded([&](RawCtx& c) {
+  return raw_guarded(stream, [&](RawCtx& c) {
     tdvp_require(ml >= 1 && mr >= 1 && wb >= 1, TDVP_ERR_SHAPE, "dims must be >= 1");
     tdvp_require(L && R && x && y && x != y, TDVP_ERR_INVALID_ARG, "null or aliased buffers");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -508,7 +518,7 @@ tdvp_status tdvp_keff_contract(int ml, int mr, int wb, const void* L, const void
 
 tdvp_status tdvp_env_contract(const tdvp_site_dims* dims, int side, const void* E, const double* W, const void* A,
                               void* out, void* stream) {
-  return raw_guarded([&](RawCtx& c) {
+  return raw_guarded(stream, [&](RawCtx& c) {
     check_dims(dims);
     tdvp_require(E && A && out && E != out, TDVP_ERR_INVALID_ARG, "null or aliased buffers");
     tdvp_require(side == 0 || side == 1, TDVP_ERR_INVALID_ARG, "side must be 0 or 1");
@@ -528,7 +538,7 @@ tdvp_status tdvp_env_contract(const tdvp_site_dims* dims, int side, const void* 
 tdvp_status tdvp_expm_contract(const tdvp_site_dims* dims, const void* L, const double* W, const void* R,
                                const void* x, void* y, double delta, tdvp_time kind, int precision, double tol,
                                int nmax, int* iters, void* stream) {
-  return raw_guarded([&](RawCtx& c) {
+  return raw_guarded(stream, [&](RawCtx& c) {
     check_dims(dims);
     tdvp_require(L && R && x && y && x != y, TDVP_ERR_INVALID_ARG, "null or aliased buffers");
     tdvp_require(kind == TDVP_REAL || kind == TDVP_IMAG, TDVP_ERR_INVALID_ARG, "bad time kind");
@@ -549,19 +559,36 @@ tdvp_status tdvp_expm_contract(const tdvp_site_dims* dims, const void* L, const 
     op.d = dims->d;
     op.env_key = (1LL << 62) + (c.key++);  // cache operands within this call only
     const long long n = (long long)dims->ml * dims->d * dims->mr;
-    int it = 0;
-    try {
-      it = lanczos_expm(
-          st, &c.pool, c.blas, c.lw, [&](const cplx* a, cplx* b) { heff_apply_prec(st, c.scr, op, a, b, precision); },
-          static_cast<const cplx*>(x), static_cast<cplx*>(y), n, delta, kind, tol, nmax);
-    } catch (...) {
-      tc_check(st, c.scr);
-      throw;
-    }
+    const int it = lanczos_expm(
+        st, &c.pool, c.blas, c.lw, c.scr,
+        [&](const cplx* a, cplx* b) { heff_apply_prec(st, c.scr, op, a, b, precision); },
+        static_cast<const cplx*>(x), static_cast<cplx*>(y), n, delta, kind, tol, nmax);
     TDVP_CUDA(cudaStreamSynchronize(st));
     tc_check(st, c.scr);
     if (iters) *iters = it;
   });
+}
+
+tdvp_status tdvp_inject_timeout(tdvp_handle* h) {
+  auto mark = [](cudaStream_t st, Scratch& s) {
+    int* word = tc_error_word(st, s);
+    const int one = 1;
+    TDVP_CUDA(cudaMemcpyAsync(word, &one, sizeof(int), cudaMemcpyHostToDevice, st));
+    TDVP_CUDA(cudaStreamSynchronize(st));
+  };
+  try {
+    if (h) {
+      mark(h->eng.st, h->eng.scr);
+    } else {
+      RawCtx& c = raw();
+      std::lock_guard<std::mutex> lk(c.mu);
+      tdvp_require(c.ready, TDVP_ERR_INVALID_ARG, "no handle-free call yet");
+      mark(nullptr, c.scr);
+    }
+    return TDVP_OK;
+  } catch (const TdvpError& e) {
+    return e.status;
+  }
 }
 
 const char* tdvp_contract_last_error(void) { return raw().err.c_str(); }

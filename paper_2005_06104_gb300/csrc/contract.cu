@@ -117,7 +117,7 @@ void LanczosWork::release() {
   live.release();
 }
 
-int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw,
+int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw, const Scratch& scr,
                  const std::function<void(const cplx*, cplx*)>& op, const cplx* x, cplx* out, long long n,
                  double delta, int kind, double tol, int nmax, int* hint) {
   nmax = std::min(std::max(1, nmax), 63);
@@ -164,11 +164,14 @@ int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw
       // alpha_j = Re <v_j, w>, w made orthogonal to V[0..j], beta_{j+1} = |w|
       blas.lanczos_step(st, V, n, j, wv, live, lw.c.data(), alpha, beta, nrm2);
     }
-    tridiag_expv(st, alpha, beta, j0 + 1, batch, delta, kind, lw.y.data(), errs);
+    const int* timed_out = scr.tc.pending ? scr.tc.err.as<int>() : nullptr;
+    tridiag_expv(st, alpha, beta, j0 + 1, batch, delta, kind, timed_out, lw.y.data(), errs);
     double h[1 + 2 * 64];
     TDVP_CUDA(cudaMemcpyAsync(h, start2, sizeof(double) * (1 + 2 * batch), cudaMemcpyDeviceToHost, st));
     TDVP_CUDA(cudaStreamSynchronize(st));
     const double* h_err = h + 1;
+    // a run on what a timed-out wait left behind ends here, and the sweep with it
+    tdvp_require(h_err[0] >= 0.0 || std::isnan(h_err[0]), TDVP_ERR_TIMEOUT, "Lanczos: a bounded device wait ran out");
     if (j0 == 0) {
       tdvp_require(std::isfinite(h[0]), TDVP_ERR_NONFINITE, "Lanczos: non-finite start vector");
       beta0 = std::sqrt(h[0]);

@@ -99,6 +99,8 @@ struct LanczosWork {
 // hint (may be null): the Krylov dimension of the previous run of the same operator kind; read
 // to size the first batch of iterations a small local problem launches without a host round
 // trip each, and updated to this run's dimension.  Results do not depend on it.
-int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw,
+// scr: whose error word the operator's bounded waits set; once it is set the run ends with
+// TDVP_ERR_TIMEOUT at its next stopping test (the word is left for tc_check).
+int lanczos_expm(cudaStream_t st, DevicePool* pool, Blas1& blas, LanczosWork& lw, const Scratch& scr,
                  const std::function<void(const cplx*, cplx*)>& op, const cplx* x, cplx* out, long long n,
                  double delta, int kind, double tol, int nmax, int* hint = nullptr);

@@ -478,23 +478,17 @@ int Engine::lanczos(const std::function<void(const cplx*, cplx*)>& op, const cpl
                     long long n, double delta, int kind, int slot) {
   int* hint = (slot >= 0 && slot < 4) ? &lanczos_hint[slot] : nullptr;
   int used = 0;
-  try {
-    for (int s = 1;; s *= 2) {
-      try {
-        used = 0;
-        for (int k = 0; k < s; ++k)
-          used += lanczos_expm(st, &pool, blas, lw, op, k == 0 ? x : out, out, n, delta / s, kind, opt.lanczos_tol,
-                               opt.lanczos_max, hint);
-        break;
-      } catch (const TdvpError& e) {
-        if (e.status != TDVP_ERR_LANCZOS_NOT_CONVERGED || 2 * s > 64) throw;
-      }
+  for (int s = 1;; s *= 2) {
+    try {
+      used = 0;
+      for (int k = 0; k < s; ++k)
+        used += lanczos_expm(st, &pool, blas, lw, scr, op, k == 0 ? x : out, out, n, delta / s, kind, opt.lanczos_tol,
+                             opt.lanczos_max, hint);
+      break;
+    } catch (const TdvpError& e) {
+      if (e.status != TDVP_ERR_LANCZOS_NOT_CONVERGED || 2 * s > 64) throw;
     }
-  } catch (...) {
-    tc_check(st, scr);  // a device timeout explains a failure better than what followed it
-    throw;
   }
-  // the error word of the bounded waits stays set until it is read: once per sweep, not per run
   lanczos_iters += used;
   lanczos_calls += 1;
   return used;
@@ -637,7 +631,6 @@ void Engine::sweep(double dt, int kind) {
     for (int j = 0; j < N; ++j) Lok[j] = Rok[j] = 0;
   env_prec = TDVP_PREC_FP64;
   sync();
-  tc_check(st, scr);
 }
 
 // ============================================================================
@@ -744,7 +737,6 @@ void Engine::sweep2(double dt, int kind) {
   env_prec = TDVP_PREC_FP64;
   ++env_epoch;
   sync();
-  tc_check(st, scr);
 }
 
 // ============================================================================
@@ -1227,7 +1219,6 @@ void Engine::expand_basis(int k, const double* weights) {
   center = 0;
   for (int j = 0; j < N; ++j) Lok[j] = Rok[j] = 0;
   sync();
-  tc_check(st, scr);
 }
 
 void Engine::apply_krylov() {

@@ -1167,7 +1167,7 @@ __device__ __noinline__ void tridiag_serial(int n, int K, double x, double delta
 
 __global__ void __launch_bounds__(128)
     k_tridiag_expv(const double* __restrict__ alpha, const double* __restrict__ beta, int n0, double delta, int kind,
-                   cplx* __restrict__ y, double* __restrict__ err) {
+                   const int* __restrict__ timed_out, cplx* __restrict__ y, double* __restrict__ err) {
   constexpr unsigned FULL = 0xffffffffu;
   __shared__ double coef[CHEB_MAX + 1];
   __shared__ double quot[128], jv[128], tk[PAR_K + 1][32], im_sum[32], phase[2];
@@ -1298,7 +1298,7 @@ __global__ void __launch_bounds__(128)
       y[i] = v;
       if (i == n - 1) {
         const double b = beta[n];
-        err[0] = bad ? 1e300 : b * sqrt(cabs2(v));
+        err[0] = timed_out && *timed_out ? -1.0 : bad ? 1e300 : b * sqrt(cabs2(v));
         err[1] = b;
       }
     }
@@ -1307,10 +1307,10 @@ __global__ void __launch_bounds__(128)
 }  // namespace
 
 void tridiag_expv(cudaStream_t st, const double* alpha, const double* beta, int n0, int count, double delta, int kind,
-                  cplx* y, double* err) {
+                  const int* timed_out, cplx* y, double* err) {
   tdvp_require(n0 >= 1 && count >= 1 && n0 + count - 1 < TRI_MAX, TDVP_ERR_INVALID_ARG,
                "tridiag_expv: n out of range");
-  k_tridiag_expv<<<count, 128, 0, st>>>(alpha, beta, n0, delta, kind, y, err);
+  k_tridiag_expv<<<count, 128, 0, st>>>(alpha, beta, n0, delta, kind, timed_out, y, err);
   TDVP_CHECK_LAUNCH();
 }
 

@@ -172,9 +172,10 @@ void fill_zero(cudaStream_t st, cplx* p, long long n);
 // For n = n0 .. n0 + count - 1 (b = n - n0): y[64 b + (0..n)) = exp(coef * T_n) e_0 for the
 // leading n x n part of the tridiagonal T (diagonal alpha, off-diagonals beta[1..n-1]);
 // kind 0: coef = -i delta, kind 1: coef = -delta.  err[2 b] = beta[n] |y[n-1]|, err[2 b + 1] =
-// beta[n], both written to device memory.
+// beta[n], both written to device memory; err[2 b] = -1 when *timed_out (device memory, may be null)
+// is set.
 void tridiag_expv(cudaStream_t st, const double* alpha, const double* beta, int n0, int count, double delta, int kind,
-                  cplx* y, double* err);
+                  const int* timed_out, cplx* y, double* err);
 
 // One-sided Jacobi SVD of a complex FP64 matrix (row-major rows x cols).
 struct SvdOut {

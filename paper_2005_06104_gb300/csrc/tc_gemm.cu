@@ -536,6 +536,7 @@ void tc_check(cudaStream_t st, Scratch& s) {
   c.pending = false;
   if (h_err != 0) {
     TDVP_CUDA(cudaMemsetAsync(c.err.as<int>(), 0, sizeof(int), st));
+    TDVP_CUDA(cudaStreamSynchronize(st));  // a handle-free call may come on another stream next
     throw TdvpError(TDVP_ERR_TIMEOUT, "tensor-core GEMM: a bounded pipeline wait ran out");
   }
 }

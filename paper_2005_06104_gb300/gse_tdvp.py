@@ -138,6 +138,18 @@ for _name, _args in _raw.items():
     _f.restype = C.c_int
 
 
+_lib.tdvp_inject_timeout.argtypes = [_h]
+_lib.tdvp_inject_timeout.restype = C.c_int
+
+
+def inject_timeout(handle=None):
+    """Marks a GseTdvp (None: the handle-free context) as if a bounded device wait had run out; its next
+    call raises TDVPError with status 6 and clears the mark.  For tests of failure handling."""
+    s = _lib.tdvp_inject_timeout(handle.h if handle is not None else None)
+    if s != 0:
+        raise TDVPError(s, "tdvp_inject_timeout")
+
+
 def _raw_chk(s):
     if s != 0:
         raise TDVPError(s, _lib.tdvp_contract_last_error().decode())
