@@ -398,7 +398,7 @@ void Engine::move_right(int i, double eps, int cap, bool trunc) {
     rule.discarded = &disc_eps;
   }
   SvdOut sv;
-  svd_jacobi(st, &pool, psi.A[i].data(), ml * d, mr, rule, sv, true, false, quick_jacobi());
+  svd_jacobi(st, &pool, psi.A[i].data(), ml * d, mr, rule, sv, true, false, quick_jacobi(trunc));
   const int r = sv.rank;
   tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "move_right: zero tensor");
   // C = U^+ A = S Vh (r x mr), one FP64 GEMM instead of rotating V in every Jacobi round;
@@ -437,7 +437,7 @@ void Engine::move_left(int i, double eps, int cap, bool trunc) {
     rule.discarded = &disc_eps;
   }
   SvdOut sv;
-  svd_jacobi(st, &pool, psi.A[i].data(), ml, d * mr, rule, sv, false, true, quick_jacobi());
+  svd_jacobi(st, &pool, psi.A[i].data(), ml, d * mr, rule, sv, false, true, quick_jacobi(trunc));
   const int r = sv.rank;
   tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "move_left: zero tensor");
   // C = A Vh^+ = U S (ml x r), one FP64 GEMM instead of rotating U in every Jacobi round
@@ -543,7 +543,7 @@ void Engine::sweep(double dt, int kind) {
           rule.discarded = &disc_eps;
         }
         SvdOut sv;
-        svd_jacobi(st, &pool, psi.A[i].data(), ml * d, mold, rule, sv, true, false, quick_jacobi());
+        svd_jacobi(st, &pool, psi.A[i].data(), ml * d, mold, rule, sv, true, false, quick_jacobi(imag));
         r = sv.rank;
         tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "sweep: zero site tensor");
         C.reset(&pool, (size_t)r * mold);
@@ -592,7 +592,7 @@ void Engine::sweep(double dt, int kind) {
           rule.discarded = &disc_eps;
         }
         SvdOut sv;
-        svd_jacobi(st, &pool, psi.A[i].data(), mold, d * mr, rule, sv, false, true, quick_jacobi());
+        svd_jacobi(st, &pool, psi.A[i].data(), mold, d * mr, rule, sv, false, true, quick_jacobi(imag));
         r = sv.rank;
         tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "sweep: zero site tensor");
         C.reset(&pool, (size_t)mold * r);
@@ -682,7 +682,7 @@ void Engine::sweep2(double dt, int kind) {
     }
     if (imag) normalize(y.data(), n);
     PhaseScope ps(tracer, PH_SVD);
-    svd_jacobi(st, &pool, y.data(), ml * d, d * mr, rule, sv, left_to_right, !left_to_right, quick_jacobi());
+    svd_jacobi(st, &pool, y.data(), ml * d, d * mr, rule, sv, left_to_right, !left_to_right, quick_jacobi(true));
     tdvp_require(sv.rank >= 1, TDVP_ERR_NONFINITE, "sweep2: zero two-site tensor");
   };
   // C <- exp(+i delta H_eff^(1)) C on site j (the backward step)
@@ -945,7 +945,7 @@ void Engine::krylov_apply(const KrylovOp& kop, const MpsDev& src, MpsDev& out) {
     SvdOut sv;
     {
       PhaseScope ps(tracer, PH_KRYLOV_EIG);
-      eig_psd_jacobi(st, &pool, rho.data(), n, rule, sv, krylov_eig_fp32(kp), quick_jacobi());
+      eig_psd_jacobi(st, &pool, rho.data(), n, rule, sv, krylov_eig_fp32(kp), quick_jacobi(imag_krylov()));
     }
     const int keep = std::max(1, sv.rank);
     tdvp_require(sv.rank >= 1, TDVP_ERR_NONFINITE, "krylov: zero density matrix");
@@ -1018,7 +1018,7 @@ void Engine::krylov_zipup(const KrylovOp& kop, const MpsDev& src, MpsDev& out) {
     SvdOut sv;
     {
       PhaseScope ps(tracer, PH_KRYLOV_EIG);
-      eig_psd_jacobi(st, &pool, rho.data(), n, rule, sv, krylov_eig_fp32(kp), quick_jacobi());
+      eig_psd_jacobi(st, &pool, rho.data(), n, rule, sv, krylov_eig_fp32(kp), quick_jacobi(imag_krylov()));
     }
     const int keep = sv.rank;
     tdvp_require(keep >= 1, TDVP_ERR_NONFINITE, "zip-up: zero site");
@@ -1045,7 +1045,7 @@ void Engine::krylov_zipup(const KrylovOp& kop, const MpsDev& src, MpsDev& out) {
   for (int i = 0; i + 1 < N; ++i) {
     const int ml = t.m[i], mr = t.m[i + 1], mr2 = t.m[i + 2];
     SvdOut sv;
-    svd_jacobi(st, &pool, t.A[i].data(), ml * d, mr, crule, sv, true, false, quick_jacobi());
+    svd_jacobi(st, &pool, t.A[i].data(), ml * d, mr, crule, sv, true, false, quick_jacobi(imag_krylov()));
     const int r = sv.rank;
     tdvp_require(r >= 1, TDVP_ERR_NONFINITE, "zip-up: zero tensor in the compression");
     DArr C(&pool, (size_t)r * mr);
@@ -1106,7 +1106,7 @@ void Engine::expand_basis(int k, const double* weights) {
         Bm = std::move(qo.Q);
       } else {
         SvdOut sv;
-        svd_jacobi(st, &pool, X, ml, cols, SvdRule{}, sv, false, true, quick_jacobi());
+        svd_jacobi(st, &pool, X, ml, cols, SvdRule{}, sv, false, true, quick_jacobi(imag_krylov()));
         r = sv.rank;
         Bm = std::move(sv.Vh);
       }
@@ -1153,7 +1153,7 @@ void Engine::expand_basis(int k, const double* weights) {
         SvdOut sy;
         {
           PhaseScope ps(tracer, PH_EXTEND_SVD);
-          svd_jacobi(st, &pool, Y.data(), rows, cols, rule, sy, false, true, quick_jacobi());
+          svd_jacobi(st, &pool, Y.data(), rows, cols, rule, sy, false, true, quick_jacobi(imag_krylov()));
         }
         nb = sy.rank;
         if (nb > 0) {
@@ -1168,7 +1168,7 @@ void Engine::expand_basis(int k, const double* weights) {
           struct KeepAll {
             int operator()(const std::vector<double>& s) const { return (int)s.size(); }
           };
-          svd_jacobi(st, &pool, sy.Vh.data(), nb, cols, KeepAll{}, so, false, true, quick_jacobi());
+          svd_jacobi(st, &pool, sy.Vh.data(), nb, cols, KeepAll{}, so, false, true, quick_jacobi(imag_krylov()));
           Bbar = std::move(so.Vh);
           nb = so.rank;
         }

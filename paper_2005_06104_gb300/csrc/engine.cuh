@@ -82,9 +82,14 @@ struct Engine {
   void build_pair_mpo();
   void env_left(int i);   // L[i+1] from L[i], A[i]
   void env_right(int i);  // R[i-1] from R[i], A[i]
-  // FP32 arithmetic for large rotation angles in FP64 Jacobi sweeps: not in a split form, whose
-  // trajectories keep their bits (see gauge_gemm)
-  bool quick_jacobi() const { return opt.precision == TDVP_PREC_FP64; }
+  // FP32 arithmetic for large rotation angles in the Jacobi sweeps of FP64 handles (see
+  // jacobi_params_quick).  Not in a split form, whose trajectories keep their bits (see gauge_gemm), and
+  // where a real-time TDVP1 trajectory meets the factors only with `truncates`: its moves decide ranks at
+  // 1e-10 of the largest singular value, where the last bits of the Krylov vectors and of the
+  // extension count (one-axis twisting of 100 spins: 12 or 13 states on a bond), so it keeps the exact
+  // angles.  Imaginary time cuts by weight and converges to a fixed point.
+  bool quick_jacobi(bool truncates) const { return truncates && opt.precision == TDVP_PREC_FP64; }
+  bool imag_krylov() const { return opt.tau_im != 0.0; }  // Krylov vectors of imaginary-time steps
   // gauge moves
   void gauge_gemm(int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A, long long lda, const cplx* B,
                   long long ldb, cplx beta, cplx* C, long long ldc);

@@ -1418,7 +1418,7 @@ __device__ __forceinline__ bool jacobi_params(T a, T b, C c, T tol, T floor2, T&
 
 // The same rotation with the angle's arithmetic in FP32 where that is enough.  GB300's FP64 unit takes 65
 // cycles per instruction of a warp: the exact angle's two reciprocal roots, root and division are about
-// 70 of them, these about 20 for a large angle and 10 for a small one.
+// 70 of them, one after the other; these are one reciprocal root, or two divisions side by side.
 //  - |sin theta| > 1e-8: any complex tangent tau = t e^{i phi} gives a unitary rotation, cs = 1 / sqrt(1 +
 //    |tau|^2), sne = cs tau, so only that normalisation has to be exact.  With tau good to FP32 about
 //    3e-7 |c| of the coupling c stays, and the angle asks for another sweep, which removes it.
@@ -1426,9 +1426,8 @@ __device__ __forceinline__ bool jacobi_params(T a, T b, C c, T tol, T floor2, T&
 //    to 1e-16 of itself (t = 1 / (2 zeta) (1 - 1 / (4 zeta^2) + ...)), with the quotient in FP64.  An FP32
 //    quotient would not do: a small angle does not mean a small coupling.  For |x_q| << |x_p| the angle
 //    is |cos(x_p, x_q)| |x_q| / |x_p|, and columns of norms 1 and 1e-8 kept a cosine of 2e-7.
-// The reciprocal of b - a is Newton's iteration from FP32's (1.8e-7, 3e-14, then rounding).
 // An imaginary-time step of 20 sites at bond dimension 40, two fifths of it Jacobi sweeps: 174 ms with the
-// exact angles, 154 ms with these.
+// exact angles, 153 ms with these.
 __device__ __forceinline__ float high_float(double x, int add) {  // x 2^add towards zero; 0 below FP32's range
   const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
   const int e = (int)((h >> 20) & 0x7ff) - 1023 + 127 + add;
@@ -1443,8 +1442,7 @@ __device__ __forceinline__ double wide_double(float x) {  // (double)x by its bi
   return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
 }
 constexpr float kSmallZeta = 5e7f;  // |zeta| from which |sin theta| <= 1e-8
-// 0: the pair stays, 1: rotate, 2: rotate, and the sweep is not the last (Jac<double>::small_angle2), -1: out
-// of this function's range
+// 0: the pair stays, 1: rotate, 2: rotate, and the sweep is not the last (Jac<double>::small_angle2)
 __device__ __forceinline__ int jacobi_params_quick(double a, double b, double2 c, double tol2, double floor2,
                                                    double& cs, double2& sne) {
   // the tests on bits, exponents and FP32 mantissas (they decide to 1e-7 of their thresholds)
@@ -1467,14 +1465,8 @@ __device__ __forceinline__ int jacobi_params_quick(double a, double b, double2 c
   const float zeta = 0.5f * high_float(diff, sh) * inv;
   const float az = fabsf(zeta);
   if (az >= kSmallZeta) {
-    const int ed = biased_exponent(diff);
-    if (ed < 50 || ed > 2000) return -1;  // 1 / (b - a) has to be a normal number
-    const double s = wide_double(1.0f / high_float(diff, 1023 - ed));  // 2^(ed - 1023) / (b - a)
-    double r = __hiloint2double(__double2hiint(s) + ((1023 - ed) << 20), __double2loint(s));
-    r = fma(r, fma(-diff, r, 1.0), r);
-    r = fma(r, fma(-diff, r, 1.0), r);
     cs = 1.0;
-    sne = make_double2(c.x * r, c.y * r);
+    sne = make_double2(c.x / diff, c.y / diff);
     return 1;
   }
   const float t = copysignf(1.0f / (az + sqrtf(1.0f + az * az)), zeta) * inv;
@@ -1488,10 +1480,7 @@ __device__ __forceinline__ int jacobi_params_quick(double a, double b, double2 c
 template <class T, class C>
 __device__ __forceinline__ int jacobi_rotation(T a, T b, C c, T tol, T floor2, int quick, T& cs, C& sne) {
   if constexpr (sizeof(T) == 8) {  // FP32 rotations have no shorter form
-    if (quick) {
-      const int r = jacobi_params_quick(a, b, c, tol * tol, floor2, cs, sne);
-      if (r >= 0) return r;
-    }
+    if (quick) return jacobi_params_quick(a, b, c, tol * tol, floor2, cs, sne);
   }
   if (!jacobi_params(a, b, c, tol, floor2, cs, sne)) return 0;
   return cabs2(sne) > Jac<T>::small_angle2 ? 2 : 1;

@@ -2,8 +2,9 @@
 
 The middle site matrix of a chain holds one block with graded columns and, in rows and columns of
 its own, a block of two equal columns, which makes the matrix rank deficient: the gauge move takes
-the SVD and not the QR.  Every singular value of the graded block is kept (above 1e-10 of the
-largest), so the left factor has to be an isometry and the state has to stay.
+the SVD and not the QR.  H = 0 (couplings of zero), so every evolution is the identity and what moves
+the state is the factorisations.  Every singular value of the graded block is kept (above 1e-10 of
+the largest), so the factors have to be isometries and the state has to stay.
 
 A Jacobi sweep that leaves every pair orthogonal to rounding gives |U^H U - 1| of a few ulp times
 sqrt(rows): 1e-15 to 4e-15 for these blocks (measured with the angles in FP64 throughout), held to
@@ -48,52 +49,74 @@ def _chain(rng, block):
     m[p:, q] = m[p:, q + 1] = v / np.linalg.norm(v)
     mps.append(m.reshape(2 ** k, 2, q + 2))
     left = q + 2
-    while left > 1:
+    while left > 1:                                # embeddings: state l goes to (s, r) = divmod(l, right)
         right = (left + 1) // 2
-        a = rng.standard_normal((left, 2 * right)) + 1j * rng.standard_normal((left, 2 * right))
-        mps.append(np.linalg.qr(a.conj().T)[0].conj().T.reshape(left, 2, right))
+        a = np.zeros((left, 2, right), dtype=complex)
+        for l in range(left):
+            a[l, l // right, l % right] = 1.0
+        mps.append(a)
         left = right
     return mps, k
+
+
+def _isometry_error(mats):
+    return max(np.max(np.abs(u.conj().T @ u - np.eye(u.shape[1]))) for u in mats)
+
+
+def _left(mps):
+    return [a.reshape(-1, a.shape[2]) for a in mps[:-1]]
+
+
+def _right(mps):
+    return [a.reshape(a.shape[0], -1).conj().T for a in mps[1:]]
+
+
+def _direction_error(mps, ref):
+    v, w = mps_to_dense(mps), mps_to_dense(ref)
+    return np.linalg.norm(v / np.linalg.norm(v) - w / np.linalg.norm(w))
 
 
 CASES = [(4, 2, 1e-4, 1.0, False), (4, 2, 1e-5, 1e-3, False), (4, 2, 1e-6, 1e-2, False), (4, 2, 1e-8, 1.0, False),
          (6, 3, 1e-7, 1.0, False), (8, 4, 1e-8, 1.0, True), (16, 8, 1e-6, 1.0, True), (60, 30, 1e-6, 1.0, True)]
 
 
+@pytest.mark.parametrize("how", ["move", "imaginary", "two-site"])
 @pytest.mark.parametrize("p,q,small,coupling,halves", CASES)
-def test_graded_block_gives_an_isometry(p, q, small, coupling, halves):
+def test_graded_block_gives_an_isometry(p, q, small, coupling, halves, how):
+    """The gauge move of a rank-deficient site (exact angles) and the truncating moves of imaginary time
+    and of the two-site integrator (large angles in FP32)."""
     assert torch.cuda.is_available()
     from paper_2005_06104_gb300 import gse_tdvp as g
-    worst = [0.0, 0.0]
+    iso = err = 0.0
     for seed in range(8):
         rng = np.random.default_rng(1000 * p + seed)
         mps, k = _chain(rng, _graded(rng, p, q, small, coupling, halves))
-        h = g.GseTdvp(mps, wl.heisenberg_mpo(wl.chain(len(mps))), chi_max=256)
+        h = g.GseTdvp(mps, wl.heisenberg_mpo(wl.chain(len(mps), 0.0)), chi_max=256)
+        if how == "imaginary":
+            h.sweep(0.1, g.IMAG)
+        elif how == "two-site":
+            h.sweep2(0.1, g.REAL)
         out = h.get_mps()
         h.close()
-        a = out[k]
-        assert a.shape[2] == q + 1                 # the two equal columns are one direction
-        u = a.reshape(-1, a.shape[2])
-        worst[0] = max(worst[0], np.max(np.abs(u.conj().T @ u - np.eye(u.shape[1]))))
-        v0, v1 = mps_to_dense(mps), mps_to_dense(out)
-        worst[1] = max(worst[1], np.linalg.norm(v1 - v0) / np.linalg.norm(v0))
-    assert worst[0] < TOL and worst[1] < TOL
+        assert out[k].shape[2] == q + 1            # the two equal columns are one direction
+        iso = max(iso, _isometry_error(_left(out) if how == "move" else _right(out)))
+        err = max(err, _direction_error(out, mps))
+    assert iso < TOL and err < TOL
 
 
+@pytest.mark.parametrize("tau", [0.1, -0.1j])
 @pytest.mark.parametrize("p,q,small", [(4, 2, 1e-4), (4, 2, 1e-5), (8, 4, 1e-5), (60, 30, 1e-5)])
-def test_graded_density_matrices_give_isometries(p, q, small):
-    """The same states through the density-matrix compression with tau = 0 (the operator is the
+def test_graded_density_matrices_give_isometries(p, q, small, tau):
+    """The same states through the density-matrix compression of the Krylov vectors (the operator is the
     identity): eigenvectors of graded positive semidefinite blocks, by Jacobi on Cholesky factors
-    whose columns are graded by themselves."""
+    whose columns are graded by themselves; in imaginary time with the large angles in FP32."""
     from paper_2005_06104_gb300 import gse_tdvp as g
     worst = 0.0
     for seed in range(8):
         rng = np.random.default_rng(500 * p + seed)
         mps, k = _chain(rng, _graded(rng, p, q, small, 1.0, True))
-        h = g.GseTdvp(mps, wl.heisenberg_mpo(wl.chain(len(mps))), chi_max=256, tau=0.0, eps_k=0.0)
+        h = g.GseTdvp(mps, wl.heisenberg_mpo(wl.chain(len(mps), 0.0)), chi_max=256, tau=tau, eps_k=0.0)
         h.apply_krylov()
-        for a in h.get_mps()[:-1]:
-            u = a.reshape(-1, a.shape[2])
-            worst = max(worst, np.max(np.abs(u.conj().T @ u - np.eye(u.shape[1]))))
+        worst = max(worst, _isometry_error(_left(h.get_mps())))
         h.close()
     assert worst < TOL
