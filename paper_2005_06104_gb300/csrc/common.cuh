@@ -10,6 +10,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <map>
+#include <mutex>
 #include <stdexcept>
 #include <string>
 #include <vector>
@@ -292,5 +293,28 @@ class Packed {
  private:
   std::vector<char> bytes_;
 };
+
+// f() once per device and call site (each lambda is a type of its own); returns what it returned there.
+// Function attributes and launch limits belong to a device: set once per process they would be missing
+// on the second one.  A call that throws is tried again next time.
+constexpr int kMaxDevices = 64;
+template <class F>
+int once_per_device(int dev, F&& f) {
+  struct Slot {
+    std::once_flag once;
+    int value = 0;
+  };
+  static Slot slots[kMaxDevices];
+  tdvp_require(dev >= 0 && dev < kMaxDevices, TDVP_ERR_INVALID_ARG, "device index out of range");
+  Slot& s = slots[dev];
+  std::call_once(s.once, [&] { s.value = (int)f(); });
+  return s.value;
+}
+template <class F>
+int per_device(F&& f) {
+  int dev = 0;
+  TDVP_CUDA(cudaGetDevice(&dev));
+  return once_per_device(dev, f);
+}
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }

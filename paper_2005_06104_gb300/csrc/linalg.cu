@@ -206,12 +206,11 @@ void zgemm_t(int tile, dim3 g, cudaStream_t st, int M, int N, int K, cplx alpha,
     cfg.numAttrs = 1;
     TDVP_CUDA(cudaLaunchKernelEx(&cfg, kernel, ZG_ARGS));
   };
-  static const bool wide = [] {  // clusters of more than 8
+  per_device([] {  // clusters of more than 8
     TDVP_CUDA(cudaFuncSetAttribute(k_zgemm<OPA, OPB, 8>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     TDVP_CUDA(cudaFuncSetAttribute(k_zgemm<OPA, OPB, 16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return true;
-  }();
-  (void)wide;
+  });
   switch (tile) {
     case 8: launch(k_zgemm<OPA, OPB, 8>, 64); break;
     case 16: launch(k_zgemm<OPA, OPB, 16>, 256); break;
@@ -264,12 +263,12 @@ void zgemm(cudaStream_t st, int opA, int opB, int M, int N, int K, cplx alpha, c
   // long K is split along K over enough blocks to occupy the GPU (needs a pool).
   const long long tiles = (long long)ceil_div(N, GB_N) * ceil_div(M, GB_M) * batch;
   int ns = 1, kc = K;
-  static const int sms = [] {  // thread-safe one-time initialisation
+  const int sms = per_device([] {
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
     return n > 0 ? n : 148;
-  }();
+  });
   if (ws && tiles < 2LL * sms && K >= 32) {
     ns = (int)std::min<long long>((2LL * sms + tiles - 1) / tiles, (K + 15) / 16);
     ns = std::max(1, std::min(ns, 65535 / batch));
@@ -958,11 +957,10 @@ void Blas1::lanczos_step(cudaStream_t st, cplx* V, long long n, int j, cplx* w, 
   const int nvec = j + 1;
   tdvp_require(j >= 0 && nvec < TRI_MAX, TDVP_ERR_INVALID_ARG, "lanczos_step: too many vectors");
   if (lanczos_step_fused(n)) {
-    static const bool attr = [] {
+    per_device([] {
       TDVP_CUDA(cudaFuncSetAttribute(k_lanczos_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
       return true;
-    }();
-    (void)attr;
+    });
     int nn = (int)n;
     cplx* pp = partial.data();
     void* args[] = {&V, &j, &w, &nn, &alpha, &beta, &nrm2, &pp};
@@ -1810,12 +1808,11 @@ void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows,
   int sweeps = 0;
   if (q > 1) {
     if (small_bytes <= 96 * 1024) {
-      static const bool attr_set = [] {
+      per_device([] {
         TDVP_CUDA(cudaFuncSetAttribute(k_jacobi_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        96 * 1024));
         return true;
-      }();
-      (void)attr_set;
+      });
       k_jacobi_small<<<1, 256, small_bytes, st>>>(X.data(), Vx.data(), p, q, qpad, tol, d_fro2,
                                                    need_acc ? 1 : 0, max_sweeps, d_flag);
       TDVP_CHECK_LAUNCH();
@@ -1825,13 +1822,13 @@ void svd_jacobi_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows,
         throw TdvpError(TDVP_ERR_SVD_NOT_CONVERGED, "Jacobi SVD did not converge");
       }
     } else {
-      static const int coop_blocks = [] {
+      const int coop_blocks = per_device([] {
         int dev = 0, sms = 0, per_sm = 0;
         TDVP_CUDA(cudaGetDevice(&dev));
         TDVP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         TDVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jacobi_coop, 256, 0));
         return std::max(1, sms * std::max(1, per_sm));
-      }();
+      });
       const int nblk = std::max(1, std::min(qpad / 2, coop_blocks));
       bar_buf.ensure(pool, sizeof(GridBar));
       GridBar* bar = bar_buf.as<GridBar>();
@@ -2572,13 +2569,13 @@ __global__ void k_to_c128(const float2* __restrict__ in, cplx* __restrict__ out,
 
 void run_pchol_groups(cudaStream_t st, DevicePool* pool, cplx* Xs, BlkDesc* d_desc, int* d_piv, std::vector<int> gsz) {
   const int nblk = (int)gsz.size();
-  static const int max_ctas = [] {
+  const int max_ctas = per_device([] {
     int dev = 0, sms = 0, per_sm = 0;
     TDVP_CUDA(cudaGetDevice(&dev));
     TDVP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     TDVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pchol_groups, 256, 0));
     return std::max(1, sms * std::min(4, std::max(1, per_sm)));
-  }();
+  });
   long long total = 0;
   for (int g : gsz) total += g;
   const int budget = std::max(max_ctas, nblk);
@@ -2614,13 +2611,13 @@ template <class T>
 void run_jacobi_multi(cudaStream_t st, DevicePool* pool, typename Jac<T>::C* Xs, typename Jac<T>::C* Vs,
                       const std::vector<BlkDesc>& desc, const BlkDesc* d_desc, bool quick, double* d_s, int* d_stat) {
   const int nblk = (int)desc.size();
-  static const int max_ctas = [] {
+  const int max_ctas = per_device([] {
     int dev = 0, sms = 0, per_sm = 0;
     TDVP_CUDA(cudaGetDevice(&dev));
     TDVP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     TDVP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jacobi_groups<T>, 256, 0));
     return std::max(1, sms * std::min(4, std::max(1, per_sm)));
-  }();
+  });
   // CTAs per block: one per pair of a round, scaled down together when they do not all fit
   std::vector<long long> pairs(nblk);
   long long total = 0;
@@ -2882,14 +2879,13 @@ void svd_blocked_keep(cudaStream_t st, DevicePool* pool, const cplx* M, int rows
       }
     }
     std::optional<ActivePhase> jac(std::in_place, PH_SVD_JACOBI);
-    static const bool attr = [] {
+    per_device([] {
       TDVP_CUDA(cudaFuncSetAttribute(k_jacobi_batched<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSmemCap));
       TDVP_CUDA(cudaFuncSetAttribute(k_jacobi_batched<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSmemCap));
       return true;
-    }();
-    (void)attr;
+    });
     if (psd && jacobi_fp32) {
       // the factor (FP64 pivoted Cholesky) is rotated in FP32: its columns are graded, so the
       // one-sided Jacobi keeps about 1e-7 relative accuracy in every eigenvalue (s^2)
@@ -3388,11 +3384,10 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
   const int cl = cluster_ctas(qmax);
   const size_t smem = (size_t)pmax * sizeof(cplx);
   tdvp_require(smem <= 200 * 1024, TDVP_ERR_INVALID_ARG, "QR: block too tall for the staged reflector");
-  static const bool attr = [] {
+  per_device([] {
     TDVP_CUDA(cudaFuncSetAttribute(k_qr_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     return true;
-  }();
-  (void)attr;
+  });
   int dev = 0, sms = 0, per_sm = 0;
   TDVP_CUDA(cudaGetDevice(&dev));
   TDVP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -3438,13 +3433,12 @@ void qr_blocked(cudaStream_t st, DevicePool* pool, const cplx* M, int rows, int 
   k_qr_gather<<<nblk, 256, 0, st>>>(M, cols, d_desc, d_r, d_c, X.data());
   TDVP_CHECK_LAUNCH();
   if (clusters) {
-    static const bool cattr = [] {
+    per_device([] {
       TDVP_CUDA(cudaFuncSetAttribute(k_qr_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
       TDVP_CUDA(cudaFuncSetAttribute(k_qr_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)(kClCols * kClP * sizeof(cplx))));
       return true;
-    }();
-    (void)cattr;
+    });
     cplx* xp = X.data();
     cplx* qp = Qb.data();
     const QrDesc* dd = d_desc;

@@ -946,7 +946,7 @@ void launch_bf16s(cudaStream_t st, const CUtensorMap& ma, const CUtensorMap& mb,
                   int kb_split, int splits, const float* sA, long long lsA, const float* sB, void* out,
                   long long ldo, long long split_stride, int out_df, int* d_err, const unsigned* maskA,
                   const unsigned* maskB, int mw) {
-  static const bool attr = [] {
+  per_device([] {
     // the register hand-over inside the kernel is sized for exactly this launch allocation
     cudaFuncAttributes fa;
     TDVP_CUDA(cudaFuncGetAttributes(&fa, k_gemm_bf16s<S>));
@@ -956,8 +956,7 @@ void launch_bf16s(cudaStream_t st, const CUtensorMap& ma, const CUtensorMap& mb,
     TDVP_CUDA(cudaFuncSetAttribute(k_gemm_bf16s<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    SCfg<S>::SMEM_BYTES));
     return true;
-  }();
-  (void)attr;
+  });
   dim3 grid(ceil_div(N, BN), ceil_div(M, BM), splits);
   tdvp_require(grid.y <= 65535 && splits <= 65535, TDVP_ERR_INVALID_ARG, "gemm_bf16s: grid too large");
   k_gemm_bf16s<S><<<grid, THREADS, SCfg<S>::SMEM_BYTES, st>>>(ma, mb, M, N, nkb, kb_split, sA, lsA, sB, out, ldo,
@@ -1037,12 +1036,12 @@ __global__ void __launch_bounds__(128) k_splitk_df(const float2* __restrict__ ws
 // Splits of K (whole 128-deep chunks) that minimise waves of CTAs x work per CTA:
 // few output tiles (a narrow product or a long K) would otherwise leave most SMs idle.
 int choose_splits(long long tiles, int nchunks) {
-  static const int sms = [] {
+  const int sms = per_device([] {
     int dev = 0, n = 0;
     TDVP_CUDA(cudaGetDevice(&dev));
     TDVP_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
     return n > 0 ? n : 148;
-  }();
+  });
   int best = 1;
   double best_t = (double)((tiles + sms - 1) / sms);
   for (int sp = 2; sp <= std::min(32, nchunks); ++sp) {

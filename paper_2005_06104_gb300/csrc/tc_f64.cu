@@ -514,7 +514,7 @@ void gemm_digits(cudaStream_t st, DevicePool* pool, const Digits& A, const Digit
                  cplx beta, cplx* C, long long ldc, int* err) {
   tdvp_require(A.ldk == B.ldk && A.mw == B.mw && M <= A.rows_pad && 2 * N <= B.rows_pad, TDVP_ERR_INVALID_ARG,
                "gemm_digits: operands differ");
-  static const int sms = [] {
+  const int sms = per_device([] {
     cudaFuncAttributes fa;
     TDVP_CUDA(cudaFuncGetAttributes(&fa, k_gemm_f64s));
     tdvp_require(fa.numRegs == REGS_LAUNCH, TDVP_ERR_CUDA,
@@ -525,7 +525,7 @@ void gemm_digits(cudaStream_t st, DevicePool* pool, const Digits& A, const Digit
     TDVP_CUDA(cudaGetDevice(&dev));
     TDVP_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
     return n > 0 ? n : 148;
-  }();
+  });
   const int nkb = A.ldk / BK, nchunks = (nkb + KC_KB - 1) / KC_KB;
   const long long tiles = (long long)ceil_div(M, BM) * ceil_div(2 * N, BN);
   // Splits of the two passes along K.  One product of one chunk takes about 0.5 us of an SM and a

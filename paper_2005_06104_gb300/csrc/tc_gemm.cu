@@ -359,11 +359,10 @@ CUtensorMap make_map(const float* base, int rows, int ld, int box_rows, int bk) 
 template <class C>
 void launch_gemm(cudaStream_t st, const float* Ahi, const float* Alo, const float* Bhi, const float* Blo, int M, int N,
                  int ldk, void* out, long long ldo, bool out_f64, int* d_err) {
-  static const bool attr = [] {
+  per_device([] {
     TDVP_CUDA(cudaFuncSetAttribute(k_gemm_tf32x3<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
     return true;
-  }();
-  (void)attr;
+  });
   // operands hold ceil(M/128)*128 and ceil(N/128)*128 rows (zero padded); a BN = 256
   // tile may reach 128 rows past the padded B operand only when N is not a multiple of
   // 256, and the host pads B to 256 rows in that case
