@@ -580,13 +580,48 @@ bool f64_on_tensor_cores(long long M, long long N, long long K) {
          K < (1LL << 29);
 }
 
+// Device memory that the digits and partial results of one product may take, and with H_eff's kept digits
+// those of an apply.  Digits take 1.75 and 3.5 times their operands and the partials twice the output:
+// 3 GB for H_eff at 1024 x 1024, w = 14, where T1 and T2 are 0.9 GB.  Beyond the limit a product runs in
+// panels of A's rows and B's columns and H_eff keeps no digits, so that a size that fits the device
+// without them still does, and a pool holding more than the limit in unused blocks gives them back.
+// (A product that large runs for 50 ms and more, its digits and the allocations for a few.)
+constexpr size_t kWorkBytes = size_t(8) << 30;
+size_t digits_bytes(long long rows, long long K) {  // of `rows` real rows
+  return sizeof(__nv_bfloat16) * NS * (size_t)((rows + 127) / 128 * 128) * (size_t)((2 * K + BK - 1) / BK * BK);
+}
+size_t partial_bytes(long long M, long long N) { return 2 * sizeof(cplx) * (size_t)M * (size_t)N; }
+void give_back(DevicePool* pool) {
+  if (pool->cached_bytes() > kWorkBytes) pool->trim();
+}
+
 void zgemm_f64s(cudaStream_t st, Scratch& s, int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A,
                 long long lda, const cplx* B, long long ldb, cplx beta, cplx* C, long long ldc) {
   int* err = tc_error_word(st, s);
+  int mp = M, np = N;  // a panel: mp x np of the output, in steps of a tile (128 real rows each)
+  while (digits_bytes(mp, K) + digits_bytes(2LL * np, K) + partial_bytes(mp, np) > kWorkBytes && (mp > 128 || np > 64)) {
+    if (mp > 128 && (np <= 64 || mp >= 2LL * np))
+      mp = pad_to((mp + 1) / 2, 128);
+    else
+      np = pad_to((np + 1) / 2, 64);
+  }
+  const bool ka = opA == OP_N || opA == OP_R, kb = opB == OP_T || opB == OP_C;
   Digits a, b;
-  make_digits(st, s.pool, 0, opA == OP_N || opA == OP_R, A, lda, M, K, opA == OP_C || opA == OP_R, a);
-  make_digits(st, s.pool, 1, opB == OP_T || opB == OP_C, B, ldb, N, K, opB == OP_C || opB == OP_R, b);
-  gemm_digits(st, s.pool, a, b, M, N, alpha, beta, C, ldc, err);
+  for (int n0 = 0; n0 < N; n0 += np) {
+    const int nn = std::min(np, N - n0);
+    make_digits(st, s.pool, 1, kb, kb ? B + n0 * ldb : B + n0, ldb, nn, K, opB == OP_C || opB == OP_R, b);
+    for (int m0 = 0; m0 < M; m0 += mp) {
+      const int mm = std::min(mp, M - m0);
+      if (n0 == 0 || mp < M)
+        make_digits(st, s.pool, 0, ka, ka ? A + m0 * lda : A + m0, lda, mm, K, opA == OP_C || opA == OP_R, a);
+      gemm_digits(st, s.pool, a, b, mm, nn, alpha, beta, C + m0 * ldc + n0, ldc, err);
+    }
+  }
+  if (mp < M || np < N) {
+    a = Digits();
+    b = Digits();
+    give_back(s.pool);
+  }
 }
 
 // H_eff with the digits of L and R kept for the applies that share op.env_key.  T1 has its rows
@@ -595,9 +630,24 @@ void zgemm_f64s(cudaStream_t st, Scratch& s, int opA, int opB, int M, int N, int
 void heff_f64s(cudaStream_t st, Scratch& s, const SiteOp& op, const cplx* x, cplx* y) {
   const int ml = op.ml, mr = op.mr, wl = op.wl, wr = op.wr, d = op.d;
   const cplx one = mkc(1.0, 0.0), zero = mkc(0.0, 0.0);
+  int* err = tc_error_word(st, s);
+  const size_t kept = digits_bytes((long long)ml * wl, ml) + digits_bytes(2LL * mr, (long long)wr * mr);
+  const size_t first = digits_bytes(2LL * d * mr, ml) + partial_bytes((long long)ml * wl, (long long)d * mr);
+  const size_t second = digits_bytes((long long)ml * d, (long long)wr * mr) + partial_bytes((long long)ml * d, mr);
+  if (kept + std::max(first, second) > kWorkBytes) {
+    s.f64.reset();
+    s.t1.ensure(s.pool, (size_t)ml * wl * d * mr);
+    s.t2.ensure(s.pool, (size_t)ml * d * wr * mr);
+    zgemm_f64s(st, s, OP_N, OP_N, ml * wl, d * mr, ml, one, op.L, ml, x, (long long)d * mr, zero, s.t1.data(),
+               (long long)d * mr);
+    wstage_left(st, *op.W, s.t1.data(), s.t2.data(), ml, mr);
+    zgemm_f64s(st, s, OP_N, OP_T, ml * d, mr, wr * mr, one, s.t2.data(), (long long)wr * mr, op.R, (long long)wr * mr,
+               zero, y, mr);
+    give_back(s.pool);
+    return;
+  }
   if (!s.f64) s.f64 = std::make_shared<F64EnvDigits>();
   F64EnvDigits& c = *s.f64;
-  int* err = tc_error_word(st, s);
   if (op.env_key < 0 || c.key != op.env_key) {
     c.key = -1;
     make_digits(st, s.pool, 0, true, op.L, ml, ml * wl, ml, false, c.L, ml, wl);
