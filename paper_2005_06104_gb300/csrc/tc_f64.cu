@@ -1,5 +1,6 @@
 // FP64 complex GEMMs on the BF16 tensor cores (sm_103a, tcgen05 kind::f16), without rounding in
-// the tensor core.
+// the tensor core: the splitting of the operands into exact slices of Ozaki, Ogita, Oishi and Rump
+// (Numer. Algorithms 59, 2012), with fixed-point slices.
 //
 // GB300 runs FP64 at 1.1 TFLOP/s and dense BF16 at 1860.  Each row of a real operand (the 4M
 // embedding of the complex one) is written as integers of 56 bits under one power of two, cut
@@ -11,9 +12,16 @@
 // integers and nothing rounds.  Groups 0..7 are kept (34 products); the first group left out is
 // 2^-64 of the operands' maxima.  The epilogue adds each chunk's group sums into 64-bit integers
 // (128-deep chunks; 256 for the groups 0..3, whose sums have room) and converts once at the end.
-// The error is the operands' rounding at 2^-56 of their row maxima whatever K is, below that of
-// FP64 multiply-adds, which grows with the square root of K.  (Groups 0..6 alone, 28 products,
-// leave 2.4e-16 of the norm: more than the split-K CUDA-core product has at K near 128.)
+// The error is the operands' rounding at 2^-56 of their row maxima whatever K is.  Against the product of
+// the operands' norms that is below the error of FP64 multiply-adds, which grows with the square root
+// of K.  It is not relative to each result: an entry below 2^-3 of its row's maximum keeps fewer than 53
+// bits, one below 2^-57 none, and a result is good to 2^-52 K of its row's times its column's maximum (a
+// row (1, 1e-12) against a column (0, 1): 1e-5 of the result, where multiply-adds are exact).
+// Operands graded against each other along K: as good as multiply-adds over six decades each (1.7e-16 to
+// 2.9e-16 of the result's norm against 3.8e-16), up to 8e-14 over fourteen.  The contractions here
+// meet no such pairs: an environment or an isometry, one factor of each, is level along K.
+// (Groups 0..6 alone, 28 products, leave 2.4e-16 of the norm: more than the split-K CUDA-core product
+// has at K near 128.)
 // Measured against 113-bit sums, bond operator (two chained products), norm-wise: 1.15e-16 here
 // and 3.4e-16 on CUDA cores at 129 x 127, w = 14; 1.4e-16 and 5.2e-16 with rows falling over six
 // decades; 1.25e-16 and 2.3e-15 at 512.

@@ -315,6 +315,30 @@ def test_fp64_digits_site(g, ml, mr):
     assert _rel(Ro.cpu().numpy(), O.env_right_step(R, A, W)) < TOL_DIGITS
 
 
+@pytest.mark.parametrize("decades", [6, 14])
+@pytest.mark.parametrize("ml,mr,w", [(64, 74, 14), (80, 70, 11)])
+def test_fp64_digits_graded_rows(g, ml, mr, w, decades):
+    """Rows and columns whose entries fall over many decades, in unrelated orders.  The digits' error is
+    bounded by the operands' maxima and not by the result: entry by entry an output stays within
+    2^-52 K of its row's and column's maxima (each operand rounded at 2^-55 of its maximum, 2 K real
+    terms per part), for each of the two chained products."""
+    rng = np.random.default_rng(decades)
+    L, R, x = _rand(rng, ml, w, ml), _rand(rng, mr, w, mr), _rand(rng, ml, mr)
+    L *= 10.0 ** -(decades * np.arange(ml) / ml)[None, None, :]
+    x *= 10.0 ** -(decades * rng.permutation(ml) / ml)[:, None]
+    Ld, Rd, xd = _dev(L, R, x)
+    yd = torch.empty_like(xd)
+    g.keff_contract(Ld, Rd, xd, yd)
+    got = yd.cpu().numpy()
+    ld = np.clongdouble
+    t = np.tensordot(L.astype(ld), x.astype(ld), axes=([2], [0]))          # [a, w, b']
+    ref = np.tensordot(t, R.astype(ld), axes=([1, 2], [1, 2]))             # [a, b]
+    top = lambda m, axes: np.max(np.abs(m), axis=axes)
+    dt = 2.0 ** -52 * ml * top(L, 2)[:, :, None] * top(x, 0)[None, None, :]   # error of t
+    bound = np.einsum("awb,cwb->ac", dt, np.abs(R)) + 2.0 ** -52 * w * mr * np.outer(top(t, (1, 2)), top(R, (1, 2)))
+    assert np.all(np.abs(got - ref) <= bound)
+
+
 def test_fp64_digits_ranges_zeros_and_non_finite(g):
     """Rows over hundreds of orders of magnitude keep their relative accuracy, zero rows and
     columns stay exact zeros, a NaN or infinity reaches the outputs it reaches in FP64."""
