@@ -365,8 +365,10 @@ void Engine::apply_op(const SiteOp& op, const cplx* x, cplx* y, int precision) {
 // CUDA-core order up to 2^28 (bond dimension about 500; 2 ms on CUDA cores there, 16 ms and a third
 // of a sweep's moves at 1024, where the digits take 1 ms): its sweeps turn a last-bit change into
 // 1e-7 of a site tensor (operand digits round at 2^-33, and the next gauge move divides by Schmidt
-// values of 1e-6; measured at chi 256), so below that line its trajectories stay those of earlier
-// releases bit by bit.
+// values of 1e-6; measured at chi 256).  Below that line the trajectories of the BF16 forms, whose
+// environments are BF16 products too, stay those of earlier releases bit by bit; above it they differ by
+// such an amount.  TF32X3 keeps FP64 environments, which take the digits by size: its trajectories
+// differ from 4 M multiply-adds on.
 void Engine::gauge_gemm(int opA, int opB, int M, int N, int K, cplx alpha, const cplx* A, long long lda, const cplx* B,
                         long long ldb, cplx beta, cplx* C, long long ldc) {
   if (opt.precision == TDVP_PREC_FP64 || (long long)M * N * K >= (1LL << 28))

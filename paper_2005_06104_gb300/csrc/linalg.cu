@@ -1063,7 +1063,9 @@ void fill_zero(cudaStream_t st, cplx* p, long long n) {
 // the stopping tests of the iterations of one batch run side by side.
 // ============================================================================
 namespace {
-constexpr int PAR_K = 95;  // orders the parallel path keeps vectors for (x up to about 15)
+// Orders the parallel path keeps vectors for.  Its recurrence starts at M < 128 (one quotient per thread),
+// which K = 74 is the last to allow: x below 11.68.  Larger x takes the serial path.
+constexpr int PAR_K = 74;
 
 // T_k(X) e_0 and the coefficients one after the other, by one warp: are, aim of its components
 __device__ __noinline__ void tridiag_serial(int n, int K, double x, double delta, int kind, double c, double h,
