@@ -447,6 +447,11 @@ def roofline_line(args, g, torch, W):
         peak = bf16 * (1.1 / 2.25)  # measured bf16 x nominal tf32/bf16 ratio
         peak_src = "measured bf16_tflops x 1.1/2.25 (nominal tf32/bf16)"
         kern = f"H_eff apply (tcgen05 kind::tf32, 3 split products) at chi={args.heff_chi}, w=14"
+    elif args.heff_chi >= 64:
+        # FP64 by exact 8-bit digits: the measured BF16 peak over the 34 digit products of an FP64 one
+        products, peak = 1, bf16 / 34
+        peak_src = ("measured bf16_tflops (MEASURED_PEAKS.json)" if peaks else "fallback 1900 TF/s bf16") + " / 34"
+        kern = f"H_eff apply (FP64 by exact 8-bit digits, tcgen05 kind::f16, 34 products) at chi={args.heff_chi}, w=14"
     else:
         products, peak, peak_src = 1, 1.097, "cuBLAS DGEMM measured on this part (bench.py --peaks)"
         kern = f"H_eff apply (FP64 CUDA cores) at chi={args.heff_chi}, w=14"
@@ -454,15 +459,14 @@ def roofline_line(args, g, torch, W):
     # chi = 1024, w = 14 in BF16X10; other configurations have no capture
     traffic, traffic_src = None, None
     if args.precision == "bf16x10" and args.heff_chi == 1024:
-        traffic = 5.121e9
+        traffic = 5.120e9
         traffic_src = ("ncu dram__bytes_read.sum + dram__bytes_write.sum over the 5 launches of one cached "
                        "apply (slice x, GEMM 1 with L channel-major, MPO stage, GEMM 3 split 4 ways, split-K "
                        "sum) of these kernels on dense random operands")
     elif args.precision == "bf16x6" and args.heff_chi == 1024:
-        traffic = 2.599e9
-        traffic_src = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the two k_gemm_bf16s<3> launches of one "
-                       "cached apply (1.264 GB GEMM 1, 1.335 GB GEMM 3; 78 % of the apply's device time in the "
-                       "launch list); the slicing, MPO-stage and split-K launches are not in this figure")
+        traffic = 3.772e9
+        traffic_src = ("ncu dram__bytes_read.sum + dram__bytes_write.sum over the 5 launches of one cached apply "
+                       "(of it 1.512 GB GEMM 1, 1.332 GB GEMM 3) of these kernels on dense random operands")
     achieved = pflops / (pms / 1e3) / 1e12
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": traffic, "kernel": kern, "peak_source": peak_src,
@@ -475,7 +479,7 @@ def roofline_line(args, g, torch, W):
 def u1_roofline(dense_roof, u1):
     """The roofline line of the H_eff apply on the U(1) state: achieved = flops over the nonzero
     blocks / measured time; the random dense-operand probe stays as context."""
-    u1_traffic = 2.147e9  # DRAM bytes of one apply on U(1) operands of this shape (ncu, see source)
+    u1_traffic = 2.122e9  # DRAM bytes of one apply on U(1) operands of this shape (ncu, see source)
     achieved = u1["tflops_blocks"]
     products = dense_roof["tensor_flops_per_algorithmic_flop"]
     return {"bound": "tensor", "achieved": achieved, "peak": dense_roof["peak"], "unit": "TFLOP/s",
