@@ -3188,6 +3188,11 @@ __global__ void __launch_bounds__(256)
 // sums.  Q is formed without barriers.  Sums in the order of k_qr_groups: the same bits.
 // The moves of a 24-site state at bond dimension 384 (blocks to 200 x 95): 705 us each by
 // k_qr_groups, 515 with one warp per column, 400 with two.
+// 34 moves of a dense 18-site state (blocks 2 q x q), ms by clusters / by k_qr_groups: q = 16: 4.7 / 7.6, 64: 12.1 /
+// 19.1, 96: 17.6 / 25.7; with kClQ at the kernel's capacity of 16 x 8 = 128 columns, 112: 21.0 / 29.3, 128: 24.6 /
+// 33.4.  So clusters win over their whole range; 96 was the widest block at hand when the line was
+// drawn.  The choice is one per call: a block beyond it sends all to k_qr_groups (480 states, charge-
+// conserving, 24 sites, 46 moves: 38 ms where 128 columns give 29).
 // kClCols columns per CTA, kClTeam warps each; a column is kClU units of 32 rows from row j on,
 // unit u with warp u % kClTeam of its team
 constexpr int kClQ = 96, kClP = 256, kClCols = 8, kClTeam = 2, kClU = kClP / 32, kClUw = kClU / kClTeam;
